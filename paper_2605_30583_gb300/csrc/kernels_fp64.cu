@@ -1,9 +1,11 @@
 // Plain all-FP64 form of the LM + PCGNR solver (the comparison baseline): the same
 // algorithm as the mixed-precision path (Sec. V of arXiv 2605.30583) written the
 // straightforward way -- FP64 everywhere, the Jacobian computed once per
-// linearisation and stored (24 doubles per observation), and one FP64 global atomic
-// per camera entry and observation for every camera-side sum.  Points are owned by
-// one thread each (the point-major index), so point sums need no atomics.
+// linearisation and stored (24 doubles per observation).  A CTA takes a tile: observations
+// in their camera-sorted order a thread (or warp) each, camera sums in registers along a
+// camera's run with one FP64 atomic per entry and run (one per entry and observation, all of a
+// camera's on the same few addresses, bound these kernels before), then a thread per point
+// (the point-major index), so point sums need no atomics.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -93,21 +95,44 @@ __global__ void k64_camera_precompute(V64 v) {
     }
 }
 
-// Linearisation: thread per point over its observations; stores r and J per
-// observation, point sums in registers, camera sums by FP64 atomics.
-__global__ void k64_linearize(V64 v, int mode, double* res_out, double* jac_out, CondHandle lm_cond, int use_cond) {
+// Linearisation, a CTA of TILE_PTS threads per tile.  First a thread per observation: r and J
+// stored.  Then the tile's observations in order, a contiguous part to a warp: lane l holds the
+// entries l and l + 32 of a camera's 54 sums (g and the J_c^T J_c triangle), so every lane works
+// on one observation's row at a time and nothing has to be reduced.  Then a thread per point.
+constexpr int T64 = TILE_PTS;
+
+__global__ void __launch_bounds__(T64) k64_linearize(V64 v, int mode, double* res_out, double* jac_out,
+                                                     CondHandle lm_cond, int use_cond) {
     if (mode == 1 && v.st->relin == 0) return;
     const double eps = v.st->opt.eps;
     // robust loss (evaluation, mode 2, is always the squared loss)
     const int loss = mode == 2 ? 0 : v.st->opt.loss;
     const double lscale = v.st->opt.loss_scale;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the row and column of this lane's two entries; entries below 9 are g (column = residual)
+    int ra[2], ca[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int t = lane + 32 * q;
+        ra[q] = ca[q] = 0;
+        if (t < 9) {
+            ra[q] = t;
+            ca[q] = -1;
+        } else {
+            for (int i = 0; i < 9; ++i)
+                if (t - 9 >= tri_index(9, i, i) && t - 9 < tri_index(9, i, i) + 9 - i) {
+                    ra[q] = i;
+                    ca[q] = i + (t - 9 - tri_index(9, i, i));
+                }
+        }
+    }
     double cost = 0.0;
-    for (int ip = gtid(); ip < v.n_pts; ip += grid_threads()) {
-        const double* X = v.x + v.pt_off + 3 * (size_t)ip;
-        double gp[3] = {0, 0, 0}, hp[6] = {0, 0, 0, 0, 0, 0};
-        for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
-            const uint32_t j = v.obs_pm[k];
-            const uint32_t c = v.obs_key[j] >> 8;
+    for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
+        const uint32_t lo = v.tile_off[tile], n = v.tile_off[tile + 1] - lo;
+        const double* Xt = v.x + v.pt_off + 3 * (size_t)tile * TILE_PTS;
+        for (uint32_t j = lo + threadIdx.x; j < lo + n; j += T64) {
+            const uint32_t key = v.obs_key[j], c = key >> 8;
+            const double* X = Xt + 3 * (key & 0xffu);
             double J[24], r0, r1;
             obs_jacobian64(v.cam64 + (size_t)c * CP_STRIDE, X[0], X[1], X[2], eps, v.obs_uv[2 * (size_t)j],
                            v.obs_uv[2 * (size_t)j + 1], r0, r1, J);
@@ -126,22 +151,49 @@ __global__ void k64_linearize(V64 v, int mode, double* res_out, double* jac_out,
             } else {
                 cost += r0 * r0 + r1 * r1;
             }
-            for (int q = 0; q < 24; ++q) v.jac[24 * (size_t)j + q] = J[q];
-            v.res[2 * (size_t)j] = r0;
-            v.res[2 * (size_t)j + 1] = r1;
-            double* gc = v.cam_lin + (size_t)c * CL_STRIDE;
-            double* hc = v.cam_H64 + (size_t)c * CH_STRIDE;
-            for (int a = 0; a < 9; ++a) {
-                atomicAdd(gc + a, J[a] * r0 + J[12 + a] * r1);
-                for (int b = a; b < 9; ++b) atomicAdd(hc + tri_index(9, a, b), J[a] * J[b] + J[12 + a] * J[12 + b]);
+            double2* Jo = reinterpret_cast<double2*>(v.jac + 24 * (size_t)j);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) Jo[q] = make_double2(J[2 * q], J[2 * q + 1]);
+            reinterpret_cast<double2*>(v.res)[j] = make_double2(r0, r1);
+        }
+        __syncthreads();   // the tile's rows are written
+        const uint32_t chunk = (n + T64 / 32 - 1) / (T64 / 32);
+        const uint32_t a = lo + min(warp * chunk, n), b = lo + min(warp * chunk + chunk, n);
+        double acc[2] = {0.0, 0.0};
+        for (uint32_t j = a; j < b; ++j) {
+            const uint32_t c = v.obs_key[j] >> 8;
+            const double* J = v.jac + 24 * (size_t)j;
+            const double* r = v.res + 2 * (size_t)j;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const double y0 = ca[q] < 0 ? r[0] : J[ca[q]], y1 = ca[q] < 0 ? r[1] : J[12 + ca[q]];
+                acc[q] = fma(J[ra[q]], y0, fma(J[12 + ra[q]], y1, acc[q]));
             }
-            for (int a = 0; a < 3; ++a) {
-                gp[a] += J[9 + a] * r0 + J[21 + a] * r1;
-                for (int b = a; b < 3; ++b) hp[tri_index(3, a, b)] += J[9 + a] * J[9 + b] + J[21 + a] * J[21 + b];
+            if (j + 1 == b || (v.obs_key[j + 1] >> 8) != c) {   // the run ends
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int t = lane + 32 * q;
+                    if (t < 9) atomicAdd(v.cam_lin + (size_t)c * CL_STRIDE + t, acc[q]);
+                    else if (t < 54) atomicAdd(v.cam_H64 + (size_t)c * CH_STRIDE + (t - 9), acc[q]);
+                    acc[q] = 0.0;
+                }
             }
         }
-        for (int a = 0; a < 3; ++a) v.g[v.pt_off + 3 * (size_t)ip + a] = gp[a];
-        for (int a = 0; a < 6; ++a) v.pt_H[(size_t)ip * PH_STRIDE + a] = hp[a];
+        const int ip = tile * TILE_PTS + (int)threadIdx.x;
+        if (ip < v.n_pts) {
+            double gp[3] = {0, 0, 0}, hp[6] = {0, 0, 0, 0, 0, 0};
+            for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
+                const uint32_t j = v.obs_pm[k];
+                const double* J = v.jac + 24 * (size_t)j;
+                const double r0 = v.res[2 * (size_t)j], r1 = v.res[2 * (size_t)j + 1];
+                for (int a = 0; a < 3; ++a) {
+                    gp[a] += J[9 + a] * r0 + J[21 + a] * r1;
+                    for (int b = a; b < 3; ++b) hp[tri_index(3, a, b)] += J[9 + a] * J[9 + b] + J[21 + a] * J[21 + b];
+                }
+            }
+            for (int a = 0; a < 3; ++a) v.g[v.pt_off + 3 * (size_t)ip + a] = gp[a];
+            for (int a = 0; a < 6; ++a) v.pt_H[(size_t)ip * PH_STRIDE + a] = hp[a];
+        }
     }
     double in[1] = {cost}, out[1];
     if (grid_reduce<1>(in, v.partials, &v.st->tickets[TK_LIN], out) && threadIdx.x == 0) {
@@ -273,37 +325,78 @@ __global__ void k64_direction(V64 v, const double* zs, int use_beta, const int32
     if (grid_reduce<1>(in, v.partials, &st->tickets[TK_DIR], out) && threadIdx.x == 0) st->pDp = out[0];
 }
 
-// q += J^T J p with the stored Jacobian: thread per point, t = J_o p per observation,
-// camera part by FP64 atomics, point part in registers.
-__global__ void k64_matvec(V64 v, const int32_t* gate) {
+// q += J^T J p with the stored Jacobian, a CTA per tile: first the tile's observations in
+// order, a contiguous part to a thread: t = J_o p (kept in the residuals' place, which nothing
+// reads after the linearisation) and the camera sums in registers along a run; then a thread per
+// point over its observations' t.
+__global__ void __launch_bounds__(T64) k64_matvec(V64 v, const int32_t* gate) {
     if (gate && *gate == 0) return;
     DevState* st = v.st;
     double jp2 = 0.0;
-    for (int ip = gtid(); ip < v.n_pts; ip += grid_threads()) {
-        const size_t ep = v.pt_off + 3 * (size_t)ip;
-        const double pp0 = v.p[ep], pp1 = v.p[ep + 1], pp2 = v.p[ep + 2];
-        double qp0 = 0.0, qp1 = 0.0, qp2 = 0.0;
-        for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
-            const uint32_t j = v.obs_pm[k];
-            const uint32_t c = v.obs_key[j] >> 8;
-            const double* J = v.jac + 24 * (size_t)j;
-            const double* pc = v.p + 9 * (size_t)c;
-            double t0 = J[9] * pp0 + J[10] * pp1 + J[11] * pp2;
-            double t1 = J[21] * pp0 + J[22] * pp1 + J[23] * pp2;
-            for (int a = 0; a < 9; ++a) {
-                t0 += J[a] * pc[a];
-                t1 += J[12 + a] * pc[a];
+    for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
+        const uint32_t lo = v.tile_off[tile], n = v.tile_off[tile + 1] - lo;
+        const uint32_t chunk = (n + T64 - 1) / T64;
+        const uint32_t a = lo + min(threadIdx.x * chunk, n), b = lo + min(threadIdx.x * chunk + chunk, n);
+        const double* Pt = v.p + v.pt_off + 3 * (size_t)tile * TILE_PTS;
+        double acc[9], pc[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] = pc[k] = 0.0;
+        uint32_t cur = 0xffffffffu;
+        for (uint32_t j = a; j < b; ++j) {
+            const uint32_t key = v.obs_key[j], c = key >> 8;
+            if (c != cur) {
+                if (cur != 0xffffffffu)
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) {
+                        atomicAdd(v.q + 9 * (size_t)cur + k, acc[k]);
+                        acc[k] = 0.0;
+                    }
+                cur = c;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) pc[k] = v.p[9 * (size_t)c + k];
+            }
+            const double2* J2 = reinterpret_cast<const double2*>(v.jac + 24 * (size_t)j);
+            double J[24];
+#pragma unroll
+            for (int q = 0; q < 12; ++q) {
+                const double2 d = J2[q];
+                J[2 * q] = d.x;
+                J[2 * q + 1] = d.y;
+            }
+            const double* pp = Pt + 3 * (key & 0xffu);
+            const double p0 = pp[0], p1 = pp[1], p2 = pp[2];
+            double t0 = J[9] * p0 + J[10] * p1 + J[11] * p2;
+            double t1 = J[21] * p0 + J[22] * p1 + J[23] * p2;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                t0 += J[k] * pc[k];
+                t1 += J[12 + k] * pc[k];
             }
             jp2 += t0 * t0 + t1 * t1;
-            double* qc = v.q + 9 * (size_t)c;
-            for (int a = 0; a < 9; ++a) atomicAdd(qc + a, J[a] * t0 + J[12 + a] * t1);
-            qp0 += J[9] * t0 + J[21] * t1;
-            qp1 += J[10] * t0 + J[22] * t1;
-            qp2 += J[11] * t0 + J[23] * t1;
+            reinterpret_cast<double2*>(v.res)[j] = make_double2(t0, t1);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) acc[k] = fma(J[k], t0, fma(J[12 + k], t1, acc[k]));
         }
-        v.q[ep] += qp0;
-        v.q[ep + 1] += qp1;
-        v.q[ep + 2] += qp2;
+        if (cur != 0xffffffffu)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) atomicAdd(v.q + 9 * (size_t)cur + k, acc[k]);
+        __syncthreads();   // the tile's t
+        const int ip = tile * TILE_PTS + (int)threadIdx.x;
+        if (ip < v.n_pts) {
+            const size_t ep = v.pt_off + 3 * (size_t)ip;
+            double q0 = 0.0, q1 = 0.0, q2 = 0.0;
+            for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
+                const uint32_t j = v.obs_pm[k];
+                const double* J = v.jac + 24 * (size_t)j;
+                const double2 t = reinterpret_cast<const double2*>(v.res)[j];
+                q0 += J[9] * t.x + J[21] * t.y;
+                q1 += J[10] * t.x + J[22] * t.y;
+                q2 += J[11] * t.x + J[23] * t.y;
+            }
+            v.q[ep] += q0;
+            v.q[ep + 1] += q1;
+            v.q[ep + 2] += q2;
+        }
     }
     double in[1] = {jp2}, out[1];
     if (grid_reduce<1>(in, v.partials, &st->tickets[TK_MV], out) && threadIdx.x == 0) {
@@ -329,21 +422,24 @@ __global__ void k64_update(V64 v, CondHandle pcg_cond, int use_cond) {
     double rz = 0.0, rr = 0.0;
     if (active) {
         const double alpha = st->alpha;
-        for (int c = gtid(); c < v.n_cams; c += grid_threads()) {
-            const size_t e = 9 * (size_t)c;
-            double rn[9];
-            for (int k = 0; k < 9; ++k) {
-                v.h[e + k] += alpha * v.p[e + k];
-                rn[k] = v.r[e + k] - alpha * v.q[e + k];
-                v.r[e + k] = rn[k];
-            }
-            const double* M = v.Minv_c + (size_t)c * MC_STRIDE;
-            for (int i = 0; i < 9; ++i) {
-                double z = 0.0;
-                for (int k = 0; k < 9; ++k) z += M[9 * i + k] * rn[k];
-                v.z[e + i] = z;
-                rz += rn[i] * z;
-                rr += rn[i] * rn[i];
+        // cameras: nine lanes each, three to a warp
+        const int lane = threadIdx.x & 31;
+        for (int cw = 3 * (gtid() >> 5); cw < v.n_cams; cw += 3 * (grid_threads() >> 5)) {
+            const int sub = lane / 9, base = 9 * sub;
+            const bool live = lane < 27 && cw + sub < v.n_cams;
+            const int c = live ? cw + sub : cw, i = live ? lane - base : 0;
+            const size_t e = 9 * (size_t)c + i;
+            const double* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * i;
+            const double rn = v.r[e] - alpha * v.q[e];
+            double z = 0.0;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) z += M[k] * __shfl_sync(0xffffffffu, rn, base + k);
+            if (live) {
+                v.h[e] += alpha * v.p[e];
+                v.r[e] = rn;
+                v.z[e] = z;
+                rz += rn * z;
+                rr += rn * rn;
             }
         }
         for (int i = gtid(); i < v.n_pts; i += grid_threads()) {
@@ -418,12 +514,12 @@ __global__ void k64_eval_candidate(V64 v, CondHandle lm_cond, int use_cond) {
     const double lscale = st->opt.loss_scale;
     double fnew = 0.0, jh2 = 0.0;
     if (active) {
-        for (int ip = gtid(); ip < v.n_pts; ip += grid_threads()) {
-            const double* Xn = v.x_new + v.pt_off + 3 * (size_t)ip;
-            const double* hp = v.h + v.pt_off + 3 * (size_t)ip;
-            for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
-                const uint32_t j = v.obs_pm[k];
-                const uint32_t c = v.obs_key[j] >> 8;
+        for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
+            const size_t base = v.pt_off + 3 * (size_t)tile * TILE_PTS;
+            for (uint32_t j = v.tile_off[tile] + threadIdx.x; j < v.tile_off[tile + 1]; j += blockDim.x) {
+                const uint32_t key = v.obs_key[j], c = key >> 8;
+                const double* Xn = v.x_new + base + 3 * (key & 0xffu);
+                const double* hp = v.h + base + 3 * (key & 0xffu);
                 double r0, r1;
                 obs_jacobian64(v.cam64_new + (size_t)c * CP_STRIDE, Xn[0], Xn[1], Xn[2], eps, v.obs_uv[2 * (size_t)j],
                                v.obs_uv[2 * (size_t)j + 1], r0, r1, nullptr);
@@ -561,6 +657,8 @@ inline int g64(const LaunchCfg& L, size_t items) {
     size_t g = (items + L.item_block - 1) / L.item_block;
     return (int)std::max<size_t>(1, std::min<size_t>(g, (size_t)L.item_grid));
 }
+// A CTA per tile, capped by the partial sums' room.
+inline int tiles64(const V64& v) { return std::max(1, std::min(v.n_tiles, MAX_GRID)); }
 }  // namespace
 
 void launch64_camera_precompute(const V64& v, const LaunchCfg& L, cudaStream_t s) {
@@ -568,7 +666,7 @@ void launch64_camera_precompute(const V64& v, const LaunchCfg& L, cudaStream_t s
 }
 void launch64_linearize(const V64& v, const LaunchCfg& L, cudaStream_t s, int mode, double* r, double* J,
                         CondHandle c, int use) {
-    k64_linearize<<<g64(L, v.n_pts), L.item_block, 0, s>>>(v, mode, r, J, c, use);
+    k64_linearize<<<tiles64(v), T64, 0, s>>>(v, mode, r, J, c, use);
 }
 void launch64_precond(const V64& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
     k64_precond<<<g64(L, std::max((size_t)v.n_pts, 32 * (size_t)v.n_cams)), L.item_block, 0, s>>>(v, c, use);
@@ -578,16 +676,16 @@ void launch64_direction(const V64& v, const LaunchCfg& L, cudaStream_t s, const 
     k64_direction<<<g64(L, v.n_vec), L.item_block, 0, s>>>(v, zs, use_beta, gate);
 }
 void launch64_matvec(const V64& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate) {
-    k64_matvec<<<g64(L, v.n_pts), L.item_block, 0, s>>>(v, gate);
+    k64_matvec<<<tiles64(v), T64, 0, s>>>(v, gate);
 }
 void launch64_update(const V64& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
-    k64_update<<<g64(L, std::max(v.n_pts, v.n_cams)), L.item_block, 0, s>>>(v, c, use);
+    k64_update<<<g64(L, std::max((size_t)v.n_pts, 11 * (size_t)v.n_cams)), L.item_block, 0, s>>>(v, c, use);
 }
 void launch64_candidate(const V64& v, const LaunchCfg& L, cudaStream_t s) {
     k64_candidate<<<g64(L, v.n_vec), L.item_block, 0, s>>>(v);
 }
 void launch64_eval_candidate(const V64& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
-    k64_eval_candidate<<<g64(L, v.n_pts), L.item_block, 0, s>>>(v, c, use);
+    k64_eval_candidate<<<tiles64(v), T64, 0, s>>>(v, c, use);
 }
 void launch64_commit(const V64& v, const LaunchCfg& L, cudaStream_t s) {
     k64_commit<<<g64(L, v.n_vec), L.item_block, 0, s>>>(v);
