@@ -31,14 +31,14 @@ __device__ __forceinline__ float warp_sumf(float v) {
 // least blockDim.x / 32 doubles.  Contains __syncthreads.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
     v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     __syncthreads();
     if (lane == 0) sh[w] = v;
     __syncthreads();
     double s = 0.0;
-    if (threadIdx.x == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        for (int i = 0; i < nw; ++i) s += sh[i];
+    if (w == 0) {   // a tree: each FP64 addition costs ~130 cycles of latency
+        s = lane < nw ? sh[lane] : 0.0;
+        for (int o = 1; o < nw; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
     return s;
 }
@@ -77,6 +77,40 @@ __device__ __forceinline__ bool grid_reduce(const double (&v)[NV], double* parti
     return true;
 }
 
+// True in every thread of the last block to come here (a ticket per block, reset by the last);
+// what the other blocks wrote before is then visible.
+__device__ __forceinline__ bool last_block(unsigned int* ticket) {
+    __shared__ bool is_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (is_last) *ticket = 0u;
+    }
+    __syncthreads();
+    if (is_last) __threadfence();
+    return is_last;
+}
+
+// grid_reduce of block sums that thread 0 holds (v in the other threads is not read).
+template <int NV>
+__device__ __forceinline__ bool grid_reduce_block(const double (&v)[NV], double* partials, unsigned int* ticket,
+                                                  double (&out)[NV]) {
+    __shared__ double sh[32];
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) partials[NV * blockIdx.x + k] = v[k];
+    if (!last_block(ticket)) return false;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        double s = 0.0;
+        for (unsigned int b = threadIdx.x; b < gridDim.x; b += blockDim.x) s += __ldcg(&partials[NV * b + k]);
+        s = block_sum(s, sh);
+        if (threadIdx.x == 0) out[k] = s;
+    }
+    return true;
+}
+
 // Slot-spread accumulation: block b adds into slot b % NSLOT.
 __device__ __forceinline__ void slot_add(double* base, int k, double v) {
     atomicAdd(&base[(blockIdx.x % NSLOT) * SLOT_STRIDE + k], v);
@@ -90,18 +124,44 @@ __device__ __forceinline__ double slot_sum_warp(const double* base, int k) {
     return v;
 }
 
-// 1/x in FP64: hardware approximation refined by two Newton-Raphson steps
-// y <- y + y (1 - x y), each roughly doubling the correct bits.  Zero, non-finite and
+// 1/x in FP64: hardware approximation (over 18 bits) refined by one third-order step
+// y <- y + y (e + e^2), e = 1 - x y, which triples the correct bits in three dependent FP64
+// operations (an FP64 operation has ~130 cycles of latency on this GPU; two Newton-Raphson
+// steps take four).  Zero, non-finite and
 // |x| outside [1e-300, 1e300] (where x y or the approximation could leave the normal
 // range, flushing or overflowing before the refinement) take the IEEE quotient.
-__device__ __forceinline__ double rcp64(double x) {
-    const double ax = fabs(x);
-    if (!(ax >= 1e-300 && ax <= 1e300)) return 1.0 / x;
+__device__ __forceinline__ double rcp64_fast(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    y = fma(y, fma(-x, y, 1.0), y);
-    return y;
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+__device__ __forceinline__ double rcp64(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;   // the range test on the high word
+    if (h - 0x01a56e20u > 0x7e37e43bu - 0x01a56e20u) return 1.0 / x;
+    return rcp64_fast(x);
+}
+
+// float -> double and double -> float (round to nearest even) with integer instructions.  The
+// conversion instruction goes through the FP64 pipe, which a warp instruction holds for 16
+// cycles on this GPU; these take 5 and ~12 full-rate instructions.  Zero and normal values of
+// the target are exact; subnormal, infinite and NaN operands or results take the instruction.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;   // subnormal, inf, NaN
+    const uint32_t hi = m ? (b & 0x80000000u) | ((m >> 3) + 0x38000000u) : b;
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e - 897u >= 254u) return (float)x;   // zero, outside the normal floats, inf, NaN
+    const uint32_t m = ((hi & 0x7fffffffu) - 0x38000000u) << 3 | lo >> 29;   // exponent and mantissa, truncated
+    const uint32_t rest = lo << 3;                                            // the bits cut off, from the top
+    const uint32_t up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (m + up));
 }
 
 // Kahan's compensated summation (W. Kahan, "Further remarks on reducing truncation
@@ -139,24 +199,45 @@ __device__ __forceinline__ double warp_sum_pair(float hi, float lo) {
     return (double)hi + (double)lo;
 }
 
+// Compensated warp sum of per-lane values hi + lo as a pair (warp_sum_pair without its FP64
+// finish), valid in lane 0.
+__device__ __forceinline__ float2 warp_pair(float hi, float lo) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_down_sync(0xffffffffu, hi, o);
+        const float l2 = __shfl_down_sync(0xffffffffu, lo, o);
+        float s, e;
+        two_sum(hi, h2, s, e);
+        hi = s;
+        lo = lo + l2 + e;
+    }
+    return make_float2(hi, lo);
+}
+
 // Block sums of two compensated per-thread partials (Kahan pairs s - c): compensated
-// FP32 pairs inside each warp, FP64 across warps.  Results valid in thread 0.  `sh`
-// holds 2 * (blockDim.x / 32) doubles.  Contains __syncthreads.
+// FP32 pairs inside each warp, FP64 across warps (in the first warp alone: FP64 work that
+// every warp repeats costs 16 cycles of the SM's FP64 pipe per instruction).  Results valid in
+// thread 0.  `sh` holds 2 * (blockDim.x / 32) doubles.  Contains __syncthreads.
 __device__ __forceinline__ void block_sum2c(float sa, float ca, float sb, float cb, double* sh, double& ra,
                                             double& rb) {
-    const double a = warp_sum_pair(sa, -ca), b = warp_sum_pair(sb, -cb);
+    const float2 a = warp_pair(sa, -ca), b = warp_pair(sb, -cb);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    float2* sp = reinterpret_cast<float2*>(sh);
     __syncthreads();
     if (lane == 0) {
-        sh[w] = a;
-        sh[nw + w] = b;
+        sp[w] = a;
+        sp[nw + w] = b;
     }
     __syncthreads();
     ra = rb = 0.0;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < nw; ++i) {
-            ra += sh[i];
-            rb += sh[nw + i];
+    if (w == 0) {
+        if (lane < nw) {
+            ra = widen(sp[lane].x) + widen(sp[lane].y);
+            rb = widen(sp[nw + lane].x) + widen(sp[nw + lane].y);
+        }
+        for (int o = 1; o < nw; o <<= 1) {
+            ra += __shfl_xor_sync(0xffffffffu, ra, o);
+            rb += __shfl_xor_sync(0xffffffffu, rb, o);
         }
     }
 }
@@ -203,58 +284,62 @@ __device__ __forceinline__ void rodrigues_coeffs(double th2, double& A, double& 
         C = 1.0 / 6.0 + th2 * (-1.0 / 120.0 + th2 * (1.0 / 5040.0 + th2 * (-1.0 / 362880.0)));
     } else {
         const double th = sqrt(th2);
-        double s, c, sh, ch;
-        sincos(th, &s, &c);
+        double sh, ch;
         sincos(0.5 * th, &sh, &ch);
-        A = s / th;
-        B = 2.0 * sh * sh / th2;
-        C = (th - s) / (th2 * th);
+        const double s = 2.0 * sh * ch, i = rcp64(th);   // sin(th); FP64 divisions are slow here
+        A = s * i;
+        B = 2.0 * (sh * i) * (sh * i);
+        C = (th - s) * i * i * i;
     }
 }
 
-// Writes one camera record (layout.h, CamPre) from 9 parameters (w, t, f, k1, k2):
-// R(w) = I + A [w]x + B [w]x^2 and J_l(w) = I + B [w]x + C [w]x^2, where J_l is the
-// left Jacobian of the rotation exponential: R(w + d) = Exp(J_l(w) d) R(w) + O(|d|^2),
-// so d(R(w) X)/dw . d = (J_l d) x (R X).
+// Writes rows [row0, row1) of one camera record (layout.h, CamPre) from 9 parameters
+// (w, t, f, k1, k2): R(w) = I + A [w]x + B [w]x^2 and J_l(w) = I + B [w]x + C [w]x^2, where J_l
+// is the left Jacobian of the rotation exponential: R(w + d) = Exp(J_l(w) d) R(w) + O(|d|^2),
+// so d(R(w) X)/dw . d = (J_l d) x (R X).  Row i also writes entry i of t and of (f, k1, k2): three
+// lanes share a camera, since the record is one long chain of FP64 operations (~130 cycles of
+// latency each, 64 of a scheduler's FP64 pipe).
 // With `retract` the record is for the tangent-space update R <- Exp(d) R(w): the
 // rotation Jacobian is then taken w.r.t. d at d = 0, i.e. J_l is replaced by I.
 // `lo` (optional, CLO_STRIDE floats): the FP32 rounding error of R, t, f, k1, k2 at the
 // same offsets as in `out`, so out + lo carries them to ~2^-48 (double-float values).
-__device__ __forceinline__ void camera_record(const double* c, float* out, bool retract = false,
-                                              float* lo = nullptr) {
+__device__ __forceinline__ void camera_record_rows(const double* c, float* out, bool retract, float* lo, int row0,
+                                                   int row1) {
     const double w0 = c[0], w1 = c[1], w2 = c[2];
     const double th2 = w0 * w0 + w1 * w1 + w2 * w2;
     double A, B, C;
     rodrigues_coeffs(th2, A, B, C);
-    // [w]x and [w]x^2 = w w^T - th2 I
-    const double K[9] = {0.0, -w2, w1, w2, 0.0, -w0, -w1, w0, 0.0};
-    const double K2[9] = {w0 * w0 - th2, w0 * w1, w0 * w2,
-                          w1 * w0, w1 * w1 - th2, w1 * w2,
-                          w2 * w0, w2 * w1, w2 * w2 - th2};
+    for (int i = row0; i < row1; ++i) {
+        // row i of [w]x and of [w]x^2 = w w^T - th2 I
+        const double wi = i == 0 ? w0 : (i == 1 ? w1 : w2);
+        const double K[3] = {i == 0 ? 0.0 : (i == 1 ? w2 : -w1), i == 0 ? -w2 : (i == 1 ? 0.0 : w0),
+                             i == 0 ? w1 : (i == 1 ? -w0 : 0.0)};
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const double I = (i % 4 == 0) ? 1.0 : 0.0;
-        out[CP_R + i] = (float)(I + A * K[i] + B * K2[i]);
-        out[CP_JL + i] = retract ? (float)I : (float)(I + B * K[i] + C * K2[i]);
-    }
-    out[CP_T + 0] = (float)c[3];
-    out[CP_T + 1] = (float)c[4];
-    out[CP_T + 2] = (float)c[5];
-    out[CP_F] = (float)c[6];
-    out[CP_K1] = (float)c[7];
-    out[CP_K2] = (float)c[8];
-    out[CP_PAD] = 0.0f;
-    if (lo) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const double I = (i % 4 == 0) ? 1.0 : 0.0;
-            const double r = I + A * K[i] + B * K2[i];
-            lo[CP_R + i] = (float)(r - (double)(float)r);
+        for (int j = 0; j < 3; ++j) {
+            const double I = i == j ? 1.0 : 0.0;
+            const double K2 = wi * (j == 0 ? w0 : (j == 1 ? w1 : w2)) - (i == j ? th2 : 0.0);
+            const double r = I + A * K[j] + B * K2;
+            const float rf = narrow(r);
+            out[CP_R + 3 * i + j] = rf;
+            if (lo) lo[CP_R + 3 * i + j] = narrow(r - widen(rf));
+            out[CP_JL + 3 * i + j] = retract ? (float)I : narrow(I + B * K[j] + C * K2);
         }
 #pragma unroll
-        for (int i = 0; i < 6; ++i) lo[CP_T + i] = (float)(c[3 + i] - (double)(float)c[3 + i]);
-        lo[CP_PAD] = 0.0f;
+        for (int k = 0; k < 6; k += 3) {   // t_i, then f, k1 or k2
+            const double d = c[3 + k + i];
+            const float df = narrow(d);
+            out[CP_T + k + i] = df;
+            if (lo) lo[CP_T + k + i] = narrow(d - widen(df));
+        }
     }
+    if (row0 == 0) {
+        out[CP_PAD] = 0.0f;
+        if (lo) lo[CP_PAD] = 0.0f;
+    }
+}
+
+__device__ __forceinline__ void camera_record(const double* c, float* out, bool retract = false, float* lo = nullptr) {
+    camera_record_rows(c, out, retract, lo, 0, 3);
 }
 
 // Unit quaternion (q0; q1 q2 q3) of the rotation vector v: (cos(t/2); sin(t/2) v / t),
@@ -391,14 +476,16 @@ __device__ __forceinline__ Geo project_geo(const Cam& c, float X0, float X1, flo
 // Inverse of one camera block, one warp per camera: lane j < 18 holds column j of
 // the augmented matrix [A | I] (A = H + mu D, 9 x 9, SPD) and Gauss-Jordan elimination
 // without pivoting runs over the 9 pivots in FP64.  Lanes 9..17 end with the columns
-// of A^-1.  Returns false (in every lane) if a pivot is not positive.
+// of A^-1.  Returns false (in every lane) if a pivot is not within [1e-300, 1e300].
 __device__ __forceinline__ bool warp_block_inverse9(double (&col)[9], int lane) {
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const double piv = __shfl_sync(0xffffffffu, col[k], k);
-        ok = ok && (piv > 0.0) && isfinite(piv);
-        const double ip = rcp64(piv > 0.0 ? piv : 1.0);
+        // positive, finite and within rcp64's range, from the high word: an integer test stays off
+        // the chain of FP64 operations (~130 cycles each)
+        ok = ok && (uint32_t)__double2hiint(piv) - 0x01a56e20u <= 0x7e37e43bu - 0x01a56e20u;
+        const double ip = rcp64_fast(piv);
         const double rk = col[k] * ip;   // row k of the updated matrix, this lane's column
 #pragma unroll
         for (int i = 0; i < 9; ++i) {

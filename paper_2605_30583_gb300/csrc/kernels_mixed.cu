@@ -29,18 +29,22 @@ namespace gbba {
 // ------------------------------------------------------------------ K0 --------
 // Camera records from the current parameters (their FP64 master copy); zeroes the
 // linearisation sums.
+// Three lanes a camera (camera_record_rows), ten cameras a warp.
+constexpr int ROW_CAMS = 10;
+
 __global__ void k_camera_precompute(Views<float> v) {
-    for (int c = 32 * (int)blockIdx.x + (int)threadIdx.x; threadIdx.x < 32 && c < v.n_cams; c += 32 * (int)gridDim.x) {
+    const int row = (int)threadIdx.x % 3;
+    for (int c = ROW_CAMS * (int)blockIdx.x + (int)threadIdx.x / 3; threadIdx.x < 3 * ROW_CAMS && c < v.n_cams;
+         c += ROW_CAMS * (int)gridDim.x) {
         double p[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) p[k] = v.xm[9 * (size_t)c + k];
-        camera_record(p, v.cam_pre + (size_t)c * CP_STRIDE, v.st->opt.retract != 0, v.cam_lo + (size_t)c * CLO_STRIDE);
+        camera_record_rows(p, v.cam_pre + (size_t)c * CP_STRIDE, v.st->opt.retract != 0,
+                           v.cam_lo + (size_t)c * CLO_STRIDE, row, row + 1);
         double* cl = v.cam_lin + (size_t)c * CL_STRIDE;
-#pragma unroll
-        for (int k = 0; k < CL_STRIDE; ++k) cl[k] = 0.0;
+        for (int k = row; k < CL_STRIDE; k += 3) cl[k] = 0.0;
         float* ch = v.cam_H + (size_t)c * CH_STRIDE;
-#pragma unroll
-        for (int k = 0; k < CH_STRIDE; ++k) ch[k] = 0.0f;
+        for (int k = row; k < CH_STRIDE; k += 3) ch[k] = 0.0f;
     }
 }
 
@@ -80,7 +84,6 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
     // robust loss (evaluation, mode 2, is always the squared loss)
     const int loss = mode == 2 ? 0 : v.st->opt.loss;
     const float lscale = (float)v.st->opt.loss_scale;
-    float cost = 0.0f, costc = 0.0f;   // Kahan pair
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
         const int pt0 = tile * TILE_PTS;
@@ -153,11 +156,9 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
                         for (int q = 0; q < 3; ++q) { Jo[9 + q] = jx0[q]; Jo[21 + q] = jx1[q]; }
                     }
                 }
-                const float s2 = fmaf(r0, r0, r1 * r1);
                 if (loss) {   // IRLS weight w = rho'(|r|^2): rows scaled by sqrt(w)
-                    const float w = loss_weight(s2, loss, lscale);
+                    const float w = loss_weight(fmaf(r0, r0, r1 * r1), loss, lscale);
                     if (mode != 2) v.obs_w[j] = w;
-                    kahan_add(cost, costc, loss_rho(s2, loss, lscale));
                     const float sw = sqrtf(w);
                     r0 *= sw;
                     r1 *= sw;
@@ -165,8 +166,6 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
                     for (int k = 0; k < 9; ++k) { j0[k] *= sw; j1[k] *= sw; }
 #pragma unroll
                     for (int q = 0; q < 3; ++q) { jx0[q] *= sw; jx1[q] *= sw; }
-                } else {
-                    kahan_add(cost, costc, s2);
                 }
 #pragma unroll
                 for (int i = 0; i < 9; ++i) acc[CL_G + i] = fmaf(j0[i], r0, fmaf(j1[i], r1, acc[CL_G + i]));
@@ -199,12 +198,10 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
             for (int q = 0; q < PH_STRIDE; ++q) v.pt_H[(size_t)(pt0 + i) * PH_STRIDE + q] = sh[6 * i + q];
         }
     }
-    double in[1] = {(double)cost - (double)costc}, out[1];
-    if (grid_reduce<1>(in, v.partials, &v.st->tickets[TK_LIN], out) && threadIdx.x == 0) {
+    if (last_block(&v.st->tickets[TK_LIN]) && threadIdx.x == 0) {
         DevState* st = v.st;
         // the cost is the residual pass's (k_residual, at these parameters); pose factors:
         // k_factor_linearize.  After an accepted step the LM decision has already set F.
-        (void)out;
         const double F = st->F_res + (v.n_fac > 0 ? st->fac_cost : 0.0);
         st->cost_out = F;
         if (mode == 0) {
@@ -393,7 +390,8 @@ __global__ void k_cam_direction(Views<float> v, const int32_t* gate, const float
         }
         v.cam_dir[(size_t)c * CD_STRIDE + k] = d;   // CD_PHI = 0, CD_T = 3, CD_I = 6
     }
-    const double bp = block_sum((double)pdp - (double)pdpc, red);
+    double bp, none;
+    block_sum2c(pdp, pdpc, 0.0f, 0.0f, red, bp, none);
     if (threadIdx.x == 0) slot_add(st->acc_mv, 1, bp);
 }
 
@@ -737,7 +735,7 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
     const int active = st->lm_active;
     const float eps = (float)st->opt.eps;
     const int loss = st->opt.loss;
-    double jh2 = 0.0;
+    float jc = 0.0f, jcc = 0.0f;   // Kahan pair
     if (active) {
         for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
             const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
@@ -748,7 +746,6 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
             uint32_t cur = NO_CAM;
             Cam co;
             float dir[9];
-            float jc = 0.0f, jcc = 0.0f;   // Kahan pair
             for (uint32_t j = a; j < b; ++j) {
                 const uint32_t key = __ldg(v.obs_key + j);
                 const uint32_t c = key >> 8, slot = key & 0xffu;
@@ -764,11 +761,12 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
                 // |J h|^2 weighted at x (F' comes from k_residual)
                 kahan_add(jc, jcc, (loss ? __ldg(v.obs_w + j) : 1.0f) * fmaf(t0, t0, t1 * t1));
             }
-            jh2 += (double)jc - (double)jcc;
         }
     }
-    double in[1] = {jh2}, out[1];
-    if (grid_reduce<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {
+    __shared__ double red[64];
+    double in[1], out[1], none;
+    block_sum2c(jc, jcc, 0.0f, 0.0f, red, in[0], none);
+    if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {
         // pose factors: k_factor_eval ran just before
         const bool fac = v.n_fac > 0;
         lm_decide(st, active, st->F_res + (fac ? st->fac_cost_new : 0.0), out[0] + (fac ? st->fac_jh2 : 0.0));
@@ -1151,6 +1149,10 @@ inline int grid_items(const LaunchCfg& L, int items) {
     return g < 1 ? 1 : (g > L.item_grid ? L.item_grid : g);
 }
 inline int grid_tiles(int cap, int n_tiles) { return n_tiles < 1 ? 1 : (n_tiles > cap ? cap : n_tiles); }
+// Blocks for a kernel with three lanes a camera, one warp of ROW_CAMS cameras per block.
+inline int grid_rows(const LaunchCfg& L, int n_cams) {
+    return std::max(1, std::min((n_cams + ROW_CAMS - 1) / ROW_CAMS, L.item_grid));
+}
 // Blocks for a camera-only kernel: one warp of 32 cameras per block (FOR_CAMERAS).
 inline int grid_cams(const LaunchCfg& L, int n_cams) {
     const int g = (n_cams + 31) / 32;
@@ -1159,7 +1161,7 @@ inline int grid_cams(const LaunchCfg& L, int n_cams) {
 }  // namespace
 
 void launch_camera_precompute(const Views<float>& v, const LaunchCfg& L, cudaStream_t s) {
-    k_camera_precompute<<<grid_cams(L, v.n_cams), 32, 0, s>>>(v);
+    k_camera_precompute<<<grid_rows(L, v.n_cams), 32, 0, s>>>(v);
 }
 void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode,
                       float* res_out, float* jac_out, CondHandle lm_cond, int use_cond) {

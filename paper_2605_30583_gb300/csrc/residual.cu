@@ -22,8 +22,8 @@
 #include <algorithm>
 
 #include "device_common.cuh"
-#include "df.cuh"
 #include "kernels.h"
+#include "residual.cuh"
 
 namespace gbba {
 namespace {
@@ -31,67 +31,17 @@ namespace {
 constexpr int RS_TB = 256;
 
 template <int TB>
-__global__ void __launch_bounds__(TB) k_residual(Views<float> v, int at_candidate, int squared) {
+__global__ void __launch_bounds__(TB, 5) k_residual(Views<float> v, int at_candidate, int squared) {
     DevState* st = v.st;
     // a candidate is only evaluated while LM runs (the decision kernel reads F' then)
     if (at_candidate && st->lm_active == 0) return;
-    __shared__ float4 sXh[TILE_PTS], sXl[TILE_PTS];   // the tile's points, double-float
-    const double* xm = at_candidate ? v.xm_new : v.xm;
-    const float* rec = at_candidate ? v.cam_pre_new : v.cam_pre;
-    const float* lor = at_candidate ? v.cam_lo_new : v.cam_lo;
-    const float eps = (float)st->opt.eps;
-    const int loss = squared ? 0 : st->opt.loss;
-    const float lscale = (float)st->opt.loss_scale;
-    const bool dfp = st->opt.res_df != 0;
-    // the cost: Kahan pair of the high parts of |r|^2 (double-float |r|^2 before any
-    // rounding, so F resolves steps far below an FP32 ulp of the residuals) and the sum
-    // of their low parts
-    float cs = 0.0f, cc = 0.0f, cl = 0.0f;
-    for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
-        const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
-        const size_t base = v.pt_off + 3 * (size_t)pt0;
-        for (int i = threadIdx.x; i < npt; i += TB) {
-            const DF a = df_from_double(xm[base + 3 * i]), b = df_from_double(xm[base + 3 * i + 1]),
-                     c = df_from_double(xm[base + 3 * i + 2]);
-            sXh[i] = make_float4(a.hi, b.hi, c.hi, 0.0f);
-            sXl[i] = make_float4(a.lo, b.lo, c.lo, 0.0f);
-        }
-        __syncthreads();
-        for (uint32_t j = lo + threadIdx.x; j < hi; j += TB) {
-            const uint32_t key = __ldg(v.obs_key + j);
-            const uint32_t c = key >> 8, slot = key & 0xffu;
-            const float2 uv = __ldg(reinterpret_cast<const float2*>(v.obs_uv) + j);
-            const float4 xh = sXh[slot];
-            float r0, r1;
-            DF s2 = {0.0f, 0.0f};
-            if (dfp) {
-                const float4 xl = sXl[slot];
-                const CamDF cam = load_cam_df(rec + (size_t)c * CP_STRIDE, lor + (size_t)c * CLO_STRIDE);
-                const DF X[3] = {{xh.x, xl.x}, {xh.y, xl.y}, {xh.z, xl.z}};
-                DF d0, d1;
-                residual_df(cam, X, eps, uv.x, uv.y, d0, d1);
-                r0 = df_to_float(d0);
-                r1 = df_to_float(d1);
-                s2 = df_add(df_mul(d0, d0), df_mul(d1, d1));
-            } else {
-                const Cam cam = load_cam(rec + (size_t)c * CP_STRIDE);
-                project_residual(cam, xh.x, xh.y, xh.z, eps, uv.x, uv.y, r0, r1);
-                s2.hi = fmaf(r0, r0, r1 * r1);
-            }
-            reinterpret_cast<float2*>(v.rbuf)[j] = make_float2(r0, r1);
-            if (loss) {   // robust loss: rho of the FP32-rounded |r|^2
-                kahan_add(cs, cc, loss_rho(df_to_float(s2), loss, lscale));
-            } else {
-                kahan_add(cs, cc, s2.hi);
-                cl += s2.lo;
-            }
-        }
-        __syncthreads();   // the next tile's staging overwrites the points
-    }
-    double in[1] = {(double)cs - (double)cc + (double)cl}, out[1];
-    if (grid_reduce<1>(in, v.partials, &st->tickets[TK_RES], out) && threadIdx.x == 0) st->F_res = 0.5 * out[0];
+    __shared__ float4 sXh[TILE_PTS], sXl[TILE_PTS];
+    float cs = 0.0f, cc = 0.0f;
+    residual_tiles<TB>(v, at_candidate, squared, blockIdx.x, gridDim.x, sXh, sXl, cs, cc);
+    __shared__ double red[2 * (TB / 32)];
+    double in[1], out[1], none;
+    block_sum2c(cs, cc, 0.0f, 0.0f, red, in[0], none);
+    if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_RES], out) && threadIdx.x == 0) st->F_res = 0.5 * out[0];
 }
 
 }  // namespace

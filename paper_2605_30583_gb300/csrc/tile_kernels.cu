@@ -576,12 +576,12 @@ __device__ __forceinline__ LinObs lin_obs(const Cam& cam, const float (&JL)[9], 
     return o;
 }
 
-// Everything one observation adds: evaluation outputs (mode 2), the IRLS weight, the cost,
+// Everything one observation adds: evaluation outputs (mode 2), the IRLS weight,
 // the camera sums (registers) and the point sums (shared memory).
 template <bool PLAIN = false>
 __device__ __forceinline__ void lin_accumulate(const Views<float>& v, LinObs& o, uint32_t j, uint32_t slot, int mode,
                                                int loss, float lscale, float* res_out, float* jac_out,
-                                               float (&acc)[TL_ACC], float* sG, float* sH, float& cs, float& cc) {
+                                               float (&acc)[TL_ACC], float* sG, float* sH) {
     if (mode == 2) {   // evaluation output: the unweighted residual and Jacobian
         const uint32_t u = v.obs_user[j];
         if (res_out) { res_out[2 * (size_t)u] = o.r0; res_out[2 * (size_t)u + 1] = o.r1; }
@@ -593,11 +593,9 @@ __device__ __forceinline__ void lin_accumulate(const Views<float>& v, LinObs& o,
             for (int q = 0; q < 3; ++q) { Jo[9 + q] = o.jx0[q]; Jo[21 + q] = o.jx1[q]; }
         }
     }
-    const float s2 = fmaf(o.r0, o.r0, o.r1 * o.r1);
     if (loss) {   // IRLS weight w = rho'(|r|^2): rows scaled by sqrt(w)
-        const float w = loss_weight(s2, loss, lscale);
+        const float w = loss_weight(fmaf(o.r0, o.r0, o.r1 * o.r1), loss, lscale);
         if (mode != 2) v.obs_w[j] = w;
-        kahan_add(cs, cc, loss_rho(s2, loss, lscale));
         const float sw = sqrtf(w);
         o.r0 *= sw;
         o.r1 *= sw;
@@ -605,8 +603,6 @@ __device__ __forceinline__ void lin_accumulate(const Views<float>& v, LinObs& o,
         for (int k = 0; k < 9; ++k) { o.j0[k] *= sw; o.j1[k] *= sw; }
 #pragma unroll
         for (int q = 0; q < 3; ++q) { o.jx0[q] *= sw; o.jx1[q] *= sw; }
-    } else {
-        kahan_add(cs, cc, s2);
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) acc[i] = fmaf(o.j0[i], o.r0, fmaf(o.j1[i], o.r1, acc[i]));
@@ -676,7 +672,6 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
     const int loss = mode == 2 ? 0 : v.st->opt.loss;
     const float lscale = (float)v.st->opt.loss_scale;
     const int lane = threadIdx.x & 31;
-    float cs = 0.0f, cc = 0.0f;   // compensated cost
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const TileRange T = tile_range(v, tile);
         for (int i = threadIdx.x; i < T.npt; i += TB)
@@ -706,7 +701,7 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
                 const uint32_t i = start + off, j = T.lo + i;
                 const uint32_t slot = sSlot[i];
                 LinObs o = lin_obs(cam, JL, sX4[slot], __ldg(rbuf + j), eps);
-                lin_accumulate<PLAIN>(v, o, j, slot, mode, loss, lscale, res_out, jac_out, acc, sGw, sHw, cs, cc);
+                lin_accumulate<PLAIN>(v, o, j, slot, mode, loss, lscale, res_out, jac_out, acc, sGw, sHw);
             }
             if (PLAIN) __syncwarp();   // the warp's next run may meet the same points
             int idx;
@@ -741,7 +736,7 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
                     load_jl(v.cam_pre + (size_t)c * CP_STRIDE, JL);
                 }
                 LinObs o = lin_obs(cam, JL, sX4[slot], __ldg(rbuf + j), eps);
-                lin_accumulate(v, o, j, slot, mode, loss, lscale, res_out, jac_out, acc, sGw, sHw, cs, cc);
+                lin_accumulate(v, o, j, slot, mode, loss, lscale, res_out, jac_out, acc, sGw, sHw);
             }
             if (cur != NO_CAM) flush_lin_global(v, cur, acc);
         }
@@ -760,12 +755,10 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
         }
         __syncthreads();   // the next tile's staging overwrites the shared sums
     }
-    double in[1] = {(double)cs - (double)cc}, out[1];
-    if (grid_reduce<1>(in, v.partials, &v.st->tickets[TK_LIN], out) && threadIdx.x == 0) {
+    if (last_block(&v.st->tickets[TK_LIN]) && threadIdx.x == 0) {
         DevState* st = v.st;
         // the cost is the residual pass's (k_residual, at these parameters); pose factors:
         // k_factor_linearize.  After an accepted step the LM decision has already set F.
-        (void)out;
         const double F = st->F_res + (v.n_fac > 0 ? st->fac_cost : 0.0);
         st->cost_out = F;
         if (mode == 0) {
