@@ -147,14 +147,8 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
                 }
                 if (mode == 2) {   // evaluation output: the unweighted residual and Jacobian
                     const uint32_t o = v.obs_user[j];
-                    if (res_out) { res_out[2 * (size_t)o] = r0; res_out[2 * (size_t)o + 1] = r1; }
-                    if (jac_out) {
-                        float* Jo = jac_out + 24 * (size_t)o;
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) { Jo[k] = j0[k]; Jo[12 + k] = j1[k]; }
-#pragma unroll
-                        for (int q = 0; q < 3; ++q) { Jo[9 + q] = jx0[q]; Jo[21 + q] = jx1[q]; }
-                    }
+                    if (res_out) store_residual(res_out + 2 * (size_t)o, r0, r1);
+                    if (jac_out) store_jacobian(jac_out + 24 * (size_t)o, j0, jx0, j1, jx1);
                 }
                 if (loss) {   // IRLS weight w = rho'(|r|^2): rows scaled by sqrt(w)
                     const float w = loss_weight(fmaf(r0, r0, r1 * r1), loss, lscale);

@@ -101,6 +101,77 @@ __device__ __forceinline__ void jdir(const Geo& g, const Cam& c, const float (&d
     t1 = fmaf(g.A[3], dP0, fmaf(g.A[4], dP1, fmaf(g.A[5], dP2, ci * g.p[1])));
 }
 
+// One observation's 2 x 12 Jacobian (camera columns, then point columns; 96 bytes) to `out`:
+// six 16-byte stores when the address allows, since the rows of neighbouring lanes go to
+// unrelated places and each store instruction costs a transaction per lane.
+__device__ __forceinline__ void store_jacobian(float* out, const float (&j0)[9], const float (&jx0)[3],
+                                               const float (&j1)[9], const float (&jx1)[3]) {
+    if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+        float4* o = reinterpret_cast<float4*>(out);
+        o[0] = make_float4(j0[0], j0[1], j0[2], j0[3]);
+        o[1] = make_float4(j0[4], j0[5], j0[6], j0[7]);
+        o[2] = make_float4(j0[8], jx0[0], jx0[1], jx0[2]);
+        o[3] = make_float4(j1[0], j1[1], j1[2], j1[3]);
+        o[4] = make_float4(j1[4], j1[5], j1[6], j1[7]);
+        o[5] = make_float4(j1[8], jx1[0], jx1[1], jx1[2]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) { out[k] = j0[k]; out[12 + k] = j1[k]; }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) { out[9 + q] = jx0[q]; out[21 + q] = jx1[q]; }
+    }
+}
+
+__device__ __forceinline__ void store_residual(float* out, float r0, float r1) {
+    if ((reinterpret_cast<uintptr_t>(out) & 7u) == 0) {
+        *reinterpret_cast<float2*>(out) = make_float2(r0, r1);
+    } else {
+        out[0] = r0;
+        out[1] = r1;
+    }
+}
+
+// Block-Jacobi inverse of one point block H + mu D (H packed xx, xy, xz, yy, yz, zz; D its
+// diagonal clamped to [lo, hi]) in FP64 by the adjugate, M = adj(A) / det(A); the inverse of
+// the diagonal where A is not positive definite.  lo_f, hi_f: the bounds as floats on the inner
+// side, so that h >= lo exactly when h >= lo_f.  Writes M (packed) and D in FP32.  FP64 runs
+// at 1/64 of the FP32 rate here (a warp instruction holds the SM's FP64 pipe for 16 cycles):
+// only the 29 instructions of the inverse itself are FP64; clamping, comparisons and
+// conversions run on the integer and FP32 units (the 28.8M-observation workload's
+// preconditioner took 688 us with them in FP64).
+__device__ __forceinline__ void point_inverse(const float (&H)[6], double mu, double lo, double hi, float lo_f,
+                                              float hi_f, float (&m)[6], float (&D)[3]) {
+    const float hd[3] = {H[0], H[3], H[5]};
+    double a[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        a[k] = widen(hd[k]);
+        D[k] = hd[k];
+        double d = a[k];
+        if (!(hd[k] >= lo_f && hd[k] <= hi_f)) {   // clamped
+            d = fmin(fmax(a[k], lo), hi);
+            D[k] = (float)d;
+        }
+        a[k] = fma(mu, d, a[k]);
+    }
+    const double a00 = a[0], a11 = a[1], a22 = a[2], a01 = widen(H[1]), a02 = widen(H[2]), a12 = widen(H[4]);
+    const double c00 = fma(a11, a22, -(a12 * a12)), c01 = fma(a02, a12, -(a01 * a22));
+    const double c02 = fma(a01, a12, -(a02 * a11)), c11 = fma(a00, a22, -(a02 * a02));
+    const double c12 = fma(a01, a02, -(a00 * a12)), c22 = fma(a00, a11, -(a01 * a01));
+    const double det = fma(a00, c00, fma(a01, c01, a02 * c02));
+    // positive and finite, from the high words (those of infinities and NaN are above)
+    const int dh = __double2hiint(det);
+    if (dh > 0 && dh < 0x7ff00000 && __double2hiint(a00) > 0 && __double2hiint(c22) > 0) {
+        const double id = rcp64(det);
+        m[0] = narrow(c00 * id); m[1] = narrow(c01 * id); m[2] = narrow(c02 * id);
+        m[3] = narrow(c11 * id); m[4] = narrow(c12 * id); m[5] = narrow(c22 * id);
+    } else {   // not SPD in FP64: inverse diagonal
+        m[0] = a00 > 0 ? (float)(1.0 / a00) : 0.0f; m[1] = 0.0f; m[2] = 0.0f;
+        m[3] = a11 > 0 ? (float)(1.0 / a11) : 0.0f; m[4] = 0.0f;
+        m[5] = a22 > 0 ? (float)(1.0 / a22) : 0.0f;
+    }
+}
+
 // Observations per thread when a CTA of `threads` threads splits `n` of them into
 // contiguous chunks, rounded up to an odd count.  A camera's run covers consecutive
 // tile slots, so lanes inside one run sit `chunk` slots apart: an odd stride sends

@@ -584,14 +584,8 @@ __device__ __forceinline__ void lin_accumulate(const Views<float>& v, LinObs& o,
                                                float (&acc)[TL_ACC], float* sG, float* sH) {
     if (mode == 2) {   // evaluation output: the unweighted residual and Jacobian
         const uint32_t u = v.obs_user[j];
-        if (res_out) { res_out[2 * (size_t)u] = o.r0; res_out[2 * (size_t)u + 1] = o.r1; }
-        if (jac_out) {
-            float* Jo = jac_out + 24 * (size_t)u;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) { Jo[k] = o.j0[k]; Jo[12 + k] = o.j1[k]; }
-#pragma unroll
-            for (int q = 0; q < 3; ++q) { Jo[9 + q] = o.jx0[q]; Jo[21 + q] = o.jx1[q]; }
-        }
+        if (res_out) store_residual(res_out + 2 * (size_t)u, o.r0, o.r1);
+        if (jac_out) store_jacobian(jac_out + 24 * (size_t)u, o.j0, o.jx0, o.j1, o.jx1);
     }
     if (loss) {   // IRLS weight w = rho'(|r|^2): rows scaled by sqrt(w)
         const float w = loss_weight(fmaf(o.r0, o.r0, o.r1 * o.r1), loss, lscale);
