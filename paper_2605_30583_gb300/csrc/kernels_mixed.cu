@@ -426,43 +426,34 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
         const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
         const uint32_t a = min(lo + threadIdx.x * chunk, hi), b = min(a + chunk, hi);
         uint32_t cur = NO_CAM;
-        float acc[9];
+        float acc[9], k1 = 0.0f, k2 = 0.0f;
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-        Cam cam;
-        float dir[9];
-        uint32_t j = a;
-        while (j < b) {
+        OpCam oc;
+        OpDir od;
+        for (uint32_t j = a; j < b; ++j) {
             const uint32_t key = __ldg(v.obs_key + j);
             const uint32_t c = key >> 8, slot = key & 0xffu;
             if (c != cur) {
-                if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
-                cur = c;
-                cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-                load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);   // from k_cam_direction
-            }
-            if (weighted) {   // robust loss: per-observation IRLS weights
-                kahan_add(jp2, jp2c, obs_normal<true>(cam, dir, sx + 3 * slot, sd + 3 * slot, eps, acc,
-                                                      sq + 3 * slot, __ldg(v.obs_w + j)));
-                j += 1;
-                continue;
-            }
-            if (j + 1 < b) {
-                const uint32_t key1 = __ldg(v.obs_key + j + 1);
-                if ((key1 >> 8) == c) {
-                    // two observations of the same camera: independent chains interleave
-                    const uint32_t slot1 = key1 & 0xffu;
-                    const float a0 = obs_normal(cam, dir, sx + 3 * slot, sd + 3 * slot, eps, acc, sq + 3 * slot);
-                    const float a1 = obs_normal(cam, dir, sx + 3 * slot1, sd + 3 * slot1, eps, acc, sq + 3 * slot1);
-                    kahan_add(jp2, jp2c, a0);
-                    kahan_add(jp2, jp2c, a1);
-                    j += 2;
-                    continue;
+                if (cur != NO_CAM) {
+                    op_finish(oc, k1, k2, acc);
+                    flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
                 }
+                cur = c;
+                const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
+                float dir[9];
+                load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);   // from k_cam_direction
+                oc = op_cam(cam);
+                od = op_dir(cam, dir);
+                k1 = cam.k1;
+                k2 = cam.k2;
             }
-            kahan_add(jp2, jp2c, obs_normal(cam, dir, sx + 3 * slot, sd + 3 * slot, eps, acc, sq + 3 * slot));
-            j += 1;
+            const float4 xs = make_float4(sx[3 * slot], sx[3 * slot + 1], sx[3 * slot + 2], 0.0f);
+            const float4 ds = make_float4(sd[3 * slot], sd[3 * slot + 1], sd[3 * slot + 2], 0.0f);
+            const float w = weighted ? __ldg(v.obs_w + j) : 1.0f;   // robust loss: IRLS weights
+            kahan_add(jp2, jp2c, obs_normal<true>(oc, od, xs, ds, eps, w, acc, sq + 3 * slot));
         }
+        if (cur != NO_CAM) op_finish(oc, k1, k2, acc);
         const bool head = seg_reduce<9>(cur, acc);
         if (head && cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
         __syncthreads();

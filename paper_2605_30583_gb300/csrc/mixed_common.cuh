@@ -69,6 +69,7 @@ __device__ __forceinline__ int warp_split_sum(float (&v)[N], int lane, int& idx)
     return rc;
 }
 
+// A thread's finished camera sums (op_finish) into the global accumulators, then cleared.
 __device__ __forceinline__ void flush_matvec(float* __restrict__ dst, float (&a)[9]) {
     atomicAdd(reinterpret_cast<float4*>(dst), make_float4(a[0], a[1], a[2], a[3]));
     atomicAdd(reinterpret_cast<float4*>(dst + 4), make_float4(a[4], a[5], a[6], a[7]));
@@ -204,6 +205,207 @@ __device__ __forceinline__ void camera_dir(const Views<float>& v, uint32_t c, co
     for (int k = 3; k < 9; ++k) dir[k] = pcv[k];
 }
 
+// ---- one observation of the normal operator ---------------------------------------------
+// J d and J^T t in camera coordinates.  With P~ = P + (0, 0, se), se = +-eps (the depth
+// guard), p = -P~.xy / P~.z and v = (-p0, -p1, 1) = P~ / P~.z:
+//   d(P)/P~.z = phi x v + (w + R dX) / P~.z,  w = d_t - phi x t  (se enters w),
+//   e = dp = -(d(P).xy + p d(P).z) / P~.z,   J d = M e + c_i p,   M = a I + b p p^T,
+//   c_i = d_f + n2 (c1 + n2 c2),  c1 = k1 d_f + f d_k1,  c2 = k2 d_f + f d_k2,
+// and the adjoint of t: y = M t, u = -(y, p.y) / P~.z, P x u from y and p alone, and the
+// intrinsic part as the three moments p.t, n2 p.t, n2^2 p.t.  The camera-constant factors
+// (fk1 = f k1, w, c1, c2) are formed once per camera run and the camera sums brought to
+// the record's form once per run (op_finish): 88 operations per observation, where the same
+// products written per observation with R X, t and the intrinsics apart took 115.
+struct OpCam {
+    float R[9], t[3], f, fk1, fk2, b1, b2;   // a = f + n2 (fk1 + n2 fk2), b = b1 + n2 b2
+};
+struct OpDir {
+    float ph[3], w[3], d6, c1, c2;
+};
+
+__device__ __forceinline__ OpCam op_cam(const Cam& m) {
+    OpCam c;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) c.R[k] = m.R[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c.t[k] = m.t[k];
+    c.f = m.f;
+    c.fk1 = m.f * m.k1;
+    c.fk2 = m.f * m.k2;
+    c.b1 = 2.0f * c.fk1;
+    c.b2 = 4.0f * c.fk2;
+    return c;
+}
+
+// From a camera's direction record (phi, d_t, d_f, d_k1, d_k2).
+__device__ __forceinline__ OpDir op_dir(const Cam& m, const float (&dir)[9]) {
+    OpDir d;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) d.ph[k] = dir[CD_PHI + k];
+    d.w[0] = dir[CD_T + 0] - fmaf(dir[1], m.t[2], -dir[2] * m.t[1]);
+    d.w[1] = dir[CD_T + 1] - fmaf(dir[2], m.t[0], -dir[0] * m.t[2]);
+    d.w[2] = dir[CD_T + 2] - fmaf(dir[0], m.t[1], -dir[1] * m.t[0]);
+    d.d6 = dir[CD_I];
+    d.c1 = fmaf(m.k1, dir[CD_I], m.f * dir[CD_I + 1]);
+    d.c2 = fmaf(m.k2, dir[CD_I], m.f * dir[CD_I + 2]);
+    return d;
+}
+
+struct OpGeo {
+    float iz, p0, p1, n2, a, b, se;
+};
+
+// EPS: the depth guard may be non-zero.
+template <bool EPS>
+__device__ __forceinline__ OpGeo op_geo(const OpCam& c, float X0, float X1, float X2, float eps) {
+    OpGeo g;
+    const float P0 = fmaf(c.R[0], X0, fmaf(c.R[1], X1, fmaf(c.R[2], X2, c.t[0])));
+    const float P1 = fmaf(c.R[3], X0, fmaf(c.R[4], X1, fmaf(c.R[5], X2, c.t[1])));
+    const float P2 = fmaf(c.R[6], X0, fmaf(c.R[7], X1, fmaf(c.R[8], X2, c.t[2])));
+    g.se = EPS ? (P2 >= 0.0f ? eps : -eps) : 0.0f;
+    g.iz = rcp_approx(EPS ? P2 + g.se : P2);
+    g.p0 = -P0 * g.iz;
+    g.p1 = -P1 * g.iz;
+    g.n2 = fmaf(g.p0, g.p0, g.p1 * g.p1);
+    g.a = fmaf(g.n2, fmaf(g.n2, c.fk2, c.fk1), c.f);
+    g.b = fmaf(g.n2, c.b2, c.b1);
+    return g;
+}
+
+// t = J d (the point's direction dx).
+template <bool EPS>
+__device__ __forceinline__ void op_forward(const OpCam& c, const OpDir& d, const OpGeo& g, float dx0, float dx1,
+                                           float dx2, float& t0, float& t1) {
+    float W0 = d.w[0], W1 = d.w[1];
+    if (EPS) {
+        W0 = fmaf(-d.ph[1], g.se, W0);
+        W1 = fmaf(d.ph[0], g.se, W1);
+    }
+    const float w0 = fmaf(c.R[0], dx0, fmaf(c.R[1], dx1, fmaf(c.R[2], dx2, W0)));
+    const float w1 = fmaf(c.R[3], dx0, fmaf(c.R[4], dx1, fmaf(c.R[5], dx2, W1)));
+    const float w2 = fmaf(c.R[6], dx0, fmaf(c.R[7], dx1, fmaf(c.R[8], dx2, d.w[2])));
+    const float ka = fmaf(d.ph[1], g.p0, -d.ph[0] * g.p1);
+    // -e
+    const float e0 = fmaf(g.iz, fmaf(g.p0, w2, w0), fmaf(g.p0, ka, fmaf(d.ph[2], g.p1, d.ph[1])));
+    const float e1 = fmaf(g.iz, fmaf(g.p1, w2, w1), fmaf(g.p1, ka, fmaf(-d.ph[2], g.p0, -d.ph[0])));
+    const float ci = fmaf(g.n2, fmaf(g.n2, d.c2, d.c1), d.d6);
+    const float m = fmaf(-g.b, fmaf(g.p0, e0, g.p1 * e1), ci);
+    t0 = fmaf(m, g.p0, -g.a * e0);
+    t1 = fmaf(m, g.p1, -g.a * e1);
+}
+
+// J^T t: camera moments into acc, and v = -u with u = A^T t (the point part is R^T u).
+template <bool EPS>
+__device__ __forceinline__ void op_adjoint(const OpGeo& g, float t0, float t1, float (&acc)[9], float& v0, float& v1,
+                                           float& v2) {
+    const float pt = fmaf(g.p0, t0, g.p1 * t1);
+    const float bp = g.b * pt;
+    const float y0 = fmaf(g.a, t0, bp * g.p0), y1 = fmaf(g.a, t1, bp * g.p1);
+    const float py = fmaf(g.p0, y0, g.p1 * y1);
+    v0 = g.iz * y0;
+    v1 = g.iz * y1;
+    v2 = g.iz * py;
+    acc[0] += fmaf(g.p1, py, y1);
+    acc[1] -= fmaf(g.p0, py, y0);
+    acc[2] = fmaf(g.p0, y1, fmaf(-g.p1, y0, acc[2]));
+    if (EPS) {
+        acc[0] = fmaf(-g.se, v1, acc[0]);
+        acc[1] = fmaf(g.se, v0, acc[1]);
+    }
+    acc[3] += v0;
+    acc[4] += v1;
+    acc[5] += v2;
+    const float np = g.n2 * pt;
+    acc[6] += pt;
+    acc[7] += np;
+    acc[8] = fmaf(g.n2, np, acc[8]);
+}
+
+// q += R^T u = -R^T v.
+__device__ __forceinline__ void op_point(const OpCam& c, float v0, float v1, float v2, float& q0, float& q1, float& q2) {
+    q0 = fmaf(-c.R[0], v0, fmaf(-c.R[3], v1, fmaf(-c.R[6], v2, q0)));
+    q1 = fmaf(-c.R[1], v0, fmaf(-c.R[4], v1, fmaf(-c.R[7], v2, q1)));
+    q2 = fmaf(-c.R[2], v0, fmaf(-c.R[5], v1, fmaf(-c.R[8], v2, q2)));
+}
+
+// Camera moments of a run -> the camera sums of the accumulators (sum R X x u, sum u, intrinsic
+// part): R X = P - t.  Linear, so it may be applied to partial sums.
+__device__ __forceinline__ void op_finish(const OpCam& c, float k1, float k2, float (&acc)[9]) {
+    const float u0 = -acc[3], u1 = -acc[4], u2 = -acc[5];
+    acc[0] -= fmaf(c.t[1], u2, -c.t[2] * u1);
+    acc[1] -= fmaf(c.t[2], u0, -c.t[0] * u2);
+    acc[2] -= fmaf(c.t[0], u1, -c.t[1] * u0);
+    acc[3] = u0;
+    acc[4] = u1;
+    acc[5] = u2;
+    const float s1 = acc[7], s2 = acc[8];
+    acc[6] = fmaf(k2, s2, fmaf(k1, s1, acc[6]));
+    acc[7] = c.f * s1;
+    acc[8] = c.f * s2;
+}
+
+// Contribution of one observation to the normal operator: t = J d (returns |t|^2), the camera
+// moments into acc, the point part R^T u into qs (shared).  GEN: the depth guard may be
+// non-zero, and the robust loss's IRLS weight w scales the observation's rows of J^T J
+// (u = A^T (w t), returns w |t|^2).  PLAIN_Q: qs belongs to the calling warp alone and
+// no other lane of it touches the same point in this step, so plain adds replace the
+// shared-memory atomics.
+template <bool GEN, bool PLAIN_Q = false>
+__device__ __forceinline__ float obs_normal(const OpCam& cam, const OpDir& dir, const float4 x, const float4 dx,
+                                            float eps, float w, float (&acc)[9], float* qs) {
+    const OpGeo g = op_geo<GEN>(cam, x.x, x.y, x.z, eps);
+    float t0, t1;
+    op_forward<GEN>(cam, dir, g, dx.x, dx.y, dx.z, t0, t1);
+    float tt = fmaf(t0, t0, t1 * t1);
+    if (GEN) {
+        tt *= w;
+        t0 *= w;
+        t1 *= w;
+    }
+    float v0, v1, v2;
+    op_adjoint<GEN>(g, t0, t1, acc, v0, v1, v2);
+    if (PLAIN_Q) {
+        op_point(cam, v0, v1, v2, qs[0], qs[1], qs[2]);
+    } else {
+        float q0 = 0.0f, q1 = 0.0f, q2 = 0.0f;
+        op_point(cam, v0, v1, v2, q0, q1, q2);
+        atomicAdd(qs + 0, q0);
+        atomicAdd(qs + 1, q1);
+        atomicAdd(qs + 2, q2);
+    }
+    return tt;
+}
+
+// One pose factor in the normal operator: t = J_f (d_a; d_b) over the (phi, t) parts of
+// the two cameras' direction records, J_f^T t added to their camera sums (phi part to
+// entries 0-2, translation part to 3-5, as the observations' sums); returns |t|^2.
+__device__ __forceinline__ float factor_normal(const float* __restrict__ Jf, const float* da, const float* db,
+                                               float* acc_a, float* acc_b) {
+    const float x[12] = {da[CD_PHI], da[CD_PHI + 1], da[CD_PHI + 2], da[CD_T], da[CD_T + 1], da[CD_T + 2],
+                         db[CD_PHI], db[CD_PHI + 1], db[CD_PHI + 2], db[CD_T], db[CD_T + 1], db[CD_T + 2]};
+    float t[6], tt = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        float ti = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) ti = fmaf(__ldg(Jf + 12 * i + j), x[j], ti);
+        t[i] = ti;
+        tt = fmaf(ti, ti, tt);
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        float ga = 0.0f, gb = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            ga = fmaf(__ldg(Jf + 12 * i + j), t[i], ga);
+            gb = fmaf(__ldg(Jf + 12 * i + 6 + j), t[i], gb);
+        }
+        atomicAdd(acc_a + j, ga);
+        atomicAdd(acc_b + j, gb);
+    }
+    return tt;
+}
+
 // Contribution of one observation to the normal operator: t = J d (returns |t|^2),
 // camera sums (RX x u, u, intrinsic part) into acc, point part R^T u into qs (shared).
 // WEIGHTED: the robust loss's IRLS weight w scales the observation's rows of J^T J
@@ -259,36 +461,6 @@ __device__ __forceinline__ float obs_normal(const Cam& cam, const float (&dir)[9
         atomicAdd(qs + 2, q2);
     }
     return WEIGHTED ? w * tt : tt;
-}
-
-// One pose factor in the normal operator: t = J_f (d_a; d_b) over the (phi, t) parts of
-// the two cameras' direction records, J_f^T t added to their camera sums (phi part to
-// entries 0-2, translation part to 3-5, as the observations' sums); returns |t|^2.
-__device__ __forceinline__ float factor_normal(const float* __restrict__ Jf, const float* da, const float* db,
-                                               float* acc_a, float* acc_b) {
-    const float x[12] = {da[CD_PHI], da[CD_PHI + 1], da[CD_PHI + 2], da[CD_T], da[CD_T + 1], da[CD_T + 2],
-                         db[CD_PHI], db[CD_PHI + 1], db[CD_PHI + 2], db[CD_T], db[CD_T + 1], db[CD_T + 2]};
-    float t[6], tt = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        float ti = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 12; ++j) ti = fmaf(__ldg(Jf + 12 * i + j), x[j], ti);
-        t[i] = ti;
-        tt = fmaf(ti, ti, tt);
-    }
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-        float ga = 0.0f, gb = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            ga = fmaf(__ldg(Jf + 12 * i + j), t[i], ga);
-            gb = fmaf(__ldg(Jf + 12 * i + 6 + j), t[i], gb);
-        }
-        atomicAdd(acc_a + j, ga);
-        atomicAdd(acc_b + j, gb);
-    }
-    return tt;
 }
 
 }  // namespace gbba

@@ -95,6 +95,80 @@ __device__ __forceinline__ void block_pair_sums(float sa, float ca, float sb, fl
     block_sum2c(sa, ca, sb, cb, sh, ra, rb);
 }
 
+// The normal operator over a tile's observations (points and directions staged in sX4, sP4):
+// long runs in camera-uniform steps of 32 observations, then the short runs in contiguous
+// per-thread chunks.  qw: the calling warp's point sums (PLAIN_Q: its own copy, plain adds in
+// the long runs).  GEN: a depth guard or weights.
+template <int TB, bool PLAIN_Q, bool GEN>
+__device__ __forceinline__ void tile_normal(const Views<float>& v, const TileRange& T, const uint32_t* sRun,
+                                            const uint32_t* sShort, const uint8_t* sSlot, const float4* sX4,
+                                            const float4* sP4, float* qw, unsigned int* s_next, float eps,
+                                            bool weighted, float& js, float& jc) {
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned int r = 0;
+        if (lane == 0) r = atomicAdd(s_next, 1u);
+        r = __shfl_sync(FULL, r, 0);
+        if (r >= T.nl) break;
+        const uint32_t start = sRun[3 * r] - T.lo, len = sRun[3 * r + 1], c = sRun[3 * r + 2];
+        const float* rec = v.cam_pre + (size_t)c * CP_STRIDE;
+        float acc[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
+        {
+            const Cam cam = load_cam(rec);
+            float dir[9];
+            load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
+            const OpCam oc = op_cam(cam);
+            const OpDir od = op_dir(cam, dir);
+            for (uint32_t off = lane; off < len; off += 32) {
+                const uint32_t slot = sSlot[start + off];
+                const float w = GEN && weighted ? __ldg(v.obs_w + T.lo + start + off) : 1.0f;
+                kahan_add(js, jc, obs_normal<GEN, PLAIN_Q>(oc, od, sX4[slot], sP4[slot], eps, w, acc, qw + 3 * slot));
+            }
+            if (PLAIN_Q) __syncwarp();   // the warp's next run may meet the same points
+            op_finish(oc, __ldg(rec + CP_K1), __ldg(rec + CP_K2), acc);
+        }
+        int idx;
+        const int nv = warp_split_sum<9>(acc, lane, idx);
+        if (nv > 0) atomicAdd(v.cam_acc + (size_t)c * CA_STRIDE + idx, acc[0]);
+    }
+    const uint32_t n = T.hi - T.ss;
+    const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
+    const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
+    uint32_t cur = NO_CAM;
+    float acc[9], k1 = 0.0f, k2 = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
+    OpCam oc;
+    OpDir od;
+    for (uint32_t j = a; j < b; ++j) {
+        const uint32_t key = sShort[j - T.ss];
+        const uint32_t c = key >> 8, slot = key & 0xffu;
+        if (c != cur) {
+            if (cur != NO_CAM) {
+                op_finish(oc, k1, k2, acc);
+                flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
+            }
+            cur = c;
+            const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
+            float dir[9];
+            load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
+            oc = op_cam(cam);
+            od = op_dir(cam, dir);
+            k1 = cam.k1;
+            k2 = cam.k2;
+        }
+        // lanes of a warp may meet one point here: atomics (into the warp's copy)
+        const float w = GEN && weighted ? __ldg(v.obs_w + j) : 1.0f;
+        kahan_add(js, jc, obs_normal<GEN>(oc, od, sX4[slot], sP4[slot], eps, w, acc, qw + 3 * slot));
+    }
+    if (cur != NO_CAM) {
+        op_finish(oc, k1, k2, acc);
+        flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
+    }
+}
+
 // ------------------------------------------------------------------ normal operator ---
 // q = J^T W J p + mu D p for the tile's points (written), camera parts J^T W J p into the
 // camera accumulators (k_update adds mu D p and applies J_l^T), |J p|^2 and the points'
@@ -123,7 +197,6 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
     const float mu = (float)st->mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;
-    const int lane = threadIdx.x & 31;
     const TileRange T = tile_range(v, blockIdx.x);
     float jp_s = 0.0f, jp_c = 0.0f, pd_s = 0.0f, pd_c = 0.0f;
     {
@@ -165,64 +238,10 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
     stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
     if (threadIdx.x == 0) s_next = 0u;
     __syncthreads();
-    // long runs: camera-uniform steps of 32 observations
-    for (;;) {
-        unsigned int r = 0;
-        if (lane == 0) r = atomicAdd(&s_next, 1u);
-        r = __shfl_sync(FULL, r, 0);
-        if (r >= T.nl) break;
-        const uint32_t start = sRun[3 * r] - T.lo, len = sRun[3 * r + 1], c = sRun[3 * r + 2];
-        const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-        float dir[9];
-        load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
-        float acc[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-        uint32_t off = lane;
-        for (; off < len; off += 32) {
-            const uint32_t j = T.lo + start + off;
-            const uint32_t slot = sSlot[start + off];
-            const float4 xp = sX4[slot], pp = sP4[slot];
-            const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {pp.x, pp.y, pp.z};
-            const float tt = weighted ? obs_normal<true, PLAIN_Q>(cam, dir, xs, ds, eps, acc, sQw + 3 * slot,
-                                                                 __ldg(v.obs_w + j))
-                                      : obs_normal<false, PLAIN_Q>(cam, dir, xs, ds, eps, acc, sQw + 3 * slot);
-            kahan_add(jp_s, jp_c, tt);
-        }
-        if (PLAIN_Q) __syncwarp();   // the warp's next run may meet the same points
-        int idx;
-        const int nv = warp_split_sum<9>(acc, lane, idx);
-        if (nv > 0) atomicAdd(v.cam_acc + (size_t)c * CA_STRIDE + idx, acc[0]);
-    }
-    // short runs: one contiguous chunk per thread
-    {
-        const uint32_t n = T.hi - T.ss;
-        const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
-        const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
-        uint32_t cur = NO_CAM;
-        float acc[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-        Cam cam;
-        float dir[9];
-        for (uint32_t j = a; j < b; ++j) {
-            const uint32_t key = sShort[j - T.ss];
-            const uint32_t c = key >> 8, slot = key & 0xffu;
-            if (c != cur) {
-                if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
-                cur = c;
-                cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-                load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
-            }
-            const float4 xp = sX4[slot], pp = sP4[slot];
-            const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {pp.x, pp.y, pp.z};
-            // lanes of a warp may meet one point here: atomics (into the warp's copy)
-            const float tt = weighted ? obs_normal<true>(cam, dir, xs, ds, eps, acc, sQw + 3 * slot, __ldg(v.obs_w + j))
-                                      : obs_normal(cam, dir, xs, ds, eps, acc, sQw + 3 * slot);
-            kahan_add(jp_s, jp_c, tt);
-        }
-        if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
-    }
+    if (weighted || eps != 0.0f)
+        tile_normal<TB, PLAIN_Q, true>(v, T, sRun, sShort, sSlot, sX4, sP4, sQw, &s_next, eps, weighted, jp_s, jp_c);
+    else
+        tile_normal<TB, PLAIN_Q, false>(v, T, sRun, sShort, sSlot, sX4, sP4, sQw, &s_next, eps, weighted, jp_s, jp_c);
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * T.npt; i += TB) {
         float qi = sQ[i];
@@ -345,7 +364,6 @@ __global__ void __launch_bounds__(TB, 6) k_tile_cg(Views<float> v, const int32_t
     const float alpha = (float)st->alpha, beta = (float)st->beta, mu = (float)st->mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;
-    const int lane = threadIdx.x & 31;
     const TileRange T = tile_range(v, blockIdx.x);
     float jp_s = 0.0f, jp_c = 0.0f, ud_s = 0.0f, ud_c = 0.0f;   // |J u|^2, u^T D u
     float ru_s = 0.0f, ru_c = 0.0f, rr_s = 0.0f, rr_c = 0.0f;   // r^T u, |r|^2
@@ -432,59 +450,11 @@ __global__ void __launch_bounds__(TB, 6) k_tile_cg(Views<float> v, const int32_t
     stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
     if (threadIdx.x == 0) s_next = 0u;
     __syncthreads();
-    // w = A u: long runs in camera-uniform steps, then the short tail by chunks
-    for (;;) {
-        unsigned int rr = 0;
-        if (lane == 0) rr = atomicAdd(&s_next, 1u);
-        rr = __shfl_sync(FULL, rr, 0);
-        if (rr >= T.nl) break;
-        const uint32_t start = sRun[3 * rr] - T.lo, len = sRun[3 * rr + 1], c = sRun[3 * rr + 2];
-        const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-        float dir[9];
-        load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
-        float acc[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
-        for (uint32_t off = lane; off < len; off += 32) {
-            const uint32_t j = T.lo + start + off;
-            const uint32_t slot = sSlot[start + off];
-            const float4 xp = sX4[slot], pp = sP4[slot];
-            const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {pp.x, pp.y, pp.z};
-            const float tt = weighted ? obs_normal<true>(cam, dir, xs, ds, eps, acc, sQ + 3 * slot, __ldg(v.obs_w + j))
-                                      : obs_normal(cam, dir, xs, ds, eps, acc, sQ + 3 * slot);
-            kahan_add(jp_s, jp_c, tt);
-        }
-        int idx;
-        const int nv = warp_split_sum<9>(acc, lane, idx);
-        if (nv > 0) atomicAdd(v.cam_acc + (size_t)c * CA_STRIDE + idx, acc[0]);
-    }
-    {
-        const uint32_t n = T.hi - T.ss;
-        const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
-        const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
-        uint32_t cur = NO_CAM;
-        float acc[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
-        Cam cam;
-        float dir[9];
-        for (uint32_t j = a; j < b; ++j) {
-            const uint32_t key = sShort[j - T.ss];
-            const uint32_t c = key >> 8, slot = key & 0xffu;
-            if (c != cur) {
-                if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
-                cur = c;
-                cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-                load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
-            }
-            const float4 xp = sX4[slot], pp = sP4[slot];
-            const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {pp.x, pp.y, pp.z};
-            const float tt = weighted ? obs_normal<true>(cam, dir, xs, ds, eps, acc, sQ + 3 * slot, __ldg(v.obs_w + j))
-                                      : obs_normal(cam, dir, xs, ds, eps, acc, sQ + 3 * slot);
-            kahan_add(jp_s, jp_c, tt);
-        }
-        if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
-    }
+    // w = A u
+    if (weighted || eps != 0.0f)
+        tile_normal<TB, false, true>(v, T, sRun, sShort, sSlot, sX4, sP4, sQ, &s_next, eps, weighted, jp_s, jp_c);
+    else
+        tile_normal<TB, false, false>(v, T, sRun, sShort, sSlot, sX4, sP4, sQ, &s_next, eps, weighted, jp_s, jp_c);
     __syncthreads();
     for (int i = threadIdx.x; i < 3 * T.npt; i += TB) v.q[T.base + i] = sQ[i];
     double b_jp, b_ud, b_ru, b_rr;
