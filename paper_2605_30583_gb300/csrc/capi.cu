@@ -248,12 +248,13 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
     if (p->precision == BA_PREC_MIXED && p->use_schur) {
         // blocks of H' (camera and point inverses, D), then the reduced right-hand side
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, pcg_c, 0, nullptr);
+        launch_precond(v, p->L, s, pcg_c, 0, nullptr, 1);
         launch_schur(v, s, 0, &v.st->lm_active);
         launch_schur_start(v, p->L, s, pcg_c, use);
     } else if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->pslots : nullptr);
+        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->pslots : nullptr,
+                       p->use_persistent ? 0 : (p->use_cg ? 2 : 1));
         if (p->use_persistent)
             launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->pslots, p->p_grid,
                                   p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one, p->p_form, s);
@@ -1146,7 +1147,7 @@ ba_status ba_apply_normal(ba_problem* p, double mu, const void* vin, void* out, 
     GBBA_CUDA(cudaMemcpyAsync(&dst->lm_active, &one, sizeof(int32_t), cudaMemcpyHostToDevice, s));
     if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, 0, 0, nullptr);
+        launch_precond(v, p->L, s, 0, 0, nullptr, 1);
         launch_set_direction(v, p->L, s, (const float*)vin);
         launch_matvec(v, p->L, s, nullptr, v.p, 0);
         launch_normal_out(v, p->L, s, (float*)out);
@@ -1272,7 +1273,7 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
         double total_ms = 0.0;
         for (int i = 0; i <= reps; ++i) {
             open_gates();
-            launch_precond(v, p->L, s, 0, 0, p->pslots);
+            launch_precond(v, p->L, s, 0, 0, p->pslots, 0);
             cudaEventRecord(e0, s);
             GBBA_CUDA(launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->pslots, p->p_grid,
                                             p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one,
@@ -1293,7 +1294,7 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
     double out[8];
     out[0] = timeit([&] { launch_camera_precompute(v, p->L, s); });
     out[1] = timeit([&] { launch_linearize(v, p->L, s, 1, nullptr, nullptr, 0, 0); });
-    out[2] = timeit([&] { launch_precond(v, p->L, s, 0, 0, nullptr); });
+    out[2] = timeit([&] { launch_precond(v, p->L, s, 0, 0, nullptr, 1); });
     out[3] = timeit([&] { launch_matvec(v, p->L, s, nullptr, v.z, 1); });
     {
         // the update skips its work once the operator sums it consumes are cleared, so

@@ -225,7 +225,11 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 // Blocks [0, cam_blocks) invert the camera blocks (a warp per camera); the others
 // invert the point blocks (a thread per point), so the long FP64 camera eliminations run
 // beside the point work instead of before it in the same warps.
-__global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, double* pslots, int cam_blocks) {
+//
+// Bound by the FP64 pipe (point_inverse).  `zero`: which PCG vectors the solver that follows wants cleared
+// (0 none, 1 h, 2 h, p and s).
+__global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, double* pslots, int cam_blocks,
+                          int zero) {
     DevState* st = v.st;
     if (pslots != nullptr && blockIdx.x == 0) {   // state of the persistent PCG kernel
         for (int i = threadIdx.x; i < PSLOT_TOTAL; i += blockDim.x) pslots[i] = 0.0;
@@ -240,7 +244,9 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, dou
         return;
     }
     const double mu = st->mu, lo = st->opt.min_diag, hi = st->opt.max_diag;
-    double rz = 0.0, rr = 0.0;
+    // the bounds as floats on the inner side: h >= lo exactly when h >= lo_f
+    const float lo_f = __double2float_ru(lo), hi_f = __double2float_rd(hi);
+    float rz = 0.0f, rr = 0.0f, rzc = 0.0f, rrc = 0.0f;   // Kahan pairs
     const int lane = threadIdx.x & 31;
     const int warps = cam_blocks * (blockDim.x >> 5);
     const bool cam_role = (int)blockIdx.x < cam_blocks;
@@ -289,8 +295,8 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, dou
             v.h[e] = 0.0f;
             v.pc[e] = 0.0f;
             v.pc[v.pc_stride + e] = 0.0f;
-            rz += (double)ri * (double)z;
-            rr += (double)ri * (double)ri;
+            kahan_add(rz, rzc, ri * z);
+            kahan_add(rr, rrc, ri * ri);
         }
         if (lane < CA_STRIDE) {
             v.cam_acc[(size_t)c * CA_STRIDE + lane] = 0.0f;
@@ -301,49 +307,44 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, dou
     }
     const int pt_stride = ((int)gridDim.x - cam_blocks) * blockDim.x;
     for (int i = ((int)blockIdx.x - cam_blocks) * blockDim.x + threadIdx.x; !cam_role && i < v.n_pts; i += pt_stride) {
-        const float* H = v.pt_H + (size_t)i * PH_STRIDE;
+        const float2* H2 = reinterpret_cast<const float2*>(v.pt_H + (size_t)i * PH_STRIDE);
         const size_t e = v.pt_off + 3 * (size_t)i;
-        double a00 = H[0], a01 = H[1], a02 = H[2], a11 = H[3], a12 = H[4], a22 = H[5];
-        const double d0 = fmin(fmax(a00, lo), hi), d1 = fmin(fmax(a11, lo), hi), d2 = fmin(fmax(a22, lo), hi);
-        a00 += mu * d0; a11 += mu * d1; a22 += mu * d2;
-        // inverse of the SPD 3x3 block by its adjugate: M = adj(A) / det(A)
-        double m[6];
-        const double c00 = a11 * a22 - a12 * a12, c01 = a02 * a12 - a01 * a22, c02 = a01 * a12 - a02 * a11;
-        const double c11 = a00 * a22 - a02 * a02, c12 = a01 * a02 - a00 * a12, c22 = a00 * a11 - a01 * a01;
-        const double det = a00 * c00 + a01 * c01 + a02 * c02;
-        if (det > 0.0 && isfinite(det) && a00 > 0.0 && c22 > 0.0) {
-            const double id = rcp64(det);
-            m[0] = c00 * id; m[1] = c01 * id; m[2] = c02 * id;
-            m[3] = c11 * id; m[4] = c12 * id; m[5] = c22 * id;
-        } else {   // not SPD in FP64: inverse diagonal
-            m[0] = a00 > 0 ? 1.0 / a00 : 0.0; m[1] = 0.0; m[2] = 0.0;
-            m[3] = a11 > 0 ? 1.0 / a11 : 0.0; m[4] = 0.0;
-            m[5] = a22 > 0 ? 1.0 / a22 : 0.0;
-        }
-        float* Mo = v.Minv_p + (size_t)i * MP_STRIDE;
-        for (int k = 0; k < 6; ++k) Mo[k] = (float)m[k];
-        v.D[e] = (float)d0; v.D[e + 1] = (float)d1; v.D[e + 2] = (float)d2;
+        const float2 h0 = H2[0], h1 = H2[1], h2 = H2[2];
         const float r0 = -v.g[e], r1 = -v.g[e + 1], r2 = -v.g[e + 2];
-        const float z0 = fmaf(Mo[0], r0, fmaf(Mo[1], r1, Mo[2] * r2));
-        const float z1 = fmaf(Mo[1], r0, fmaf(Mo[3], r1, Mo[4] * r2));
-        const float z2 = fmaf(Mo[2], r0, fmaf(Mo[4], r1, Mo[5] * r2));
+        const float Hp[6] = {h0.x, h0.y, h1.x, h1.y, h2.x, h2.y};
+        float m[6], dd[3];
+        point_inverse(Hp, mu, lo, hi, lo_f, hi_f, m, dd);
+        float2* Mo = reinterpret_cast<float2*>(v.Minv_p + (size_t)i * MP_STRIDE);
+        Mo[0] = make_float2(m[0], m[1]);
+        Mo[1] = make_float2(m[2], m[3]);
+        Mo[2] = make_float2(m[4], m[5]);
+        v.D[e] = dd[0]; v.D[e + 1] = dd[1]; v.D[e + 2] = dd[2];
+        const float z0 = fmaf(m[0], r0, fmaf(m[1], r1, m[2] * r2));
+        const float z1 = fmaf(m[1], r0, fmaf(m[3], r1, m[4] * r2));
+        const float z2 = fmaf(m[2], r0, fmaf(m[4], r1, m[5] * r2));
         v.r[e] = r0; v.r[e + 1] = r1; v.r[e + 2] = r2;
         v.z[e] = z0; v.z[e + 1] = z1; v.z[e + 2] = z2;
-        v.p[e] = 0.0f; v.p[e + 1] = 0.0f; v.p[e + 2] = 0.0f;
-        v.s[e] = 0.0f; v.s[e + 1] = 0.0f; v.s[e + 2] = 0.0f;
-        v.h[e] = 0.0f; v.h[e + 1] = 0.0f; v.h[e + 2] = 0.0f;
-        rz += (double)(r0 * z0 + r1 * z1 + r2 * z2);
-        rr += (double)(r0 * r0 + r1 * r1 + r2 * r2);
+        if (zero > 0) { v.h[e] = 0.0f; v.h[e + 1] = 0.0f; v.h[e + 2] = 0.0f; }
+        if (zero > 1) {
+            v.p[e] = 0.0f; v.p[e + 1] = 0.0f; v.p[e + 2] = 0.0f;
+            v.s[e] = 0.0f; v.s[e + 1] = 0.0f; v.s[e + 2] = 0.0f;
+        }
+        kahan_add(rz, rzc, fmaf(r0, z0, fmaf(r1, z1, r2 * z2)));
+        kahan_add(rr, rrc, fmaf(r0, r0, fmaf(r1, r1, r2 * r2)));
     }
-    double in[2] = {rz, rr}, out[2];
-    if (grid_reduce<2>(in, v.partials, &st->tickets[TK_PRE], out) && threadIdx.x == 0) {
+    __shared__ double red[64];
+    double in[2], out[2];
+    block_sum2c(rz, rzc, rr, rrc, red, in[0], in[1]);
+    if (!grid_reduce_block<2>(in, v.partials, &st->tickets[TK_PRE], out)) return;
+    for (int k = threadIdx.x; k < NSLOT * SLOT_STRIDE; k += blockDim.x) st->acc_mv[k] = st->acc_up[k] = 0.0;
+    if (threadIdx.x == 0) {
         st->rz = out[0];
         st->rr0 = out[1];
         st->rr = out[1];
         st->beta = 0.0;
         st->alpha = 0.0;
+        st->h_alpha = 0.0f;
         st->pcg_iter = 0;
-        for (int k = 0; k < NSLOT * SLOT_STRIDE; ++k) st->acc_mv[k] = st->acc_up[k] = 0.0;
         // a non-finite r^T z means a non-finite gradient or block (a Jacobian that
         // overflowed, e.g. a point at a camera centre): a numeric failure, not a stall
         if (!isfinite(out[0]) || !isfinite(out[1])) st->status = 4;
@@ -403,6 +404,7 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
     __shared__ double red[32];
     DevState* st = v.st;
     const float beta = use_beta ? (float)st->beta : 0.0f;
+    const float ha = use_beta ? st->h_alpha : 0.0f;
     const float mu = (float)st->mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;
@@ -414,6 +416,7 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
         const int npt = min(TILE_PTS, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         for (int i = threadIdx.x; i < 3 * npt; i += TB) {
+            if (ha != 0.0f) v.h[base + i] = fmaf(ha, v.p[base + i], v.h[base + i]);   // the last update's step
             const float pn = beta != 0.0f ? fmaf(beta, v.p[base + i], zs[base + i]) : zs[base + i];
             v.p[base + i] = pn;
             sd[i] = pn;
@@ -469,81 +472,91 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
 }
 
 // ------------------------------------------------------------------ K5 --------
-// alpha = r^T z / (|J p|^2 + mu p^T D p); h += alpha p; r -= alpha q; z = M^-1 r; the
+// alpha = r^T z / (|J p|^2 + mu p^T D p); h += alpha p (cameras; the points' step is left to
+// the next operator, which reads p anyway and has memory bandwidth to spare, or to the
+// candidate: st->h_alpha); r -= alpha q; z = M^-1 r; the
 // sums r^T z and |r|^2 go to st->acc_up.  Cameras first finish
 // q = (J_l^T sum RX x u, sum u, intrinsic part) + mu D p from the K4 accumulators.
-// Points run four at a time with float4 accesses.  Never gated: its last block
-// decides whether PCG continues, sets the loop flag and clears the accumulators.
-__global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int cameras_only) {
+// Blocks [0, cam_blocks) take the cameras, nine lanes each and three to a warp: a camera's sums, r
+// and z travel by shuffles, so its update is one round of loads (a thread per camera, with its 81
+// preconditioner entries one after the other, took ~8 us of this kernel whatever the size).  The
+// other blocks take the points, four at a time with float4 accesses.  Never gated: its last
+// block decides whether PCG continues, sets the loop flag and clears the accumulators.
+__global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int cam_blocks, int cameras_only) {
     DevState* st = v.st;
-    __shared__ double red[32];
-    __shared__ double sh_mv[2];
-    __shared__ bool is_last;
+    __shared__ double red[64];
+    __shared__ double sh_mv[3];   // |J p|^2, p^T D p, alpha
+    __shared__ float sh_f[2];     // alpha, mu
+    __shared__ bool is_last, sh_bad;
     const int active = st->pcg_active;
     float rz = 0.0f, rr = 0.0f, rzc = 0.0f, rrc = 0.0f;   // Kahan pairs
-    double alpha_d = 0.0;
-    bool bad = false;
+    // the scalars are FP64: one thread of the CTA computes them for all
     if (active) {
         if (threadIdx.x < 32) {
             const double a0 = slot_sum_warp(st->acc_mv, 0), a1 = slot_sum_warp(st->acc_mv, 1);
-            if (threadIdx.x == 0) { sh_mv[0] = a0; sh_mv[1] = a1; }
+            if (threadIdx.x == 0) {
+                const double denom = a0 + st->mu * a1;
+                sh_bad = !(denom > 0.0) || !isfinite(denom);
+                const double alpha = sh_bad ? 0.0 : st->rz / denom;
+                sh_mv[0] = a0;
+                sh_mv[1] = a1;
+                sh_mv[2] = alpha;
+                sh_f[0] = (float)alpha;
+                sh_f[1] = (float)st->mu;
+            }
         }
         __syncthreads();
-        const double denom = sh_mv[0] + st->mu * sh_mv[1];
-        bad = !(denom > 0.0) || !isfinite(denom);
-        alpha_d = bad ? 0.0 : st->rz / denom;
     }
+    const bool bad = active && sh_bad;
     if (active && !bad) {
-        const float alpha = (float)alpha_d;
-        const float mu = (float)st->mu;
+        const float alpha = sh_f[0];
+        const float mu = sh_f[1];
         const float* pcur = v.pc + (size_t)((st->pcg_iter & 1) ^ 1) * v.pc_stride;
-        FOR_CAMERAS(c, v) {
-            const size_t e = 9 * (size_t)c;
+        const int lane = threadIdx.x & 31;
+        const int wpb = blockDim.x >> 5;
+        for (int cw = 3 * ((int)blockIdx.x * wpb + ((int)threadIdx.x >> 5)); (int)blockIdx.x < cam_blocks && cw < v.n_cams;
+             cw += 3 * wpb * cam_blocks) {
+            const int sub = lane / 9, base = 9 * sub;
+            const bool live = lane < 27 && cw + sub < v.n_cams;
+            const int c = live ? cw + sub : cw, i = live ? lane - base : 0, i3 = i < 3 ? i : 0;
+            const size_t e = 9 * (size_t)c + i;
             float* ca = v.cam_acc + (size_t)c * CA_STRIDE;
             const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
-            float q[9];
+            const float* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * i;
+            const float a = ca[i], pk = pcur[e], Dk = v.D[e], hk = v.h[e], rk = v.r[e];
+            const float j0 = JL[i3], j1 = JL[3 + i3], j2 = JL[6 + i3];
+            float m[9];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = fmaf(JL[k], ca[0], fmaf(JL[3 + k], ca[1], JL[6 + k] * ca[2]));
+            for (int k = 0; k < 9; ++k) m[k] = M[k];
+            const float a0 = __shfl_sync(FULL, a, base), a1 = __shfl_sync(FULL, a, base + 1);
+            const float a2 = __shfl_sync(FULL, a, base + 2);
+            const float q = i < 3 ? fmaf(j0, a0, fmaf(j1, a1, j2 * a2)) : a;
+            const float rn = fmaf(-alpha, fmaf(mu, Dk * pk, q), rk);
+            float z = 0.0f;
 #pragma unroll
-            for (int k = 3; k < 9; ++k) q[k] = ca[k];
-#pragma unroll
-            for (int k = 0; k < CA_STRIDE; ++k) ca[k] = 0.0f;
-            float rn[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const float pk = pcur[e + k];
-                const float qk = fmaf(mu, v.D[e + k] * pk, q[k]);
-                v.p[e + k] = pk;
-                v.h[e + k] = fmaf(alpha, pk, v.h[e + k]);
-                rn[k] = fmaf(-alpha, qk, v.r[e + k]);
-                v.r[e + k] = rn[k];
-            }
-            const float* M = v.Minv_c + (size_t)c * MC_STRIDE;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                float z = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) z = fmaf(M[9 * i + k], rn[k], z);
-                v.z[e + i] = z;
-                kahan_add(rz, rzc, rn[i] * z);
-                kahan_add(rr, rrc, rn[i] * rn[i]);
+            for (int k = 0; k < 9; ++k) z = fmaf(m[k], __shfl_sync(FULL, rn, base + k), z);
+            if (live) {
+                ca[i] = 0.0f;
+                v.p[e] = pk;
+                v.h[e] = fmaf(alpha, pk, hk);
+                v.r[e] = rn;
+                v.z[e] = z;
+                kahan_add(rz, rzc, rn * z);
+                kahan_add(rr, rrc, rn * rn);
             }
         }
-        for (int qd = blockIdx.x * blockDim.x + threadIdx.x; !cameras_only && qd < v.n_quads;
-             qd += gridDim.x * blockDim.x) {
+        const int pt_blocks = (int)gridDim.x - cam_blocks;
+        for (int qd = ((int)blockIdx.x - cam_blocks) * (int)blockDim.x + (int)threadIdx.x;
+             (int)blockIdx.x >= cam_blocks && !cameras_only && qd < v.n_quads; qd += pt_blocks * (int)blockDim.x) {
             const size_t e = v.pt_off + 12 * (size_t)qd;
-            float4* p4 = reinterpret_cast<float4*>(v.p + e);
-            float4* h4 = reinterpret_cast<float4*>(v.h + e);
             float4* r4 = reinterpret_cast<float4*>(v.r + e);
             const float4* q4 = reinterpret_cast<const float4*>(v.q + e);
             float4* z4 = reinterpret_cast<float4*>(v.z + e);
             const float4* m4 = reinterpret_cast<const float4*>(v.Minv_p + 24 * (size_t)qd);
-            float P[12], H[12], R[12], Q[12], M[24];
+            float R[12], Q[12], M[24];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const float4 a = p4[k], b = h4[k], c = r4[k], d = q4[k];
-                P[4 * k] = a.x; P[4 * k + 1] = a.y; P[4 * k + 2] = a.z; P[4 * k + 3] = a.w;
-                H[4 * k] = b.x; H[4 * k + 1] = b.y; H[4 * k + 2] = b.z; H[4 * k + 3] = b.w;
+                const float4 c = r4[k], d = q4[k];
                 R[4 * k] = c.x; R[4 * k + 1] = c.y; R[4 * k + 2] = c.z; R[4 * k + 3] = c.w;
                 Q[4 * k] = d.x; Q[4 * k + 1] = d.y; Q[4 * k + 2] = d.z; Q[4 * k + 3] = d.w;
             }
@@ -554,10 +567,7 @@ __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int 
             }
             float Z[12];
 #pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                H[k] = fmaf(alpha, P[k], H[k]);
-                R[k] = fmaf(-alpha, Q[k], R[k]);
-            }
+            for (int k = 0; k < 12; ++k) R[k] = fmaf(-alpha, Q[k], R[k]);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float* m = M + 6 * j;
@@ -573,14 +583,13 @@ __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int 
             }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                h4[k] = make_float4(H[4 * k], H[4 * k + 1], H[4 * k + 2], H[4 * k + 3]);
                 r4[k] = make_float4(R[4 * k], R[4 * k + 1], R[4 * k + 2], R[4 * k + 3]);
                 z4[k] = make_float4(Z[4 * k], Z[4 * k + 1], Z[4 * k + 2], Z[4 * k + 3]);
             }
         }
     }
-    const double brz = block_sum((double)rz - (double)rzc, red);
-    const double brr = block_sum((double)rr - (double)rrc, red);
+    double brz, brr;
+    block_sum2c(rz, rzc, rr, rrc, red, brz, brr);
     if (threadIdx.x == 0) {
         if (active && !bad) {
             slot_add(st->acc_up, 0, brz);
@@ -598,11 +607,12 @@ __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int 
     for (int k = threadIdx.x; k < NSLOT * SLOT_STRIDE; k += 32) st->acc_mv[k] = st->acc_up[k] = 0.0;
     if (threadIdx.x != 0) return;
     if (active) {
+        if (!cameras_only) st->h_alpha = bad ? 0.0f : sh_f[0];
         if (bad) {
             st->pcg_active = 0;
             if (!isfinite(sh_mv[0]) || !isfinite(sh_mv[1])) st->status = 4;
         } else {
-            st->alpha = alpha_d;
+            st->alpha = sh_mv[2];
             st->jp2 = sh_mv[0];
             st->pDp = sh_mv[1];
             st->pcg_iter += 1;
@@ -634,45 +644,53 @@ __global__ void k_candidate(Views<float> v) {
         v.cam_acc[i] = 0.0f;
     if (st->lm_active == 0) return;
     const bool retract = st->opt.retract != 0;
-    double gh = 0.0;
-    FOR_CAMERAS(c, v) {
-        {
-            const size_t e = 9 * (size_t)c;
-            const double* cl = v.cam_lin + (size_t)c * CL_STRIDE;
-            // the step applied to the FP64 master copy; the FP32 copy is its rounding
-            double xn[9];
-            float hc[9];
+    const float ha = st->h_alpha;
+    double gh = 0.0;                 // cameras
+    float ghp = 0.0f, ghc = 0.0f;    // points, a Kahan pair
+    // cameras: three lanes each (camera_record_rows), in the first warp of a block
+    const int row = (int)threadIdx.x % 3;
+    for (int c = ROW_CAMS * (int)blockIdx.x + (int)threadIdx.x / 3; threadIdx.x < 3 * ROW_CAMS && c < v.n_cams;
+         c += ROW_CAMS * (int)gridDim.x) {
+        const size_t e = 9 * (size_t)c;
+        const double* cl = v.cam_lin + (size_t)c * CL_STRIDE;
+        // the step applied to the FP64 master copy; the FP32 copy is its rounding
+        double xn[9];
+        float hc[9];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                hc[k] = v.h[e + k];
-                xn[k] = v.xm[e + k] + (double)hc[k];
-                gh += cl[CL_G + k] * (double)hc[k];
-            }
-            if (retract) {   // R' = Exp(h_w) R(w)
-                const double w[3] = {v.xm[e], v.xm[e + 1], v.xm[e + 2]};
-                const double hw[3] = {hc[0], hc[1], hc[2]};
-                compose_rotvec(hw, w, xn);
-            }
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                v.xm_new[e + k] = xn[k];
-                v.x_new[e + k] = (float)xn[k];
-            }
-            camera_record(xn, v.cam_pre_new + (size_t)c * CP_STRIDE, retract, v.cam_lo_new + (size_t)c * CLO_STRIDE);
-            const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
-            float* d = v.cam_dir + (size_t)c * CD_STRIDE;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-                d[CD_PHI + i] = fmaf(JL[3 * i], hc[0], fmaf(JL[3 * i + 1], hc[1], JL[3 * i + 2] * hc[2]));
-#pragma unroll
-            for (int k = 0; k < 6; ++k) d[CD_T + k] = hc[3 + k];
+        for (int k = 0; k < 9; ++k) {
+            hc[k] = v.h[e + k];
+            xn[k] = v.xm[e + k] + widen(hc[k]);
         }
+        if (retract) {   // R' = Exp(h_w) R(w)
+            const double w[3] = {v.xm[e], v.xm[e + 1], v.xm[e + 2]};
+            const double hw[3] = {hc[0], hc[1], hc[2]};
+            compose_rotvec(hw, w, xn);
+        }
+        for (int k = row; k < 9; k += 3) {
+            double xk = xn[0];
+            float hk = hc[0];
+#pragma unroll
+            for (int q = 1; q < 9; ++q) {
+                xk = q == k ? xn[q] : xk;
+                hk = q == k ? hc[q] : hk;
+            }
+            gh += cl[CL_G + k] * widen(hk);
+            v.xm_new[e + k] = xk;
+            v.x_new[e + k] = narrow(xk);
+        }
+        camera_record_rows(xn, v.cam_pre_new + (size_t)c * CP_STRIDE, retract, v.cam_lo_new + (size_t)c * CLO_STRIDE, row,
+                           row + 1);
+        const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
+        float* d = v.cam_dir + (size_t)c * CD_STRIDE;
+        d[CD_PHI + row] = fmaf(JL[3 * row], hc[0], fmaf(JL[3 * row + 1], hc[1], JL[3 * row + 2] * hc[2]));
+        d[CD_T + row] = row == 0 ? hc[3] : (row == 1 ? hc[4] : hc[5]);
+        d[CD_I + row] = row == 0 ? hc[6] : (row == 1 ? hc[7] : hc[8]);
     }
     // points four at a time (a quad's twelve entries as 16-byte accesses; the padding
     // entries of the last quad are zero and stay zero)
     for (int qd = blockIdx.x * blockDim.x + threadIdx.x; qd < v.n_quads; qd += gridDim.x * blockDim.x) {
         const size_t e = v.pt_off + 12 * (size_t)qd;
-        const float4* h4 = reinterpret_cast<const float4*>(v.h + e);
+        float4* h4 = reinterpret_cast<float4*>(v.h + e);
         const float4* g4 = reinterpret_cast<const float4*>(v.g + e);
         const double2* m2 = reinterpret_cast<const double2*>(v.xm + e);
         float H[12], G[12];
@@ -683,6 +701,18 @@ __global__ void k_candidate(Views<float> v) {
             H[4 * k] = a.x; H[4 * k + 1] = a.y; H[4 * k + 2] = a.z; H[4 * k + 3] = a.w;
             G[4 * k] = b.x; G[4 * k + 1] = b.y; G[4 * k + 2] = b.z; G[4 * k + 3] = b.w;
         }
+        if (ha != 0.0f) {   // the last PCG update's step
+            const float4* p4 = reinterpret_cast<const float4*>(v.p + e);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float4 a = p4[k];
+                H[4 * k] = fmaf(ha, a.x, H[4 * k]);
+                H[4 * k + 1] = fmaf(ha, a.y, H[4 * k + 1]);
+                H[4 * k + 2] = fmaf(ha, a.z, H[4 * k + 2]);
+                H[4 * k + 3] = fmaf(ha, a.w, H[4 * k + 3]);
+                h4[k] = make_float4(H[4 * k], H[4 * k + 1], H[4 * k + 2], H[4 * k + 3]);
+            }
+        }
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             const double2 a = m2[k];
@@ -692,7 +722,7 @@ __global__ void k_candidate(Views<float> v) {
         float sgh = 0.0f;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            X[k] += (double)H[k];
+            X[k] += widen(H[k]);
             sgh = fmaf(G[k], H[k], sgh);
         }
         double2* n2 = reinterpret_cast<double2*>(v.xm_new + e);
@@ -701,11 +731,14 @@ __global__ void k_candidate(Views<float> v) {
         for (int k = 0; k < 6; ++k) n2[k] = make_double2(X[2 * k], X[2 * k + 1]);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            x4[k] = make_float4((float)X[4 * k], (float)X[4 * k + 1], (float)X[4 * k + 2], (float)X[4 * k + 3]);
-        gh += (double)sgh;
+            x4[k] = make_float4(narrow(X[4 * k]), narrow(X[4 * k + 1]), narrow(X[4 * k + 2]), narrow(X[4 * k + 3]));
+        kahan_add(ghp, ghc, sgh);
     }
-    double in[1] = {gh}, out[1];
-    if (grid_reduce<1>(in, v.partials, &st->tickets[TK_CAND], out) && threadIdx.x == 0) st->gh = out[0];
+    __shared__ double red[64];
+    double in[1], out[1], none;
+    block_sum2c(ghp, ghc, 0.0f, 0.0f, red, in[0], none);
+    if (threadIdx.x < 32) in[0] += warp_sum(gh);   // only the first warp has cameras
+    if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_CAND], out) && threadIdx.x == 0) st->gh = out[0];
 }
 
 // ------------------------------------------------------------------ K2 --------
@@ -1158,12 +1191,12 @@ void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s,
                                                                                  lm_cond, use_cond);
 }
 void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
-                    double* pslots) {
+                    double* pslots, int zero) {
     // camera blocks: a warp per camera; point blocks: a thread per point
     const int wpb = L.item_block / 32;
     const int cam_blocks = std::max(1, std::min((v.n_cams + wpb - 1) / wpb, L.item_grid / 2));
     const int pt_blocks = std::max(1, std::min(grid_items(L, v.n_pts), L.item_grid - cam_blocks));
-    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, pslots, cam_blocks);
+    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, pslots, cam_blocks, zero);
 }
 void launch_matvec(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
                    const float* zs, int use_beta) {
@@ -1187,11 +1220,13 @@ void launch_schur_start(const Views<float>& v, const LaunchCfg& L, cudaStream_t 
 }
 void launch_update(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
                    int cameras_only) {
-    k_update<<<cameras_only ? std::max(grid_cams(L, v.n_cams), 1) : std::max(grid_items(L, v.n_quads), grid_cams(L, v.n_cams)),
-               L.item_block, 0, s>>>(v, c, use, cameras_only);
+    const int cpb = 3 * (L.item_block / 32);   // cameras a block takes at a time
+    const int cam_blocks = std::max(1, std::min((v.n_cams + cpb - 1) / cpb, L.item_grid / 2));
+    const int pt_blocks = cameras_only ? 0 : std::max(1, std::min(grid_items(L, v.n_quads), L.item_grid - cam_blocks));
+    k_update<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, cam_blocks, cameras_only);
 }
 void launch_candidate(const Views<float>& v, const LaunchCfg& L, cudaStream_t s) {
-    k_candidate<<<std::max(grid_items(L, v.n_quads), grid_cams(L, v.n_cams)), L.item_block, 0, s>>>(v);
+    k_candidate<<<std::max(grid_items(L, v.n_quads), grid_rows(L, v.n_cams)), L.item_block, 0, s>>>(v);
 }
 void launch_eval_candidate(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
     launch_factor_eval(v, L, s);

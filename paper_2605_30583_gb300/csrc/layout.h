@@ -84,6 +84,10 @@ struct DevState {
     double fac_cost, fac_cost_new, fac_jh2;
     // mixed form: 1/2 sum rho(|r|^2) of the observations at the candidate (k_residual)
     double F_res;
+    // separate-kernel textbook PCG: alpha of the last update, whose step h += alpha p of the
+    // points is still to be taken (by the next operator or the candidate); 0: none
+    float h_alpha;
+    int32_t pad2;
     // Per-iteration sums, spread over NSLOT slots (block b adds into slot b % NSLOT,
     // one 128-byte line each) so concurrent atomics do not queue on one address.
     double acc_mv[NSLOT * SLOT_STRIDE];   // k = 0: |J p|^2, k = 1: p^T D p

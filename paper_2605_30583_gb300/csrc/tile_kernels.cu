@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
     __shared__ double red[2 * (TB / 32)];
     DevState* st = v.st;
     const float beta = use_beta ? (float)st->beta : 0.0f;
+    const float ha = use_beta ? st->h_alpha : 0.0f;
     const float mu = (float)st->mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;
@@ -206,13 +207,14 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
         const int ne = 3 * T.npt;
         float* sPf = reinterpret_cast<float*>(sP4);
         float* sXf = reinterpret_cast<float*>(sX4);
-        float Z[EPT], P[EPT], Dd[EPT], X[EPT];
+        float Z[EPT], P[EPT], Dd[EPT], X[EPT], H[EPT];
 #pragma unroll
         for (int t = 0; t < EPT; ++t) {
             const int i = threadIdx.x + t * TB;
             if (i < ne) {
                 Z[t] = zs[T.base + i];
-                P[t] = beta != 0.0f ? v.p[T.base + i] : 0.0f;
+                P[t] = beta != 0.0f || ha != 0.0f ? v.p[T.base + i] : 0.0f;
+                H[t] = ha != 0.0f ? v.h[T.base + i] : 0.0f;
                 Dd[t] = v.D[T.base + i];
                 X[t] = v.x[T.base + i];
             }
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
         for (int t = 0; t < EPT; ++t) {
             const int i = threadIdx.x + t * TB;
             if (i < ne) {
+                if (ha != 0.0f) v.h[T.base + i] = fmaf(ha, P[t], H[t]);   // the last update's step
                 const float pn = beta != 0.0f ? fmaf(beta, P[t], Z[t]) : Z[t];
                 v.p[T.base + i] = pn;
                 const int slot = i / 3, k = i - 3 * slot;
