@@ -271,7 +271,8 @@ static void step_lm_tail(ba_problem* p, cudaStream_t s, CondHandle lm_c, int use
         const Views<float>& v = p->vf;
         if (p->use_schur) launch_schur(v, s, 2, &v.st->lm_active);   // points back-substituted
         launch_candidate(v, p->L, s);
-        launch_residual(v, p->L, s, 1);   // r(x') and F'; the relinearisation reuses r
+        // r(x') and F' (the relinearisation reuses r); few tiles: in the evaluation's launch
+        if (!p->L.wide_tiles) launch_residual(v, p->L, s, 1);
         launch_eval_candidate(v, p->L, s, lm_c, use);
         launch_commit(v, p->L, s);
         launch_linearize(v, p->L, s, 1, nullptr, nullptr, lm_c, 0);

@@ -45,6 +45,8 @@ struct LaunchCfg {
     // no camera observes a point twice (checked at bind): the operator's warps add their
     // point sums into private copies with plain adds
     int tn_plain_q = 0;
+    // few tiles: 512 threads per tile in the linearisation and the evaluations
+    bool wide_tiles = false;
 };
 
 // residual pass of the mixed form (residual.cu): r at x (at_candidate 0) or at x' (1),

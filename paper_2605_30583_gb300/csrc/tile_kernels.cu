@@ -34,6 +34,7 @@
 #include "device_common.cuh"
 #include "kernels.h"
 #include "mixed_common.cuh"
+#include "residual.cuh"
 
 namespace gbba {
 
@@ -515,6 +516,10 @@ __global__ void __launch_bounds__(TB, 6) k_tile_cg(Views<float> v, const int32_t
 // st->relin), 2 evaluation only (squared loss; optional r and J in the caller's order).
 constexpr int TL_ACC = 9 + 45;   // per-lane camera sums: g, upper triangle of J_c^T J_c
 constexpr int TL_TB = 128;
+// Few tiles: a tile's runs spread over more warps.  With at most this many tiles per SM the
+// linearisation and the candidate's evaluation (k_tile_step) run 512 threads per tile.
+constexpr int WIDE_TILES = 2;
+constexpr int WIDE_TB = 512;
 
 struct LinObs {
     float r0, r1, j0[9], j1[9], jx0[3], jx1[3];
@@ -623,14 +628,17 @@ __device__ __forceinline__ void flush_lin_global(const Views<float>& v, uint32_t
 // PLAIN: every warp keeps its own copy of the tile's point sums, added to with plain
 // shared-memory adds in its long runs (as in k_tile_normal).
 template <int TB, bool PLAIN>
-__global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mode, float* res_out, float* jac_out,
+__global__ void __launch_bounds__(TB, TB == 128 ? 4 : 1) k_tile_linearize(Views<float> v, int mode, float* res_out, float* jac_out,
                                                        CondHandle lm_cond, int use_cond, Caps cap) {
     if (mode == 1 && v.st->relin == 0) return;
     constexpr int NQ = PLAIN ? TB / 32 : 1;   // point-sum copies
     extern __shared__ __align__(16) unsigned char dsm[];
     const float2* rbuf = reinterpret_cast<const float2*>(v.rbuf);   // residuals (k_residual)
     __shared__ float4 sX4[TILE_PTS];
-    __shared__ float sG[NQ * 3 * TILE_PTS], sH[NQ * PH_STRIDE * TILE_PTS];   // J_p^T W r, J_p^T W J_p (upper)
+    // J_p^T W r, J_p^T W J_p (upper); the observation table follows
+    float* const sG = reinterpret_cast<float*>(dsm);
+    float* const sH = sG + NQ * 3 * TILE_PTS;
+    unsigned char* const tab = dsm + 4 * NQ * (3 + PH_STRIDE) * TILE_PTS;
     float* const sGw = sG + (PLAIN ? (threadIdx.x >> 5) * 3 * TILE_PTS : 0);
     float* const sHw = sH + (PLAIN ? (threadIdx.x >> 5) * PH_STRIDE * TILE_PTS : 0);
     __shared__ unsigned int s_next;
@@ -647,7 +655,7 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
         for (int i = threadIdx.x; i < NQ * PH_STRIDE * TILE_PTS; i += TB) sH[i] = 0.0f;
         uint32_t *sRun, *sShort;
         uint8_t* sSlot;
-        stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
+        stage_compact<TB>(v, T, cap, tab, sRun, sShort, sSlot);
         if (threadIdx.x == 0) s_next = 0u;
         __syncthreads();
         // long runs: camera-uniform steps of 32 observations
@@ -745,46 +753,33 @@ __global__ void __launch_bounds__(TB, 4) k_tile_linearize(Views<float> v, int mo
 // LM loop flag.
 constexpr int TE_TB = 128;
 
-struct EvalCam {
-    Cam co;       // record at x
-    float dir[9]; // direction record of h (k_candidate)
-};
-
-__device__ __forceinline__ EvalCam load_eval_cam(const Views<float>& v, uint32_t c) {
-    EvalCam e;
-    e.co = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
-    const float4* d4 = reinterpret_cast<const float4*>(v.cam_dir + (size_t)c * CD_STRIDE);
-    const float4 a = __ldcg(d4), b = __ldcg(d4 + 1), cc = __ldcg(d4 + 2);
-    e.dir[0] = a.x; e.dir[1] = a.y; e.dir[2] = a.z; e.dir[3] = a.w;
-    e.dir[4] = b.x; e.dir[5] = b.y; e.dir[6] = b.z; e.dir[7] = b.w; e.dir[8] = cc.x;
-    return e;
-}
-
-__device__ __forceinline__ void eval_obs(const Views<float>& v, const EvalCam& e, const float4* sXo,
-                                         const float4* sHp, uint32_t j, uint32_t slot, float eps, int loss, float& js_,
-                                         float& jc_) {
-    const float4 xo = sXo[slot], hp = sHp[slot];
-    const Geo g = project_geo(e.co, xo.x, xo.y, xo.z, eps);
-    float t0, t1;
-    jdir(g, e.co, e.dir, hp.x, hp.y, hp.z, t0, t1);
-    // |J h|^2 weighted at x
-    kahan_add(js_, jc_, (loss ? __ldg(v.obs_w + j) : 1.0f) * fmaf(t0, t0, t1 * t1));
-}
-
-// Six CTAs per SM (at most 85 registers per thread; 240 -> 220 us on the large workload
-// against four).
+// |J h|^2 of tiles first, first + stride, ... as a Kahan pair (js, jc).  sXo, sHp: TILE_PTS entries
+// each (x and h of the tile's points).
 template <int TB>
-__global__ void __launch_bounds__(TB, 6) k_tile_eval(Views<float> v, CondHandle lm_cond, int use_cond, Caps cap) {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ float4 sXo[TILE_PTS], sHp[TILE_PTS];                // x and h of the tile's points
-    __shared__ unsigned int s_next;
-    DevState* st = v.st;
-    const int active = st->lm_active;
-    const float eps = (float)st->opt.eps;
-    const int loss = st->opt.loss;
+__device__ __forceinline__ void eval_tiles(const Views<float>& v, const Caps& cap, unsigned char* dsm, float4* sXo,
+                                           float4* sHp, unsigned int* s_next, int first, int stride, float& js,
+                                           float& jc) {
+    const float eps = (float)v.st->opt.eps;
+    const int loss = v.st->opt.loss;
     const int lane = threadIdx.x & 31;
-    float js_ = 0.0f, jc_ = 0.0f;   // compensated |J h|^2
-    for (int tile = blockIdx.x; active && tile < v.n_tiles; tile += gridDim.x) {
+    struct EvalCam {
+        OpCam c;
+        OpDir d;   // of h (k_candidate)
+    };
+    auto load = [&](uint32_t c) {
+        const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
+        float dir[9];
+        load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
+        return EvalCam{op_cam(cam), op_dir(cam, dir)};
+    };
+    auto visit = [&](const EvalCam& e, uint32_t j, uint32_t slot) {   // |J h|^2 weighted at x
+        const float4 x = sXo[slot], h = sHp[slot];
+        float t0, t1;
+        if (eps != 0.0f) op_forward<true>(e.c, e.d, op_geo<true>(e.c, x.x, x.y, x.z, eps), h.x, h.y, h.z, t0, t1);
+        else op_forward<false>(e.c, e.d, op_geo<false>(e.c, x.x, x.y, x.z, 0.0f), h.x, h.y, h.z, t0, t1);
+        kahan_add(js, jc, (loss ? __ldg(v.obs_w + j) : 1.0f) * fmaf(t0, t0, t1 * t1));
+    };
+    for (int tile = first; tile < v.n_tiles; tile += stride) {
         const TileRange T = tile_range(v, tile);
         for (int i = threadIdx.x; i < T.npt; i += TB) {
             const size_t e = T.base + 3 * i;
@@ -794,44 +789,85 @@ __global__ void __launch_bounds__(TB, 6) k_tile_eval(Views<float> v, CondHandle 
         uint32_t *sRun, *sShort;
         uint8_t* sSlot;
         stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
-        if (threadIdx.x == 0) s_next = 0u;
+        if (threadIdx.x == 0) *s_next = 0u;
         __syncthreads();
         for (;;) {
             unsigned int r = 0;
-            if (lane == 0) r = atomicAdd(&s_next, 1u);
+            if (lane == 0) r = atomicAdd(s_next, 1u);
             r = __shfl_sync(FULL, r, 0);
             if (r >= T.nl) break;
             const uint32_t start = sRun[3 * r] - T.lo, len = sRun[3 * r + 1];
-            const EvalCam e = load_eval_cam(v, sRun[3 * r + 2]);
-            for (uint32_t off = lane; off < len; off += 32) {
-                const uint32_t i = start + off;
-                eval_obs(v, e, sXo, sHp, T.lo + i, sSlot[i], eps, loss, js_, jc_);
-            }
+            const EvalCam e = load(sRun[3 * r + 2]);
+            for (uint32_t off = lane; off < len; off += 32) visit(e, T.lo + start + off, sSlot[start + off]);
         }
-        {
-            const uint32_t n = T.hi - T.ss;
-            const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
-            const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
-            uint32_t cur = NO_CAM;
-            EvalCam e;
-            for (uint32_t j = a; j < b; ++j) {
-                const uint32_t key = sShort[j - T.ss];
-                const uint32_t c = key >> 8;
-                if (c != cur) {
-                    cur = c;
-                    e = load_eval_cam(v, c);
-                }
-                eval_obs(v, e, sXo, sHp, j, key & 0xffu, eps, loss, js_, jc_);
+        const uint32_t n = T.hi - T.ss;
+        const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
+        const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
+        uint32_t cur = NO_CAM;
+        EvalCam e;
+        for (uint32_t j = a; j < b; ++j) {
+            const uint32_t key = sShort[j - T.ss];
+            const uint32_t c = key >> 8;
+            if (c != cur) {
+                cur = c;
+                e = load(c);
             }
+            visit(e, j, key & 0xffu);
         }
         __syncthreads();   // the next tile's staging overwrites the points
     }
-    double in[1] = {(double)js_ - (double)jc_}, out[1];
-    if (grid_reduce<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {
-        // pose factors: k_factor_eval ran just before
-        const bool fac = v.n_fac > 0;
-        lm_decide(st, active, st->F_res + (fac ? st->fac_cost_new : 0.0), out[0] + (fac ? st->fac_jh2 : 0.0));
-        if (use_cond) cudaGraphSetConditional(lm_cond, st->lm_active ? 1u : 0u);
+}
+
+// The LM decision from F' (F_res) and |J h|^2, by one thread.
+__device__ __forceinline__ void tile_decide(const Views<float>& v, int active, double F_res, double jh2, CondHandle lm_cond,
+                                            int use_cond) {
+    DevState* st = v.st;
+    // pose factors: k_factor_eval ran just before
+    const bool fac = v.n_fac > 0;
+    lm_decide(st, active, F_res + (fac ? st->fac_cost_new : 0.0), jh2 + (fac ? st->fac_jh2 : 0.0));
+    if (use_cond) cudaGraphSetConditional(lm_cond, st->lm_active ? 1u : 0u);
+}
+
+// Six CTAs per SM (at most 85 registers per thread; 240 -> 220 us on the large workload
+// against four).
+template <int TB>
+__global__ void __launch_bounds__(TB, 6) k_tile_eval(Views<float> v, CondHandle lm_cond, int use_cond, Caps cap) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ float4 sXo[TILE_PTS], sHp[TILE_PTS];
+    __shared__ unsigned int s_next;
+    __shared__ double red[2 * (TB / 32)];
+    DevState* st = v.st;
+    const int active = st->lm_active;
+    float js = 0.0f, jc = 0.0f;
+    if (active) eval_tiles<TB>(v, cap, dsm, sXo, sHp, &s_next, blockIdx.x, gridDim.x, js, jc);
+    double in[1], out[1], none;
+    block_sum2c(js, jc, 0.0f, 0.0f, red, in[0], none);
+    if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0)
+        tile_decide(v, active, st->F_res, out[0], lm_cond, use_cond);
+}
+
+// Few tiles: the residual pass at x' and the evaluation of |J h|^2 in one launch (both are bound by
+// latency there, and neither needs the other): blocks below n_tiles take a tile's residuals, the
+// others a tile's |J h|^2.
+template <int TB>
+__global__ void __launch_bounds__(TB, 1) k_tile_step(Views<float> v, CondHandle lm_cond, int use_cond, Caps cap) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ float4 sA[TILE_PTS], sB[TILE_PTS];
+    __shared__ unsigned int s_next;
+    __shared__ double red[2 * (TB / 32)];
+    DevState* st = v.st;
+    const int active = st->lm_active;
+    const bool res = (int)blockIdx.x < v.n_tiles;
+    float s = 0.0f, c = 0.0f;
+    if (active && res) residual_tiles<TB>(v, 1, 0, blockIdx.x, v.n_tiles, sA, sB, s, c);
+    if (active && !res) eval_tiles<TB>(v, cap, dsm, sA, sB, &s_next, (int)blockIdx.x - v.n_tiles, v.n_tiles, s, c);
+    double b, none, in[2], out[2];
+    block_sum2c(s, c, 0.0f, 0.0f, red, b, none);
+    in[0] = res ? b : 0.0;
+    in[1] = res ? 0.0 : b;
+    if (grid_reduce_block<2>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {
+        if (active) st->F_res = 0.5 * out[0];
+        tile_decide(v, active, 0.5 * out[0], out[1], lm_cond, use_cond);
     }
 }
 
@@ -849,6 +885,23 @@ int prepare(K kernel, int tb, size_t dyn) {
     return n;
 }
 
+// Dynamic shared memory of the linearisation: the copies of the point sums, the table.
+size_t lin_smem(const LaunchCfg& L, int tb, bool plain) {
+    return 4 * (size_t)(plain ? tb / 32 : 1) * (3 + PH_STRIDE) * TILE_PTS + L.tl_smem;
+}
+
+template <int TB>
+void tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, float* res_out, float* jac_out,
+                    CondHandle lm_cond, int use_cond) {
+    const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
+    const int grid = TB == TL_TB ? L.tl_grid : std::max(1, v.n_tiles);
+    if (L.tn_plain_q)
+        k_tile_linearize<TB, true><<<grid, TB, lin_smem(L, TB, true), s>>>(v, mode, res_out, jac_out, lm_cond, use_cond, cap);
+    else
+        k_tile_linearize<TB, false><<<grid, TB, lin_smem(L, TB, false), s>>>(v, mode, res_out, jac_out, lm_cond, use_cond,
+                                                                            cap);
+}
+
 }  // namespace
 
 // The tile kernels stage a whole tile's observation table (compact form); a problem
@@ -856,6 +909,7 @@ int prepare(K kernel, int tb, size_t dyn) {
 // (all grids 0).
 void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int max_short_obs, int max_long_runs) {
     L.tn_grid = L.tl_grid = L.te_grid = 0;
+    L.wide_tiles = false;
     L.tk_run_cap = std::max(1, max_long_runs);
     L.tk_short_cap = std::max(1, max_short_obs);
     L.tk_long_cap = (std::max(1, max_long_obs) + 15) / 16 * 16;
@@ -865,10 +919,14 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
     const int bn = std::min(prepare(k_tile_normal<TN_TB, true>, TN_TB, L.tn_smem),
                             prepare(k_tile_normal<TN_TB, false>, TN_TB, L.tn_smem));
     const int bc = prepare(k_tile_cg<TN_TB>, TN_TB, L.tn_smem);
-    const int bl = std::min(prepare(k_tile_linearize<TL_TB, true>, TL_TB, L.tl_smem),
-                            prepare(k_tile_linearize<TL_TB, false>, TL_TB, L.tl_smem));
+    const int bl = std::min(prepare(k_tile_linearize<TL_TB, true>, TL_TB, lin_smem(L, TL_TB, true)),
+                            prepare(k_tile_linearize<TL_TB, false>, TL_TB, lin_smem(L, TL_TB, false)));
     const int be = prepare(k_tile_eval<TE_TB>, TE_TB, L.te_smem);
     if (bn < 1 || bl < 1 || be < 1 || bc < 1) return;
+    L.wide_tiles = n_tiles <= WIDE_TILES * sms &&
+                   std::min({prepare(k_tile_linearize<WIDE_TB, true>, WIDE_TB, lin_smem(L, WIDE_TB, true)),
+                             prepare(k_tile_linearize<WIDE_TB, false>, WIDE_TB, lin_smem(L, WIDE_TB, false)),
+                             prepare(k_tile_step<WIDE_TB>, WIDE_TB, L.te_smem)}) >= 1;
     const int nt = std::max(1, n_tiles);
     L.tn_grid = nt;   // one CTA per tile
     L.tl_grid = std::max(1, std::min({nt, sms * bl, MAX_GRID}));
@@ -892,18 +950,14 @@ void launch_cg_round(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, 
 
 void launch_tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, float* res_out,
                            float* jac_out, CondHandle lm_cond, int use_cond) {
-    const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
-    if (L.tn_plain_q)
-        k_tile_linearize<TL_TB, true><<<L.tl_grid, TL_TB, L.tl_smem, s>>>(v, mode, res_out, jac_out, lm_cond, use_cond,
-                                                                        cap);
-    else
-        k_tile_linearize<TL_TB, false><<<L.tl_grid, TL_TB, L.tl_smem, s>>>(v, mode, res_out, jac_out, lm_cond,
-                                                                         use_cond, cap);
+    if (L.wide_tiles) tile_linearize<WIDE_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
+    else tile_linearize<TL_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
 }
 
 void launch_tile_eval(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle lm_cond, int use_cond) {
-    k_tile_eval<TE_TB><<<L.te_grid, TE_TB, L.te_smem, s>>>(v, lm_cond, use_cond,
-                                                           Caps{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap});
+    const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
+    if (L.wide_tiles) k_tile_step<WIDE_TB><<<2 * std::max(1, v.n_tiles), WIDE_TB, L.te_smem, s>>>(v, lm_cond, use_cond, cap);
+    else k_tile_eval<TE_TB><<<L.te_grid, TE_TB, L.te_smem, s>>>(v, lm_cond, use_cond, cap);
 }
 
 }  // namespace gbba
