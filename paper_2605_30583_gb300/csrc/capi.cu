@@ -227,7 +227,7 @@ static void step_init(ba_problem* p, cudaStream_t s, CondHandle lm_c, int use) {
 static void step_pcg_iter(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int use) {
     if (p->precision == BA_PREC_MIXED && p->use_schur) {   // reduced camera system
         const Views<float>& v = p->vf;
-        launch_schur(v, s, 1, &v.st->pcg_active);
+        launch_schur(v, p->L, s, SCHUR_MV, &v.st->pcg_active);
         launch_update(v, p->L, s, pcg_c, use, 1);
     } else if (p->precision == BA_PREC_MIXED && p->use_cg) {
         const Views<float>& v = p->vf;
@@ -249,7 +249,7 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
         // blocks of H' (camera and point inverses, D), then the reduced right-hand side
         const Views<float>& v = p->vf;
         launch_precond(v, p->L, s, pcg_c, 0, nullptr, 1);
-        launch_schur(v, s, 0, &v.st->lm_active);
+        launch_schur(v, p->L, s, SCHUR_RHS, &v.st->lm_active);
         launch_schur_start(v, p->L, s, pcg_c, use);
     } else if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
@@ -269,7 +269,7 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
 static void step_lm_tail(ba_problem* p, cudaStream_t s, CondHandle lm_c, int use) {
     if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        if (p->use_schur) launch_schur(v, s, 2, &v.st->lm_active);   // points back-substituted
+        if (p->use_schur) launch_schur(v, p->L, s, SCHUR_BACK, &v.st->lm_active);   // points back-substituted
         launch_candidate(v, p->L, s);
         // r(x') and F' (the relinearisation reuses r); few tiles: in the evaluation's launch
         if (!p->L.wide_tiles) launch_residual(v, p->L, s, 1);

@@ -78,7 +78,9 @@ void launch_cg_round(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, 
 void launch_tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, float* res_out,
                            float* jac_out, CondHandle lm_cond, int use_cond);
 // Schur-complement PCG (kernels_mixed.cu): mode 0 right-hand side, 1 operator, 2 back-substitution
-void launch_schur(const Views<float>& v, cudaStream_t s, int mode, const int32_t* gate);
+enum : int { SCHUR_RHS = 0, SCHUR_MV = 1, SCHUR_BACK = 2 };
+void launch_schur(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, const int32_t* gate);
+void launch_tile_schur(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, const int32_t* gate);
 void launch_schur_start(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use);
 // pose factors (pose_factor.cu); no-ops without factors
 void launch_factor_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode);

@@ -828,8 +828,6 @@ __global__ void k_commit(Views<float> v) {
 // J_c^T W (J_c d - J_p z).  The camera PCG vectors use the camera segments of r z p h
 // and k_update in its cameras-only form.
 
-enum : int { SCHUR_RHS = 0, SCHUR_MV = 1, SCHUR_BACK = 2 };
-
 // t = J_c d for a camera direction record d (no point part)
 __device__ __forceinline__ void jc_apply(const GeoLite& g, const Cam& c, const float (&dir)[9], float& t0, float& t1) {
     const float dP0 = fmaf(dir[1], g.RX[2], -dir[2] * g.RX[1]) + dir[CD_T + 0];
@@ -1018,34 +1016,32 @@ __global__ void k_schur_start(Views<float> v, CondHandle pcg_cond, int use_cond)
         return;
     }
     double rz = 0.0, rr = 0.0;
-    FOR_CAMERAS(c, v) {
-        const size_t e = 9 * (size_t)c;
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    // nine lanes a camera, three cameras a warp (as k_update)
+    for (int cw = 3 * ((int)blockIdx.x * wpb + ((int)threadIdx.x >> 5)); cw < v.n_cams; cw += 3 * wpb * (int)gridDim.x) {
+        const int sub = lane / 9, base = 9 * sub;
+        const bool live = lane < 27 && cw + sub < v.n_cams;
+        const int c = live ? cw + sub : cw, i = live ? lane - base : 0, i3 = i < 3 ? i : 0;
+        const size_t e = 9 * (size_t)c + i;
         float* ca = v.cam_acc + (size_t)c * CA_STRIDE;
         const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
-        const double* cl = v.cam_lin + (size_t)c * CL_STRIDE;
-        float q[9], rn[9];
+        const float* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * i;
+        const float a = ca[i];
+        const float a0 = __shfl_sync(FULL, a, base), a1 = __shfl_sync(FULL, a, base + 1);
+        const float a2 = __shfl_sync(FULL, a, base + 2);
+        const float q = i < 3 ? fmaf(JL[i3], a0, fmaf(JL[3 + i3], a1, JL[6 + i3] * a2)) : a;
+        const float rn = (float)(-v.cam_lin[(size_t)c * CL_STRIDE + CL_G + i]) + q;
+        float z = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) q[k] = fmaf(JL[k], ca[0], fmaf(JL[3 + k], ca[1], JL[6 + k] * ca[2]));
-#pragma unroll
-        for (int k = 3; k < 9; ++k) q[k] = ca[k];
-#pragma unroll
-        for (int k = 0; k < CA_STRIDE; ++k) ca[k] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            rn[k] = (float)(-cl[CL_G + k]) + q[k];
-            v.r[e + k] = rn[k];
-            v.p[e + k] = 0.0f;
-            v.h[e + k] = 0.0f;
-        }
-        const float* M = v.Minv_c + (size_t)c * MC_STRIDE;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            float z = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) z = fmaf(M[9 * i + k], rn[k], z);
-            v.z[e + i] = z;
-            rz += (double)rn[i] * (double)z;
-            rr += (double)rn[i] * (double)rn[i];
+        for (int k = 0; k < 9; ++k) z = fmaf(M[k], __shfl_sync(FULL, rn, base + k), z);
+        if (live) {
+            ca[i] = 0.0f;
+            v.r[e] = rn;
+            v.p[e] = 0.0f;
+            v.h[e] = 0.0f;
+            v.z[e] = z;
+            rz += (double)rn * (double)z;
+            rr += (double)rn * (double)rn;
         }
     }
     double in[2] = {rz, rr}, out[2];
@@ -1198,25 +1194,37 @@ void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, C
     const int pt_blocks = std::max(1, std::min(grid_items(L, v.n_pts), L.item_grid - cam_blocks));
     k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, pslots, cam_blocks, zero);
 }
-void launch_matvec(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
-                   const float* zs, int use_beta) {
+static void launch_cam_direction(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
+                                 const float* zs, int use_beta) {
     // one thread per camera entry, no more blocks than that needs (each adds one slot sum)
     const int cd_grid = std::max(1, std::min(L.item_grid, (9 * v.n_cams + L.item_block - 1) / L.item_block));
     k_cam_direction<<<cd_grid, L.item_block, 0, s>>>(v, gate, zs, use_beta);
+}
+void launch_matvec(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
+                   const float* zs, int use_beta) {
+    launch_cam_direction(v, L, s, gate, zs, use_beta);
     if (L.tn_grid > 0)   // tiles with their camera tables in shared memory
         launch_tile_normal(v, L, s, gate, zs, use_beta);
     else
         k_matvec<MV_TB><<<v.n_tiles > 0 ? v.n_tiles : 1, MV_TB, 0, s>>>(v, gate, zs, use_beta);
     launch_factor_matvec(v, L, s, gate, zs, use_beta);   // pose factors, if any
 }
-void launch_schur(const Views<float>& v, cudaStream_t s, int mode, const int32_t* gate) {
+void launch_schur(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, const int32_t* gate) {
+    if (L.tn_grid > 0 && L.tn_plain_q) {   // tables in shared memory, no camera observes a point twice
+        // p_c = z + beta p_c (its p^T D p goes to the slot sums), or the record of h_c (whose
+        // sum nothing reads: the next preconditioner clears it)
+        if (mode != SCHUR_RHS) launch_cam_direction(v, L, s, gate, mode == SCHUR_MV ? v.z : v.h, mode == SCHUR_MV);
+        launch_tile_schur(v, L, s, mode, gate);
+        return;
+    }
     const int grid = v.n_tiles > 0 ? v.n_tiles : 1;
     if (mode == SCHUR_RHS) k_schur<MV_TB, SCHUR_RHS><<<grid, MV_TB, 0, s>>>(v, gate);
     else if (mode == SCHUR_MV) k_schur<MV_TB, SCHUR_MV><<<grid, MV_TB, 0, s>>>(v, gate);
     else k_schur<MV_TB, SCHUR_BACK><<<grid, MV_TB, 0, s>>>(v, gate);
 }
 void launch_schur_start(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
-    k_schur_start<<<grid_cams(L, v.n_cams), L.item_block, 0, s>>>(v, c, use);
+    const int cpb = 3 * (L.item_block / 32);
+    k_schur_start<<<std::max(1, std::min((v.n_cams + cpb - 1) / cpb, L.item_grid)), L.item_block, 0, s>>>(v, c, use);
 }
 void launch_update(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
                    int cameras_only) {

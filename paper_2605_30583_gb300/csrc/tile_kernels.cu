@@ -871,6 +871,191 @@ __global__ void __launch_bounds__(TB, 1) k_tile_step(Views<float> v, CondHandle 
     }
 }
 
+// ------------------------------------------------------------------ Schur complement ---
+// k_schur (kernels_mixed.cu) in the tile kernels' form: the camera direction records come from
+// k_cam_direction, a tile's long runs are walked in camera-uniform steps and every warp adds its
+// point sums into a copy of its own.  Modes as there: SCHUR_RHS camera sums of J_c^T W J_p z,
+// z = H'pp^-1 g_p; SCHUR_MV camera sums of J_c^T W (J_c d - J_p z), z = H'pp^-1 y,
+// y = J_p^T W J_c d, and sum w |J_c d|^2 - sum y^T z; SCHUR_BACK h_p = H'pp^-1 (-g_p - y).
+constexpr int TS_TB = 256;
+
+// One pass over the tile: visit(camera, direction, geometry, slot, weight, observation's sums).
+template <int TB, bool GEN, bool DIR, bool CAMS, typename F>
+__device__ __forceinline__ void schur_pass(const Views<float>& v, const TileRange& T, const uint32_t* sRun,
+                                           const uint32_t* sShort, const uint8_t* sSlot, const float4* sX4,
+                                           unsigned int* s_next, float eps, bool weighted, F&& visit) {
+    const int lane = threadIdx.x & 31;
+    const OpDir none = {};
+    float acc[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
+    for (;;) {
+        unsigned int r = 0;
+        if (lane == 0) r = atomicAdd(s_next, 1u);
+        r = __shfl_sync(FULL, r, 0);
+        if (r >= T.nl) break;
+        const uint32_t start = sRun[3 * r] - T.lo, len = sRun[3 * r + 1], c = sRun[3 * r + 2];
+        const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
+        const OpCam oc = op_cam(cam);
+        OpDir od = none;
+        if (DIR) {
+            float dir[9];
+            load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
+            od = op_dir(cam, dir);
+        }
+        for (uint32_t off = lane; off < len; off += 32) {
+            const uint32_t slot = sSlot[start + off];
+            const float4 x = sX4[slot];
+            visit(oc, od, op_geo<GEN>(oc, x.x, x.y, x.z, eps), slot,
+                  GEN && weighted ? __ldg(v.obs_w + T.lo + start + off) : 1.0f, acc, true);
+        }
+        __syncwarp();   // the warp's next run may meet the same points
+        if (CAMS) {
+            op_finish(oc, cam.k1, cam.k2, acc);
+            int idx;
+            const int nv = warp_split_sum<9>(acc, lane, idx);
+            if (nv > 0) atomicAdd(v.cam_acc + (size_t)c * CA_STRIDE + idx, acc[0]);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
+        }
+    }
+    const uint32_t n = T.hi - T.ss;
+    const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
+    const uint32_t a = T.ss + min(threadIdx.x * chunk, n), b = T.ss + min(threadIdx.x * chunk + chunk, n);
+    uint32_t cur = NO_CAM;
+    OpCam oc;
+    OpDir od = none;
+    float k1 = 0.0f, k2 = 0.0f;
+    for (uint32_t j = a; j < b; ++j) {
+        const uint32_t key = sShort[j - T.ss];
+        const uint32_t c = key >> 8, slot = key & 0xffu;
+        if (c != cur) {
+            if (CAMS && cur != NO_CAM) {
+                op_finish(oc, k1, k2, acc);
+                flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
+            }
+            cur = c;
+            const Cam cam = load_cam(v.cam_pre + (size_t)c * CP_STRIDE);
+            oc = op_cam(cam);
+            k1 = cam.k1;
+            k2 = cam.k2;
+            if (DIR) {
+                float dir[9];
+                load_dir(v.cam_dir + (size_t)c * CD_STRIDE, dir);
+                od = op_dir(cam, dir);
+            }
+        }
+        const float4 x = sX4[slot];
+        visit(oc, od, op_geo<GEN>(oc, x.x, x.y, x.z, eps), slot, GEN && weighted ? __ldg(v.obs_w + j) : 1.0f, acc, false);
+    }
+    if (CAMS && cur != NO_CAM) {
+        op_finish(oc, k1, k2, acc);
+        flush_matvec(v.cam_acc + (size_t)cur * CA_STRIDE, acc);
+    }
+}
+
+template <int TB, int MODE, bool GEN>
+__device__ __forceinline__ void tile_schur(const Views<float>& v, const TileRange& T, const Caps& cap,
+                                           unsigned char* dsm, float4* sX4, float* sY, float4* sZ4,
+                                           unsigned int* s_next, float eps, bool weighted, float& ts, float& tc) {
+    constexpr int NW = TB / 32;
+    float* const y = sY + (threadIdx.x >> 5) * 3 * TILE_PTS;   // this warp's copy
+    uint32_t *sRun, *sShort;
+    uint8_t* sSlot;
+    for (int i = threadIdx.x; i < T.npt; i += TB) {
+        const size_t e = T.base + 3 * i;
+        sX4[i] = make_float4(v.x[e], v.x[e + 1], v.x[e + 2], 0.0f);
+    }
+    for (int i = threadIdx.x; MODE != SCHUR_RHS && i < NW * 3 * TILE_PTS; i += TB) sY[i] = 0.0f;
+    stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
+    if (threadIdx.x < 2) s_next[threadIdx.x] = 0u;
+    __syncthreads();
+    if (MODE != SCHUR_RHS) {
+        schur_pass<TB, GEN, true, false>(v, T, sRun, sShort, sSlot, sX4, s_next, eps, weighted,
+            [&](const OpCam& oc, const OpDir& od, const OpGeo& g, uint32_t slot, float w, float (&)[9], bool plain) {
+                float t0, t1, u[9], v0, v1, v2;
+                op_forward<GEN>(oc, od, g, 0.0f, 0.0f, 0.0f, t0, t1);
+                if (MODE == SCHUR_MV) kahan_add(ts, tc, w * fmaf(t0, t0, t1 * t1));
+#pragma unroll
+                for (int k = 0; k < 9; ++k) u[k] = 0.0f;   // camera part: not wanted
+                op_adjoint<GEN>(g, w * t0, w * t1, u, v0, v1, v2);
+                float* q = y + 3 * slot;
+                if (plain) {
+                    op_point(oc, v0, v1, v2, q[0], q[1], q[2]);
+                } else {   // lanes of a warp may meet one point in the short runs
+                    float q0 = 0.0f, q1 = 0.0f, q2 = 0.0f;
+                    op_point(oc, v0, v1, v2, q0, q1, q2);
+                    atomicAdd(q, q0);
+                    atomicAdd(q + 1, q1);
+                    atomicAdd(q + 2, q2);
+                }
+            });
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < T.npt; i += TB) {
+        const size_t e = T.base + 3 * i;
+        const float* m = v.Minv_p + MP_STRIDE * (size_t)(T.pt0 + i);
+        float b[3] = {0.0f, 0.0f, 0.0f};
+        if (MODE != SCHUR_RHS) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                for (int w = 0; w < NW; ++w) b[k] += sY[w * 3 * TILE_PTS + 3 * i + k];
+        }
+        if (MODE == SCHUR_RHS) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) b[k] = v.g[e + k];
+        } else if (MODE == SCHUR_BACK) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) b[k] = -v.g[e + k] - b[k];
+        }
+        const float z0 = fmaf(m[0], b[0], fmaf(m[1], b[1], m[2] * b[2]));
+        const float z1 = fmaf(m[1], b[0], fmaf(m[3], b[1], m[4] * b[2]));
+        const float z2 = fmaf(m[2], b[0], fmaf(m[4], b[1], m[5] * b[2]));
+        if (MODE == SCHUR_BACK) {
+            v.h[e] = z0;
+            v.h[e + 1] = z1;
+            v.h[e + 2] = z2;
+        } else {
+            sZ4[i] = make_float4(z0, z1, z2, 0.0f);
+            if (MODE == SCHUR_MV) kahan_add(ts, tc, -fmaf(b[0], z0, fmaf(b[1], z1, b[2] * z2)));
+        }
+    }
+    if (MODE != SCHUR_BACK) {
+        __syncthreads();
+        schur_pass<TB, GEN, MODE == SCHUR_MV, true>(v, T, sRun, sShort, sSlot, sX4, s_next + 1, eps, weighted,
+            [&](const OpCam& oc, const OpDir& od, const OpGeo& g, uint32_t slot, float w, float (&acc)[9], bool) {
+                const float4 z = sZ4[slot];
+                const float sg = MODE == SCHUR_MV ? -1.0f : 1.0f;
+                float t0, t1, v0, v1, v2;
+                op_forward<GEN>(oc, od, g, sg * z.x, sg * z.y, sg * z.z, t0, t1);
+                op_adjoint<GEN>(g, w * t0, w * t1, acc, v0, v1, v2);
+            });
+    }
+}
+
+template <int TB, int MODE>
+__global__ void __launch_bounds__(TB) k_tile_schur(Views<float> v, const int32_t* gate, Caps cap) {
+    if (gated_off(gate)) return;
+    constexpr int NW = TB / 32;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ float4 sX4[TILE_PTS], sZ4[TILE_PTS];
+    __shared__ float sY[NW * 3 * TILE_PTS];
+    __shared__ unsigned int s_next[2];
+    __shared__ double red[2 * NW];
+    DevState* st = v.st;
+    const float eps = (float)st->opt.eps;
+    const bool weighted = st->opt.loss != 0;
+    const TileRange T = tile_range(v, blockIdx.x);
+    float ts = 0.0f, tc = 0.0f;   // Kahan pair
+    if (weighted || eps != 0.0f) tile_schur<TB, MODE, true>(v, T, cap, dsm, sX4, sY, sZ4, s_next, eps, weighted, ts, tc);
+    else tile_schur<TB, MODE, false>(v, T, cap, dsm, sX4, sY, sZ4, s_next, eps, weighted, ts, tc);
+    if (MODE == SCHUR_MV) {
+        double b, none;
+        block_sum2c(ts, tc, 0.0f, 0.0f, red, b, none);
+        if (threadIdx.x == 0) slot_add(st->acc_mv, 0, b);
+    }
+}
+
 template <typename K>
 int prepare(K kernel, int tb, size_t dyn) {
     if (ensure_dynamic_smem((const void*)kernel, (int)dyn) != cudaSuccess) {
@@ -922,7 +1107,10 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
     const int bl = std::min(prepare(k_tile_linearize<TL_TB, true>, TL_TB, lin_smem(L, TL_TB, true)),
                             prepare(k_tile_linearize<TL_TB, false>, TL_TB, lin_smem(L, TL_TB, false)));
     const int be = prepare(k_tile_eval<TE_TB>, TE_TB, L.te_smem);
-    if (bn < 1 || bl < 1 || be < 1 || bc < 1) return;
+    const int bs = std::min({prepare(k_tile_schur<TS_TB, SCHUR_RHS>, TS_TB, L.tn_smem),
+                             prepare(k_tile_schur<TS_TB, SCHUR_MV>, TS_TB, L.tn_smem),
+                             prepare(k_tile_schur<TS_TB, SCHUR_BACK>, TS_TB, L.tn_smem)});
+    if (bn < 1 || bl < 1 || be < 1 || bc < 1 || bs < 1) return;
     L.wide_tiles = n_tiles <= WIDE_TILES * sms &&
                    std::min({prepare(k_tile_linearize<WIDE_TB, true>, WIDE_TB, lin_smem(L, WIDE_TB, true)),
                              prepare(k_tile_linearize<WIDE_TB, false>, WIDE_TB, lin_smem(L, WIDE_TB, false)),
@@ -952,6 +1140,13 @@ void launch_tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream
                            float* jac_out, CondHandle lm_cond, int use_cond) {
     if (L.wide_tiles) tile_linearize<WIDE_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
     else tile_linearize<TL_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
+}
+
+void launch_tile_schur(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, const int32_t* gate) {
+    const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
+    if (mode == SCHUR_RHS) k_tile_schur<TS_TB, SCHUR_RHS><<<L.tn_grid, TS_TB, L.tn_smem, s>>>(v, gate, cap);
+    else if (mode == SCHUR_MV) k_tile_schur<TS_TB, SCHUR_MV><<<L.tn_grid, TS_TB, L.tn_smem, s>>>(v, gate, cap);
+    else k_tile_schur<TS_TB, SCHUR_BACK><<<L.tn_grid, TS_TB, L.tn_smem, s>>>(v, gate, cap);
 }
 
 void launch_tile_eval(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle lm_cond, int use_cond) {
