@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <iterator>
 #include <new>
 #include <thread>
 #include <vector>
@@ -77,12 +78,15 @@ Layout compute_layout(int32_t n_cams, int32_t n_pts, int64_t n_obs, int32_t prec
     l.staging = b.take(8 * (9 * nc + 3 * np));
     l.blk_tile = b.take(4 * (MAX_PBLOCKS + 1));
     l.blk_cam_off = b.take(4 * (MAX_PBLOCKS + 1));
+    l.blk_fac = b.take(4 * (MAX_PBLOCKS + 1));
     // per-CTA camera lists of the persistent PCG kernel: each CTA lists the cameras of
     // its observations and pose factors, and every other camera is listed once, so
     // n_obs + 2 n_fac + n_cams + MAX_PBLOCKS entries always suffice; the plan is only
     // used when they fit in shared memory, so cap the region
     const size_t nfc = 2 * (size_t)std::max(0, n_fac);
     l.blk_cams = b.take(4 * std::min(no + nfc + nc + MAX_PBLOCKS, (size_t)(MAX_PBLOCKS * 4096)));
+    // bitmap of the cameras that each CTA's observations see (while the plan is made)
+    l.blk_seen = precision == BA_PREC_FP64 ? 0 : b.take(4 * (size_t)MAX_PBLOCKS * ((nc + 31) / 32));
     l.pslots = b.take(8 * PSLOT_TOTAL);
     // long-run tables: a tile holds at most (its observations / LONG_RUN) long runs
     l.long_off = b.take(4 * (n_tiles + 1));
@@ -256,7 +260,7 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
         launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->pslots : nullptr,
                        p->use_persistent ? 0 : (p->use_cg ? 2 : 1));
         if (p->use_persistent)
-            launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->pslots, p->p_grid,
+            launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->pslots, p->p_grid,
                                   p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one, p->p_form, s);
     } else {
         launch64_precond(p->vd, p->L, s, pcg_c, use);
@@ -460,9 +464,9 @@ ba_status ba_options_default(ba_options* o) {
 namespace {
 
 // Validation of the observation arrays and their copy into the problem, split over the
-// host's cores for large problems (one pass over 28.8M observations on one core takes
-// ~0.2 s).  Each thread takes a contiguous range of observations: it checks the indices
-// and pixels up to its first bad observation, copies its range, and marks the points it
+// host's cores (one pass over 28.8M observations on one core takes ~0.2 s).  Each thread
+// takes a contiguous range of observations: it checks the indices and pixels up to its first
+// bad observation, copies its range, and marks the points it
 // sees in two bitmaps of its own (seen once, seen at least twice).  The bitmaps are then
 // merged word by word over the threads, and the first bad observation or the first point
 // seen fewer than twice is reported, as a sequential pass would report it.
@@ -477,7 +481,8 @@ ObsCheck check_and_copy_observations(int32_t n_cams, int32_t n_pts, int64_t n_ob
                                      const uint32_t* pt_idx, const double* pixels, uint32_t* cam_out,
                                      uint32_t* pt_out, double* px_out) {
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const int nt = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)hw, 16, n_obs >> 20}));
+    // a thread per 128K observations: below that its start costs what it saves
+    const int nt = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)hw, 16, n_obs >> 17}));
     const size_t words = ((size_t)n_pts + 63) / 64;
     std::vector<uint64_t> once((size_t)nt * words, 0ull), twice((size_t)nt * words, 0ull);
     std::vector<int64_t> first_bad(nt, -1);
@@ -698,8 +703,9 @@ static ba_status write_options(ba_problem* p, const ba_options* o);
 
 // Persistent PCG plan: one CTA per SM, contiguous tile runs balanced by observation
 // count; a form is used only when every CTA's keys and point state fit in its shared
-// memory.  Each CTA lists the cameras of its observations and of its pose factors
-// (factor k runs in CTA k % G); a camera that neither sees is listed by CTA c % G, and
+// memory.  Each CTA lists the cameras of its observations and of its pose factors (a factor
+// goes to a CTA whose observations see both of its cameras, where there is one, so that the
+// list hardly grows); a camera that neither sees is listed by CTA c % G, and
 // the first list holding a camera owns it.
 static ba_status plan_persistent(ba_problem* p, int sms) {
     const int nt = p->n_tiles;
@@ -717,38 +723,59 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
     }
     bt[G] = (uint32_t)nt;
     const size_t limit = (size_t)std::max(0, persistent_max_smem() - 4096);
-    auto point_bytes = [&](int b) {
+    auto smem_bytes = [&](bool one, int b, size_t ncb) {
         const size_t no = off[bt[b + 1]] - off[bt[b]];
         const long pb = (long)bt[b] * TILE_PTS, pe = std::min((long)bt[b + 1] * TILE_PTS, (long)p->n_pts);
-        const size_t np = pe > pb ? (size_t)(pe - pb) : 0;
-        const size_t n3p = (3 * np + 3) & ~(size_t)3;
-        // keys, X and p as float4, D r z h q as 3-float arrays, M^-1 (6 per point)
-        return ((4 * no + 15) & ~(size_t)15) + 32 * np + 4 * (5 * n3p + ((6 * np + 3) & ~(size_t)3));
+        return pcg_smem_bytes(one, no, pe > pb ? (size_t)(pe - pb) : 0, ncb);
     };
-    size_t worst = 0;
-    for (int b = 0; b < G; ++b) worst = std::max(worst, point_bytes(b));
-    if (worst > limit) return BA_OK;   // too large: the multi-kernel PCG path is used
-    // distinct cameras of each CTA's observations (sorted), then the unseen ones
-    std::vector<uint32_t> keys((size_t)p->n_obs);
-    GBBA_CUDA(cudaMemcpy(keys.data(), p->vf.obs_key, 4 * keys.size(), cudaMemcpyDeviceToHost));
+    for (int b = 0; b < G; ++b)   // too large: the multi-kernel PCG path is used
+        if (bt[b + 1] - bt[b] > (uint32_t)MAX_CTA_TILES || smem_bytes(false, b, 0) > limit) return BA_OK;
+    // distinct cameras of each CTA's observations: a bit per CTA and camera, set on the device
+    // (bringing the keys to the host and sorting them there took most of a bind), read here in
+    // camera order; then the unseen cameras
+    GBBA_CUDA(cudaMemcpyAsync(p->blk_tile, bt.data(), 4 * bt.size(), cudaMemcpyHostToDevice, p->stream));
+    const size_t words = ((size_t)p->n_cams + 31) / 32;
+    uint32_t* seen_dev = (uint32_t*)(p->ws + p->lay.blk_seen);
+    GBBA_CUDA(cudaMemsetAsync(seen_dev, 0, 4 * words * (size_t)G, p->stream));
+    launch_mark_cameras(p->vf, p->blk_tile, G, seen_dev, p->stream);
+    GBBA_CUDA(cudaGetLastError());
+    std::vector<uint32_t> bits(words * (size_t)G);
+    GBBA_CUDA(cudaMemcpyAsync(bits.data(), seen_dev, 4 * bits.size(), cudaMemcpyDeviceToHost, p->stream));
+    GBBA_CUDA(cudaStreamSynchronize(p->stream));
     std::vector<std::vector<uint32_t>> lists((size_t)G);
     std::vector<char> seen((size_t)p->n_cams, 0);
-    for (int b = 0; b < G; ++b) {
-        std::vector<uint32_t>& cb = lists[b];
-        for (uint32_t j = off[bt[b]]; j < off[bt[b + 1]]; ++j) cb.push_back(keys[j] >> 8);
-        std::sort(cb.begin(), cb.end());
-        cb.erase(std::unique(cb.begin(), cb.end()), cb.end());
-        for (uint32_t c : cb) seen[c] = 1;
-    }
-    // pose factor k runs in CTA k % G, which lists both of its cameras
-    for (int32_t k = 0; k < p->n_fac; ++k)
-        for (int e = 0; e < 2; ++e) {
-            const uint32_t c = p->fac_cam[2 * (size_t)k + e];
-            std::vector<uint32_t>& cb = lists[k % G];
-            auto it = std::lower_bound(cb.begin(), cb.end(), c);
-            if (it == cb.end() || *it != c) cb.insert(it, c);
-            seen[c] = 1;
+    for (int b = 0; b < G; ++b)
+        for (size_t w = 0; w < words; ++w)
+            for (uint32_t m = bits[words * (size_t)b + w]; m; m &= m - 1) {
+                const uint32_t c = (uint32_t)(32 * w) + (uint32_t)__builtin_ctz(m);
+                lists[b].push_back(c);
+                seen[c] = 1;
+            }
+    // pose factors: to the least loaded CTA that sees both cameras, else one that sees one of them
+    std::vector<std::vector<int32_t>> fac_of((size_t)G);
+    if (p->n_fac > 0) {
+        std::vector<std::vector<int>> where((size_t)p->n_cams);
+        for (int b = 0; b < G; ++b)
+            for (uint32_t c : lists[b]) where[c].push_back(b);
+        for (int32_t k = 0; k < p->n_fac; ++k) {
+            const uint32_t ca = p->fac_cam[2 * (size_t)k], cb = p->fac_cam[2 * (size_t)k + 1];
+            std::vector<int> both;
+            std::set_intersection(where[ca].begin(), where[ca].end(), where[cb].begin(), where[cb].end(),
+                                  std::back_inserter(both));
+            const std::vector<int>& cand = !both.empty() ? both : (!where[ca].empty() ? where[ca] : where[cb]);
+            int best = k % G;
+            if (!cand.empty())
+                best = *std::min_element(cand.begin(), cand.end(),
+                                         [&](int x, int y) { return fac_of[x].size() < fac_of[y].size(); });
+            fac_of[best].push_back(k);
+            for (const uint32_t c : {ca, cb}) {
+                std::vector<uint32_t>& list = lists[best];
+                auto it = std::lower_bound(list.begin(), list.end(), c);
+                if (it == list.end() || *it != c) list.insert(it, c);
+                seen[c] = 1;
+            }
         }
+    }
     for (int c = 0; c < p->n_cams; ++c)
         if (!seen[c]) {
             std::vector<uint32_t>& cb = lists[c % G];
@@ -763,14 +790,10 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
             seen[c] = 1;
         }
         coff[b + 1] = (uint32_t)cams.size();
-        const size_t ncb = lists[b].size();
-        const size_t no = off[bt[b + 1]] - off[bt[b]];
-        const long pb = (long)bt[b] * TILE_PTS, pe = std::min((long)bt[b + 1] * TILE_PTS, (long)p->n_pts);
-        const size_t np = pe > pb ? (size_t)(pe - pb) : 0;
-        worst_two = std::max(worst_two, point_bytes(b) + 4 * ((ncb + 3) & ~(size_t)3) + 4 * 28 * ncb);
-        worst_one = std::max(worst_one, pcg1_smem_bytes(no, np, ncb));
+        worst_two = std::max(worst_two, smem_bytes(false, b, lists[b].size()));
+        worst_one = std::max(worst_one, smem_bytes(true, b, lists[b].size()));
     }
-    const size_t cap = (p->lay.pslots - p->lay.blk_cams) / 4;
+    const size_t cap = (p->lay.blk_seen - p->lay.blk_cams) / 4;
     if (cams.size() > cap) return BA_OK;
     auto fits = [&](int form, size_t bytes) {
         int bps = 0;
@@ -784,9 +807,25 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
     p->fits_one = fits(PCG_ONE_EXCHANGE, worst_one);
     p->fits_two = fits(PCG_TWO_EXCHANGE, worst_two);
     if (!p->fits_one && !p->fits_two) return BA_OK;
-    GBBA_CUDA(cudaMemcpy(p->blk_tile, bt.data(), 4 * bt.size(), cudaMemcpyHostToDevice));
     GBBA_CUDA(cudaMemcpy(p->blk_cam_off, coff.data(), 4 * coff.size(), cudaMemcpyHostToDevice));
     GBBA_CUDA(cudaMemcpy(p->blk_cams, cams.data(), 4 * cams.size(), cudaMemcpyHostToDevice));
+    // the factors in the order of their CTAs
+    std::vector<uint32_t> foff((size_t)G + 1, 0), fcam;
+    std::vector<double> fmeas, fsqrt;
+    for (int b = 0; b < G; ++b) {
+        for (const int32_t k : fac_of[b]) {
+            fcam.insert(fcam.end(), &p->fac_cam[2 * (size_t)k], &p->fac_cam[2 * (size_t)k] + 2);
+            fmeas.insert(fmeas.end(), &p->fac_meas[6 * (size_t)k], &p->fac_meas[6 * (size_t)k] + 6);
+            fsqrt.insert(fsqrt.end(), &p->fac_sqrt[6 * (size_t)k], &p->fac_sqrt[6 * (size_t)k] + 6);
+        }
+        foff[b + 1] = foff[b] + (uint32_t)fac_of[b].size();
+    }
+    GBBA_CUDA(cudaMemcpy(p->blk_fac, foff.data(), 4 * foff.size(), cudaMemcpyHostToDevice));
+    if (p->n_fac > 0) {
+        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_cam, fcam.data(), 4 * fcam.size(), cudaMemcpyHostToDevice));
+        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_meas, fmeas.data(), 8 * fmeas.size(), cudaMemcpyHostToDevice));
+        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_sqrt, fsqrt.data(), 8 * fsqrt.size(), cudaMemcpyHostToDevice));
+    }
     p->persistent = true;
     p->p_grid = G;
     p->p_smem_one = (int)worst_one;
@@ -877,6 +916,7 @@ ba_status ba_bind_workspace(ba_problem* p, void* ws, size_t bytes, void* stream)
     p->blk_tile = (uint32_t*)(w + l.blk_tile);
     p->blk_cam_off = (uint32_t*)(w + l.blk_cam_off);
     p->blk_cams = (uint32_t*)(w + l.blk_cams);
+    p->blk_fac = (uint32_t*)(w + l.blk_fac);
     p->pslots = (double*)(w + l.pslots);
     p->persistent = p->fits_one = p->fits_two = false;
     if (p->precision == BA_PREC_MIXED) {
@@ -1276,8 +1316,8 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
             open_gates();
             launch_precond(v, p->L, s, 0, 0, p->pslots, 0);
             cudaEventRecord(e0, s);
-            GBBA_CUDA(launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->pslots, p->p_grid,
-                                            p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one,
+            GBBA_CUDA(launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->pslots,
+                                            p->p_grid, p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one,
                                             p->p_form, s));
             cudaEventRecord(e1, s);
             cudaEventSynchronize(e1);

@@ -112,20 +112,24 @@ void launch_selftest_rcp64(const double* x, double* y, int64_t n, cudaStream_t s
 cudaError_t launch_selftest_wait(void* scratch, int grid, long long timeout_ns, cudaStream_t s);
 cudaError_t persistent_prepare(int form, int smem_bytes, int* blocks_per_sm);
 cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_tile, const uint32_t* blk_cam_off,
-                                  const uint32_t* blk_cams, double* pslots, int grid, int smem_bytes, int form,
-                                  cudaStream_t s);
-// Dynamic shared memory of the one-exchange kernel for a CTA with `no` observations,
-// `np` points and `ncb` listed cameras, in the order the kernel carves it.
-__host__ __device__ inline size_t pcg1_smem_bytes(size_t no, size_t np, size_t ncb) {
+                                  const uint32_t* blk_cams, const uint32_t* blk_fac, double* pslots, int grid,
+                                  int smem_bytes, int form, cudaStream_t s);
+// Dynamic shared memory of the persistent kernels for a CTA with `no` observations, `np`
+// points and `ncb` listed cameras, in the order the kernels carve it: keys; X and the
+// direction as float4 (their fourth entries hold D_0 and D_1 in the one-exchange form); five
+// vectors (and D_2); M^-1 blocks; camera ids (and owner bits), records and directions, and in
+// the one-exchange form the cameras' u, p, s, r, h.
+__host__ __device__ inline size_t pcg_smem_bytes(bool one_exchange, size_t no, size_t np, size_t ncb) {
     const size_t n3p = (3 * np + 3) & ~(size_t)3;
-    size_t b = (4 * no + 15) & ~(size_t)15;          // observation keys
-    b += 32 * np;                                     // (X, D_0) and (u, D_1) as float4
-    b += 4 * ((np + 3) & ~(size_t)3);                 // D_2
-    b += 4 * 5 * n3p;                                 // p, s, r, h, q
-    b += 4 * ((6 * np + 3) & ~(size_t)3);             // M^-1 blocks
-    b += 4 * ((ncb + 3) & ~(size_t)3);                // camera ids
-    b += 4 * ((((ncb + 31) >> 5) + 3) & ~(size_t)3);  // owner bits
-    b += 4 * (16 + 12 + 5 * 9) * ncb;                 // records, directions, u p s r h
+    size_t b = (4 * no + 15) & ~(size_t)15;
+    b += 32 * np + 4 * 5 * n3p;
+    b += 4 * ((6 * np + 3) & ~(size_t)3);
+    b += 4 * ((ncb + 3) & ~(size_t)3) + 4 * (16 + 12) * ncb;
+    if (one_exchange) {
+        b += 4 * ((np + 3) & ~(size_t)3);
+        b += 4 * ((((ncb + 31) >> 5) + 3) & ~(size_t)3);
+        b += 4 * 5 * 9 * ncb;
+    }
     return b;
 }
 int occupancy_blocks_linearize();
@@ -179,6 +183,9 @@ void build_order(const Views<T>& v, const OrderBuffers& b, cudaStream_t s);
 // same camera and slot on both sides of a tile boundary; a false alarm only costs the
 // operator its plain point sums).  order.cu.
 void flag_repeated_keys(const uint32_t* obs_key, int64_t n_obs, uint32_t* flag, cudaStream_t s);
+// Sets bit c of row b (rows of (n_cams + 31) / 32 words, zeroed by the caller) for every camera
+// c that an observation of the tiles [blk_tile[b], blk_tile[b + 1]), b < n_blk, sees (order.cu).
+void launch_mark_cameras(const Views<float>& v, const uint32_t* blk_tile, int n_blk, uint32_t* rows, cudaStream_t s);
 // Ascending sort of (key, value) pairs, n a power of two >= 2 (order.cu).
 void sort_pairs(uint64_t* keys, uint32_t* vals, size_t n, cudaStream_t s);
 

@@ -20,7 +20,8 @@ constexpr int MAX_GRID = 4096;      // upper bound on blocks of any reduction ke
 constexpr int NPART = 4;            // doubles of partial sums per block
 constexpr int NSLOT = 32;           // atomic accumulator slots per scalar sum
 constexpr int SLOT_STRIDE = 16;     // doubles between slots (one 128-byte line)
-constexpr int MAX_PBLOCKS = 1024;   // CTAs of the persistent PCG kernel
+constexpr int MAX_CTA_TILES = 16;   // tiles of one of its CTAs
+constexpr int MAX_PBLOCKS = 256;    // CTAs of the persistent PCG kernel (one per SM)
 // Exchange area of the persistent PCG kernels: three rotating slot sets of NSLOT
 // slots, each slot XCH_NV sums (doubles), cleared before every launch.
 constexpr int XCH_NV = 4;

@@ -514,6 +514,22 @@ void flag_repeated_keys(const uint32_t* obs_key, int64_t n_obs, uint32_t* flag, 
     k_repeated_keys<<<blocks_for((size_t)n_obs, 256), 256, 0, s>>>(obs_key, n_obs, flag);
 }
 
+namespace {
+__global__ void k_mark_cameras(Views<float> v, const uint32_t* __restrict__ blk_tile, int words, uint32_t* rows) {
+    const uint32_t ob = v.tile_off[blk_tile[blockIdx.x]], oe = v.tile_off[blk_tile[blockIdx.x + 1]];
+    uint32_t* row = rows + (size_t)words * blockIdx.x;
+    for (uint32_t j = ob + threadIdx.x; j < oe; j += blockDim.x) {
+        const uint32_t c = __ldg(v.obs_key + j) >> 8;
+        // once per camera run
+        if (j == ob || (__ldg(v.obs_key + j - 1) >> 8) != c) atomicOr(row + (c >> 5), 1u << (c & 31u));
+    }
+}
+}  // namespace
+
+void launch_mark_cameras(const Views<float>& v, const uint32_t* blk_tile, int n_blk, uint32_t* rows, cudaStream_t s) {
+    k_mark_cameras<<<n_blk, 512, 0, s>>>(v, blk_tile, (v.n_cams + 31) / 32, rows);
+}
+
 template void build_order<float>(const Views<float>&, const OrderBuffers&, cudaStream_t);
 template void build_order<double>(const Views<double>&, const OrderBuffers&, cudaStream_t);
 

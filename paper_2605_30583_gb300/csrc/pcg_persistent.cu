@@ -45,80 +45,125 @@ namespace gbba {
 
 namespace {
 
-// Grid-wide barrier number `epoch` (1, 2, ... within a launch) for a co-resident
-// (cooperative) grid.  Each CTA adds one to a counter, cleared before the launch, with
-// release semantics, and waits until it reaches epoch * nblocks: the count can only
+// Arrival at grid-wide barrier number `epoch` (1, 2, ... within a launch) of a co-resident
+// (cooperative) grid, and the wait for the others, by one thread whose CTA's writes happen
+// before (a CTA or warp barrier).  Each CTA adds one to a counter, cleared before the launch,
+// with release semantics, and waits until it reaches epoch * nblocks: the count can only
 // get there once every CTA has arrived, and a CTA that has already moved on to the
 // next barrier only raises it further.  False on time-out or when another CTA has
 // already reported one.  Limits below 1 ms are checked at every poll (0: give up at the
-// first poll that finds the barrier incomplete), longer ones every 16th poll.
+// first poll that finds the barrier incomplete), longer ones every 64th poll; the limit
+// counts from the first check, so a wait that ends sooner never reads the (slow) timer.
+__device__ __forceinline__ bool grid_arrive_wait(unsigned long long* cnt, int* err, unsigned int nblocks,
+                                                 unsigned long long epoch, long long timeout_ns) {
+    bool ok = true;
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(cnt), "l"(1ull) : "memory");
+    const unsigned long long target = epoch * nblocks;
+    long long t0 = -1;
+    unsigned spins = 0;
+    for (;;) {
+        unsigned long long c;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(cnt) : "memory");
+        if (c >= target) break;
+        if (timeout_ns < 1000000LL || (++spins & 63u) == 0u) {
+            if (*reinterpret_cast<volatile int*>(err)) { ok = false; break; }
+            const long long now = global_ns();
+            if (t0 < 0) t0 = now;
+            if (now - t0 >= timeout_ns) {
+                atomicExch(err, 1);
+                ok = false;
+                break;
+            }
+        }
+    }
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return ok;
+}
+
 __device__ __forceinline__ bool grid_sync_on(unsigned long long* cnt, int* err, unsigned int nblocks,
                                              unsigned long long epoch, long long timeout_ns) {
     __shared__ int s_ok;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(cnt), "l"(1ull) : "memory");
-        const unsigned long long target = epoch * nblocks;
-        const long long t0 = global_ns();
-        unsigned spins = 0;
-        for (;;) {
-            unsigned long long c;
-            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(cnt) : "memory");
-            if (c >= target) break;
-            if (timeout_ns < 1000000LL || (++spins & 15u) == 0u) {
-                if (*reinterpret_cast<volatile int*>(err)) { ok = 0; break; }
-                if (global_ns() - t0 >= timeout_ns) {
-                    atomicExch(err, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-            __nanosleep(32);
-        }
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        s_ok = ok;
-    }
+    if (threadIdx.x == 0) s_ok = grid_arrive_wait(cnt, err, nblocks, epoch, timeout_ns) ? 1 : 0;
     __syncthreads();
     return s_ok != 0;
 }
 
-__device__ __forceinline__ bool grid_sync(DevState* st, unsigned int nblocks, unsigned long long epoch) {
-    return grid_sync_on(&st->bar_count, &st->bar_err, nblocks, epoch, st->opt.wait_ns);
-}
+// What the CTA does after an exchange, decided by one thread for all.  FP64 runs at 1/64 of
+// the FP32 rate on this GPU: a warp instruction holds its pipe for 16 cycles, so scalar
+// recurrences repeated by all 16 warps cost 4-5 us per iteration; here one lane runs them.
+enum : int { ACT_STOP = 0, ACT_UPDATE, ACT_VERIFY, ACT_TIMEOUT };
+struct PcgStep {
+    int act;
+    float alpha, beta;
+};
 
-// Grid-wide sums of XCH_NV per-CTA values, then the grid barrier.  Exchange e adds
-// into slot set e % 3 (CTA b into slot b % NSLOT, so concurrent atomics spread over
-// NSLOT lines); every CTA then reads the same totals.  Block 0 clears set (e + 1) % 3
-// before it arrives: that set was last read right after exchange e - 2, which every
-// CTA has left, and is next filled after exchange e.  `mine` is read in thread 0;
-// `sh` holds XCH_NV doubles.  False on time-out.
-__device__ bool exchange(DevState* st, double* pslots, unsigned long long epoch, const double (&mine)[XCH_NV],
-                         double (&tot)[XCH_NV], double* sh) {
+// Grid-wide sums of XCH_NV per-warp values, the grid barrier, and the decision.  red holds the
+// CTA's compensated partials, value k of warp w at red[NW k + w]; with `last_only` the values
+// before the last count as zero.  Exchange e adds into slot set e % 3 (CTA b into slot
+// b % NSLOT, so concurrent atomics spread over NSLOT lines); every CTA then reads the same
+// totals, and lane 0 calls decide(totals), which writes the shared step.  After the barrier
+// block 0 clears set (e + 2) % 3: it was last read before barrier e, which every CTA has
+// reached, and is next filled past barrier e + 1, which waits for block 0.  Call with the
+// partials published (a barrier before); returns after a barrier.
+template <int NW, typename F>
+__device__ __forceinline__ void exchange(DevState* st, double* pslots, unsigned long long epoch, const float2* red,
+                                         bool last_only, PcgStep* step, F&& decide) {
+    static_assert(XCH_NV == 4 && NSLOT == 32, "lane l holds value l % 4 of every eighth warp or slot");
     double* cur = pslots + (size_t)(epoch % 3ull) * NSLOT * SLOT_STRIDE;
-    if (blockIdx.x == 0) {
-        double* nx = pslots + (size_t)((epoch + 1ull) % 3ull) * NSLOT * SLOT_STRIDE;
-        for (int i = threadIdx.x; i < NSLOT * SLOT_STRIDE; i += blockDim.x) nx[i] = 0.0;
-    }
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < XCH_NV; ++k)
-            if (mine[k] != 0.0) slot_add(cur, k, mine[k]);
-    }
-    if (!grid_sync(st, gridDim.x, epoch)) return false;
     if (threadIdx.x < 32) {
-        double x[XCH_NV];
+        const int lane = threadIdx.x, k = lane & 3, q = lane >> 2;
+        // the warps' pairs summed as pairs (an FP64 addition has ~130 cycles of latency, a pair's
+        // six FP32 operations ~30), one FP64 value per sum to the slot
+        float hi = 0.0f, lo = 0.0f;
+        if (!last_only || k == XCH_NV - 1)
+            for (int w = q; w < NW; w += 8) {
+                float s, e;
+                const float2 p = red[NW * k + w];
+                two_sum(hi, p.x, s, e);
+                hi = s;
+                lo += p.y + e;
+            }
 #pragma unroll
-        for (int k = 0; k < XCH_NV; ++k) x[k] = slot_sum_warp(cur, k);
-        if (threadIdx.x == 0) {
+        for (int o = 4; o < 32; o <<= 1) {
+            const float h2 = __shfl_xor_sync(FULL, hi, o), l2 = __shfl_xor_sync(FULL, lo, o);
+            float s, e;
+            two_sum(hi, h2, s, e);
+            hi = s;
+            lo = lo + l2 + e;
+        }
+        if (q == 0 && (hi != 0.0f || lo != 0.0f)) slot_add(cur, k, widen(hi) + widen(lo));
+        __syncwarp();
+        int ok = 1;
+        if (lane == 0) ok = grid_arrive_wait(&st->bar_count, &st->bar_err, gridDim.x, epoch, st->opt.wait_ns) ? 1 : 0;
+        ok = __shfl_sync(FULL, ok, 0);
+        __syncwarp();
+        if (ok) {
+            double x[NSLOT / 8];
 #pragma unroll
-            for (int k = 0; k < XCH_NV; ++k) sh[k] = x[k];
+            for (int s = 0; s < NSLOT / 8; ++s) x[s] = __ldcg(&cur[(q + 8 * s) * SLOT_STRIDE + k]);
+            double d = (x[0] + x[1]) + (x[2] + x[3]);
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) d += __shfl_xor_sync(FULL, d, o);
+            double tot[XCH_NV];
+#pragma unroll
+            for (int i = 0; i < XCH_NV; ++i) tot[i] = __shfl_sync(FULL, d, i);
+            if (lane == 0) decide(tot);
+        } else if (lane == 0) {
+            step->act = ACT_TIMEOUT;
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < XCH_NV; ++k) tot[k] = sh[k];
-    return true;
+    if (blockIdx.x == 0 && threadIdx.x >= 32) {
+        double* nx = pslots + (size_t)((epoch + 2ull) % 3ull) * NSLOT * SLOT_STRIDE;
+        for (int i = threadIdx.x - 32; i < NSLOT * SLOT_STRIDE; i += blockDim.x - 32) nx[i] = 0.0;
+    }
+}
+
+// Tests on the high word, off the chain of FP64 operations.
+__device__ __forceinline__ bool finite64(double x) { return ((uint32_t)__double2hiint(x) & 0x7fffffffu) < 0x7ff00000u; }
+__device__ __forceinline__ bool positive_finite64(double x) {
+    return (uint32_t)__double2hiint(x) - 1u < 0x7ff00000u - 1u;
 }
 
 // Local index of camera c in the CTA's sorted camera list (c must be listed).
@@ -131,12 +176,12 @@ __device__ __forceinline__ uint32_t local_cam(const uint32_t* sCid, uint32_t ncb
     return lo;
 }
 
-// Pose factors k = b, b + G, ... of CTA b through the operator (both cameras of each
-// are in the CTA's list): returns this thread's part of |J_f d|^2.
+// CTA b's pose factors [f0, f1) through the operator (both cameras of each are in the CTA's
+// list): returns this thread's part of |J_f d|^2.
 __device__ __forceinline__ float factor_pass(const Views<float>& v, const uint32_t* sCid, uint32_t ncb,
-                                          const float* sDir, float* acc, int stride) {
+                                          const float* sDir, float* acc, uint32_t f0, uint32_t f1) {
     float jj = 0.0f;
-    for (int k = blockIdx.x + (int)gridDim.x * (int)threadIdx.x; k < v.n_fac; k += stride) {
+    for (uint32_t k = f0 + threadIdx.x; k < f1; k += blockDim.x) {
         const uint32_t ca = v.fac_cam[2 * (size_t)k], cb = v.fac_cam[2 * (size_t)k + 1];
         jj += factor_normal(v.fac_J + 72 * (size_t)k, sDir + 12 * local_cam(sCid, ncb, ca),
                             sDir + 12 * local_cam(sCid, ncb, cb), acc + (size_t)ca * CA_STRIDE,
@@ -145,24 +190,127 @@ __device__ __forceinline__ float factor_pass(const Views<float>& v, const uint32
     return jj;
 }
 
+// The CTA's tiles: block-local first observation, first short-run observation, and the number
+// of long- and short-run observations in the tiles before.
+struct TileTab {
+    uint32_t lo[MAX_CTA_TILES + 1], ss[MAX_CTA_TILES], nl[MAX_CTA_TILES + 1], ns[MAX_CTA_TILES + 1];
+};
+
+__device__ __forceinline__ void make_tile_tab(const Views<float>& v, uint32_t t0, int tiles, uint32_t ob, TileTab& T) {
+    if (threadIdx.x != 0) return;
+    uint32_t nl = 0, ns = 0;
+    for (int t = 0; t < tiles; ++t) {
+        const uint32_t lo = v.tile_off[t0 + t], ss = v.short_start[t0 + t], hi = v.tile_off[t0 + t + 1];
+        T.lo[t] = lo - ob;
+        T.ss[t] = ss - ob;
+        T.nl[t] = nl;
+        T.ns[t] = ns;
+        nl += ss - lo;
+        ns += hi - ss;
+        T.lo[t + 1] = hi - ob;
+    }
+    T.nl[tiles] = nl;
+    T.ns[tiles] = ns;
+}
+
+// A camera's records from the CTA's tables (128-bit shared loads; both arrays are 16-byte
+// aligned).
+__device__ __forceinline__ void resident_cam(const float* sCam, const float* sDir, uint32_t lc, OpCam& oc, OpDir& od) {
+    const float4* r4 = reinterpret_cast<const float4*>(sCam + 16 * lc);
+    const float4 ra = r4[0], rb = r4[1], rc = r4[2], rd = r4[3];
+    Cam cam;
+    cam.R[0] = ra.x; cam.R[1] = ra.y; cam.R[2] = ra.z; cam.R[3] = ra.w;
+    cam.R[4] = rb.x; cam.R[5] = rb.y; cam.R[6] = rb.z; cam.R[7] = rb.w;
+    cam.R[8] = rc.x; cam.t[0] = rc.y; cam.t[1] = rc.z; cam.t[2] = rc.w;
+    cam.f = rd.x; cam.k1 = rd.y; cam.k2 = rd.z;
+    const float4* d4 = reinterpret_cast<const float4*>(sDir + 12 * lc);
+    const float4 da = d4[0], db = d4[1], dc = d4[2];
+    const float dir[9] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w, dc.x};
+    oc = op_cam(cam);
+    od = op_dir(cam, dir);
+}
+
+// The normal operator over the CTA's observations (the keys carry CTA-local camera indices):
+// points and directions from shared memory, point sums into sQ, camera sums into `cacc`.  Bound
+// by latency: 16 warps, each a serial chain of keys, points and shared atomics.  Every thread
+// takes an equal contiguous chunk of the long runs' observations (it meets few cameras there) and
+// one of the short runs' (nearly every observation another camera): with one chunk over both, the
+// two warps that held a tile's short runs took three times as long as the others (20k against
+// 7k cycles on 200 cameras and 50,000 points) and the grid waited for them; 688 -> 667 us per 50
+// iterations there.  One short-run observation per thread and step, neighbouring lanes of a camera
+// combined by shuffles, took 961 us.
+template <int TB>
+__device__ __forceinline__ void resident_normal(const Views<float>& v, const uint32_t* skey, const float4* sX4,
+                                                const float4* sD4, float* sQ, const TileTab& T, int tiles,
+                                                const uint32_t* sCid, const float* sCam, const float* sDir, float* cacc,
+                                                uint32_t ob, float eps, bool weighted, float& js, float& jc) {
+    const bool general = weighted || eps != 0.0f;
+    uint32_t cur = NO_CAM;
+    float acc[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
+    OpCam oc;
+    OpDir od;
+    for (int part = 0; part < 2; ++part) {
+        const uint32_t* cnt = part ? T.ns : T.nl;
+        const uint32_t* first = part ? T.ss : T.lo;
+        const uint32_t n = cnt[tiles], chunk = odd_chunk<uint32_t>(n, TB);
+        const uint32_t a = min(threadIdx.x * chunk, n), b = min(a + chunk, n);
+        int t = -1;
+        uint32_t tend = 0, off = 0;
+        for (uint32_t i = a; i < b; ++i) {
+            while (i >= tend) {
+                ++t;
+                off = first[t] - cnt[t];
+                tend = cnt[t + 1];
+            }
+            const uint32_t j = i + off;
+            const uint32_t key = skey[j], lc = key >> 8;
+            if (lc != cur) {
+                if (cur != NO_CAM) {
+                    op_finish(oc, sCam[16 * cur + CP_K1], sCam[16 * cur + CP_K2], acc);
+                    flush_matvec(cacc + (size_t)sCid[cur] * CA_STRIDE, acc);
+                }
+                cur = lc;
+                resident_cam(sCam, sDir, lc, oc, od);
+            }
+            const int lp = t * TILE_PTS + (int)(key & 0xffu);
+            const float4 x = sX4[lp], dx = sD4[lp];
+            const float tt = general ? obs_normal<true>(oc, od, x, dx, eps, weighted ? __ldg(v.obs_w + ob + j) : 1.0f,
+                                                        acc, sQ + 3 * lp)
+                                     : obs_normal<false>(oc, od, x, dx, 0.0f, 1.0f, acc, sQ + 3 * lp);
+            kahan_add(js, jc, tt);
+        }
+    }
+    if (cur != NO_CAM) op_finish(oc, sCam[16 * cur + CP_K1], sCam[16 * cur + CP_K2], acc);
+    // every lane of the warp reaches this one collective
+    const bool head = seg_reduce<9>(cur, acc);
+    if (head && cur != NO_CAM) flush_matvec(cacc + (size_t)sCid[cur] * CA_STRIDE, acc);
+}
+
 }  // namespace
 
 template <int TB>
 __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const uint32_t* __restrict__ blk_tile,
                                                          const uint32_t* __restrict__ blk_cam_off,
                                                          const uint32_t* __restrict__ blk_cams,
+                                                         const uint32_t* __restrict__ blk_fac,
                                                          double* __restrict__ pslots) {
+    const uint32_t f0 = __ldg(blk_fac + blockIdx.x), f1 = __ldg(blk_fac + blockIdx.x + 1);
     DevState* st = v.st;
     if (st->pcg_active == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int CAMS_PER_PASS = TB / 9;
-    __shared__ double red[64];
-    __shared__ double shx[XCH_NV + 1];
+    constexpr int NW = TB / 32;
+    __shared__ float2 red[XCH_NV * NW];
+    __shared__ PcgStep step;
     __shared__ float s_cam_r[9 * CAMS_PER_PASS];
     const int tid = threadIdx.x;
     // cameras owned by this CTA: blockIdx.x + gridDim.x * j, j < n_own
     const int n_own = v.n_cams > (int)blockIdx.x ? (v.n_cams - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const uint32_t t0 = blk_tile[blockIdx.x], t1 = blk_tile[blockIdx.x + 1];
+    const int tiles = (int)(t1 - t0);
+    __shared__ TileTab tab;
     const uint32_t ob = v.tile_off[t0], oe = v.tile_off[t1];
     const uint32_t no = oe - ob;
     const int pb = (int)(t0 * TILE_PTS);
@@ -186,6 +334,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
     float* sCam = reinterpret_cast<float*>(sCid + ((ncb + 3) & ~3u));   // 16 per camera
     float* sDir = sCam + 16 * (size_t)ncb;                              // 12 per camera
     const size_t g0 = v.pt_off + 3 * (size_t)pb;
+    make_tile_tab(v, t0, tiles, ob, tab);
     for (uint32_t i = tid; i < ncb; i += TB) sCid[i] = __ldg(blk_cams + cb + i) & ~BLK_CAM_OWNER;
     for (uint32_t i = tid; i < 16 * ncb; i += TB)
         sCam[i] = __ldg(v.cam_pre + (size_t)(__ldg(blk_cams + cb + i / 16) & ~BLK_CAM_OWNER) * CP_STRIDE + i % 16);
@@ -213,26 +362,16 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
     const float muf = (float)mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;   // robust loss: IRLS weights per observation
-    const double tol2 = st->opt.tol * st->opt.tol;
-    const double rr0 = st->rr0;
     const int max_pcg = st->opt.max_pcg;
-    double rz = st->rz, rr = rr0, alpha = 0.0;
+    // the recurrences' scalars, kept by thread 0 (lane 0 of the deciding warp)
+    double rz = st->rz, rr = st->rr0, alpha = 0.0, beta_d = 0.0;
+    const double stop_rr = st->opt.tol * st->opt.tol * rr;
+    bool numeric_fail = false;
     float beta = 0.0f;
     unsigned long long epoch = 0ull;
     int k = 0;
-    bool ok = true, numeric_fail = false;
-    // this thread's observation chunk (block-local indices) and its first tile
-    const uint32_t chunk = odd_chunk<uint32_t>(no, TB);
-    const uint32_t ja = min(tid * chunk, no), jb = min(ja + chunk, no);
-    uint32_t tfirst = t0;
-    {
-        uint32_t lo = t0, hi = t1;   // largest t in [t0, t1) with tile_off[t] - ob <= ja
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (__ldg(v.tile_off + mid) - ob <= ja) lo = mid; else hi = mid;
-        }
-        tfirst = lo;
-    }
+    bool ok = true;
+    for (int i = tid; i < XCH_NV * NW; i += TB) red[i] = make_float2(0.0f, 0.0f);
 
     while (k < max_pcg) {
         const float* pc_old = v.pc + (size_t)(k & 1) * v.pc_stride;
@@ -268,69 +407,33 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
             kahan_add(pdp, pdpc, fmaf(sD[3 * i] * p0, p0, fmaf(sD[3 * i + 1] * p1, p1, sD[3 * i + 2] * p2 * p2)));
         }
         __syncthreads();
+        resident_normal<TB>(v, skey, sX4, sP4, sQ, tab, tiles, sCid, sCam, sDir, v.cam_acc, ob, eps, weighted, jp2, jp2c);
+        if (v.n_fac > 0) kahan_add(jp2, jp2c, factor_pass(v, sCid, ncb, sDir, v.cam_acc, f0, f1));
         {
-            uint32_t cur = NO_CAM;
-            float acc[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
-            if (ja < jb) {
-                uint32_t tcur = tfirst;
-                uint32_t tend = __ldg(v.tile_off + tcur + 1) - ob;
-                int tpt = (int)(tcur * TILE_PTS) - pb;
-                Cam cam;
-                float dir[9];
-                for (uint32_t j = ja; j < jb; ++j) {
-                    while (j >= tend) {
-                        ++tcur;
-                        tend = __ldg(v.tile_off + tcur + 1) - ob;
-                        tpt = (int)(tcur * TILE_PTS) - pb;
-                    }
-                    const uint32_t key = skey[j];
-                    const uint32_t lc = key >> 8;   // the CTA's local camera index
-                    const int lp = tpt + (int)(key & 0xffu);
-                    if (lc != cur) {
-                        if (cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)sCid[cur] * CA_STRIDE, acc);
-                        cur = lc;
-                        // records as 128-bit shared loads (both arrays are 16-byte aligned)
-                        const float4* r4 = reinterpret_cast<const float4*>(sCam + 16 * lc);
-                        const float4 ra = r4[0], rb = r4[1], rc = r4[2], rd = r4[3];
-                        cam.R[0] = ra.x; cam.R[1] = ra.y; cam.R[2] = ra.z; cam.R[3] = ra.w;
-                        cam.R[4] = rb.x; cam.R[5] = rb.y; cam.R[6] = rb.z; cam.R[7] = rb.w;
-                        cam.R[8] = rc.x; cam.t[0] = rc.y; cam.t[1] = rc.z; cam.t[2] = rc.w;
-                        cam.f = rd.x; cam.k1 = rd.y; cam.k2 = rd.z;
-                        const float4* d4 = reinterpret_cast<const float4*>(sDir + 12 * lc);
-                        const float4 da = d4[0], db = d4[1], dc = d4[2];
-                        dir[0] = da.x; dir[1] = da.y; dir[2] = da.z; dir[3] = da.w;
-                        dir[4] = db.x; dir[5] = db.y; dir[6] = db.z; dir[7] = db.w; dir[8] = dc.x;
-                    }
-                    const float4 xp = sX4[lp], pp = sP4[lp];
-                    const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {pp.x, pp.y, pp.z};
-                    kahan_add(jp2, jp2c, weighted ? obs_normal<true>(cam, dir, xs, ds, eps, acc, sQ + 3 * lp,
-                                                                     __ldg(v.obs_w + ob + j))
-                                                  : obs_normal(cam, dir, xs, ds, eps, acc, sQ + 3 * lp));
-                }
+            const float2 a = warp_pair(jp2, -jp2c), b = warp_pair(pdp, -pdpc);
+            if ((tid & 31) == 0) {
+                red[tid >> 5] = a;
+                red[NW + (tid >> 5)] = b;
             }
-            // every lane of the warp reaches this one collective
-            const bool head = seg_reduce<9>(cur, acc);
-            if (head && cur != NO_CAM) flush_matvec(v.cam_acc + (size_t)sCid[cur] * CA_STRIDE, acc);
         }
-        if (v.n_fac > 0) kahan_add(jp2, jp2c, factor_pass(v, sCid, ncb, sDir, v.cam_acc, (int)gridDim.x * TB));
-        double sj, sp;
-        {
-            double mine[XCH_NV] = {0.0, 0.0, 0.0, 0.0}, tot[XCH_NV];
-            block_sum2c(jp2, jp2c, pdp, pdpc, red, mine[0], mine[1]);
-            if (!exchange(st, pslots, ++epoch, mine, tot, shx)) { ok = false; break; }
-            sj = tot[0];
-            sp = tot[1];
-        }
+        __syncthreads();
+        exchange<NW>(st, pslots, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
+            const double denom = tot[0] + mu * tot[1];
+            if (!positive_finite64(denom)) {
+                numeric_fail = !finite64(denom);
+                step.act = ACT_STOP;
+            } else {
+                alpha = rz * rcp64(denom);
+                step.act = ACT_UPDATE;
+                step.alpha = (float)alpha;
+            }
+        });
         // ------------------------------------------------------------ phase B
-        const double denom = sj + mu * sp;
-        if (!(denom > 0.0) || !isfinite(denom)) {
-            numeric_fail = !isfinite(denom);
-            break;   // every CTA sees the same sums and leaves here
+        if (step.act != ACT_UPDATE) {   // every CTA takes the same step
+            ok = step.act != ACT_TIMEOUT;
+            break;
         }
-        alpha = rz / denom;
-        const float af = (float)alpha;
+        const float af = step.alpha;
         float lrz = 0.0f, lrzc = 0.0f, lrr = 0.0f, lrrc = 0.0f;   // Kahan pairs
         // points: all of it in shared memory
         auto update_points = [&]() {
@@ -440,21 +543,37 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
             }
             update_points();
         }
-        double rzn, rrn;
         {
-            double mine[XCH_NV] = {0.0, 0.0, 0.0, 0.0}, tot[XCH_NV];
-            block_sum2c(lrz, lrzc, lrr, lrrc, red, mine[0], mine[1]);
-            if (!exchange(st, pslots, ++epoch, mine, tot, shx)) { ok = false; break; }
-            rzn = tot[0];
-            rrn = tot[1];
+            const float2 a = warp_pair(lrz, -lrzc), b = warp_pair(lrr, -lrrc);
+            if ((tid & 31) == 0) {
+                red[tid >> 5] = a;
+                red[NW + (tid >> 5)] = b;
+            }
         }
-        // ------------------------------------------------------------ phase C
+        __syncthreads();
         ++k;
-        rr = rrn;
-        if (!isfinite(rzn) || !isfinite(rrn)) { numeric_fail = true; break; }
-        if (rrn <= tol2 * rr0) break;
-        beta = (float)(rzn / rz);
-        rz = rzn;
+        exchange<NW>(st, pslots, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
+            // ------------------------------------------------------------ phase C
+            const double rzn = tot[0];
+            rr = tot[1];
+            step.act = ACT_UPDATE;
+            if (!finite64(rzn) || !finite64(rr)) {
+                numeric_fail = true;
+                step.act = ACT_STOP;
+            } else if (rr <= stop_rr) {
+                step.act = ACT_STOP;
+            } else {
+                beta_d = rzn * rcp64(rz);
+                rz = rzn;
+                step.beta = (float)beta_d;
+            }
+        });
+        if (step.act != ACT_UPDATE) {
+            ok = step.act != ACT_TIMEOUT;
+            if (!ok) --k;
+            break;
+        }
+        beta = step.beta;
     }
     // points' h back to global for the candidate step
     for (int i = tid; i < n3; i += TB) v.h[g0 + i] = sH[i];
@@ -464,7 +583,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
         st->rz = rz;
         st->rr = rr;
         st->alpha = alpha;
-        st->beta = beta;
+        st->beta = beta_d;
         st->pcg_active = 0;
         if (!ok) st->status = 5;
         else if (numeric_fail) st->status = 4;
@@ -497,87 +616,123 @@ __device__ __forceinline__ void camera_dirs(const Views<float>& v, const uint32_
     }
 }
 
-// Warp sums of the update's three compensated partials (Kahan pairs s - c) into
-// red[3 * warp + k]: compensated FP32 pairs inside the warp (warp_sum_pair).
-__device__ __forceinline__ void warp_partials3(float a, float ac, float b, float bc, float c, float cc,
-                                               double* red) {
-    const double sa = warp_sum_pair(a, -ac), sb = warp_sum_pair(b, -bc), sc = warp_sum_pair(c, -cc);
-    if ((threadIdx.x & 31) == 0) {
-        const int w = threadIdx.x >> 5;
-        red[3 * w] = sa;
-        red[3 * w + 1] = sb;
-        red[3 * w + 2] = sc;
-    }
-}
+// The CTA's tables of the one-exchange form (shared memory).
+struct Tables1x {
+    const float4* sX4;   // (X, D_0)
+    float4* sU4;         // (u, D_1)
+    const float* sD2;
+    float *sP, *sS, *sR, *sH, *sQ;
+    const float* sM;
+    const uint32_t *sCid, *sOwn;
+    float *sDir, *sCu, *sCp, *sCs, *sCr, *sCh;
+};
 
-// Residual replacement of the one-exchange form: with A h assembled (points in sQ,
-// cameras in the accumulator set `cacc`), r = b - A h with b = -g and u = M^-1 r (p and
-// s are kept); the partials of r^T u, |r|^2 and u^T D u go to red_u as the update phase
-// leaves them, and the owners clear the accumulator set `clear` as it does.
-template <int TB>
-__device__ void replace_residual(const Views<float>& v, const float* cacc, const uint32_t* sCid, const uint32_t* sOwn,
-                                 int ne, int np, size_t g0, float muf, const float4* sX4, float4* sU4,
-                                 const float* sD2, float* sR, const float* sH, float* sQ, const float* sM, float* sCu,
-                                 float* sCr, const float* sCh, float* clear, double* red_u) {
-    const int tid = threadIdx.x;
+// Update phase of the one-exchange form, from the assembled operator sums (points in sQ,
+// cameras in the accumulator set `cacc`): w = A u, then p, s, h, r and u = M^-1 r; with
+// TRUE_R (residual replacement) the sums are A h instead, r = b - A h with b = -g, and p, s,
+// h are kept.  The cameras' direction records follow, the owner of a camera clears the
+// accumulator set `clear` (filled by the iteration after next: its last readers are past
+// the exchange), and the warps' partials of r^T u, |r|^2 and u^T D u go to `red`.
+// A camera is nine lanes, three cameras a warp: its sums, r and u travel by shuffles, so no
+// block barrier separates the steps.  The last warps take the cameras, the first ones hold
+// the most points.
+template <int TB, bool TRUE_R>
+__device__ __forceinline__ void update_1x(const Views<float>& v, const Tables1x& T, const float* cacc, float* clear,
+                                          int ncb, int np, size_t g0, float muf, float af, float beta, float2* red) {
+    constexpr int NW = TB / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float lg = 0.0f, lr = 0.0f, lu = 0.0f, lgc = 0.0f, lrc = 0.0f, luc = 0.0f;   // Kahan pairs
-    // cameras, step 1: r = -g - (J^T J h + mu D h)
-    for (int e = tid; e < ne; e += TB) {
-        const int lc = e / 9, i = e - 9 * lc;
-        const uint32_t c = sCid[lc];
-        const float* ca = cacc + (size_t)c * CA_STRIDE;
-        float q;
-        if (i < 3) {
-            const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
-            q = fmaf(__ldg(JL + i), __ldcg(ca + 0), fmaf(__ldg(JL + 3 + i), __ldcg(ca + 1),
-                                                       __ldg(JL + 6 + i) * __ldcg(ca + 2)));
-        } else {
-            q = __ldcg(ca + i);
+    for (int cw = 3 * (NW - 1 - warp); cw < ncb; cw += 3 * NW) {
+        const int sub = lane / 9, i = lane - 9 * sub, base = 9 * sub;
+        const bool live = lane < 27 && cw + sub < ncb;
+        const int lc = live ? cw + sub : cw;
+        const int ii = live ? i : 0;
+        const int e = 9 * lc + ii;
+        const uint32_t c = T.sCid[lc];
+        const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
+        const float* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * ii;
+        const float ca = __ldcg(cacc + (size_t)c * CA_STRIDE + ii);
+        const float Dc = __ldg(v.D + 9 * (size_t)c + ii);
+        float m[9], jc[3], jr[3];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) m[q] = __ldg(M + q);
+        const int i3 = ii < 3 ? ii : 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            jc[q] = __ldg(JL + 3 * q + i3);
+            jr[q] = __ldg(JL + 3 * i3 + q);
         }
-        const float ah = fmaf(muf, __ldg(v.D + 9 * (size_t)c + i) * sCh[e], q);
-        sCr[e] = (float)(-v.cam_lin[(size_t)c * CL_STRIDE + CL_G + i]) - ah;
+        const float c0 = __shfl_sync(FULL, ca, base), c1 = __shfl_sync(FULL, ca, base + 1);
+        const float c2 = __shfl_sync(FULL, ca, base + 2);
+        const float q = ii < 3 ? fmaf(jc[0], c0, fmaf(jc[1], c1, jc[2] * c2)) : ca;
+        float r;
+        if (TRUE_R) {
+            r = (float)(-v.cam_lin[(size_t)c * CL_STRIDE + CL_G + ii]) - fmaf(muf, Dc * T.sCh[e], q);
+        } else {
+            const float u = T.sCu[e];
+            const float pk = fmaf(beta, T.sCp[e], u);
+            const float sk = fmaf(beta, T.sCs[e], fmaf(muf, Dc * u, q));
+            r = fmaf(-af, sk, T.sCr[e]);
+            if (live) {
+                T.sCp[e] = pk;
+                T.sCs[e] = sk;
+                T.sCh[e] = fmaf(af, pk, T.sCh[e]);
+            }
+        }
+        float z = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) z = fmaf(m[k], __shfl_sync(FULL, r, base + k), z);
+        const float z0 = __shfl_sync(FULL, z, base), z1 = __shfl_sync(FULL, z, base + 1);
+        const float z2 = __shfl_sync(FULL, z, base + 2);
+        if (live) {
+            T.sCr[e] = r;
+            T.sCu[e] = z;
+            T.sDir[12 * lc + ii] = ii < 3 ? fmaf(jr[0], z0, fmaf(jr[1], z1, jr[2] * z2)) : z;
+            if (owns(T.sOwn, lc)) {
+                kahan_add(lg, lgc, r * z);
+                kahan_add(lr, lrc, r * r);
+                kahan_add(lu, luc, Dc * z * z);
+                clear[(size_t)c * CA_STRIDE + ii] = 0.0f;
+            }
+        }
     }
-    // points
+    // points: all of it in shared memory
     for (int i = tid; i < np; i += TB) {
-        const float Dq[3] = {sX4[i].w, sU4[i].w, sD2[i]};
+        const float4 u4 = T.sU4[i];
+        const float Dq[3] = {T.sX4[i].w, u4.w, T.sD2[i]};
+        const float uq[3] = {u4.x, u4.y, u4.z};
         float r3[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const int e = 3 * i + q;
-            const float ah = fmaf(muf, Dq[q] * sH[e], sQ[e]);
-            r3[q] = -v.g[g0 + e] - ah;
-            sR[e] = r3[q];
-            sQ[e] = 0.0f;
+            if (TRUE_R) {
+                r3[q] = -v.g[g0 + e] - fmaf(muf, Dq[q] * T.sH[e], T.sQ[e]);
+            } else {
+                const float pk = fmaf(beta, T.sP[e], uq[q]);
+                const float sk = fmaf(beta, T.sS[e], fmaf(muf, Dq[q] * uq[q], T.sQ[e]));
+                T.sP[e] = pk;
+                T.sS[e] = sk;
+                T.sH[e] = fmaf(af, pk, T.sH[e]);
+                r3[q] = fmaf(-af, sk, T.sR[e]);
+            }
+            T.sQ[e] = 0.0f;
+            T.sR[e] = r3[q];
         }
-        const float* m = sM + 6 * i;
+        const float* m = T.sM + 6 * i;
         const float z0 = fmaf(m[0], r3[0], fmaf(m[1], r3[1], m[2] * r3[2]));
         const float z1 = fmaf(m[1], r3[0], fmaf(m[3], r3[1], m[4] * r3[2]));
         const float z2 = fmaf(m[2], r3[0], fmaf(m[4], r3[1], m[5] * r3[2]));
-        sU4[i] = make_float4(z0, z1, z2, Dq[1]);
+        T.sU4[i] = make_float4(z0, z1, z2, u4.w);
         kahan_add(lg, lgc, fmaf(r3[0], z0, fmaf(r3[1], z1, r3[2] * z2)));
         kahan_add(lr, lrc, fmaf(r3[0], r3[0], fmaf(r3[1], r3[1], r3[2] * r3[2])));
         kahan_add(lu, luc, fmaf(Dq[0] * z0, z0, fmaf(Dq[1] * z1, z1, Dq[2] * z2 * z2)));
     }
-    __syncthreads();   // camera r
-    // cameras, step 2: u = M^-1 r
-    for (int e = tid; e < ne; e += TB) {
-        const int lc = e / 9, i = e - 9 * lc;
-        const uint32_t c = sCid[lc];
-        const float* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * i;
-        const float* r9 = sCr + 9 * lc;
-        float z = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) z = fmaf(__ldg(M + q), r9[q], z);
-        sCu[e] = z;
-        if (owns(sOwn, lc)) {
-            const float ri = r9[i];
-            kahan_add(lg, lgc, ri * z);
-            kahan_add(lr, lrc, ri * ri);
-            kahan_add(lu, luc, __ldg(v.D + 9 * (size_t)c + i) * z * z);
-            clear[(size_t)c * CA_STRIDE + i] = 0.0f;
-        }
+    const float2 a = warp_pair(lg, -lgc), b = warp_pair(lr, -lrc), d = warp_pair(lu, -luc);
+    if (lane == 0) {
+        red[warp] = a;
+        red[NW + warp] = b;
+        red[2 * NW + warp] = d;
     }
-    warp_partials3(lg, lgc, lr, lrc, lu, luc, red_u);
 }
 
 }  // namespace
@@ -586,14 +741,19 @@ template <int TB>
 __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, const uint32_t* __restrict__ blk_tile,
                                                          const uint32_t* __restrict__ blk_cam_off,
                                                          const uint32_t* __restrict__ blk_cams,
+                                                         const uint32_t* __restrict__ blk_fac,
                                                          double* __restrict__ pslots) {
+    const uint32_t f0 = __ldg(blk_fac + blockIdx.x), f1 = __ldg(blk_fac + blockIdx.x + 1);
     DevState* st = v.st;
     if (st->pcg_active == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int NW = TB / 32;
-    __shared__ double red_u[3 * NW], red_m[NW], shx[XCH_NV + 1];
+    __shared__ float2 red[XCH_NV * NW];   // r^T u, |r|^2, u^T D u (update phase), |J u|^2 (operator)
+    __shared__ PcgStep step;
     const int tid = threadIdx.x;
     const uint32_t t0 = blk_tile[blockIdx.x], t1 = blk_tile[blockIdx.x + 1];
+    const int tiles = (int)(t1 - t0);
+    __shared__ TileTab tab;
     const uint32_t ob = v.tile_off[t0], oe = v.tile_off[t1];
     const uint32_t no = oe - ob;
     const int pb = (int)(t0 * TILE_PTS);
@@ -625,6 +785,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     const size_t g0 = v.pt_off + 3 * (size_t)pb;
     const size_t cas = (size_t)CA_STRIDE * v.n_cams;   // floats between accumulator sets
 
+    make_tile_tab(v, t0, tiles, ob, tab);
     for (uint32_t i = tid; i < ncb; i += TB) sCid[i] = __ldg(blk_cams + cb + i) & ~BLK_CAM_OWNER;
     for (uint32_t w = tid; w < (ncb + 31) / 32; w += TB) {
         uint32_t m = 0u;
@@ -678,20 +839,29 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
             kahan_add(lu, luc, __ldg(v.D + ge) * u * u);
         }
     }
-    warp_partials3(lg, lgc, lr, lrc, lu, luc, red_u);
+    {
+        const float2 a = warp_pair(lg, -lgc), b = warp_pair(lr, -lrc), d = warp_pair(lu, -luc);
+        if ((tid & 31) == 0) {
+            red[tid >> 5] = a;
+            red[NW + (tid >> 5)] = b;
+            red[2 * NW + (tid >> 5)] = d;
+        }
+    }
     __syncthreads();   // camera u
     camera_dirs<TB>(v, sCid, sCu, sDir, ne);
     __syncthreads();
+    const Tables1x T{sX4, sU4, sD2, sP, sS, sR, sH, sQ, sM, sCid, sOwn, sDir, sCu, sCp, sCs, sCr, sCh};
 
     const double mu = st->mu;
     const float muf = (float)mu;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;   // robust loss: IRLS weights per observation
-    const double tol2 = st->opt.tol * st->opt.tol;
-    const double rr0 = st->rr0;
     const int max_pcg = st->opt.max_pcg;
-    double gam = st->rz, gam_prev = 1.0, alpha = 0.0, alpha_prev = 1.0, rr = rr0;
-    float beta = 0.0f;
+    // the recurrences' scalars, kept by thread 0 (lane 0 of the deciding warp)
+    double gam = st->rz, igam = 0.0, alpha = 0.0, ialpha = 0.0, beta_d = 0.0, dprev = 0.0, rr = st->rr0;
+    const double stop_rr = st->opt.tol * st->opt.tol * rr;
+    bool numeric_fail = false;
+    int checks = 0;
     unsigned long long epoch = 0ull;
     int k = 0;    // PCG updates
     int it = 0;   // operator passes (they rotate the camera accumulator sets)
@@ -702,222 +872,103 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     // meets the tolerance.  At most MAX_CHECKS such checks per solve; past them the
     // recursive residual decides.
     constexpr int MAX_CHECKS = 4;
-    int checks = 0;
     bool verify = false;   // the coming operator pass applies A to h
     bool true_r = false;   // r was just replaced by the true residual
-    bool ok = true, numeric_fail = false;
-    // this thread's observation chunk (block-local indices) and its first tile
-    const uint32_t chunk = odd_chunk<uint32_t>(no, TB);
-    const uint32_t ja = min(tid * chunk, no), jb = min(ja + chunk, no);
-    uint32_t tfirst = t0;
-    {
-        uint32_t lo = t0, hi = t1;   // largest t in [t0, t1) with tile_off[t] - ob <= ja
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (__ldg(v.tile_off + mid) - ob <= ja) lo = mid; else hi = mid;
-        }
-        tfirst = lo;
-    }
+    bool ok = true;
 
     while (k < max_pcg) {
         float* cacc = v.cam_acc + (size_t)(it % CA_SETS) * cas;
         // ------------------------------------------------------------ M: w = A u (A h when verifying)
         float jj = 0.0f, jjc = 0.0f;   // Kahan pair
-        {
-            uint32_t cur = NO_CAM;
-            float acc[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
-            if (ja < jb) {
-                uint32_t tcur = tfirst;
-                uint32_t tend = __ldg(v.tile_off + tcur + 1) - ob;
-                int tpt = (int)(tcur * TILE_PTS) - pb;
-                Cam cam;
-                float dir[9];
-                for (uint32_t j = ja; j < jb; ++j) {
-                    while (j >= tend) {
-                        ++tcur;
-                        tend = __ldg(v.tile_off + tcur + 1) - ob;
-                        tpt = (int)(tcur * TILE_PTS) - pb;
-                    }
-                    const uint32_t key = skey[j];
-                    const uint32_t lc = key >> 8;   // the CTA's local camera index
-                    const int lp = tpt + (int)(key & 0xffu);
-                    if (lc != cur) {
-                        if (cur != NO_CAM) flush_matvec(cacc + (size_t)sCid[cur] * CA_STRIDE, acc);
-                        cur = lc;
-                        // records as 128-bit shared loads (both arrays are 16-byte aligned)
-                        const float4* r4 = reinterpret_cast<const float4*>(sCam + 16 * lc);
-                        const float4 ra = r4[0], rb = r4[1], rc = r4[2], rd = r4[3];
-                        cam.R[0] = ra.x; cam.R[1] = ra.y; cam.R[2] = ra.z; cam.R[3] = ra.w;
-                        cam.R[4] = rb.x; cam.R[5] = rb.y; cam.R[6] = rb.z; cam.R[7] = rb.w;
-                        cam.R[8] = rc.x; cam.t[0] = rc.y; cam.t[1] = rc.z; cam.t[2] = rc.w;
-                        cam.f = rd.x; cam.k1 = rd.y; cam.k2 = rd.z;
-                        const float4* d4 = reinterpret_cast<const float4*>(sDir + 12 * lc);
-                        const float4 da = d4[0], db = d4[1], dc = d4[2];
-                        dir[0] = da.x; dir[1] = da.y; dir[2] = da.z; dir[3] = da.w;
-                        dir[4] = db.x; dir[5] = db.y; dir[6] = db.z; dir[7] = db.w; dir[8] = dc.x;
-                    }
-                    const float4 xp = sX4[lp], up = sU4[lp];
-                    const float xs[3] = {xp.x, xp.y, xp.z}, ds[3] = {up.x, up.y, up.z};
-                    kahan_add(jj, jjc, weighted ? obs_normal<true>(cam, dir, xs, ds, eps, acc, sQ + 3 * lp,
-                                                                   __ldg(v.obs_w + ob + j))
-                                                : obs_normal(cam, dir, xs, ds, eps, acc, sQ + 3 * lp));
-                }
-            }
-            // every lane of the warp reaches this one collective
-            const bool head = seg_reduce<9>(cur, acc);
-            if (head && cur != NO_CAM) flush_matvec(cacc + (size_t)sCid[cur] * CA_STRIDE, acc);
-        }
-        if (v.n_fac > 0) kahan_add(jj, jjc, factor_pass(v, sCid, ncb, sDir, cacc, (int)gridDim.x * TB));
-        const double jw = warp_sum_pair(jj, -jjc);
-        if ((tid & 31) == 0) red_m[tid >> 5] = jw;
+        resident_normal<TB>(v, skey, sX4, sU4, sQ, tab, tiles, sCid, sCam, sDir, cacc, ob, eps, weighted, jj, jjc);
+        if (v.n_fac > 0) kahan_add(jj, jjc, factor_pass(v, sCid, ncb, sDir, cacc, f0, f1));
+        const float2 jw = warp_pair(jj, -jjc);
+        if ((tid & 31) == 0) red[3 * NW + (tid >> 5)] = jw;
         __syncthreads();
         // ------------------------------------------------------------ X: exchange
-        double mine[XCH_NV] = {0.0, 0.0, 0.0, 0.0}, tot[XCH_NV];
-        if (tid == 0) {
-            for (int w = 0; w < NW; ++w) {
-                if (!verify) {   // a verification pass carries only its operator sums
-                    mine[0] += red_u[3 * w];
-                    mine[1] += red_u[3 * w + 1];
-                    mine[2] += red_u[3 * w + 2];
-                }
-                mine[3] += red_m[w];
+        exchange<NW>(st, pslots, ++epoch, red, verify, &step, [&](const double (&tot)[XCH_NV]) {
+            if (verify) {   // a verification pass only assembles A h
+                step.act = ACT_UPDATE;
+                return;
             }
+            const double g_k = tot[0], udu = tot[2], jju = tot[3];
+            if (!finite64(g_k) || !finite64(tot[1])) {
+                numeric_fail = true;
+                step.act = ACT_STOP;
+                return;
+            }
+            rr = tot[1];
+            if (k > 0 && rr <= stop_rr) {
+                // a true residual (or no checks left) ends the solve; else the recursive one is
+                // checked against the true one: the next pass applies A to h
+                step.act = true_r || checks >= MAX_CHECKS ? ACT_STOP : ACT_VERIFY;
+                ++checks;
+                return;
+            }
+            beta_d = k > 0 ? g_k * igam : 0.0;
+            const double delta = jju + mu * udu;                                     // u^T A u
+            const double denom = k > 0 ? fma(-beta_d, g_k * ialpha, delta) : delta;   // p^T A p
+            if (!positive_finite64(denom)) {
+                numeric_fail = !finite64(denom);
+                step.act = ACT_STOP;
+                return;
+            }
+            gam = g_k;
+            alpha = g_k * rcp64(denom);
+            step.act = ACT_UPDATE;
+            step.alpha = narrow(alpha);
+            step.beta = narrow(beta_d);
+            dprev = denom;   // 1 / gamma and 1 / alpha: taken off the other warps' path, below
+        });
+        const int act = step.act;   // every CTA takes the same step
+        if (act == ACT_STOP || act == ACT_TIMEOUT) {
+            ok = act == ACT_STOP;
+            break;
         }
-        if (!exchange(st, pslots, ++epoch, mine, tot, shx)) { ok = false; break; }
+        if (act == ACT_VERIFY) {
+            verify = true;
+            for (int i = tid; i < np; i += TB) {
+                sU4[i] = make_float4(sH[3 * i], sH[3 * i + 1], sH[3 * i + 2], sU4[i].w);
+                // w = A u of the pass that found the tolerance met is not applied
+                sQ[3 * i] = sQ[3 * i + 1] = sQ[3 * i + 2] = 0.0f;
+            }
+            float* clear = v.cam_acc + (size_t)((it + 2) % CA_SETS) * cas;   // as the update would
+            for (int e = tid; e < ne; e += TB) {
+                sCu[e] = sCh[e];
+                const int lc = e / 9;
+                if (owns(sOwn, lc)) clear[(size_t)sCid[lc] * CA_STRIDE + (e - 9 * lc)] = 0.0f;
+            }
+            __syncthreads();
+            camera_dirs<TB>(v, sCid, sCu, sDir, ne);
+            __syncthreads();
+            ++it;
+            continue;
+        }
+        float* clear = v.cam_acc + (size_t)((it + 2) % CA_SETS) * cas;
         if (verify) {
             // ---------------------------------------------------- R: r = b - A h, restart
-            replace_residual<TB>(v, cacc, sCid, sOwn, ne, np, g0, muf, sX4, sU4, sD2, sR, sH, sQ, sM, sCu, sCr, sCh,
-                                 v.cam_acc + (size_t)((it + 2) % CA_SETS) * cas, red_u);
-            __syncthreads();   // camera u
-            camera_dirs<TB>(v, sCid, sCu, sDir, ne);
-            __syncthreads();
+            update_1x<TB, true>(v, T, cacc, clear, (int)ncb, np, g0, muf, 0.0f, 0.0f, red);
             verify = false;
             true_r = true;
-            ++it;
-            continue;
-        }
-        const double g_k = tot[0], rr_k = tot[1], udu = tot[2], jju = tot[3];
-        if (!isfinite(g_k) || !isfinite(rr_k)) { numeric_fail = true; break; }
-        rr = rr_k;
-        if (k > 0 && rr_k <= tol2 * rr0) {
-            if (true_r || checks >= MAX_CHECKS) break;   // a true residual (or no checks left)
-            // check the recursive residual against the true one: the next pass applies A to h
-            ++checks;
-            verify = true;
-            for (int i = tid; i < np; i += TB)
-                sU4[i] = make_float4(sH[3 * i], sH[3 * i + 1], sH[3 * i + 2], sU4[i].w);
-            for (int e = tid; e < ne; e += TB) sCu[e] = sCh[e];
-            __syncthreads();
-            camera_dirs<TB>(v, sCid, sCu, sDir, ne);
-            __syncthreads();
-            ++it;
-            continue;
-        }
-        const double b_k = k > 0 ? g_k / gam_prev : 0.0;
-        const double delta = jju + mu * udu;                                  // u^T A u
-        const double denom = k > 0 ? delta - b_k * g_k / alpha_prev : delta;   // p^T A p
-        if (!(denom > 0.0) || !isfinite(denom)) {
-            numeric_fail = !isfinite(denom);
-            break;   // every CTA sees the same sums and leaves here
-        }
-        gam = g_k;
-        alpha = g_k / denom;
-        beta = (float)b_k;
-        const float af = (float)alpha;
-        // ------------------------------------------------------------ U: update
-        lg = lr = lu = lgc = lrc = luc = 0.0f;
-        // cameras, step 1: w from the assembled sums, then p, s, h, r
-        for (int e = tid; e < ne; e += TB) {
-            const int lc = e / 9, i = e - 9 * lc;
-            const uint32_t c = sCid[lc];
-            const float* ca = cacc + (size_t)c * CA_STRIDE;
-            float q;
-            if (i < 3) {
-                const float* JL = v.cam_pre + (size_t)c * CP_STRIDE + CP_JL;
-                q = fmaf(__ldg(JL + i), __ldcg(ca + 0), fmaf(__ldg(JL + 3 + i), __ldcg(ca + 1),
-                                                           __ldg(JL + 6 + i) * __ldcg(ca + 2)));
-            } else {
-                q = __ldcg(ca + i);
+        } else {
+            // ------------------------------------------------------------ U: update
+            if (tid == 0) {
+                igam = rcp64(gam);
+                ialpha = dprev * igam;
             }
-            const float u = sCu[e];
-            const float w = fmaf(muf, __ldg(v.D + 9 * (size_t)c + i) * u, q);
-            const float pk = fmaf(beta, sCp[e], u);
-            const float sk = fmaf(beta, sCs[e], w);
-            sCp[e] = pk;
-            sCs[e] = sk;
-            sCh[e] = fmaf(af, pk, sCh[e]);
-            sCr[e] = fmaf(-af, sk, sCr[e]);
+            update_1x<TB, false>(v, T, cacc, clear, (int)ncb, np, g0, muf, step.alpha, step.beta, red);
+            true_r = false;
+            ++k;
         }
-        // points: all of it in shared memory
-        for (int i = tid; i < np; i += TB) {
-            const float4 x4 = sX4[i], u4 = sU4[i];
-            const float Dq[3] = {x4.w, u4.w, sD2[i]};
-            const float uq[3] = {u4.x, u4.y, u4.z};
-            float r3[3];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int e = 3 * i + q;
-                const float w = fmaf(muf, Dq[q] * uq[q], sQ[e]);
-                const float pk = fmaf(beta, sP[e], uq[q]);
-                const float sk = fmaf(beta, sS[e], w);
-                sP[e] = pk;
-                sS[e] = sk;
-                sQ[e] = 0.0f;
-                sH[e] = fmaf(af, pk, sH[e]);
-                r3[q] = fmaf(-af, sk, sR[e]);
-                sR[e] = r3[q];
-            }
-            const float* m = sM + 6 * i;
-            const float z0 = fmaf(m[0], r3[0], fmaf(m[1], r3[1], m[2] * r3[2]));
-            const float z1 = fmaf(m[1], r3[0], fmaf(m[3], r3[1], m[4] * r3[2]));
-            const float z2 = fmaf(m[2], r3[0], fmaf(m[4], r3[1], m[5] * r3[2]));
-            sU4[i] = make_float4(z0, z1, z2, u4.w);
-            kahan_add(lg, lgc, fmaf(r3[0], z0, fmaf(r3[1], z1, r3[2] * z2)));
-            kahan_add(lr, lrc, fmaf(r3[0], r3[0], fmaf(r3[1], r3[1], r3[2] * r3[2])));
-            kahan_add(lu, luc, fmaf(Dq[0] * z0, z0, fmaf(Dq[1] * z1, z1, Dq[2] * z2 * z2)));
-        }
-        __syncthreads();   // camera r
-        // cameras, step 2: u = M^-1 r; the owner adds the partials and clears the
-        // accumulator set that the iteration after next fills (its last readers are
-        // past the exchange above)
-        {
-            float* clear = v.cam_acc + (size_t)((it + 2) % CA_SETS) * cas;
-            for (int e = tid; e < ne; e += TB) {
-                const int lc = e / 9, i = e - 9 * lc;
-                const uint32_t c = sCid[lc];
-                const float* M = v.Minv_c + (size_t)c * MC_STRIDE + 9 * i;
-                const float* r9 = sCr + 9 * lc;
-                float z = 0.0f;
-#pragma unroll
-                for (int q = 0; q < 9; ++q) z = fmaf(__ldg(M + q), r9[q], z);
-                sCu[e] = z;
-                if (owns(sOwn, lc)) {
-                    const float ri = r9[i];
-                    kahan_add(lg, lgc, ri * z);
-                    kahan_add(lr, lrc, ri * ri);
-                    kahan_add(lu, luc, __ldg(v.D + 9 * (size_t)c + i) * z * z);
-                    clear[(size_t)c * CA_STRIDE + i] = 0.0f;
-                }
-            }
-        }
-        warp_partials3(lg, lgc, lr, lrc, lu, luc, red_u);
-        __syncthreads();   // camera u
-        camera_dirs<TB>(v, sCid, sCu, sDir, ne);
-        __syncthreads();
-        gam_prev = g_k;
-        alpha_prev = alpha;
-        true_r = false;
-        ++k;
+        __syncthreads();   // u and the direction records
         ++it;
     }
     // closing exchange: past it no CTA reads an accumulator set any more, so the
     // owners leave all of them cleared
     if (ok) {
-        double z4[XCH_NV] = {0.0, 0.0, 0.0, 0.0}, t4[XCH_NV];
         __syncthreads();
-        ok = exchange(st, pslots, ++epoch, z4, t4, shx);
+        exchange<NW>(st, pslots, ++epoch, red, true, &step, [&](const double (&)[XCH_NV]) { step.act = ACT_STOP; });
+        ok = step.act != ACT_TIMEOUT;
     }
     for (int e = tid; e < ne; e += TB) {
         const int lc = e / 9, i = e - 9 * lc;
@@ -934,7 +985,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
         st->rz = gam;
         st->rr = rr;
         st->alpha = alpha;
-        st->beta = beta;
+        st->beta = beta_d;
         st->pcg_active = 0;
         if (!ok) st->status = 5;
         else if (numeric_fail) st->status = 4;
@@ -959,8 +1010,8 @@ cudaError_t persistent_prepare(int form, int smem_bytes, int* blocks_per_sm) {
 }
 
 cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_tile, const uint32_t* blk_cam_off,
-                                  const uint32_t* blk_cams, double* pslots, int grid, int smem_bytes, int form,
-                                  cudaStream_t s) {
+                                  const uint32_t* blk_cams, const uint32_t* blk_fac, double* pslots, int grid,
+                                  int smem_bytes, int form, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(PCG_TB);
@@ -972,8 +1023,8 @@ cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_til
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (form == PCG_TWO_EXCHANGE)
-        return cudaLaunchKernelEx(&cfg, k_pcg_persistent<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, pslots);
-    return cudaLaunchKernelEx(&cfg, k_pcg_persistent_1x<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, pslots);
+        return cudaLaunchKernelEx(&cfg, k_pcg_persistent<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, pslots);
+    return cudaLaunchKernelEx(&cfg, k_pcg_persistent_1x<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, pslots);
 }
 
 // Self-test of the bounded grid wait: a cooperative grid of `grid` CTAs waits at a
