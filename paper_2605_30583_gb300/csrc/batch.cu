@@ -80,29 +80,49 @@ __device__ __forceinline__ Cam cam_plain(const float* rec) {
     return m;
 }
 
-// Block-wide sums broadcast to every thread: two FP32 values (FP32 within a warp, FP64
-// across warps) or two FP64 values.
-__device__ __forceinline__ void bsum2(float a, float b, double* sh, double& ra, double& rb) {
-    block_sum2(a, b, sh, ra, rb);
-    if (threadIdx.x == 0) { sh[62] = ra; sh[63] = rb; }
-    __syncthreads();
-    ra = sh[62];
-    rb = sh[63];
-    __syncthreads();
-}
-
-__device__ __forceinline__ void bsum2d(double a, double b, double* sh, double& ra, double& rb) {
+// Block sums of two FP32 per-thread values (FP32 inside a warp, FP64 across warps), given to
+// lane 0 of the first warp, which takes the decision they feed (decide(sum a, sum b)) for the
+// CTA: FP64 scalars repeated by every warp would each hold the SM's FP64 pipe for 16 cycles.
+// `sh` holds 64 floats.  The barriers publish what decide writes to shared memory.
+template <typename F>
+__device__ __forceinline__ void bdecide(float a, float b, float* sh, F&& decide) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_down_sync(0xffffffffu, a, o);
         b += __shfl_down_sync(0xffffffffu, b, o);
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) {
+        sh[w] = a;
+        sh[32 + w] = b;
+    }
     __syncthreads();
-    if (lane == 0) { sh[w] = a; sh[nw + w] = b; }
+    if (w == 0) {
+        double ra = lane < nw ? widen(sh[lane]) : 0.0, rb = lane < nw ? widen(sh[32 + lane]) : 0.0;
+        for (int o = 1; o < nw; o <<= 1) {
+            ra += __shfl_xor_sync(0xffffffffu, ra, o);
+            rb += __shfl_xor_sync(0xffffffffu, rb, o);
+        }
+        if (lane == 0) decide(ra, rb);
+    }
     __syncthreads();
-    ra = rb = 0.0;
-    for (int i = 0; i < nw; ++i) { ra += sh[i]; rb += sh[nw + i]; }
+}
+
+// Block sums of two FP32 per-thread values, or of two compensated ones (Kahan pairs s - c),
+// broadcast to every thread.  `sh` holds 64 doubles.
+__device__ __forceinline__ void bsum2(float a, float b, double* sh, double& ra, double& rb) {
+    bdecide(a, b, reinterpret_cast<float*>(sh), [&](double x, double y) { sh[62] = x; sh[63] = y; });
+    ra = sh[62];
+    rb = sh[63];
+    __syncthreads();
+}
+
+__device__ __forceinline__ void bsum2c(float sa, float ca, float sb, float cb, double* sh, double& ra, double& rb) {
+    block_sum2c(sa, ca, sb, cb, sh, ra, rb);
+    if (threadIdx.x == 0) { sh[62] = ra; sh[63] = rb; }
+    __syncthreads();
+    ra = sh[62];
+    rb = sh[63];
     __syncthreads();
 }
 
@@ -207,7 +227,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
         const bool head = seg_reduce<BLIN>(cur, acc);
         if (head && cur != NO_CAM) b_flush_lin(b, P.c0 + cur, acc);
     }
-    double cost = 0.0;
+    float cost = 0.0f, costc = 0.0f;   // Kahan pair
     for (int i = threadIdx.x; i < P.np; i += blockDim.x) {
         const int gp = P.p0 + i;
         const float* X = b.x + P.v0 + 9 * P.nc + 3 * i;
@@ -221,7 +241,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
             const float fs = cam.f * g.s;
             const float r0 = fmaf(fs, g.p[0], -b.obs_uv[2 * (size_t)j]);
             const float r1 = fmaf(fs, g.p[1], -b.obs_uv[2 * (size_t)j + 1]);
-            cost += (double)fmaf(r0, r0, r1 * r1);
+            kahan_add(cost, costc, fmaf(r0, r0, r1 * r1));
             float jx0[3], jx1[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
@@ -242,7 +262,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
         for (int q = 0; q < 6; ++q) b.pt_H[(size_t)gp * 6 + q] = hq[q];
     }
     double F, unused;
-    bsum2d(cost, 0.0, sh, F, unused);   // its barriers also publish the camera sums
+    bsum2c(cost, costc, 0.0f, 0.0f, sh, F, unused);   // its barriers also publish the camera sums
     return 0.5 * F;
 }
 
@@ -257,6 +277,7 @@ __device__ void b_precond(const BatchView& b, const Prob& P, double mu, double* 
     float* h = b.h + P.v0;
     const float* gv = b.g + P.v0;
     float lrz = 0.0f, lrr = 0.0f;
+    const float lo_f = __double2float_ru(o.min_diag), hi_f = __double2float_rd(o.max_diag);
     const int lane = threadIdx.x & 31;
     for (int c = threadIdx.x >> 5; c < P.nc; c += blockDim.x >> 5) {   // one warp per camera
         const float* Hc = b.cam_H + (size_t)(P.c0 + c) * CH_STRIDE;
@@ -295,29 +316,14 @@ __device__ void b_precond(const BatchView& b, const Prob& P, double mu, double* 
         __syncwarp();
     }
     for (int i = threadIdx.x; i < P.np; i += blockDim.x) {
-        const float* Hp = b.pt_H + (size_t)(P.p0 + i) * 6;
+        const float* Hg = b.pt_H + (size_t)(P.p0 + i) * 6;
         const int e = 9 * P.nc + 3 * i;
-        double a00 = Hp[0], a01 = Hp[1], a02 = Hp[2], a11 = Hp[3], a12 = Hp[4], a22 = Hp[5];
-        const double d0 = fmin(fmax(a00, o.min_diag), o.max_diag), d1 = fmin(fmax(a11, o.min_diag), o.max_diag),
-                     d2 = fmin(fmax(a22, o.min_diag), o.max_diag);
-        a00 += mu * d0; a11 += mu * d1; a22 += mu * d2;
-        // inverse of the SPD 3x3 block by its adjugate
-        const double c00 = a11 * a22 - a12 * a12, c01 = a02 * a12 - a01 * a22, c02 = a01 * a12 - a02 * a11;
-        const double c11 = a00 * a22 - a02 * a02, c12 = a01 * a02 - a00 * a12, c22 = a00 * a11 - a01 * a01;
-        const double det = a00 * c00 + a01 * c01 + a02 * c02;
-        double m[6];
-        if (det > 0.0 && isfinite(det) && a00 > 0.0 && c22 > 0.0) {
-            const double id = rcp64(det);
-            m[0] = c00 * id; m[1] = c01 * id; m[2] = c02 * id; m[3] = c11 * id; m[4] = c12 * id; m[5] = c22 * id;
-        } else {
-            m[0] = a00 > 0 ? 1.0 / a00 : 0.0; m[1] = 0.0; m[2] = 0.0;
-            m[3] = a11 > 0 ? 1.0 / a11 : 0.0; m[4] = 0.0; m[5] = a22 > 0 ? 1.0 / a22 : 0.0;
-        }
-        float Mo[6];
-        for (int k = 0; k < 6; ++k) Mo[k] = (float)m[k];
+        const float Hp[6] = {Hg[0], Hg[1], Hg[2], Hg[3], Hg[4], Hg[5]};
+        float Mo[6], dd[3];
+        point_inverse(Hp, mu, o.min_diag, o.max_diag, lo_f, hi_f, Mo, dd);
         float* Mg = b.Minv_p + (size_t)(P.p0 + i) * 6;
         for (int k = 0; k < 6; ++k) Mg[k] = Mo[k];
-        Dv[e] = (float)d0; Dv[e + 1] = (float)d1; Dv[e + 2] = (float)d2;
+        Dv[e] = dd[0]; Dv[e + 1] = dd[1]; Dv[e + 2] = dd[2];
         const float r0 = -gv[e], r1 = -gv[e + 1], r2 = -gv[e + 2];
         const float z0 = fmaf(Mo[0], r0, fmaf(Mo[1], r1, Mo[2] * r2));
         const float z1 = fmaf(Mo[1], r0, fmaf(Mo[3], r1, Mo[4] * r2));
@@ -339,6 +345,26 @@ struct Shm {
     float *q, *x, *p;                      // per point, 3 each (x and p only with staged points)
 };
 
+// Camera work of the PCG loop: nine lanes a camera, three cameras (cw, cw + 1, cw + 2) a warp, so
+// that a camera's vectors travel by shuffles.  Idle lanes read what camera cw's first lane reads.
+__device__ __forceinline__ int cam_base() { return 9 * ((int)(threadIdx.x & 31) / 9); }
+__device__ __forceinline__ bool cam_lane_live(int cw, int nc) {
+    const int lane = threadIdx.x & 31;
+    return lane < 27 && cw + lane / 9 < nc;
+}
+__device__ __forceinline__ int live_cam(int cw, int nc) {
+    return cam_lane_live(cw, nc) ? cw + (int)(threadIdx.x & 31) / 9 : cw;
+}
+__device__ __forceinline__ int live_cam_entry(int cw, int nc) {
+    return cam_lane_live(cw, nc) ? (int)(threadIdx.x & 31) % 9 : 0;
+}
+
+// A decision of the PCG loop: stop (0 no, 1 yes, 4 a non-finite sum) and alpha or beta.
+struct BStep {
+    int stop;
+    float a;
+};
+
 // PCGNR on (J^T J + mu D) h = -g from h = 0 (Sec. V): p = z + beta p;
 // alpha = r^T z / (|J p|^2 + mu p^T D p); h += alpha p; r -= alpha (J^T J p + mu D p);
 // z = M^-1 r; stop when |r| <= tol |r0| or after max_pcg iterations.  J p and J^T (J p)
@@ -349,7 +375,7 @@ struct Shm {
 // so do the points' parameters X and the point part of p, and the per-observation
 // gathers of the product never leave the SM.  The loops over points issue all their
 // loads before any store (several elements per thread) so that global-memory latency
-// overlaps; camera work goes to the last threads, which hold the fewest points.
+// overlaps; camera work goes to the last warps, which hold the fewest points.
 //
 // mu is folded into every product with D before it is summed or applied: once the cost
 // reaches the FP32 noise floor, rejected steps drive mu to 1e20 and beyond, where p
@@ -387,29 +413,25 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
     const float* Xp = SP ? S.x : xg;            // point parameters
     float* Pp = SP ? S.p : b.p + P.v0 + nc9;    // point part of the direction (zero after the preconditioner)
     __syncthreads();
-    const double tol2 = o.tol * o.tol;
+    __shared__ BStep step;
+    float* shf = reinterpret_cast<float*>(sh);
     int k = 0;
-    double beta = 0.0;
+    float bf = 0.0f;
     for (;;) {
         // ---- direction p = z + beta p, camera direction records, mu p^T D p
         float pdp = 0.0f;
-        const float bf = (float)beta;
-        for (int c = TB - 1 - tid; c < P.nc; c += TB) {
-            float pc[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                pc[q] = fmaf(bf, S.pc[9 * c + q], S.zc[9 * c + q]);
-                S.pc[9 * c + q] = pc[q];
-                pdp = fmaf(muf * (S.dc[9 * c + q] * pc[q]), pc[q], pdp);
+        for (int cw = 3 * (TB / 32 - 1 - (tid >> 5)); cw < P.nc; cw += 3 * (TB / 32)) {
+            const int c = live_cam(cw, P.nc), i = live_cam_entry(cw, P.nc), e = 9 * c + i, base = cam_base();
+            const float pk = fmaf(bf, S.pc[e], S.zc[e]);
+            const float p0 = __shfl_sync(FULL, pk, base), p1 = __shfl_sync(FULL, pk, base + 1);
+            const float p2 = __shfl_sync(FULL, pk, base + 2);
+            if (cam_lane_live(cw, P.nc)) {
+                const float* JL = S.jl + 9 * c + 3 * (i < 3 ? i : 0);
+                S.pc[e] = pk;
+                pdp = fmaf(muf * (S.dc[e] * pk), pk, pdp);
+                S.dir[SDIR * c + i] = i < 3 ? fmaf(JL[0], p0, fmaf(JL[1], p1, JL[2] * p2)) : pk;
+                S.acc[SACC * c + i] = 0.0f;
             }
-            const float* JL = S.jl + 9 * c;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-                S.dir[SDIR * c + i] = fmaf(JL[3 * i], pc[0], fmaf(JL[3 * i + 1], pc[1], JL[3 * i + 2] * pc[2]));
-#pragma unroll
-            for (int q = 3; q < 9; ++q) S.dir[SDIR * c + q] = pc[q];
-#pragma unroll
-            for (int q = 0; q < SACC; ++q) S.acc[SACC * c + q] = 0.0f;
         }
         for (int e0 = tid; e0 < n3; e0 += 4 * TB) {
             float zv[4], dv[4], pv[4];
@@ -444,8 +466,8 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
             float acc[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) acc[q] = 0.0f;
-            Cam cam;
-            float dir[9];
+            OpCam oc;
+            OpDir od;
             uint32_t kn[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) kn[u] = (a + u < e) ? keys[a + u] : NO_CAM;
@@ -462,6 +484,7 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
                     const uint32_t c = kc[u] >> 16, lp = kc[u] & 0xffffu;
                     if (c != cur) {
                         if (cur != NO_CAM) {
+                            op_finish(oc, S.cam[SCAM * cur + CP_K1], S.cam[SCAM * cur + CP_K2], acc);
 #pragma unroll
                             for (int q = 0; q < 9; ++q) {
                                 atomicAdd(S.acc + SACC * cur + q, acc[q]);
@@ -469,59 +492,60 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
                             }
                         }
                         cur = c;
-                        const float4* r4 = reinterpret_cast<const float4*>(S.cam + SCAM * c);
-                        const float4 c0 = r4[0], c1 = r4[1], c2 = r4[2], c3 = r4[3];
-                        cam.R[0] = c0.x; cam.R[1] = c0.y; cam.R[2] = c0.z; cam.R[3] = c0.w;
-                        cam.R[4] = c1.x; cam.R[5] = c1.y; cam.R[6] = c1.z; cam.R[7] = c1.w;
-                        cam.R[8] = c2.x; cam.t[0] = c2.y; cam.t[1] = c2.z; cam.t[2] = c2.w;
-                        cam.f = c3.x; cam.k1 = c3.y; cam.k2 = c3.z;
+                        const Cam cam = cam_plain(S.cam + SCAM * c);
+                        float dir[9];
 #pragma unroll
                         for (int q = 0; q < 9; ++q) dir[q] = S.dir[SDIR * c + q];
+                        oc = op_cam(cam);
+                        od = op_dir(cam, dir);
                     }
-                    jp2 += obs_normal(cam, dir, Xp + 3 * lp, Pp + 3 * lp, eps, acc, S.q + 3 * lp);
+                    const float4 xs = make_float4(Xp[3 * lp], Xp[3 * lp + 1], Xp[3 * lp + 2], 0.0f);
+                    const float4 ds = make_float4(Pp[3 * lp], Pp[3 * lp + 1], Pp[3 * lp + 2], 0.0f);
+                    jp2 += eps != 0.0f ? obs_normal<true>(oc, od, xs, ds, eps, 1.0f, acc, S.q + 3 * lp)
+                                       : obs_normal<false>(oc, od, xs, ds, 0.0f, 1.0f, acc, S.q + 3 * lp);
                 }
             }
+            if (cur != NO_CAM) op_finish(oc, S.cam[SCAM * cur + CP_K1], S.cam[SCAM * cur + CP_K2], acc);
             const bool head = seg_reduce<9>(cur, acc);
             if (head && cur != NO_CAM)
 #pragma unroll
                 for (int q = 0; q < 9; ++q) atomicAdd(S.acc + SACC * cur + q, acc[q]);
         }
-        double sj, sp;
-        bsum2(jp2, pdp, sh, sj, sp);   // barriers publish S.acc / S.q
-        const double denom = sj + sp;
-        if (!(denom > 0.0) || !isfinite(denom)) {
-            if (!isfinite(denom)) status = 4;
+        bdecide(jp2, pdp, shf, [&](double sj, double sp) {   // its barriers publish S.acc / S.q
+            const double denom = sj + sp;
+            const bool fine = denom > 0.0 && isfinite(denom);
+            step.stop = fine ? 0 : (isfinite(denom) ? 1 : 4);
+            step.a = fine ? (float)(rz * rcp64(denom)) : 0.0f;
+        });
+        if (step.stop) {
+            if (step.stop == 4) status = 4;
             break;
         }
         // ---- h += alpha p, r -= alpha (q + mu D p), z = M^-1 r
-        const float af = (float)(rz / denom);
+        const float af = step.a;
         float lrz = 0.0f, lrr = 0.0f;
-        for (int c = TB - 1 - tid; c < P.nc; c += TB) {
-            const float* JL = S.jl + 9 * c;
-            const float* ca = S.acc + SACC * c;
-            float qv[9], rn[9], M[81];
+        for (int cw = 3 * (TB / 32 - 1 - (tid >> 5)); cw < P.nc; cw += 3 * (TB / 32)) {
+            const int c = live_cam(cw, P.nc), i = live_cam_entry(cw, P.nc), e = 9 * c + i, base = cam_base();
+            const float* M = Mc + 81 * c + 9 * i;
+            float m[9];
 #pragma unroll
-            for (int t = 0; t < 81; ++t) M[t] = Mc[81 * c + t];
+            for (int q = 0; q < 9; ++q) m[q] = M[q];
+            const float a = S.acc[SACC * c + i];
+            const float a0 = __shfl_sync(FULL, a, base), a1 = __shfl_sync(FULL, a, base + 1);
+            const float a2 = __shfl_sync(FULL, a, base + 2);
+            const float* JL = S.jl + 9 * c + (i < 3 ? i : 0);
+            const float q = i < 3 ? fmaf(JL[0], a0, fmaf(JL[3], a1, JL[6] * a2)) : a;
+            const float pk = S.pc[e];
+            const float rn = fmaf(-af, fmaf(muf, S.dc[e] * pk, q), S.rc[e]);
+            float z = 0.0f;
 #pragma unroll
-            for (int q = 0; q < 3; ++q) qv[q] = fmaf(JL[q], ca[0], fmaf(JL[3 + q], ca[1], JL[6 + q] * ca[2]));
-#pragma unroll
-            for (int q = 3; q < 9; ++q) qv[q] = ca[q];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                const int e = 9 * c + q;
-                const float pk = S.pc[e];
+            for (int k2 = 0; k2 < 9; ++k2) z = fmaf(m[k2], __shfl_sync(FULL, rn, base + k2), z);
+            if (cam_lane_live(cw, P.nc)) {
                 S.hc[e] = fmaf(af, pk, S.hc[e]);
-                rn[q] = fmaf(-af, fmaf(muf, S.dc[e] * pk, qv[q]), S.rc[e]);
-                S.rc[e] = rn[q];
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                float zz = 0.0f;
-#pragma unroll
-                for (int q = 0; q < 9; ++q) zz = fmaf(M[9 * i + q], rn[q], zz);
-                S.zc[9 * c + i] = zz;
-                lrz = fmaf(rn[i], zz, lrz);
-                lrr = fmaf(rn[i], rn[i], lrr);
+                S.rc[e] = rn;
+                S.zc[e] = z;
+                lrz = fmaf(rn, z, lrz);
+                lrr = fmaf(rn, rn, lrr);
             }
         }
         for (int i0 = tid; i0 < P.np; i0 += 2 * TB) {
@@ -564,16 +588,20 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
                 }
             }
         }
-        double rzn, rrn;
-        bsum2(lrz, lrr, sh, rzn, rrn);
         ++k;
-        if (!isfinite(rzn) || !isfinite(rrn)) {
-            status = 4;
+        bdecide(lrz, lrr, shf, [&](double rzn, double rrn) {
+            step.stop = !isfinite(rzn) || !isfinite(rrn) ? 4
+                        : (rrn <= o.tol * o.tol * rr0 || k >= o.max_pcg || !(rzn > 0.0) ? 1 : 0);
+            if (!step.stop) {
+                step.a = (float)(rzn * rcp64(rz));
+                rz = rzn;   // thread 0's; the others' is not read
+            }
+        });
+        if (step.stop) {
+            if (step.stop == 4) status = 4;
             break;
         }
-        if (rrn <= tol2 * rr0 || k >= o.max_pcg || !(rzn > 0.0)) break;
-        beta = rzn / rz;
-        rz = rzn;
+        bf = step.a;
     }
     // camera block of h back to the global vector for the candidate step
     for (int i = tid; i < nc9; i += TB) hg[i] = S.hc[i];
@@ -592,11 +620,18 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
     float* xn = b.x_new + P.v0;
     const float* h = b.h + P.v0;
     const float* gv = b.g + P.v0;
-    double lgh = 0.0;
+    double lgh = 0.0;                 // cameras
+    float sgh = 0.0f, cgh = 0.0f;     // points: exact products, summed as a Kahan pair
     for (int e = tid; e < n; e += TB) {
-        xn[e] = x[e] + h[e];
-        const double ge = e < 9 * P.nc ? b.cam_g[(size_t)(P.c0 + e / 9) * CL_STRIDE + e % 9] : (double)gv[e];
-        lgh += ge * (double)h[e];
+        const float he = h[e];
+        xn[e] = x[e] + he;
+        if (e < 9 * P.nc) {
+            lgh += b.cam_g[(size_t)(P.c0 + e / 9) * CL_STRIDE + e % 9] * (double)he;
+        } else {
+            const float ge = gv[e], pr = ge * he;
+            kahan_add(sgh, cgh, pr);
+            cgh -= fmaf(ge, he, -pr);
+        }
     }
     __syncthreads();
     if (b.opt.retract) {   // rotations: R' = Exp(h_w) R(w)
@@ -618,7 +653,7 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         for (int q = 3; q < 9; ++q) sDir[SDIR * c + q] = hc[q];
     }
     __syncthreads();
-    double lf = 0.0, ljh = 0.0;
+    float lf = 0.0f, lfc = 0.0f, ljh = 0.0f, ljhc = 0.0f;   // Kahan pairs
     for (int64_t j = P.o0 + tid; j < P.o0 + P.no; j += TB) {
         const uint32_t key = b.obs_key[j];
         const uint32_t c = key >> 16, lp = key & 0xffffu;
@@ -626,7 +661,7 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         const Cam cn = cam_plain(b.cam_pre_new + (size_t)(P.c0 + c) * CP_STRIDE);
         float r0, r1;
         project_residual(cn, xn[e3], xn[e3 + 1], xn[e3 + 2], eps, b.obs_uv[2 * j], b.obs_uv[2 * j + 1], r0, r1);
-        lf += (double)fmaf(r0, r0, r1 * r1);
+        kahan_add(lf, lfc, fmaf(r0, r0, r1 * r1));
         const float4* r4 = reinterpret_cast<const float4*>(sCam + SCAM * c);
         const float4 c0 = r4[0], c1 = r4[1], c2 = r4[2], c3 = r4[3];
         Cam co;
@@ -650,12 +685,16 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         apply_A(g, dP0, dP1, dP2, t0, t1);
         t0 = fmaf(ci, g.p[0], t0);
         t1 = fmaf(ci, g.p[1], t1);
-        ljh += (double)fmaf(t0, t0, t1 * t1);
+        kahan_add(ljh, ljhc, fmaf(t0, t0, t1 * t1));
     }
     double fs;
-    bsum2d(lf, ljh, sh, fs, jh2);
-    double unused;
-    bsum2d(lgh, 0.0, sh, gh, unused);
+    bsum2c(lf, lfc, ljh, ljhc, sh, fs, jh2);
+    double gc = block_sum(lgh, sh), gp, none;   // in thread 0
+    block_sum2c(sgh, cgh, 0.0f, 0.0f, sh, gp, none);
+    if (tid == 0) sh[62] = gc + gp;
+    __syncthreads();
+    gh = sh[62];
+    __syncthreads();
     Fn = 0.5 * fs;
 }
 
@@ -684,6 +723,7 @@ __global__ void __launch_bounds__(TB, MINB) k_batch_solve(BatchView b) {
     float* sDir = S.dir;
     __shared__ double sh[64];
     __shared__ int s_q;
+    __shared__ struct { double mu, nu, F; int acc, active; } lm;
     const DevOptions& o = b.opt;
     const float eps = (float)o.eps;
     const int tid = threadIdx.x;
@@ -712,23 +752,33 @@ __global__ void __launch_bounds__(TB, MINB) k_batch_solve(BatchView b) {
             pcg_total += b_pcg<TB, SP>(b, P, mu, rz, rr0, S, sh, status);
             double Fn, jh2, gh;
             b_candidate<TB>(b, P, sCam, sDir, sh, Fn, jh2, gh);
-            // LM decision (Madsen): the same rule as the single-problem solver
-            const double L = -gh - 0.5 * jh2;
-            const double rho = L > 0.0 ? (F - Fn) / L : -1.0;
-            const bool acc = isfinite(Fn) && L > 0.0 && rho > 0.0;
+            // LM decision (Madsen): the same rule as the single-problem solver, by one thread
             ++it;
-            if (acc) {
-                const double t = 2.0 * rho - 1.0;
-                mu *= fmax(1.0 / 3.0, 1.0 - t * t * t);
-                nu = 2.0;
-                F = Fn;
-                ++n_acc;
-            } else {
-                mu *= nu;
-                nu *= 2.0;
+            if (tid == 0) {
+                const double L = -gh - 0.5 * jh2;
+                const double rho = L > 0.0 ? (F - Fn) / L : -1.0;
+                const bool ok = isfinite(Fn) && L > 0.0 && rho > 0.0;
+                if (ok) {
+                    const double t = 2.0 * rho - 1.0;
+                    lm.mu = mu * fmax(1.0 / 3.0, 1.0 - t * t * t);
+                    lm.nu = 2.0;
+                    lm.F = Fn;
+                } else {
+                    lm.mu = mu * nu;
+                    lm.nu = 2.0 * nu;
+                    lm.F = F;
+                }
+                lm.acc = ok ? 1 : 0;
+                lm.active = it < o.max_lm && lm.mu <= o.max_mu && lm.F > 0.0 && status == 0 ? 1 : 0;
             }
-            active = it < o.max_lm && mu <= o.max_mu && F > 0.0 && status == 0;
-            if (acc) {   // every thread took the same decision from the same sums
+            __syncthreads();
+            mu = lm.mu;
+            nu = lm.nu;
+            F = lm.F;
+            active = lm.active != 0;
+            const bool acc = lm.acc != 0;
+            n_acc += acc ? 1 : 0;
+            if (acc) {
                 float* x = b.x + P.v0;
                 const float* xn = b.x_new + P.v0;
                 for (int e = tid; e < n; e += TB) x[e] = xn[e];

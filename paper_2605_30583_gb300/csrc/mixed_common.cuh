@@ -406,61 +406,4 @@ __device__ __forceinline__ float factor_normal(const float* __restrict__ Jf, con
     return tt;
 }
 
-// Contribution of one observation to the normal operator: t = J d (returns |t|^2),
-// camera sums (RX x u, u, intrinsic part) into acc, point part R^T u into qs (shared).
-// WEIGHTED: the robust loss's IRLS weight w scales the observation's rows of J^T J
-// (u = A^T (w t), returns w |t|^2).  PLAIN_Q: qs belongs to the calling warp alone and
-// no other lane of it touches the same point in this step, so plain adds replace the
-// shared-memory atomics.
-template <bool WEIGHTED = false, bool PLAIN_Q = false>
-__device__ __forceinline__ float obs_normal(const Cam& cam, const float (&dir)[9], const float* xs,
-                                            const float* ds, float eps, float (&acc)[9], float* qs,
-                                            float w = 1.0f) {
-    const GeoLite g = project_lite(cam, xs[0], xs[1], xs[2], eps);
-    // J d = A (phi x RX + d_t + R d_X) + c_i p
-    float dP0 = fmaf(dir[1], g.RX[2], -dir[2] * g.RX[1]) + dir[CD_T + 0];
-    float dP1 = fmaf(dir[2], g.RX[0], -dir[0] * g.RX[2]) + dir[CD_T + 1];
-    float dP2 = fmaf(dir[0], g.RX[1], -dir[1] * g.RX[0]) + dir[CD_T + 2];
-    dP0 = fmaf(cam.R[0], ds[0], fmaf(cam.R[1], ds[1], fmaf(cam.R[2], ds[2], dP0)));
-    dP1 = fmaf(cam.R[3], ds[0], fmaf(cam.R[4], ds[1], fmaf(cam.R[5], ds[2], dP1)));
-    dP2 = fmaf(cam.R[6], ds[0], fmaf(cam.R[7], ds[1], fmaf(cam.R[8], ds[2], dP2)));
-    const float fn2 = cam.f * g.n2;
-    const float ci = fmaf(g.s, dir[CD_I + 0], fmaf(fn2, dir[CD_I + 1], fn2 * g.n2 * dir[CD_I + 2]));
-    float t0, t1;
-    apply_A(g, dP0, dP1, dP2, t0, t1);
-    t0 = fmaf(ci, g.p[0], t0);
-    t1 = fmaf(ci, g.p[1], t1);
-    const float tt = fmaf(t0, t0, t1 * t1);
-    if (WEIGHTED) {
-        t0 *= w;
-        t1 *= w;
-    }
-    // adjoint: u = A^T t
-    float u0, u1, u2;
-    apply_At(g, t0, t1, u0, u1, u2);
-    acc[0] += fmaf(g.RX[1], u2, -g.RX[2] * u1);
-    acc[1] += fmaf(g.RX[2], u0, -g.RX[0] * u2);
-    acc[2] += fmaf(g.RX[0], u1, -g.RX[1] * u0);
-    acc[3] += u0;
-    acc[4] += u1;
-    acc[5] += u2;
-    const float pt = fmaf(g.p[0], t0, g.p[1] * t1);
-    acc[6] = fmaf(g.s, pt, acc[6]);
-    acc[7] = fmaf(fn2, pt, acc[7]);
-    acc[8] = fmaf(fn2 * g.n2, pt, acc[8]);
-    const float q0 = fmaf(cam.R[0], u0, fmaf(cam.R[3], u1, cam.R[6] * u2));
-    const float q1 = fmaf(cam.R[1], u0, fmaf(cam.R[4], u1, cam.R[7] * u2));
-    const float q2 = fmaf(cam.R[2], u0, fmaf(cam.R[5], u1, cam.R[8] * u2));
-    if (PLAIN_Q) {
-        qs[0] += q0;
-        qs[1] += q1;
-        qs[2] += q2;
-    } else {
-        atomicAdd(qs + 0, q0);
-        atomicAdd(qs + 1, q1);
-        atomicAdd(qs + 2, q2);
-    }
-    return WEIGHTED ? w * tt : tt;
-}
-
 }  // namespace gbba
