@@ -45,6 +45,7 @@ struct LaunchCfg {
     // no camera observes a point twice (checked at bind): the operator's warps add their
     // point sums into private copies with plain adds
     int tn_plain_q = 0;
+    int tn_ahead = 0;   // the operator's CTAs in flight
     // few tiles: 512 threads per tile in the linearisation and the evaluations
     bool wide_tiles = false;
 };

@@ -71,22 +71,68 @@ __host__ __device__ __forceinline__ size_t compact_bytes(const Caps& c) {
     return 12 * (size_t)c.run + 4 * (size_t)c.shrt + (size_t)c.lng;
 }
 
+// The keys come four to a load (aligned down; what lies outside the tile is dropped), the first
+// KEY_LOADS of a thread before anything is stored, so that their latency is paid once.  sSlot
+// starts at the byte that makes four packed slots an aligned word.
+constexpr int KEY_LOADS = 2;
+struct KeyLoads {
+    uint4 k[KEY_LOADS];
+};
+
+template <int TB>
+__device__ __forceinline__ KeyLoads load_keys(const Views<float>& v, const TileRange& T) {
+    KeyLoads L;
+    const uint4* src = reinterpret_cast<const uint4*>(v.obs_key);
+#pragma unroll
+    for (int t = 0; t < KEY_LOADS; ++t) {
+        const uint32_t i = (T.lo & ~3u) + 4 * (threadIdx.x + t * TB);
+        L.k[t] = i < T.hi ? __ldg(src + i / 4) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    return L;
+}
+
+template <int TB>
+__device__ __forceinline__ void store_compact(const Views<float>& v, const TileRange& T, const Caps& cap,
+                                              const KeyLoads& L, unsigned char* dsm, uint32_t*& sRun,
+                                              uint32_t*& sShort, uint8_t*& sSlot) {
+    sRun = reinterpret_cast<uint32_t*>(dsm);
+    sShort = sRun + 3 * cap.run;
+    uint8_t* const words = reinterpret_cast<uint8_t*>(sShort + cap.shrt);
+    sSlot = words + (T.lo & 3u);
+    uint32_t* const short_to = sShort;
+    const uint32_t lo4 = T.lo & ~3u;
+    auto put = [&](uint32_t i, const uint4& k) {
+        if (i < T.ss)
+            *reinterpret_cast<uint32_t*>(words + (i - lo4)) =
+                (k.x & 0xffu) | (k.y & 0xffu) << 8 | (k.z & 0xffu) << 16 | k.w << 24;
+        if (i + 3 >= T.ss) {
+            const uint32_t key[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q)
+                if (i + q >= T.ss && i + q < T.hi) short_to[i + q - T.ss] = key[q];
+        }
+    };
+#pragma unroll
+    for (int t = 0; t < KEY_LOADS; ++t) {
+        const uint32_t i = lo4 + 4 * (threadIdx.x + t * TB);
+        if (i < T.hi) put(i, L.k[t]);
+    }
+    for (uint32_t i = lo4 + 4 * (threadIdx.x + KEY_LOADS * TB); i < T.hi; i += 4 * TB)
+        put(i, __ldg(reinterpret_cast<const uint4*>(v.obs_key) + i / 4));
+    for (uint32_t i = threadIdx.x; i < 3 * T.nl; i += TB) sRun[i] = __ldg(v.long_run + 3 * (size_t)T.l0 + i);
+}
+
 template <int TB>
 __device__ __forceinline__ void stage_compact(const Views<float>& v, const TileRange& T, const Caps& cap,
                                               unsigned char* dsm, uint32_t*& sRun, uint32_t*& sShort,
                                               uint8_t*& sSlot) {
-    sRun = reinterpret_cast<uint32_t*>(dsm);
-    sShort = sRun + 3 * cap.run;
-    sSlot = reinterpret_cast<uint8_t*>(sShort + cap.shrt);
-    const uint32_t nlo = T.ss - T.lo, n = T.hi - T.lo;
-    for (uint32_t i = threadIdx.x; i < n; i += TB) {
-        const uint32_t key = __ldg(v.obs_key + T.lo + i);
-        if (i < nlo) sSlot[i] = (uint8_t)(key & 0xffu);
-        else sShort[i - nlo] = key;
-    }
-    for (uint32_t i = threadIdx.x; i < 3 * T.nl; i += TB) sRun[i] = __ldg(v.long_run + 3 * (size_t)T.l0 + i);
+    store_compact<TB>(v, T, cap, load_keys<TB>(v, T), dsm, sRun, sShort, sSlot);
 }
 
+// Brings [p, p + bytes) into the L2 (16-byte aligned, a multiple of 16 bytes).
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 
 // Block sums of compensated per-thread partials (Kahan pairs s - c): FP32 pairs inside
 // each warp, FP64 across the warps; valid in thread 0.  `sh` holds 2 * (TB / 32) doubles.
@@ -183,14 +229,19 @@ __device__ __forceinline__ void tile_normal(const Views<float>& v, const TileRan
 // shared-memory adds (valid when no camera observes a point twice; see the file head).
 // Replacing the point-sum atomics of the long runs this way took the operator from 302
 // to 289 us on the 28.8M-observation workload.
+//
+// Of 281 us (19.8M observations, 4.5M points), staging and outputs took 117, the long runs 121 and
+// the short ones 33.  The staging is bound by the latency of its loads: vectors as float4, four
+// keys to a load, and the data of the tile that takes this one's place (`ahead` tiles on, all
+// CTAs in flight) brought into the L2 meanwhile: 281 -> 269 us.  Its bytes alone take 75 us.
 template <int TB, bool PLAIN_Q>
 __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int32_t* gate, const float* zs,
-                                                       int use_beta, Caps cap) {
+                                                       int use_beta, int ahead, Caps cap) {
     if (gated_off(gate)) return;
     constexpr int NQ = PLAIN_Q ? TB / 32 : 1;   // point-sum copies
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ float4 sX4[TILE_PTS], sP4[TILE_PTS];
-    __shared__ float sQ[NQ * 3 * TILE_PTS];
+    __shared__ __align__(16) float sQ[NQ * 3 * TILE_PTS];
     __shared__ unsigned int s_next;
     __shared__ double red[2 * (TB / 32)];
     DevState* st = v.st;
@@ -201,45 +252,72 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
     const bool weighted = st->opt.loss != 0;
     const TileRange T = tile_range(v, blockIdx.x);
     float jp_s = 0.0f, jp_c = 0.0f, pd_s = 0.0f, pd_c = 0.0f;
+    const KeyLoads keys = load_keys<TB>(v, T);
+    // the tile that takes this one's place on the SM: its data into the L2 meanwhile
+    if (threadIdx.x == TB - 1 && (int)blockIdx.x + ahead < v.n_tiles) {
+        const TileRange N = tile_range(v, blockIdx.x + ahead);
+        const uint32_t bytes = 12u * (uint32_t)N.npt & ~15u, k0 = N.lo & ~3u;
+        prefetch_l2(v.obs_key + k0, 4 * (N.hi - k0) & ~15u);
+        prefetch_l2(zs + N.base, bytes);
+        prefetch_l2(v.D + N.base, bytes);
+        prefetch_l2(v.x + N.base, bytes);
+        if (beta != 0.0f || ha != 0.0f) prefetch_l2(v.p + N.base, bytes);
+        if (ha != 0.0f) prefetch_l2(v.h + N.base, bytes);
+    }
+    const int ne4 = (3 * T.npt + 3) / 4;   // float4 entries (a tile's end falls on a quad of points)
     {
         // every load before the stores of p (which may alias them)
-        static_assert((3 * TILE_PTS) % TB == 0, "whole entry steps");
-        constexpr int EPT = 3 * TILE_PTS / TB;
-        const int ne = 3 * T.npt;
+        static_assert(3 * TILE_PTS / 4 <= 2 * TB, "two entries a thread");
         float* sPf = reinterpret_cast<float*>(sP4);
         float* sXf = reinterpret_cast<float*>(sX4);
-        float Z[EPT], P[EPT], Dd[EPT], X[EPT], H[EPT];
+        float4 Z[2], P[2], Dd[2], X[2], H[2];
+        const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int t = 0; t < EPT; ++t) {
-            const int i = threadIdx.x + t * TB;
-            if (i < ne) {
-                Z[t] = zs[T.base + i];
-                P[t] = beta != 0.0f || ha != 0.0f ? v.p[T.base + i] : 0.0f;
-                H[t] = ha != 0.0f ? v.h[T.base + i] : 0.0f;
-                Dd[t] = v.D[T.base + i];
-                X[t] = v.x[T.base + i];
+        for (int t = 0; t < 2; ++t) {
+            const int g = threadIdx.x + t * TB;
+            if (g < ne4) {
+                const size_t e = T.base + 4 * (size_t)g;
+                Z[t] = *reinterpret_cast<const float4*>(zs + e);
+                P[t] = beta != 0.0f || ha != 0.0f ? *reinterpret_cast<const float4*>(v.p + e) : zero;
+                H[t] = ha != 0.0f ? *reinterpret_cast<const float4*>(v.h + e) : zero;
+                Dd[t] = *reinterpret_cast<const float4*>(v.D + e);
+                X[t] = *reinterpret_cast<const float4*>(v.x + e);
             }
         }
 #pragma unroll
-        for (int t = 0; t < EPT; ++t) {
-            const int i = threadIdx.x + t * TB;
-            if (i < ne) {
-                if (ha != 0.0f) v.h[T.base + i] = fmaf(ha, P[t], H[t]);   // the last update's step
-                const float pn = beta != 0.0f ? fmaf(beta, P[t], Z[t]) : Z[t];
-                v.p[T.base + i] = pn;
-                const int slot = i / 3, k = i - 3 * slot;
-                sPf[4 * slot + k] = pn;
-                sXf[4 * slot + k] = X[t];
-                sQ[i] = mu * (Dd[t] * pn);
-                kahan_add(pd_s, pd_c, Dd[t] * pn * pn);
+        for (int t = 0; t < 2; ++t) {
+            const int g = threadIdx.x + t * TB;
+            if (g < ne4) {
+                const size_t e = T.base + 4 * (size_t)g;
+                const float4 z = Z[t], po = P[t], d = Dd[t];
+                if (ha != 0.0f)   // the last update's step
+                    *reinterpret_cast<float4*>(v.h + e) = make_float4(fmaf(ha, po.x, H[t].x), fmaf(ha, po.y, H[t].y),
+                                                                      fmaf(ha, po.z, H[t].z), fmaf(ha, po.w, H[t].w));
+                const float4 pn = beta != 0.0f ? make_float4(fmaf(beta, po.x, z.x), fmaf(beta, po.y, z.y),
+                                                             fmaf(beta, po.z, z.z), fmaf(beta, po.w, z.w))
+                                               : z;
+                *reinterpret_cast<float4*>(v.p + e) = pn;
+                const float pk[4] = {pn.x, pn.y, pn.z, pn.w}, xk[4] = {X[t].x, X[t].y, X[t].z, X[t].w};
+                const int slot = 4 * g / 3, k = 4 * g - 3 * slot;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {   // entry (slot, k + q) in rows of four floats
+                    const int o = 4 * slot + k + q + (k + q >= 3 ? 1 : 0) + (k + q >= 6 ? 1 : 0);
+                    sPf[o] = pk[q];
+                    sXf[o] = xk[q];
+                }
+                reinterpret_cast<float4*>(sQ)[g] =
+                    make_float4(mu * (d.x * pn.x), mu * (d.y * pn.y), mu * (d.z * pn.z), mu * (d.w * pn.w));
+                kahan_add(pd_s, pd_c, fmaf(d.x * pn.x, pn.x, d.y * pn.y * pn.y));
+                kahan_add(pd_s, pd_c, fmaf(d.z * pn.z, pn.z, d.w * pn.w * pn.w));
             }
         }
     }
-    for (int i = threadIdx.x; i < (NQ - 1) * 3 * TILE_PTS; i += TB) sQ[3 * TILE_PTS + i] = 0.0f;
+    for (int i = threadIdx.x; i < (NQ - 1) * 3 * TILE_PTS / 4; i += TB)
+        reinterpret_cast<float4*>(sQ + 3 * TILE_PTS)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     float* const sQw = sQ + (PLAIN_Q ? (threadIdx.x >> 5) * 3 * TILE_PTS : 0);   // this warp's copy
     uint32_t *sRun, *sShort;
     uint8_t* sSlot;
-    stage_compact<TB>(v, T, cap, dsm, sRun, sShort, sSlot);
+    store_compact<TB>(v, T, cap, keys, dsm, sRun, sShort, sSlot);
     if (threadIdx.x == 0) s_next = 0u;
     __syncthreads();
     if (weighted || eps != 0.0f)
@@ -247,11 +325,17 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
     else
         tile_normal<TB, PLAIN_Q, false>(v, T, sRun, sShort, sSlot, sX4, sP4, sQw, &s_next, eps, weighted, jp_s, jp_c);
     __syncthreads();
-    for (int i = threadIdx.x; i < 3 * T.npt; i += TB) {
-        float qi = sQ[i];
+    for (int i = threadIdx.x; i < ne4; i += TB) {
+        float4 qi = reinterpret_cast<const float4*>(sQ)[i];
 #pragma unroll
-        for (int w = 1; w < NQ; ++w) qi += sQ[w * 3 * TILE_PTS + i];
-        v.q[T.base + i] = qi;
+        for (int w = 1; w < NQ; ++w) {
+            const float4 a = reinterpret_cast<const float4*>(sQ + w * 3 * TILE_PTS)[i];
+            qi.x += a.x;
+            qi.y += a.y;
+            qi.z += a.z;
+            qi.w += a.w;
+        }
+        *reinterpret_cast<float4*>(v.q + T.base + 4 * (size_t)i) = qi;
     }
     double bj, bp;
     block_pair_sums<TB>(jp_s, jp_c, pd_s, pd_c, red, bj, bp);
@@ -1097,7 +1181,7 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
     L.wide_tiles = false;
     L.tk_run_cap = std::max(1, max_long_runs);
     L.tk_short_cap = std::max(1, max_short_obs);
-    L.tk_long_cap = (std::max(1, max_long_obs) + 15) / 16 * 16;
+    L.tk_long_cap = (std::max(1, max_long_obs) + 7 + 15) / 16 * 16;   // whole words (store_compact)
     const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
     if (compact_bytes(cap) > 160 * 1024) return;
     L.tn_smem = L.tl_smem = L.te_smem = (int)compact_bytes(cap);
@@ -1117,6 +1201,7 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
                              prepare(k_tile_step<WIDE_TB>, WIDE_TB, L.te_smem)}) >= 1;
     const int nt = std::max(1, n_tiles);
     L.tn_grid = nt;   // one CTA per tile
+    L.tn_ahead = sms * bn;
     L.tl_grid = std::max(1, std::min({nt, sms * bl, MAX_GRID}));
     L.te_grid = std::max(1, std::min({nt, sms * be, MAX_GRID}));
 }
@@ -1124,8 +1209,8 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
 void launch_tile_normal(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
                         const float* zs, int use_beta) {
     const Caps cap{L.tk_run_cap, L.tk_short_cap, L.tk_long_cap};
-    if (L.tn_plain_q) k_tile_normal<TN_TB, true><<<L.tn_grid, TN_TB, L.tn_smem, s>>>(v, gate, zs, use_beta, cap);
-    else k_tile_normal<TN_TB, false><<<L.tn_grid, TN_TB, L.tn_smem, s>>>(v, gate, zs, use_beta, cap);
+    if (L.tn_plain_q) k_tile_normal<TN_TB, true><<<L.tn_grid, TN_TB, L.tn_smem, s>>>(v, gate, zs, use_beta, L.tn_ahead, cap);
+    else k_tile_normal<TN_TB, false><<<L.tn_grid, TN_TB, L.tn_smem, s>>>(v, gate, zs, use_beta, L.tn_ahead, cap);
 }
 
 void launch_cg_round(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate, CondHandle c,
