@@ -87,7 +87,7 @@ Layout compute_layout(int32_t n_cams, int32_t n_pts, int64_t n_obs, int32_t prec
     l.blk_cams = b.take(4 * std::min(no + nfc + nc + MAX_PBLOCKS, (size_t)(MAX_PBLOCKS * 4096)));
     // bitmap of the cameras that each CTA's observations see (while the plan is made)
     l.blk_seen = precision == BA_PREC_FP64 ? 0 : b.take(4 * (size_t)MAX_PBLOCKS * ((nc + 31) / 32));
-    l.pslots = b.take(8 * PSLOT_TOTAL);
+    l.xch = b.take(XCH_BYTES);
     // long-run tables: a tile holds at most (its observations / LONG_RUN) long runs
     l.long_off = b.take(4 * (n_tiles + 1));
     l.long_run = b.take(12 * (no / LONG_RUN + n_tiles));
@@ -257,10 +257,10 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
         launch_schur_start(v, p->L, s, pcg_c, use);
     } else if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->pslots : nullptr,
+        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->xch : nullptr,
                        p->use_persistent ? 0 : (p->use_cg ? 2 : 1));
         if (p->use_persistent)
-            launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->pslots, p->p_grid,
+            launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->xch, p->p_grid,
                                   p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one, p->p_form, s);
     } else {
         launch64_precond(p->vd, p->L, s, pcg_c, use);
@@ -917,7 +917,7 @@ ba_status ba_bind_workspace(ba_problem* p, void* ws, size_t bytes, void* stream)
     p->blk_cam_off = (uint32_t*)(w + l.blk_cam_off);
     p->blk_cams = (uint32_t*)(w + l.blk_cams);
     p->blk_fac = (uint32_t*)(w + l.blk_fac);
-    p->pslots = (double*)(w + l.pslots);
+    p->xch = (ulonglong2*)(w + l.xch);
     p->persistent = p->fits_one = p->fits_two = false;
     if (p->precision == BA_PREC_MIXED) {
         ba_status pst = plan_persistent(p, sms);
@@ -1314,9 +1314,9 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
         double total_ms = 0.0;
         for (int i = 0; i <= reps; ++i) {
             open_gates();
-            launch_precond(v, p->L, s, 0, 0, p->pslots, 0);
+            launch_precond(v, p->L, s, 0, 0, p->xch, 0);
             cudaEventRecord(e0, s);
-            GBBA_CUDA(launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->pslots,
+            GBBA_CUDA(launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->xch,
                                             p->p_grid, p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one,
                                             p->p_form, s));
             cudaEventRecord(e1, s);

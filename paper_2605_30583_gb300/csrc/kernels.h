@@ -61,7 +61,7 @@ void launch_camera_precompute(const Views<float>& v, const LaunchCfg& L, cudaStr
 void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode,
                       float* res_out, float* jac_out, CondHandle lm_cond, int use_cond);
 void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
-                    double* pslots, int zero);
+                    ulonglong2* words, int zero);
 void launch_matvec(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
                    const float* zs, int use_beta);
 void launch_update(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
@@ -113,7 +113,7 @@ void launch_selftest_rcp64(const double* x, double* y, int64_t n, cudaStream_t s
 cudaError_t launch_selftest_wait(void* scratch, int grid, long long timeout_ns, cudaStream_t s);
 cudaError_t persistent_prepare(int form, int smem_bytes, int* blocks_per_sm);
 cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_tile, const uint32_t* blk_cam_off,
-                                  const uint32_t* blk_cams, const uint32_t* blk_fac, double* pslots, int grid,
+                                  const uint32_t* blk_cams, const uint32_t* blk_fac, ulonglong2* words, int grid,
                                   int smem_bytes, int form, cudaStream_t s);
 // Dynamic shared memory of the persistent kernels for a CTA with `no` observations, `np`
 // points and `ncb` listed cameras, in the order the kernels carve it: keys; X and the

@@ -22,11 +22,10 @@ constexpr int NSLOT = 32;           // atomic accumulator slots per scalar sum
 constexpr int SLOT_STRIDE = 16;     // doubles between slots (one 128-byte line)
 constexpr int MAX_CTA_TILES = 16;   // tiles of one of its CTAs
 constexpr int MAX_PBLOCKS = 256;    // CTAs of the persistent PCG kernel (one per SM)
-// Exchange area of the persistent PCG kernels: three rotating slot sets of NSLOT
-// slots, each slot XCH_NV sums (doubles), cleared before every launch.
+// Exchange area of the persistent PCG kernels: two alternating sets of XCH_NV sums of every CTA,
+// 16 bytes each (two 64-bit words), cleared before every launch.
 constexpr int XCH_NV = 4;
-constexpr int PSLOT_TOTAL = 3 * NSLOT * SLOT_STRIDE;
-static_assert(XCH_NV <= SLOT_STRIDE, "a slot holds every sum of one exchange");
+constexpr int XCH_BYTES = 2 * XCH_NV * MAX_PBLOCKS * 16;
 // Camera accumulator sets of the one-exchange kernel (rotating over iterations).
 constexpr int CA_SETS = 3;
 // A camera run of a tile this long or longer is walked in camera-uniform warp steps.
@@ -97,8 +96,7 @@ struct DevState {
     int32_t pcg_iter, pcg_active, pcg_total, pad0;
     int64_t t_start, t_end;
     uint32_t tickets[TK_COUNT];
-    unsigned long long bar_count;   // arrivals at the grid barriers of the persistent PCG kernel
-    int32_t bar_err, pad1;
+    int32_t bar_err, pad1;   // a wait of the persistent PCG kernel ran out of time
     IterRec hist[HIST_CAP];
 };
 

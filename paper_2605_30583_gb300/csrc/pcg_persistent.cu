@@ -4,9 +4,9 @@
 // One cooperative launch runs every PCG iteration of one LM step.  The grid is one
 // CTA per SM; CTA b owns a contiguous run of tiles (balanced by observation count)
 // and keeps, for the whole solve, its observation keys and its points' X, D, M^-1
-// and PCG vectors in shared memory.  Grid-wide sums travel through an exchange:
-// slot-spread atomic sums followed by a grid barrier, after which every CTA reads the
-// same totals and so takes the same stop decision.  Every wait is time-bounded: on a
+// and PCG vectors in shared memory.  Grid-wide sums travel through an exchange: every CTA
+// publishes its sums and waits for those of all others, which it adds up in the same
+// order and so takes the same stop decision.  Every wait is time-bounded: on a
 // time-out the CTA sets an error flag, every CTA leaves, and the solve reports
 // BA_ERR_TIMEOUT.
 //
@@ -45,48 +45,82 @@ namespace gbba {
 
 namespace {
 
-// Arrival at grid-wide barrier number `epoch` (1, 2, ... within a launch) of a co-resident
-// (cooperative) grid, and the wait for the others, by one thread whose CTA's writes happen
-// before (a CTA or warp barrier).  Each CTA adds one to a counter, cleared before the launch,
-// with release semantics, and waits until it reaches epoch * nblocks: the count can only
-// get there once every CTA has arrived, and a CTA that has already moved on to the
-// next barrier only raises it further.  False on time-out or when another CTA has
-// already reported one.  Limits below 1 ms are checked at every poll (0: give up at the
-// first poll that finds the barrier incomplete), longer ones every 64th poll; the limit
-// counts from the first check, so a wait that ends sooner never reads the (slow) timer.
-__device__ __forceinline__ bool grid_arrive_wait(unsigned long long* cnt, int* err, unsigned int nblocks,
-                                                 unsigned long long epoch, long long timeout_ns) {
-    bool ok = true;
-    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(cnt), "l"(1ull) : "memory");
-    const unsigned long long target = epoch * nblocks;
-    long long t0 = -1;
+// The limit of a wait for other CTAs, asked by one thread after each poll that found something
+// missing: true when the wait is over because it ran out of time (the shared error word is then
+// set) or another CTA's did.  Limits below 1 ms are checked at every poll (0: give up at the first
+// one), longer ones every 64th; the limit counts from the first check, so a wait that ends
+// sooner never reads the (slow) timer.
+struct WaitLimit {
+    int* err;
+    long long limit_ns, t0 = -1;
     unsigned spins = 0;
-    for (;;) {
-        unsigned long long c;
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(cnt) : "memory");
-        if (c >= target) break;
-        if (timeout_ns < 1000000LL || (++spins & 63u) == 0u) {
-            if (*reinterpret_cast<volatile int*>(err)) { ok = false; break; }
-            const long long now = global_ns();
-            if (t0 < 0) t0 = now;
-            if (now - t0 >= timeout_ns) {
-                atomicExch(err, 1);
-                ok = false;
-                break;
-            }
-        }
+    __device__ __forceinline__ bool over() {
+        if (limit_ns >= 1000000LL && (++spins & 63u) != 0u) return false;
+        if (*reinterpret_cast<volatile int*>(err)) return true;
+        const long long now = global_ns();
+        if (t0 < 0) t0 = now;
+        if (now - t0 < limit_ns) return false;
+        atomicExch(err, 1);
+        return true;
     }
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    return ok;
+};
+
+// One published sum: a float pair, each half in a 64-bit word with the exchange's number in its
+// upper 32 bits (64-bit accesses are not torn, so a reader needs no order between the words).
+__device__ __forceinline__ void publish(ulonglong2* to, float hi, float lo, uint32_t epoch) {
+    const unsigned long long e = (unsigned long long)epoch << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(to), "l"(e | __float_as_uint(hi)),
+                 "l"(e | __float_as_uint(lo))
+                 : "memory");
 }
 
-__device__ __forceinline__ bool grid_sync_on(unsigned long long* cnt, int* err, unsigned int nblocks,
-                                             unsigned long long epoch, long long timeout_ns) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) s_ok = grid_arrive_wait(cnt, err, nblocks, epoch, timeout_ns) ? 1 : 0;
-    __syncthreads();
-    return s_ok != 0;
+// Waits until the sums of `n` <= MAX_PBLOCKS CTAs at `from` carry `epoch` and adds them up, in the
+// same order in every CTA; one warp, the total in every lane.  False when the wait's limit ran out.
+__device__ __forceinline__ bool gather(const ulonglong2* from, int n, uint32_t epoch, WaitLimit limit, float& hi,
+                                       float& lo) {
+    constexpr int PER = MAX_PBLOCKS / 32;
+    const int lane = threadIdx.x & 31;
+    float h[PER], l[PER];
+    unsigned missing = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        h[i] = l[i] = 0.0f;
+        if (lane + 32 * i < n) missing |= 1u << i;
+    }
+    for (;;) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (missing >> i & 1u) {
+                unsigned long long a, b;
+                asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(from + lane + 32 * i) : "memory");
+                if ((uint32_t)(a >> 32) == epoch && (uint32_t)(b >> 32) == epoch) {
+                    h[i] = __uint_as_float((uint32_t)a);
+                    l[i] = __uint_as_float((uint32_t)b);
+                    missing &= ~(1u << i);
+                }
+            }
+        if (__all_sync(FULL, missing == 0u)) break;
+        int over = 0;
+        if (lane == 0) over = limit.over() ? 1 : 0;
+        if (__shfl_sync(FULL, over, 0)) return false;
+    }
+    hi = lo = 0.0f;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        float s, e;
+        two_sum(hi, h[i], s, e);
+        hi = s;
+        lo += l[i] + e;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float h2 = __shfl_xor_sync(FULL, hi, o), l2 = __shfl_xor_sync(FULL, lo, o);
+        float s, e;
+        two_sum(hi, h2, s, e);
+        hi = s;
+        lo = (lo + l2) + e;
+    }
+    return true;
 }
 
 // What the CTA does after an exchange, decided by one thread for all.  FP64 runs at 1/64 of
@@ -100,64 +134,64 @@ struct PcgStep {
 
 // Grid-wide sums of XCH_NV per-warp values, the grid barrier, and the decision.  red holds the
 // CTA's compensated partials, value k of warp w at red[NW k + w]; with `last_only` the values
-// before the last count as zero.  Exchange e adds into slot set e % 3 (CTA b into slot
-// b % NSLOT, so concurrent atomics spread over NSLOT lines); every CTA then reads the same
-// totals, and lane 0 calls decide(totals), which writes the shared step.  After the barrier
-// block 0 clears set (e + 2) % 3: it was last read before barrier e, which every CTA has
-// reached, and is next filled past barrier e + 1, which waits for block 0.  Call with the
-// partials published (a barrier before); returns after a barrier.
+// before the last count as zero.  Warp k adds up the CTA's value k and publishes it with the
+// number of the exchange, then gathers the value k of every CTA: there is no counter to arrive
+// at and no second read, the sums themselves say that their CTA has arrived.  (Slot-spread FP64
+// atomics, a release on a counter, the wait and the read of the slots: ~5.5 us.)  Two sets of
+// words alternate: a CTA that publishes exchange e + 2 has seen every CTA's e + 1, which each
+// published after reading all of e.  What the CTAs wrote before (camera sums) is visible after:
+// the last value's publisher and readers carry the fences.  Thread 0 calls decide(totals), which
+// writes the shared step.  Call with the partials published (a barrier before); returns after
+// a barrier.
 template <int NW, typename F>
-__device__ __forceinline__ void exchange(DevState* st, double* pslots, unsigned long long epoch, const float2* red,
+__device__ __forceinline__ void exchange(DevState* st, ulonglong2* words, uint32_t epoch, const float2* red,
                                          bool last_only, PcgStep* step, F&& decide) {
-    static_assert(XCH_NV == 4 && NSLOT == 32, "lane l holds value l % 4 of every eighth warp or slot");
-    double* cur = pslots + (size_t)(epoch % 3ull) * NSLOT * SLOT_STRIDE;
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x, k = lane & 3, q = lane >> 2;
-        // the warps' pairs summed as pairs (an FP64 addition has ~130 cycles of latency, a pair's
-        // six FP32 operations ~30), one FP64 value per sum to the slot
+    static_assert(NW >= XCH_NV && NW <= 32 && (NW & (NW - 1)) == 0, "a warp per value, a lane per warp");
+    __shared__ double s_tot[XCH_NV];
+    __shared__ int s_ok[XCH_NV];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < XCH_NV) {
+        const bool last = w == XCH_NV - 1;
+        ulonglong2* cur = words + (size_t)((epoch & 1u) * XCH_NV + w) * MAX_PBLOCKS;
         float hi = 0.0f, lo = 0.0f;
-        if (!last_only || k == XCH_NV - 1)
-            for (int w = q; w < NW; w += 8) {
-                float s, e;
-                const float2 p = red[NW * k + w];
-                two_sum(hi, p.x, s, e);
-                hi = s;
-                lo += p.y + e;
-            }
+        if (lane < NW && (last || !last_only)) {
+            const float2 p = red[NW * w + lane];
+            hi = p.x;
+            lo = p.y;
+        }
 #pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            const float h2 = __shfl_xor_sync(FULL, hi, o), l2 = __shfl_xor_sync(FULL, lo, o);
+        for (int o = NW / 2; o > 0; o >>= 1) {
+            const float h2 = __shfl_down_sync(FULL, hi, o), l2 = __shfl_down_sync(FULL, lo, o);
             float s, e;
             two_sum(hi, h2, s, e);
             hi = s;
-            lo = lo + l2 + e;
+            lo = (lo + l2) + e;
         }
-        if (q == 0 && (hi != 0.0f || lo != 0.0f)) slot_add(cur, k, widen(hi) + widen(lo));
+        if (lane == 0) {
+            if (last) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            publish(cur + blockIdx.x, hi, lo, epoch);
+        }
         __syncwarp();
-        int ok = 1;
-        if (lane == 0) ok = grid_arrive_wait(&st->bar_count, &st->bar_err, gridDim.x, epoch, st->opt.wait_ns) ? 1 : 0;
-        ok = __shfl_sync(FULL, ok, 0);
-        __syncwarp();
-        if (ok) {
-            double x[NSLOT / 8];
-#pragma unroll
-            for (int s = 0; s < NSLOT / 8; ++s) x[s] = __ldcg(&cur[(q + 8 * s) * SLOT_STRIDE + k]);
-            double d = (x[0] + x[1]) + (x[2] + x[3]);
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) d += __shfl_xor_sync(FULL, d, o);
+        const bool ok = gather(cur, gridDim.x, epoch, WaitLimit{&st->bar_err, st->opt.wait_ns}, hi, lo);
+        if (last) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        if (lane == 0) {
+            s_tot[w] = widen(hi) + widen(lo);
+            s_ok[w] = ok;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * XCH_NV) : "memory");
+        if (threadIdx.x == 0) {
             double tot[XCH_NV];
+            bool all = true;
 #pragma unroll
-            for (int i = 0; i < XCH_NV; ++i) tot[i] = __shfl_sync(FULL, d, i);
-            if (lane == 0) decide(tot);
-        } else if (lane == 0) {
-            step->act = ACT_TIMEOUT;
+            for (int i = 0; i < XCH_NV; ++i) {
+                tot[i] = s_tot[i];
+                all = all && s_ok[i] != 0;
+            }
+            if (all) decide(tot);
+            else step->act = ACT_TIMEOUT;
         }
     }
     __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x >= 32) {
-        double* nx = pslots + (size_t)((epoch + 2ull) % 3ull) * NSLOT * SLOT_STRIDE;
-        for (int i = threadIdx.x - 32; i < NSLOT * SLOT_STRIDE; i += blockDim.x - 32) nx[i] = 0.0;
-    }
 }
 
 // Tests on the high word, off the chain of FP64 operations.
@@ -295,7 +329,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
                                                          const uint32_t* __restrict__ blk_cam_off,
                                                          const uint32_t* __restrict__ blk_cams,
                                                          const uint32_t* __restrict__ blk_fac,
-                                                         double* __restrict__ pslots) {
+                                                         ulonglong2* __restrict__ words) {
     const uint32_t f0 = __ldg(blk_fac + blockIdx.x), f1 = __ldg(blk_fac + blockIdx.x + 1);
     DevState* st = v.st;
     if (st->pcg_active == 0) return;
@@ -368,7 +402,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
     const double stop_rr = st->opt.tol * st->opt.tol * rr;
     bool numeric_fail = false;
     float beta = 0.0f;
-    unsigned long long epoch = 0ull;
+    uint32_t epoch = 0u;
     int k = 0;
     bool ok = true;
     for (int i = tid; i < XCH_NV * NW; i += TB) red[i] = make_float2(0.0f, 0.0f);
@@ -417,7 +451,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
             }
         }
         __syncthreads();
-        exchange<NW>(st, pslots, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
+        exchange<NW>(st, words, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
             const double denom = tot[0] + mu * tot[1];
             if (!positive_finite64(denom)) {
                 numeric_fail = !finite64(denom);
@@ -552,7 +586,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
         }
         __syncthreads();
         ++k;
-        exchange<NW>(st, pslots, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
+        exchange<NW>(st, words, ++epoch, red, false, &step, [&](const double (&tot)[XCH_NV]) {
             // ------------------------------------------------------------ phase C
             const double rzn = tot[0];
             rr = tot[1];
@@ -742,7 +776,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
                                                          const uint32_t* __restrict__ blk_cam_off,
                                                          const uint32_t* __restrict__ blk_cams,
                                                          const uint32_t* __restrict__ blk_fac,
-                                                         double* __restrict__ pslots) {
+                                                         ulonglong2* __restrict__ words) {
     const uint32_t f0 = __ldg(blk_fac + blockIdx.x), f1 = __ldg(blk_fac + blockIdx.x + 1);
     DevState* st = v.st;
     if (st->pcg_active == 0) return;
@@ -862,7 +896,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     const double stop_rr = st->opt.tol * st->opt.tol * rr;
     bool numeric_fail = false;
     int checks = 0;
-    unsigned long long epoch = 0ull;
+    uint32_t epoch = 0u;
     int k = 0;    // PCG updates
     int it = 0;   // operator passes (they rotate the camera accumulator sets)
     // Residual replacement (van der Vorst and Ye, SIAM J. Sci. Comput. 22, 2000): when the
@@ -886,7 +920,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
         if ((tid & 31) == 0) red[3 * NW + (tid >> 5)] = jw;
         __syncthreads();
         // ------------------------------------------------------------ X: exchange
-        exchange<NW>(st, pslots, ++epoch, red, verify, &step, [&](const double (&tot)[XCH_NV]) {
+        exchange<NW>(st, words, ++epoch, red, verify, &step, [&](const double (&tot)[XCH_NV]) {
             if (verify) {   // a verification pass only assembles A h
                 step.act = ACT_UPDATE;
                 return;
@@ -967,7 +1001,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     // owners leave all of them cleared
     if (ok) {
         __syncthreads();
-        exchange<NW>(st, pslots, ++epoch, red, true, &step, [&](const double (&)[XCH_NV]) { step.act = ACT_STOP; });
+        exchange<NW>(st, words, ++epoch, red, true, &step, [&](const double (&)[XCH_NV]) { step.act = ACT_STOP; });
         ok = step.act != ACT_TIMEOUT;
     }
     for (int e = tid; e < ne; e += TB) {
@@ -1010,7 +1044,7 @@ cudaError_t persistent_prepare(int form, int smem_bytes, int* blocks_per_sm) {
 }
 
 cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_tile, const uint32_t* blk_cam_off,
-                                  const uint32_t* blk_cams, const uint32_t* blk_fac, double* pslots, int grid,
+                                  const uint32_t* blk_cams, const uint32_t* blk_fac, ulonglong2* words, int grid,
                                   int smem_bytes, int form, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -1023,19 +1057,21 @@ cudaError_t launch_pcg_persistent(const Views<float>& v, const uint32_t* blk_til
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (form == PCG_TWO_EXCHANGE)
-        return cudaLaunchKernelEx(&cfg, k_pcg_persistent<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, pslots);
-    return cudaLaunchKernelEx(&cfg, k_pcg_persistent_1x<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, pslots);
+        return cudaLaunchKernelEx(&cfg, k_pcg_persistent<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, words);
+    return cudaLaunchKernelEx(&cfg, k_pcg_persistent_1x<PCG_TB>, v, blk_tile, blk_cam_off, blk_cams, blk_fac, words);
 }
 
-// Self-test of the bounded grid wait: a cooperative grid of `grid` CTAs waits at a
-// barrier that counts one CTA more than it has, which nothing will ever complete.
-// Every CTA must give up after `timeout_ns`, set the shared error word and return;
-// scratch = {arrival count (u64), error word (i32), CTAs that gave up (u32)}.
+// Self-test of the bounded wait: every CTA of a cooperative grid waits for a sum that nothing will
+// ever publish.  Every CTA must give up after `timeout_ns`, set the shared error word and
+// return; scratch = {unused (u64), error word (i32), CTAs that gave up (u32)}.
+__device__ ulonglong2 selftest_words[1];
+
 __global__ void k_selftest_wait(unsigned long long* scratch, long long timeout_ns) {
     int* err = reinterpret_cast<int*>(scratch + 1);
-    unsigned int* gave_up = reinterpret_cast<unsigned int*>(scratch + 1) + 1;
-    const bool ok = grid_sync_on(scratch, err, gridDim.x + 1, 1ull, timeout_ns);
-    if (!ok && threadIdx.x == 0) atomicAdd(gave_up, 1u);
+    if (threadIdx.x >= 32) return;
+    float hi, lo;
+    const bool ok = gather(selftest_words, 1, 1u, WaitLimit{err, timeout_ns}, hi, lo);
+    if (!ok && threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned int*>(err) + 1, 1u);
 }
 
 __global__ void k_selftest_rcp64(const double* __restrict__ x, double* __restrict__ y, int64_t n) {

@@ -27,7 +27,7 @@ ba_status cuda_status(cudaError_t e, const char* what);
 struct Layout {
     size_t state, partials, obs_key, obs_uv, obs_user, tile_off, pt_user, pt_internal, obs_pm, pt_obs_off;
     size_t vec[10];                      // x, x_new, h, r, z, p, q, g, D, s
-    size_t blk_tile, blk_cam_off, blk_cams, blk_seen, blk_fac, pslots;
+    size_t blk_tile, blk_cam_off, blk_cams, blk_seen, blk_fac, xch;
     size_t long_off, long_run, short_start;
     size_t xm, xm_new;                   // mixed form: FP64 master parameters (0 in the plain form)
     size_t cam_lo, cam_lo_new, rbuf;     // mixed form: low-order camera records, residuals
@@ -107,7 +107,7 @@ struct ba_problem {
     uint32_t* blk_cam_off = nullptr;   // device, [p_grid + 1]: per-CTA camera list offsets
     uint32_t* blk_cams = nullptr;      // device, the lists (inside the ordering region of the workspace)
     uint32_t* blk_fac = nullptr;    // device, [p_grid + 1]: first pose factor of each CTA
-    double* pslots = nullptr;       // device, [PSLOT_TOTAL]
+    ulonglong2* xch = nullptr;      // device, [XCH_BYTES]
 
 };
 
