@@ -228,15 +228,12 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 //
 // Bound by the FP64 pipe (point_inverse).  `zero`: which PCG vectors the solver that follows wants cleared
 // (0 none, 1 h, 2 h, p and s).
-__global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, double* pslots, int cam_blocks,
+__global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulonglong2* words, int cam_blocks,
                           int zero) {
     DevState* st = v.st;
-    if (pslots != nullptr && blockIdx.x == 0) {   // state of the persistent PCG kernel
-        for (int i = threadIdx.x; i < PSLOT_TOTAL; i += blockDim.x) pslots[i] = 0.0;
-        if (threadIdx.x == 0) {
-            st->bar_count = 0ull;
-            st->bar_err = 0;
-        }
+    if (words != nullptr && blockIdx.x == 0) {   // state of the persistent PCG kernel
+        for (int i = threadIdx.x; i < XCH_BYTES / 16; i += blockDim.x) words[i] = make_ulonglong2(0ull, 0ull);
+        if (threadIdx.x == 0) st->bar_err = 0;
     }
     if (st->lm_active == 0) {
         // the PCG loop that follows must see a cleared flag
@@ -300,7 +297,7 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, dou
         }
         if (lane < CA_STRIDE) {
             v.cam_acc[(size_t)c * CA_STRIDE + lane] = 0.0f;
-            if (pslots != nullptr)   // the persistent kernel rotates over all the sets
+            if (words != nullptr)   // the persistent kernel rotates over all the sets
                 for (int set = 1; set < CA_SETS; ++set)
                     v.cam_acc[((size_t)set * v.n_cams + c) * CA_STRIDE + lane] = 0.0f;
         }
@@ -1187,12 +1184,12 @@ void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s,
                                                                                  lm_cond, use_cond);
 }
 void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
-                    double* pslots, int zero) {
+                    ulonglong2* words, int zero) {
     // camera blocks: a warp per camera; point blocks: a thread per point
     const int wpb = L.item_block / 32;
     const int cam_blocks = std::max(1, std::min((v.n_cams + wpb - 1) / wpb, L.item_grid / 2));
     const int pt_blocks = std::max(1, std::min(grid_items(L, v.n_pts), L.item_grid - cam_blocks));
-    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, pslots, cam_blocks, zero);
+    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, words, cam_blocks, zero);
 }
 static void launch_cam_direction(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
                                  const float* zs, int use_beta) {
