@@ -278,37 +278,29 @@ __device__ void b_precond(const BatchView& b, const Prob& P, double mu, double* 
     const float* gv = b.g + P.v0;
     float lrz = 0.0f, lrr = 0.0f;
     const float lo_f = __double2float_ru(o.min_diag), hi_f = __double2float_rd(o.max_diag);
-    const int lane = threadIdx.x & 31;
-    for (int c = threadIdx.x >> 5; c < P.nc; c += blockDim.x >> 5) {   // one warp per camera
-        const float* Hc = b.cam_H + (size_t)(P.c0 + c) * CH_STRIDE;
-        const int j = lane < 18 ? lane : 17;
-        double col[9];
-        for (int i = 0; i < 9; ++i) {
-            if (j < 9) {
-                double hv = Hc[tri_index(9, i < j ? i : j, i < j ? j : i)];
-                if (i == j) hv += mu * fmin(fmax(hv, o.min_diag), o.max_diag);
-                col[i] = hv;
-            } else {
-                col[i] = (i == j - 9) ? 1.0 : 0.0;
+    for (int c0 = 3 * (int)(threadIdx.x >> 5); c0 < P.nc; c0 += 3 * (int)(blockDim.x >> 5)) {
+        const CamLane L = cam_lane(c0, P.nc);
+        double col[9], D, diag;
+        const bool ok = camera_inverse9(b.cam_H + (size_t)(P.c0 + L.cam) * CH_STRIDE, mu, o.min_diag, o.max_diag, L, col, D,
+                                        diag);
+        float* Mo = b.Minv_c + (size_t)(P.c0 + L.cam) * 81;
+        if (L.live) {
+            if (ok) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) Mo[i * 9 + L.i] = narrow(col[i]);
+            } else {   // not SPD in FP64: inverse diagonal
+#pragma unroll
+                for (int i = 0; i < 9; ++i) Mo[i * 9 + L.i] = (i == L.i && diag > 0.0) ? (float)(1.0 / diag) : 0.0f;
             }
         }
-        const double hd = lane < 9 ? (double)Hc[tri_index(9, lane, lane)] : 0.0;
-        const bool ok = warp_block_inverse9(col, lane);
-        float* Mo = b.Minv_c + (size_t)(P.c0 + c) * 81;
-        if (lane >= 9 && lane < 18)
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + (lane - 9)] = (float)col[i];
-        if (!ok && lane < 9) {   // not SPD in FP64: inverse diagonal
-            const double dd = hd + mu * fmin(fmax(hd, o.min_diag), o.max_diag);
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + lane] = (i == lane && dd > 0.0) ? (float)(1.0 / dd) : 0.0f;
-        }
         __syncwarp();
-        if (lane < 9) {
-            const int e = 9 * c + lane;
-            Dv[e] = (float)fmin(fmax(hd, o.min_diag), o.max_diag);
-            const double* gc = b.cam_g + (size_t)(P.c0 + c) * CL_STRIDE;
-            const float ri = (float)(-gc[lane]);
-            float zz = 0.0f;
-            for (int k = 0; k < 9; ++k) zz = fmaf(Mo[lane * 9 + k], (float)(-gc[k]), zz);
+        const int e = 9 * L.cam + L.i;
+        const float ri = narrow(-b.cam_g[(size_t)(P.c0 + L.cam) * CL_STRIDE + L.i]);
+        float zz = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) zz = fmaf(Mo[L.i * 9 + k], __shfl_sync(0xffffffffu, ri, L.base + k), zz);
+        if (L.live) {
+            Dv[e] = narrow(D);
             r[e] = ri; z[e] = zz; pv[e] = 0.0f; h[e] = 0.0f;
             lrz = fmaf(ri, zz, lrz);
             lrr = fmaf(ri, ri, lrr);

@@ -473,28 +473,58 @@ __device__ __forceinline__ Geo project_geo(const Cam& c, float X0, float X1, flo
     return g;
 }
 
-// Inverse of one camera block, one warp per camera: lane j < 18 holds column j of
-// the augmented matrix [A | I] (A = H + mu D, 9 x 9, SPD) and Gauss-Jordan elimination
-// without pivoting runs over the 9 pivots in FP64.  Lanes 9..17 end with the columns
-// of A^-1.  Returns false (in every lane) if a pivot is not within [1e-300, 1e300].
-__device__ __forceinline__ bool warp_block_inverse9(double (&col)[9], int lane) {
+// Three cameras a warp, nine lanes each: lane `i` of the group that starts at lane `base` works on
+// column i of camera `cam`; a lane without a camera (live false) repeats lane 0's work.
+struct CamLane {
+    int cam, i, base;
+    bool live;
+};
+
+__device__ __forceinline__ CamLane cam_lane(int c0, int n_cams) {
+    const int lane = threadIdx.x & 31, sub = lane / 9;
+    const bool live = lane < 27 && c0 + sub < n_cams;
+    return {live ? c0 + sub : c0, live ? lane - 9 * sub : 0, live ? 9 * sub : 0, live};
+}
+
+__device__ __forceinline__ double to_fp64(float x) { return widen(x); }
+__device__ __forceinline__ double to_fp64(double x) { return x; }
+
+// Inverse of camera blocks A = H + mu D (9 x 9, SPD), H given by its upper triangle: column i of
+// A^-1 to `col` of lane i, D_i = H_ii clamped to [lo, hi] to `D`, A_ii to `diag`.  In-place
+// Gauss-Jordan elimination without pivoting in FP64: step k multiplies row k by 1 / a_kk,
+// takes a_ik times it from the other rows and leaves column k of the inverse in column k's place
+// (the operations of the elimination of [A | I], without its columns that are still those of
+// I).  Bound by the FP64 pipe, which a warp instruction holds for 16 cycles: one camera a warp
+// with its 18 columns took three times as long.  False if a pivot is not within [1e-300, 1e300].
+// Every lane of the warp calls it.
+template <typename T>
+__device__ __forceinline__ bool camera_inverse9(const T* __restrict__ H, double mu, double lo, double hi,
+                                                const CamLane& L, double (&col)[9], double& D, double& diag) {
+    const double h = to_fp64(H[tri_index(9, L.i, L.i)]);
+    D = fmin(fmax(h, lo), hi);
+    diag = fma(mu, D, h);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const double x = to_fp64(H[tri_index(9, q < L.i ? q : L.i, q < L.i ? L.i : q)]);
+        col[q] = q == L.i ? diag : x;
+    }
     bool ok = true;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const double piv = __shfl_sync(0xffffffffu, col[k], k);
+        const double piv = __shfl_sync(0xffffffffu, col[k], L.base + k);
         // positive, finite and within rcp64's range, from the high word: an integer test stays off
         // the chain of FP64 operations (~130 cycles each)
         ok = ok && (uint32_t)__double2hiint(piv) - 0x01a56e20u <= 0x7e37e43bu - 0x01a56e20u;
         const double ip = rcp64_fast(piv);
-        const double rk = col[k] * ip;   // row k of the updated matrix, this lane's column
+        const bool own = L.i == k;
+        const double rk = own ? ip : col[k] * ip;   // row k of the updated matrix, this lane's column
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            const double aik = __shfl_sync(0xffffffffu, col[i], k);
-            if (i != k) col[i] = fma(-aik, rk, col[i]);
+            const double aik = __shfl_sync(0xffffffffu, col[i], L.base + k);
+            if (i != k) col[i] = fma(-aik, rk, own ? 0.0 : col[i]);
         }
         col[k] = rk;
     }
-    (void)lane;
     return ok;
 }
 

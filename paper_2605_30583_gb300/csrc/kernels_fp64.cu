@@ -223,38 +223,24 @@ __global__ void k64_precond(V64 v, CondHandle pcg_cond, int use_cond) {
     }
     const double mu = st->mu, lo = st->opt.min_diag, hi = st->opt.max_diag;
     double rz = 0.0, rr = 0.0;
-    const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
-    for (int c = gtid() >> 5; c < v.n_cams; c += warps) {
-        const double* H = v.cam_H64 + (size_t)c * CH_STRIDE;
-        double col[9];
-        const int j = lane < 18 ? lane : 17;
-        for (int i = 0; i < 9; ++i) {
-            if (j < 9) {
-                double h = H[tri_index(9, i < j ? i : j, i < j ? j : i)];
-                if (i == j) h += mu * fmin(fmax(h, lo), hi);
-                col[i] = h;
-            } else {
-                col[i] = (i == j - 9) ? 1.0 : 0.0;
-            }
-        }
-        const double hdiag = lane < 9 ? H[tri_index(9, lane, lane)] : 0.0;
-        const bool ok = warp_block_inverse9(col, lane);
+    for (int c0 = 3 * (int)(gtid() >> 5); c0 < v.n_cams; c0 += 3 * warps) {
+        const CamLane L = cam_lane(c0, v.n_cams);
+        const int c = L.cam;
+        double col[9], D, diag;
+        const bool ok = camera_inverse9(v.cam_H64 + (size_t)c * CH_STRIDE, mu, lo, hi, L, col, D, diag);
         double* Mo = v.Minv_c + (size_t)c * MC_STRIDE;
-        if (lane >= 9 && lane < 18)
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + (lane - 9)] = col[i];
-        if (!ok && lane < 9) {
-            const double dd = hdiag + mu * fmin(fmax(hdiag, lo), hi);
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + lane] = (i == lane && dd > 0.0) ? 1.0 / dd : 0.0;
-        }
+        if (L.live)
+            for (int i = 0; i < 9; ++i)
+                Mo[i * 9 + L.i] = ok ? col[i] : (i == L.i && diag > 0.0) ? 1.0 / diag : 0.0;
         __syncwarp();
-        if (lane < 9) {
-            const size_t e = 9 * (size_t)c + lane;
-            v.D[e] = fmin(fmax(hdiag, lo), hi);
+        if (L.live) {
+            const size_t e = 9 * (size_t)c + L.i;
+            v.D[e] = D;
             const double* gc = v.cam_lin + (size_t)c * CL_STRIDE;
-            const double ri = -gc[lane];
+            const double ri = -gc[L.i];
             double z = 0.0;
-            for (int k = 0; k < 9; ++k) z += Mo[lane * 9 + k] * (-gc[k]);
+            for (int k = 0; k < 9; ++k) z += Mo[L.i * 9 + k] * (-gc[k]);
             v.r[e] = ri;
             v.z[e] = z;
             v.p[e] = 0.0;
@@ -669,7 +655,7 @@ void launch64_linearize(const V64& v, const LaunchCfg& L, cudaStream_t s, int mo
     k64_linearize<<<tiles64(v), T64, 0, s>>>(v, mode, r, J, c, use);
 }
 void launch64_precond(const V64& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use) {
-    k64_precond<<<g64(L, std::max((size_t)v.n_pts, 32 * (size_t)v.n_cams)), L.item_block, 0, s>>>(v, c, use);
+    k64_precond<<<g64(L, std::max((size_t)v.n_pts, 11 * (size_t)v.n_cams)), L.item_block, 0, s>>>(v, c, use);
 }
 void launch64_direction(const V64& v, const LaunchCfg& L, cudaStream_t s, const double* zs, int use_beta,
                         const int32_t* gate) {

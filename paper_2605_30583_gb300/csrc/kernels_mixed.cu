@@ -244,47 +244,32 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
     // the bounds as floats on the inner side: h >= lo exactly when h >= lo_f
     const float lo_f = __double2float_ru(lo), hi_f = __double2float_rd(hi);
     float rz = 0.0f, rr = 0.0f, rzc = 0.0f, rrc = 0.0f;   // Kahan pairs
-    const int lane = threadIdx.x & 31;
     const int warps = cam_blocks * (blockDim.x >> 5);
     const bool cam_role = (int)blockIdx.x < cam_blocks;
-    for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; cam_role && c < v.n_cams; c += warps) {
-        const double* cl = v.cam_lin + (size_t)c * CL_STRIDE;
-        double col[9];
-        const int j = lane < 18 ? lane : 17;
+    for (int c0 = 3 * (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); cam_role && c0 < v.n_cams; c0 += 3 * warps) {
+        const CamLane L = cam_lane(c0, v.n_cams);
+        const int c = L.cam;
+        double col[9], D, diag;
+        const bool ok = camera_inverse9(v.cam_H + (size_t)c * CH_STRIDE, mu, lo, hi, L, col, D, diag);
+        float* Mo = v.Minv_c + (size_t)c * MC_STRIDE;
+        if (L.live) {
+            if (ok) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            if (j < 9) {
-                const int lo_i = i < j ? i : j, hi_i = i < j ? j : i;
-                double h = (double)v.cam_H[(size_t)c * CH_STRIDE + tri_index(9, lo_i, hi_i)];
-                if (i == j) h += mu * fmin(fmax(h, lo), hi);
-                col[i] = h;
-            } else {
-                col[i] = (i == j - 9) ? 1.0 : 0.0;
+                for (int i = 0; i < 9; ++i) Mo[i * 9 + L.i] = narrow(col[i]);
+            } else {   // not SPD in FP64: inverse diagonal
+#pragma unroll
+                for (int i = 0; i < 9; ++i) Mo[i * 9 + L.i] = (i == L.i && diag > 0.0) ? (float)(1.0 / diag) : 0.0f;
             }
         }
-        // diagonal of J^T J for D and for the fallback, before elimination
-        const double hdiag = (lane < 9) ? (double)v.cam_H[(size_t)c * CH_STRIDE + tri_index(9, lane, lane)] : 0.0;
-        const bool ok = warp_block_inverse9(col, lane);
-        float* Mo = v.Minv_c + (size_t)c * MC_STRIDE;
-        if (lane >= 9 && lane < 18) {
-            const int jj = lane - 9;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + jj] = (float)col[i];
-        }
-        if (!ok && lane < 9) {   // not SPD in FP64: inverse diagonal
-            const double dd = hdiag + mu * fmin(fmax(hdiag, lo), hi);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) Mo[i * 9 + lane] = (i == lane && dd > 0.0) ? (float)(1.0 / dd) : 0.0f;
-        }
         __syncwarp();
-        if (lane < 9) {
-            const size_t e = 9 * (size_t)c + lane;
-            v.D[e] = (float)fmin(fmax(hdiag, lo), hi);
-            const float ri = (float)(-cl[CL_G + lane]);
-            // z_i = sum_k M[i][k] r_k
-            float z = 0.0f;
+        const size_t e = 9 * (size_t)c + L.i;
+        const float ri = narrow(-v.cam_lin[(size_t)c * CL_STRIDE + CL_G + L.i]);
+        // z_i = sum_k M[i][k] r_k
+        float z = 0.0f;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) z = fmaf(Mo[lane * 9 + k], (float)(-cl[CL_G + k]), z);
+        for (int k = 0; k < 9; ++k) z = fmaf(Mo[L.i * 9 + k], __shfl_sync(FULL, ri, L.base + k), z);
+        if (L.live) {
+            v.D[e] = narrow(D);
             v.r[e] = ri;
             v.z[e] = z;
             v.p[e] = 0.0f;
@@ -294,12 +279,12 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
             v.pc[v.pc_stride + e] = 0.0f;
             kahan_add(rz, rzc, ri * z);
             kahan_add(rr, rrc, ri * ri);
-        }
-        if (lane < CA_STRIDE) {
-            v.cam_acc[(size_t)c * CA_STRIDE + lane] = 0.0f;
-            if (words != nullptr)   // the persistent kernel rotates over all the sets
-                for (int set = 1; set < CA_SETS; ++set)
-                    v.cam_acc[((size_t)set * v.n_cams + c) * CA_STRIDE + lane] = 0.0f;
+            for (int k = L.i; k < CA_STRIDE; k += 9) {
+                v.cam_acc[(size_t)c * CA_STRIDE + k] = 0.0f;
+                if (words != nullptr)   // the persistent kernel rotates over all the sets
+                    for (int set = 1; set < CA_SETS; ++set)
+                        v.cam_acc[((size_t)set * v.n_cams + c) * CA_STRIDE + k] = 0.0f;
+            }
         }
     }
     const int pt_stride = ((int)gridDim.x - cam_blocks) * blockDim.x;
@@ -1185,9 +1170,9 @@ void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s,
 }
 void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
                     ulonglong2* words, int zero) {
-    // camera blocks: a warp per camera; point blocks: a thread per point
-    const int wpb = L.item_block / 32;
-    const int cam_blocks = std::max(1, std::min((v.n_cams + wpb - 1) / wpb, L.item_grid / 2));
+    // camera blocks: a warp per three cameras; point blocks: a thread per point
+    const int cpb = 3 * (L.item_block / 32);
+    const int cam_blocks = std::max(1, std::min((v.n_cams + cpb - 1) / cpb, L.item_grid / 2));
     const int pt_blocks = std::max(1, std::min(grid_items(L, v.n_pts), L.item_grid - cam_blocks));
     k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, words, cam_blocks, zero);
 }
