@@ -59,7 +59,7 @@ Layout compute_layout(int32_t n_cams, int32_t n_pts, int64_t n_obs, int32_t prec
     Layout l{};
     const size_t T = precision == BA_PREC_FP64 ? 8 : 4;
     const size_t nc = (size_t)n_cams, np = (size_t)n_pts, no = (size_t)n_obs;
-    const size_t n_tiles = (np + TILE_PTS - 1) / TILE_PTS;
+    const size_t tp = (size_t)tile_points(n_pts), n_tiles = (np + tp - 1) / tp;
     const size_t n_quads = (np + 3) / 4;
     const size_t pt_off = align_up(9 * nc, 4);
     const size_t n_vec = pt_off + 12 * n_quads;
@@ -151,6 +151,7 @@ Views<T> make_views(ba_problem* p) {
     v.n_cams = p->n_cams;
     v.n_pts = p->n_pts;
     v.n_tiles = p->n_tiles;
+    v.tile_pts = tile_points(p->n_pts);
     v.n_quads = (p->n_pts + 3) / 4;
     v.n_obs = p->n_obs;
     v.pc_stride = (int64_t)((9 * (size_t)p->n_cams + 63) / 64 * 64);
@@ -607,7 +608,7 @@ ba_status ba_problem_create(int32_t n_cams, int32_t n_pts, int64_t n_obs, const 
     p->n_cams = n_cams;
     p->n_pts = n_pts;
     p->n_obs = n_obs;
-    p->n_tiles = (n_pts + TILE_PTS - 1) / TILE_PTS;
+    p->n_tiles = (n_pts + tile_points(n_pts) - 1) / tile_points(n_pts);
     p->precision = precision;
     p->pt_off = (int64_t)((9 * (size_t)n_cams + 3) / 4 * 4);
     p->n_vec = p->pt_off + 12 * (int64_t)(((size_t)n_pts + 3) / 4);
@@ -725,7 +726,7 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
     const size_t limit = (size_t)std::max(0, persistent_max_smem() - 4096);
     auto smem_bytes = [&](bool one, int b, size_t ncb) {
         const size_t no = off[bt[b + 1]] - off[bt[b]];
-        const long pb = (long)bt[b] * TILE_PTS, pe = std::min((long)bt[b + 1] * TILE_PTS, (long)p->n_pts);
+        const long tp = p->vf.tile_pts, pb = (long)bt[b] * tp, pe = std::min((long)bt[b + 1] * tp, (long)p->n_pts);
         return pcg_smem_bytes(one, no, pe > pb ? (size_t)(pe - pb) : 0, ncb);
     };
     for (int b = 0; b < G; ++b)   // too large: the multi-kernel PCG path is used

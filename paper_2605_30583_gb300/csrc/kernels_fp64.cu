@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(T64) k64_linearize(V64 v, int mode, double* re
     double cost = 0.0;
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], n = v.tile_off[tile + 1] - lo;
-        const double* Xt = v.x + v.pt_off + 3 * (size_t)tile * TILE_PTS;
+        const double* Xt = v.x + v.pt_off + 3 * (size_t)tile * v.tile_pts;
         for (uint32_t j = lo + threadIdx.x; j < lo + n; j += T64) {
             const uint32_t key = v.obs_key[j], c = key >> 8;
             const double* X = Xt + 3 * (key & 0xffu);
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(T64) k64_linearize(V64 v, int mode, double* re
                 }
             }
         }
-        const int ip = tile * TILE_PTS + (int)threadIdx.x;
-        if (ip < v.n_pts) {
+        const int ip = tile * v.tile_pts + (int)threadIdx.x;
+        if ((int)threadIdx.x < v.tile_pts && ip < v.n_pts) {
             double gp[3] = {0, 0, 0}, hp[6] = {0, 0, 0, 0, 0, 0};
             for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
                 const uint32_t j = v.obs_pm[k];
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(T64) k64_matvec(V64 v, const int32_t* gate) {
         const uint32_t lo = v.tile_off[tile], n = v.tile_off[tile + 1] - lo;
         const uint32_t chunk = (n + T64 - 1) / T64;
         const uint32_t a = lo + min(threadIdx.x * chunk, n), b = lo + min(threadIdx.x * chunk + chunk, n);
-        const double* Pt = v.p + v.pt_off + 3 * (size_t)tile * TILE_PTS;
+        const double* Pt = v.p + v.pt_off + 3 * (size_t)tile * v.tile_pts;
         double acc[9], pc[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[k] = pc[k] = 0.0;
@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(T64) k64_matvec(V64 v, const int32_t* gate) {
 #pragma unroll
             for (int k = 0; k < 9; ++k) atomicAdd(v.q + 9 * (size_t)cur + k, acc[k]);
         __syncthreads();   // the tile's t
-        const int ip = tile * TILE_PTS + (int)threadIdx.x;
-        if (ip < v.n_pts) {
+        const int ip = tile * v.tile_pts + (int)threadIdx.x;
+        if ((int)threadIdx.x < v.tile_pts && ip < v.n_pts) {
             const size_t ep = v.pt_off + 3 * (size_t)ip;
             double q0 = 0.0, q1 = 0.0, q2 = 0.0;
             for (uint32_t k = v.pt_obs_off[ip]; k < v.pt_obs_off[ip + 1]; ++k) {
@@ -501,7 +501,7 @@ __global__ void k64_eval_candidate(V64 v, CondHandle lm_cond, int use_cond) {
     double fnew = 0.0, jh2 = 0.0;
     if (active) {
         for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
-            const size_t base = v.pt_off + 3 * (size_t)tile * TILE_PTS;
+            const size_t base = v.pt_off + 3 * (size_t)tile * v.tile_pts;
             for (uint32_t j = v.tile_off[tile] + threadIdx.x; j < v.tile_off[tile + 1]; j += blockDim.x) {
                 const uint32_t key = v.obs_key[j], c = key >> 8;
                 const double* Xn = v.x_new + base + 3 * (key & 0xffu);

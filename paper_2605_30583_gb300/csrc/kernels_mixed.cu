@@ -86,8 +86,8 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
     const float lscale = (float)v.st->opt.loss_scale;
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
+        const int pt0 = tile * v.tile_pts;
+        const int npt = min(v.tile_pts, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         __syncthreads();
         for (int i = threadIdx.x; i < npt; i += TB) {
@@ -394,8 +394,8 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
     float pdp = 0.0f, jp2 = 0.0f, pdpc = 0.0f, jp2c = 0.0f;
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
+        const int pt0 = tile * v.tile_pts;
+        const int npt = min(v.tile_pts, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         for (int i = threadIdx.x; i < 3 * npt; i += TB) {
             if (ha != 0.0f) v.h[base + i] = fmaf(ha, v.p[base + i], v.h[base + i]);   // the last update's step
@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
     if (active) {
         for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
             const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-            const int pt0 = tile * TILE_PTS;
+            const int pt0 = tile * v.tile_pts;
             const uint32_t n = hi - lo;
             const uint32_t chunk = odd_chunk<uint32_t>(n, TB);
             const uint32_t a = min(lo + threadIdx.x * chunk, hi), b = min(a + chunk, hi);
@@ -884,8 +884,8 @@ __global__ void __launch_bounds__(TB) k_schur(Views<float> v, const int32_t* gat
             }
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
+        const int pt0 = tile * v.tile_pts;
+        const int npt = min(v.tile_pts, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         for (int i = threadIdx.x; i < 3 * npt; i += TB) {
             sx[i] = v.x[base + i];
@@ -1308,8 +1308,8 @@ __global__ void __launch_bounds__(TB) k_cost_grad(Views<float> v, const float* _
     float cost = 0.0f;
     for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
+        const int pt0 = tile * v.tile_pts;
+        const int npt = min(v.tile_pts, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         __syncthreads();
         for (int i = threadIdx.x; i < npt; i += TB)

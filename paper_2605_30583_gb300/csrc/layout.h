@@ -14,7 +14,20 @@
 
 namespace gbba {
 
-constexpr int TILE_PTS = 256;       // points per tile; an observation's tile slot fits 8 bits
+constexpr int TILE_PTS = 256;       // most points of a tile; an observation's tile slot fits 8 bits
+constexpr int TILE_MIN = 64;        // fewest, see tile_points
+constexpr int TILE_SMS = 152;       // SMs that small problems are spread over
+// Points per tile.  Up to 16 tiles per SM the tiles are cut so that every SM gets the same number
+// of them (whole tiles of 256 points leave SMs with one more than others: 50,000 points are 196
+// tiles, two for 44 SMs and one for 108, now 298 of 168; 1,000 points fill 4 SMs, now 16).  A
+// multiple of 4, so that every tile starts on a 16-byte boundary of the point vectors.
+__host__ __device__ inline int tile_points(int n_pts) {
+    const int64_t full = ((int64_t)n_pts + TILE_PTS - 1) / TILE_PTS;
+    if (full > 16 * TILE_SMS) return TILE_PTS;
+    const int64_t per_sm = (full + TILE_SMS - 1) / TILE_SMS, tiles = per_sm * TILE_SMS;
+    const int64_t t = (((n_pts + tiles - 1) / tiles) + 3) / 4 * 4;
+    return (int)(t < TILE_MIN ? TILE_MIN : t > TILE_PTS ? TILE_PTS : t);
+}
 constexpr int HIST_CAP = 1024;      // LM iterations recorded in the device history
 constexpr int MAX_GRID = 4096;      // upper bound on blocks of any reduction kernel
 constexpr int NPART = 4;            // doubles of partial sums per block
@@ -104,6 +117,7 @@ struct DevState {
 template <typename T>
 struct Views {
     int32_t n_cams, n_pts, n_tiles, n_quads;
+    int32_t tile_pts;            // points per tile (tile_points)
     int64_t n_obs;
     int64_t pt_off, n_vec;
     int64_t pc_stride;           // floats between the two camera-direction buffers

@@ -3,7 +3,7 @@
 //
 //  1. each point's key is the smallest camera index observing it; points are
 //     sorted by (key, caller index), giving the internal point order;
-//  2. tiles are TILE_PTS consecutive internal points;
+//  2. tiles are tile_points(n_pts) consecutive internal points;
 //  3. observations are sorted by (tile, camera, tile slot, caller index), so a
 //     tile's observations are contiguous and grouped into camera runs;
 //  4. inside each tile the runs of at least LONG_RUN observations move to the front.
@@ -67,9 +67,9 @@ __global__ void k_point_perm(const uint32_t* vals, int n_pts, uint32_t* pt_user,
 }
 
 __global__ void k_tile_count(const uint32_t* pt_idx, const uint32_t* pt_internal, int64_t n_obs,
-                             uint32_t* tile_cnt) {
+                             int tile_pts, uint32_t* tile_cnt) {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_obs; o += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&tile_cnt[pt_internal[pt_idx[o]] / TILE_PTS], 1u);
+        atomicAdd(&tile_cnt[pt_internal[pt_idx[o]] / (uint32_t)tile_pts], 1u);
 }
 
 // Exclusive scan of cnt[0..n) into off[0..n] with one block of 1024 threads.
@@ -99,11 +99,11 @@ __global__ void __launch_bounds__(1024) k_scan_single(const uint32_t* cnt, int n
 }
 
 __global__ void k_obs_sort_keys(const uint32_t* cam_idx, const uint32_t* pt_idx, const uint32_t* pt_internal,
-                                int64_t n_obs, size_t sort_n, uint64_t* keys, uint32_t* vals) {
+                                int64_t n_obs, int tile_pts, size_t sort_n, uint64_t* keys, uint32_t* vals) {
     for (size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x; o < sort_n; o += (size_t)gridDim.x * blockDim.x) {
         if (o < (size_t)n_obs) {
             const uint32_t ip = pt_internal[pt_idx[o]];
-            const uint64_t tile = ip / TILE_PTS, slot = ip % TILE_PTS;
+            const uint64_t tile = ip / (uint32_t)tile_pts, slot = ip % (uint32_t)tile_pts;
             // within a camera's run the points are ordered from a camera-dependent
             // starting slot: threads that walk different cameras' runs of one tile in
             // step then touch different points (no same-address shared atomics)
@@ -122,10 +122,11 @@ __global__ void k_obs_sort_keys(const uint32_t* cam_idx, const uint32_t* pt_idx,
 // index); then one CTA per tile sorts the bucket in shared memory (bitonic network on the
 // bucket padded to a power of two) and writes the keys and values k_obs_gather reads.
 __global__ void k_obs_bucket(const uint32_t* cam_idx, const uint32_t* pt_idx, const uint32_t* pt_internal,
-                             int64_t n_obs, const uint32_t* tile_off, uint32_t* cursor, uint64_t* keys) {
+                             int64_t n_obs, int tile_pts, const uint32_t* tile_off, uint32_t* cursor,
+                             uint64_t* keys) {
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_obs; o += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t ip = pt_internal[pt_idx[o]];
-        const uint32_t tile = ip / TILE_PTS, slot = ip % TILE_PTS, cam = cam_idx[o];
+        const uint32_t tile = ip / (uint32_t)tile_pts, slot = ip % (uint32_t)tile_pts, cam = cam_idx[o];
         const uint64_t rslot = (slot + SLOT_ROTATION * (uint64_t)cam) % TILE_PTS;
         const uint32_t at = tile_off[tile] + atomicAdd(&cursor[tile], 1u);
         keys[at] = ((uint64_t)cam << 40) | (rslot << 32) | (uint64_t)o;
@@ -270,7 +271,7 @@ __global__ void k_copy_back(const uint32_t* tmp_key, const T* tmp_uv, const uint
 }
 
 // Point-major index by a counting sort inside each tile: a tile's observation range
-// holds exactly the observations of its TILE_PTS points, so the point offsets are the
+// holds exactly the observations of its points, so the point offsets are the
 // tile's first observation plus an exclusive scan of per-slot counts, and each point's
 // observations are placed in increasing position j (lanes of a 32-observation step
 // ranked among equal slots, steps in order): the same index as sorting (point, j).
@@ -279,7 +280,7 @@ constexpr int PM_WARPS = 4;
 
 __global__ void __launch_bounds__(32 * PM_WARPS) k_pm_tiles(const uint32_t* __restrict__ obs_key,
                                                             const uint32_t* __restrict__ tile_off, int n_tiles,
-                                                            int n_pts, int64_t n_obs, uint32_t* obs_pm,
+                                                            int tile_pts, int n_pts, int64_t n_obs, uint32_t* obs_pm,
                                                             uint32_t* pt_obs_off) {
     static_assert(TILE_PTS == 256, "one-byte point slots");
     __shared__ uint32_t cnt_all[PM_WARPS][TILE_PTS];
@@ -306,12 +307,12 @@ __global__ void __launch_bounds__(32 * PM_WARPS) k_pm_tiles(const uint32_t* __re
             if (lane >= d) incl += o;
         }
         uint32_t base = incl - run;
-        const int pt0 = t * TILE_PTS;
+        const int pt0 = t * tile_pts;
 #pragma unroll
         for (int k = 0; k < TILE_PTS / 32; ++k) {
             const int s2 = lane * (TILE_PTS / 32) + k;
             cnt[s2] = base;
-            if (pt0 + s2 < n_pts) pt_obs_off[pt0 + s2] = lo + base;
+            if (s2 < tile_pts && pt0 + s2 < n_pts) pt_obs_off[pt0 + s2] = lo + base;
             base += c[k];
         }
         __syncwarp();
@@ -437,7 +438,7 @@ void build_order(const Views<T>& v, const OrderBuffers& b, cudaStream_t s) {
     k_point_perm<<<blocks_for(v.n_pts, TB), TB, 0, s>>>(b.vals, v.n_pts, pt_user, pt_internal);
     // 2. tiles
     k_fill_u32<<<blocks_for(v.n_tiles, TB), TB, 0, s>>>(b.tile_cnt, (size_t)v.n_tiles, 0u);
-    k_tile_count<<<blocks_for(v.n_obs, TB), TB, 0, s>>>(b.pt_idx, pt_internal, v.n_obs, b.tile_cnt);
+    k_tile_count<<<blocks_for(v.n_obs, TB), TB, 0, s>>>(b.pt_idx, pt_internal, v.n_obs, v.tile_pts, b.tile_cnt);
     k_scan_single<<<1, 1024, 0, s>>>(b.tile_cnt, v.n_tiles, tile_off);
     // 3. observation order: sorted inside each tile's bucket in shared memory when the
     //    largest tile fits TILE_SORT_MAX observations, else one global sort
@@ -455,15 +456,15 @@ void build_order(const Views<T>& v, const OrderBuffers& b, cudaStream_t s) {
         uint32_t pn = 2;
         while (pn < most) pn <<= 1;
         k_fill_u32<<<blocks_for(v.n_tiles, TB), TB, 0, s>>>(b.tile_cnt, (size_t)v.n_tiles, 0u);
-        k_obs_bucket<<<blocks_for(v.n_obs, TB), TB, 0, s>>>(b.cam_idx, b.pt_idx, pt_internal, v.n_obs, tile_off,
-                                                             b.tile_cnt, b.keys);
+        k_obs_bucket<<<blocks_for(v.n_obs, TB), TB, 0, s>>>(b.cam_idx, b.pt_idx, pt_internal, v.n_obs, v.tile_pts,
+                                                             tile_off, b.tile_cnt, b.keys);
         const size_t smem = 8 * (size_t)pn;
         if (smem > 48 * 1024) cudaFuncSetAttribute(k_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_tile_sort<<<std::max(1, std::min(v.n_tiles, 65535)), 512, smem, s>>>(tile_off, v.n_tiles, b.keys, b.vals);
     } else {
         const size_t no2 = pow2_at_least((size_t)v.n_obs);
-        k_obs_sort_keys<<<blocks_for(no2, TB), TB, 0, s>>>(b.cam_idx, b.pt_idx, pt_internal, v.n_obs, no2, b.keys,
-                                                           b.vals);
+        k_obs_sort_keys<<<blocks_for(no2, TB), TB, 0, s>>>(b.cam_idx, b.pt_idx, pt_internal, v.n_obs, v.tile_pts,
+                                                           no2, b.keys, b.vals);
         bitonic_sort(b.keys, b.vals, no2, s);
     }
     k_obs_gather<T><<<blocks_for(v.n_obs, TB), TB, 0, s>>>(b.keys, b.vals, b.pixels, v.n_obs,
@@ -491,7 +492,7 @@ void build_order(const Views<T>& v, const OrderBuffers& b, cudaStream_t s) {
     //    so every internal point owns a non-empty run), one counting sort per tile
     {
         const int grid = (int)std::min<int64_t>(8192, ((int64_t)v.n_tiles + PM_WARPS - 1) / PM_WARPS);
-        k_pm_tiles<<<std::max(1, grid), 32 * PM_WARPS, 0, s>>>(v.obs_key, tile_off, v.n_tiles, v.n_pts, v.n_obs,
+        k_pm_tiles<<<std::max(1, grid), 32 * PM_WARPS, 0, s>>>(v.obs_key, tile_off, v.n_tiles, v.tile_pts, v.n_pts, v.n_obs,
                                                                const_cast<uint32_t*>(v.obs_pm),
                                                                const_cast<uint32_t*>(v.pt_obs_off));
     }

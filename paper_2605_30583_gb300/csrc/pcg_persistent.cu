@@ -308,7 +308,7 @@ __device__ __forceinline__ void resident_normal(const Views<float>& v, const uin
                 cur = lc;
                 resident_cam(sCam, sDir, lc, oc, od);
             }
-            const int lp = t * TILE_PTS + (int)(key & 0xffu);
+            const int lp = t * v.tile_pts + (int)(key & 0xffu);
             const float4 x = sX4[lp], dx = sD4[lp];
             const float tt = general ? obs_normal<true>(oc, od, x, dx, eps, weighted ? __ldg(v.obs_w + ob + j) : 1.0f,
                                                         acc, sQ + 3 * lp)
@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent(Views<float> v, const 
     __shared__ TileTab tab;
     const uint32_t ob = v.tile_off[t0], oe = v.tile_off[t1];
     const uint32_t no = oe - ob;
-    const int pb = (int)(t0 * TILE_PTS);
-    const int pe = min((int)(t1 * TILE_PTS), v.n_pts);
+    const int pb = (int)t0 * v.tile_pts;
+    const int pe = min((int)t1 * v.tile_pts, v.n_pts);
     const int np = pe > pb ? pe - pb : 0;
     const int n3 = 3 * np;
     const int n3p = (n3 + 3) & ~3;
@@ -790,8 +790,8 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     __shared__ TileTab tab;
     const uint32_t ob = v.tile_off[t0], oe = v.tile_off[t1];
     const uint32_t no = oe - ob;
-    const int pb = (int)(t0 * TILE_PTS);
-    const int pe = min((int)(t1 * TILE_PTS), v.n_pts);
+    const int pb = (int)t0 * v.tile_pts;
+    const int pe = min((int)t1 * v.tile_pts, v.n_pts);
     const int np = pe > pb ? pe - pb : 0;
     const int n3p = (3 * np + 3) & ~3;
     const uint32_t cb = blk_cam_off[blockIdx.x], ncb = blk_cam_off[blockIdx.x + 1] - cb;

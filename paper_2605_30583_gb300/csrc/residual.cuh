@@ -26,8 +26,8 @@ __device__ __forceinline__ void residual_tiles(const Views<float>& v, int at_can
     float cl = 0.0f;
     for (int tile = first; tile < v.n_tiles; tile += stride) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
-        const int pt0 = tile * TILE_PTS;
-        const int npt = min(TILE_PTS, v.n_pts - pt0);
+        const int pt0 = tile * v.tile_pts;
+        const int npt = min(v.tile_pts, v.n_pts - pt0);
         const size_t base = v.pt_off + 3 * (size_t)pt0;
         for (int i = threadIdx.x; i < npt; i += TB) {
             const DF a = df_from_double(xm[base + 3 * i]), b = df_from_double(xm[base + 3 * i + 1]),

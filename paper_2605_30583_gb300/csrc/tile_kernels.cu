@@ -53,8 +53,8 @@ __device__ __forceinline__ TileRange tile_range(const Views<float>& v, int tile)
     r.l0 = v.long_off[tile];
     r.nl = v.long_off[tile + 1] - r.l0;
     r.ss = v.short_start[tile];
-    r.pt0 = tile * TILE_PTS;
-    r.npt = min(TILE_PTS, v.n_pts - r.pt0);
+    r.pt0 = tile * v.tile_pts;
+    r.npt = min(v.tile_pts, v.n_pts - r.pt0);
     r.base = v.pt_off + 3 * (size_t)r.pt0;
     return r;
 }
