@@ -230,10 +230,10 @@ __device__ __forceinline__ void tile_normal(const Views<float>& v, const TileRan
 // Replacing the point-sum atomics of the long runs this way took the operator from 302
 // to 289 us on the 28.8M-observation workload.
 //
-// Of 281 us (19.8M observations, 4.5M points), staging and outputs took 117, the long runs 121 and
+// Of 281 us (28.8M observations, 4.5M points), staging and outputs took 117, the long runs 121 and
 // the short ones 33.  The staging is bound by the latency of its loads: vectors as float4, four
 // keys to a load, and the data of the tile that takes this one's place (`ahead` tiles on, all
-// CTAs in flight) brought into the L2 meanwhile: 281 -> 269 us.  Its bytes alone take 75 us.
+// CTAs in flight) brought into the L2 meanwhile: 281 -> 269 us.  Its bytes alone take 81 us.
 template <int TB, bool PLAIN_Q>
 __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int32_t* gate, const float* zs,
                                                        int use_beta, int ahead, Caps cap) {

@@ -148,3 +148,57 @@ def test_unaligned_evaluation_outputs(B):
         cost = ctypes.c_double()
         B.check(B.lib().ba_evaluate(p._h, ctypes.byref(cost), r2.data_ptr(), J2.data_ptr()))
         assert torch.equal(r2.view_as(r), r) and torch.equal(J2.view_as(J), J)
+
+
+@pytest.mark.parametrize("n_pts", [63, 64, 65, 2 * 64 + 1, 152 * 64, 152 * 64 + 1])
+def test_tile_size_rule(B, n_pts):
+    """Small problems are cut into tiles of 64 to 256 points, a multiple of four."""
+    import torch
+    prob = _scene(24, n_pts, 300 + n_pts)
+    p = _bind(B, prob)
+    p.evaluate()
+    lin = O.linearize(*_args(prob))
+    D = O.damping_diag(lin.J)
+    v = np.random.default_rng(2).standard_normal(9 * 24 + 3 * n_pts).astype(np.float32).astype(np.float64)
+    out, _ = p.apply_normal(0.01, torch.from_numpy(v))
+    Ja = abs(lin.J)
+    scale = Ja.T @ (Ja @ np.abs(v)) + 0.01 * D * np.abs(v)
+    err = np.abs(out.double().cpu().numpy() - O.normal_matvec(lin, D, 0.01, v))
+    assert np.all(err <= 1e-4 * scale), np.max(err / scale)
+    opts = dict(max_lm_iters=2, max_pcg_iters=8)
+    res = p.solve(**opts)
+    ref = O.ba_solve(*_args(prob), O.LMOptions(**opts))
+    assert abs(res.final_cost - ref.final_cost) <= 1e-4 * ref.final_cost
+
+
+def test_the_operator_and_the_gradient_share_their_jacobian(B):
+    """A point 0.5 to 1 in front of a camera that is 1000 from the origin has ~5 digits left in
+    P = R X + t.  g = J^T r and J^T J use the same rounded P: with r = J d in the linearisation's
+    arithmetic, J^T J d and J^T r agree to FP32 rounding of the sums, 2e-6 of their norm, where
+    Jacobians that round P differently disagree by ~1e-4."""
+    import torch
+    rng = np.random.default_rng(5)
+    n_cams, n_pts = 4, 300
+    cams = np.zeros((n_cams, 9))
+    cams[:, :3] = 0.3 * rng.standard_normal((n_cams, 3))
+    cams[:, 6] = 700.0
+    from scipy.spatial.transform import Rotation
+    R = Rotation.from_rotvec(cams[:, :3]).as_matrix()
+    pts = 1000.0 * np.array([0.6, -0.5, 0.62]) + rng.uniform(-0.2, 0.2, size=(n_pts, 3))
+    centre = 1000.0 * np.array([0.6, -0.5, 0.62])
+    P0 = np.array([0.0, 0.0, -0.75])   # the centre of the points in each camera
+    cams[:, 3:6] = P0 - R @ centre
+    cams, pts = cams.astype(np.float32).astype(np.float64), pts.astype(np.float32).astype(np.float64)
+    ci, pi = np.tile(np.arange(n_cams), n_pts), np.repeat(np.arange(n_pts), n_cams)
+    p = B.Problem(n_cams, n_pts, ci.astype(np.uint32), pi.astype(np.uint32), np.zeros((len(ci), 2)))
+    p.set_params(cams, pts)
+    _, _, J = p.evaluate(jacobian=True)
+    J = J.double().cpu().numpy()
+    d = np.concatenate([np.zeros(9 * n_cams), rng.standard_normal(3 * n_pts)]).astype(np.float32).astype(np.float64)
+    dp = d[9 * n_cams:].reshape(-1, 3)
+    r = np.einsum("oij,oj->oi", J[:, :, 9:], dp[pi])
+    want = np.zeros((n_pts, 3))
+    np.add.at(want, pi, np.einsum("oij,oi->oj", J[:, :, 9:], r))
+    out, _ = p.apply_normal(0.0, torch.from_numpy(d))
+    got = out.double().cpu().numpy()[9 * n_cams:].reshape(-1, 3)
+    assert np.linalg.norm(got - want) <= 2e-6 * np.linalg.norm(want)
