@@ -118,7 +118,8 @@ __device__ __forceinline__ CamDF load_cam_df(const float* __restrict__ rec, cons
 // few units of 2^-46 of the ~500 px terms, so rounded to FP32 it is the exact residual
 // to within an ulp of itself.  Low parts are gathered and renormalised only where a
 // cancellation (R X + t, f s p - u) or a division follows: 210 FP32 operations, where
-// renormalising every sum and product took 305.
+// renormalising every sum and product took 305
+// (28.8M residuals: 475 -> 381 us).
 __device__ __forceinline__ void residual_df(const CamDF& c, const DF (&X)[3], float eps, float u0, float u1,
                                             DF& r0, DF& r1) {
     DF P[3];

@@ -99,6 +99,9 @@ __global__ void k64_camera_precompute(V64 v) {
 // stored.  Then the tile's observations in order, a contiguous part to a warp: lane l holds the
 // entries l and l + 32 of a camera's 54 sums (g and the J_c^T J_c triangle), so every lane works
 // on one observation's row at a time and nothing has to be reduced.  Then a thread per point.
+// Bound by the FP64 pipe.  (A thread per point over its scattered observations, with 54 atomics
+// each, and the operator below in the same form: 11.4 ms for a solve of 3 x 15 iterations of 200
+// cameras and 50,000 points, 5.3 ms so.)
 constexpr int T64 = TILE_PTS;
 
 __global__ void __launch_bounds__(T64) k64_linearize(V64 v, int mode, double* res_out, double* jac_out,
