@@ -46,8 +46,8 @@ struct LaunchCfg {
     // point sums into private copies with plain adds
     int tn_plain_q = 0;
     int tn_ahead = 0;   // the operator's CTAs in flight
-    // few tiles: 512 threads per tile in the linearisation and the evaluations
-    bool wide_tiles = false;
+    // few tiles: 512 threads per tile in the linearisation; residuals and evaluation in one launch
+    bool wide_lin = false, wide_tiles = false;
 };
 
 // residual pass of the mixed form (residual.cu): r at x (at_candidate 0) or at x' (1),

@@ -600,8 +600,12 @@ __global__ void __launch_bounds__(TB, 6) k_tile_cg(Views<float> v, const int32_t
 // st->relin), 2 evaluation only (squared loss; optional r and J in the caller's order).
 constexpr int TL_ACC = 9 + 45;   // per-lane camera sums: g, upper triangle of J_c^T J_c
 constexpr int TL_TB = 128;
-// Few tiles: a tile's runs spread over more warps.  With at most this many tiles per SM the
-// linearisation and the candidate's evaluation (k_tile_step) run 512 threads per tile.
+// Few tiles: a tile's runs spread over the warps of 512 threads.  The linearisation does so up to
+// one tile per SM (16 tiles: 18.0 -> 13.8 us; 298 tiles 22.9 against 23.6, 302 tiles 23.3 against
+// 25.8, 910 tiles 43.7 against 61.9), the candidate's residuals and evaluation in one launch
+// (k_tile_step) up to two (against both launches: 25.3 -> 14.2 us, 31.8 -> 30.6, 32.5 -> 32.5 and
+// a launch gap of 2 us each; 910 tiles 45.8 against 77.7).
+constexpr int WIDE_LIN_TILES = 1;
 constexpr int WIDE_TILES = 2;
 constexpr int WIDE_TB = 512;
 
@@ -1181,7 +1185,7 @@ void tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, i
 // (all grids 0).
 void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int max_short_obs, int max_long_runs) {
     L.tn_grid = L.tl_grid = L.te_grid = 0;
-    L.wide_tiles = false;
+    L.wide_lin = L.wide_tiles = false;
     L.tk_run_cap = std::max(1, max_long_runs);
     L.tk_short_cap = std::max(1, max_short_obs);
     L.tk_long_cap = (std::max(1, max_long_obs) + 7 + 15) / 16 * 16;   // whole words (store_compact)
@@ -1198,10 +1202,10 @@ void plan_tile_kernels(LaunchCfg& L, int n_tiles, int sms, int max_long_obs, int
                              prepare(k_tile_schur<TS_TB, SCHUR_MV>, TS_TB, L.tn_smem),
                              prepare(k_tile_schur<TS_TB, SCHUR_BACK>, TS_TB, L.tn_smem)});
     if (bn < 1 || bl < 1 || be < 1 || bc < 1 || bs < 1) return;
-    L.wide_tiles = n_tiles <= WIDE_TILES * sms &&
-                   std::min({prepare(k_tile_linearize<WIDE_TB, true>, WIDE_TB, lin_smem(L, WIDE_TB, true)),
-                             prepare(k_tile_linearize<WIDE_TB, false>, WIDE_TB, lin_smem(L, WIDE_TB, false)),
-                             prepare(k_tile_step<WIDE_TB>, WIDE_TB, L.te_smem)}) >= 1;
+    L.wide_lin = n_tiles <= WIDE_LIN_TILES * sms &&
+                 std::min(prepare(k_tile_linearize<WIDE_TB, true>, WIDE_TB, lin_smem(L, WIDE_TB, true)),
+                          prepare(k_tile_linearize<WIDE_TB, false>, WIDE_TB, lin_smem(L, WIDE_TB, false))) >= 1;
+    L.wide_tiles = n_tiles <= WIDE_TILES * sms && prepare(k_tile_step<WIDE_TB>, WIDE_TB, L.te_smem) >= 1;
     const int nt = std::max(1, n_tiles);
     L.tn_grid = nt;   // one CTA per tile
     L.tn_ahead = sms * bn;
@@ -1226,7 +1230,7 @@ void launch_cg_round(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, 
 
 void launch_tile_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, int mode, float* res_out,
                            float* jac_out, CondHandle lm_cond, int use_cond) {
-    if (L.wide_tiles) tile_linearize<WIDE_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
+    if (L.wide_lin) tile_linearize<WIDE_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
     else tile_linearize<TL_TB>(v, L, s, mode, res_out, jac_out, lm_cond, use_cond);
 }
 
