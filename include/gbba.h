@@ -124,12 +124,12 @@ typedef struct {
                                      only (BA_ERR_NOT_IMPLEMENTED for the FP64 form and
                                      the batched mode).                                 */
     int32_t wait_timeout_ms;      /* limit on each grid-wide wait of the persistent PCG
-                                     kernel (its CTAs meet at a barrier twice per
-                                     iteration), default 2000.  A wait that does not end
+                                     kernel (its CTAs wait for one another's sums once or
+                                     twice per iteration), default 2000.  A wait that does not end
                                      within it gives up: every CTA leaves the kernel and
                                      the solve reports BA_ERR_TIMEOUT (the context stays
                                      usable).  0 gives up at the first poll that finds
-                                     the barrier incomplete.  0..60000.  The separate-
+                                     a sum missing.  0..60000.  The separate-
                                      kernel PCG and the batched mode have no grid-wide
                                      waits and ignore it.                              */
     int32_t residual_precision;   /* arithmetic of the mixed form's residuals r = f s p - u
@@ -175,9 +175,9 @@ const char* ba_status_string(int32_t status);
 int32_t ba_abi_version(void);
 
 /* Self-test of the bounded grid waits that every cooperative kernel of this library
- * uses (the persistent PCG kernel's barriers).  Launches a cooperative grid of `grid`
- * CTAs (1 <= grid <= the SM count) that waits at a barrier counting one CTA more than
- * it has, which nothing completes; each CTA must give up after timeout_ms (1..2000)
+ * uses (the persistent PCG kernel's exchanges).  Launches a cooperative grid of `grid`
+ * CTAs (1 <= grid <= the SM count) that waits, through the same code, for a sum that
+ * nothing ever publishes; each CTA must give up after timeout_ms (1..2000)
  * and return, leaving the context usable.  scratch: 16 bytes of caller-owned device
  * memory, 16-byte aligned.  On BA_OK, *gave_up is the number of CTAs that gave up
  * (grid when the mechanism works) and *error_word the shared error flag (1).  No GPU
@@ -186,7 +186,7 @@ ba_status ba_selftest_wait_timeout(void* scratch, int32_t grid, int32_t timeout_
                                    int32_t* error_word);
 
 /* Self-test of the FP64 reciprocal that the block-Jacobi inversions use (a hardware
- * approximation refined by two Newton-Raphson steps).  y[i] = 1/x[i] for i < n, with
+ * approximation refined by one third-order step).  y[i] = 1/x[i] for i < n, with
  * x and y device arrays of n doubles (n >= 1), enqueued on `stream` (cudaStream_t).
  * Zero, non-finite and |x| outside [1e-300, 1e300] take the IEEE quotient 1.0 / x. */
 ba_status ba_selftest_rcp64(const double* x, double* y, int64_t n, void* stream);

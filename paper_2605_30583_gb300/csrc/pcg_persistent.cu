@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
     const int n3p = (3 * np + 3) & ~3;
     const uint32_t cb = blk_cam_off[blockIdx.x], ncb = blk_cam_off[blockIdx.x + 1] - cb;
     const int ne = 9 * (int)ncb;   // camera vector entries of this CTA
-    // shared memory, carved in the order pcg1_smem_bytes counts it
+    // shared memory, carved in the order pcg_smem_bytes counts it
     uint32_t* skey = reinterpret_cast<uint32_t*>(smem);
     float4* sX4 = reinterpret_cast<float4*>(smem + (((size_t)no * 4 + 15) & ~(size_t)15));   // (X, D_0)
     float4* sU4 = sX4 + np;                                                                  // (u, D_1)
