@@ -253,13 +253,12 @@ static void step_lm_head(ba_problem* p, cudaStream_t s, CondHandle pcg_c, int us
     if (p->precision == BA_PREC_MIXED && p->use_schur) {
         // blocks of H' (camera and point inverses, D), then the reduced right-hand side
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, pcg_c, 0, nullptr, 1);
+        launch_precond(v, p->L, s, pcg_c, 0, nullptr, 0);
         launch_schur(v, p->L, s, SCHUR_RHS, &v.st->lm_active);
         launch_schur_start(v, p->L, s, pcg_c, use);
     } else if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->xch : nullptr,
-                       p->use_persistent ? 0 : (p->use_cg ? 2 : 1));
+        launch_precond(v, p->L, s, pcg_c, use, p->use_persistent ? p->xch : nullptr, p->use_cg ? 1 : 0);
         if (p->use_persistent)
             launch_pcg_persistent(v, p->blk_tile, p->blk_cam_off, p->blk_cams, p->blk_fac, p->xch, p->p_grid,
                                   p->p_form == PCG_TWO_EXCHANGE ? p->p_smem_two : p->p_smem_one, p->p_form, s);
@@ -1189,7 +1188,7 @@ ba_status ba_apply_normal(ba_problem* p, double mu, const void* vin, void* out, 
     GBBA_CUDA(cudaMemcpyAsync(&dst->lm_active, &one, sizeof(int32_t), cudaMemcpyHostToDevice, s));
     if (p->precision == BA_PREC_MIXED) {
         const Views<float>& v = p->vf;
-        launch_precond(v, p->L, s, 0, 0, nullptr, 1);
+        launch_precond(v, p->L, s, 0, 0, nullptr, 0);
         launch_set_direction(v, p->L, s, (const float*)vin);
         launch_matvec(v, p->L, s, nullptr, v.p, 0);
         launch_normal_out(v, p->L, s, (float*)out);
@@ -1336,7 +1335,7 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
     double out[8];
     out[0] = timeit([&] { launch_camera_precompute(v, p->L, s); });
     out[1] = timeit([&] { launch_linearize(v, p->L, s, 1, nullptr, nullptr, 0, 0); });
-    out[2] = timeit([&] { launch_precond(v, p->L, s, 0, 0, nullptr, 1); });
+    out[2] = timeit([&] { launch_precond(v, p->L, s, 0, 0, nullptr, 0); });
     out[3] = timeit([&] { launch_matvec(v, p->L, s, nullptr, v.z, 1); });
     {
         // the update skips its work once the operator sums it consumes are cleared, so

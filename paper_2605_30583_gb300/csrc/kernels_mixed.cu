@@ -229,10 +229,11 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 //
 // Bound by the FP64 pipe (80 % active: 28 operations a point, ~42 a camera's share of a warp):
 // 687 -> 488 us on 13,000 cameras and 4.5M points with integer conversions, one reciprocal a
-// point, compensated FP32 sums and three cameras a warp.  `zero`: which PCG vectors the solver that
-// follows wants cleared (0 none, 1 h, 2 h, p and s).
+// point, compensated FP32 sums and three cameras a warp.  h is always cleared: a PCG that runs no
+// iteration (cap 0, a zero or non-finite residual) leaves the step at 0, and the candidate and its
+// evaluation read it.  `zero_ps`: the solver that follows wants the points' p and s cleared too.
 __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulonglong2* words, int cam_blocks,
-                          int zero) {
+                          int zero_ps) {
     DevState* st = v.st;
     if (words != nullptr && blockIdx.x == 0) {   // state of the persistent PCG kernel
         for (int i = threadIdx.x; i < XCH_BYTES / 16; i += blockDim.x) words[i] = make_ulonglong2(0ull, 0ull);
@@ -309,8 +310,8 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
         const float z2 = fmaf(m[2], r0, fmaf(m[4], r1, m[5] * r2));
         v.r[e] = r0; v.r[e + 1] = r1; v.r[e + 2] = r2;
         v.z[e] = z0; v.z[e + 1] = z1; v.z[e + 2] = z2;
-        if (zero > 0) { v.h[e] = 0.0f; v.h[e + 1] = 0.0f; v.h[e + 2] = 0.0f; }
-        if (zero > 1) {
+        v.h[e] = 0.0f; v.h[e + 1] = 0.0f; v.h[e + 2] = 0.0f;
+        if (zero_ps) {
             v.p[e] = 0.0f; v.p[e + 1] = 0.0f; v.p[e + 2] = 0.0f;
             v.s[e] = 0.0f; v.s[e + 1] = 0.0f; v.s[e + 2] = 0.0f;
         }
@@ -1173,12 +1174,12 @@ void launch_linearize(const Views<float>& v, const LaunchCfg& L, cudaStream_t s,
                                                                                  lm_cond, use_cond);
 }
 void launch_precond(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, CondHandle c, int use,
-                    ulonglong2* words, int zero) {
+                    ulonglong2* words, int zero_ps) {
     // camera blocks: a warp per three cameras; point blocks: a thread per point
     const int cpb = 3 * (L.item_block / 32);
     const int cam_blocks = std::max(1, std::min((v.n_cams + cpb - 1) / cpb, L.item_grid / 2));
     const int pt_blocks = std::max(1, std::min(grid_items(L, v.n_pts), L.item_grid - cam_blocks));
-    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, words, cam_blocks, zero);
+    k_precond<<<cam_blocks + pt_blocks, L.item_block, 0, s>>>(v, c, use, words, cam_blocks, zero_ps);
 }
 static void launch_cam_direction(const Views<float>& v, const LaunchCfg& L, cudaStream_t s, const int32_t* gate,
                                  const float* zs, int use_beta) {
