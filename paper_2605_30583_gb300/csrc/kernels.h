@@ -133,6 +133,7 @@ __host__ __device__ inline size_t pcg_smem_bytes(bool one_exchange, size_t no, s
     }
     return b;
 }
+static_assert(MAX_CTA_TILES * TILE_MIN * (32 + 4 * 5 * 3 + 4 * 6) > 227 * 1024, "a CTA's tiles are bounded by its points");
 int occupancy_blocks_linearize();
 int occupancy_blocks_matvec();
 int occupancy_blocks_eval();

@@ -33,7 +33,9 @@ constexpr int MAX_GRID = 4096;      // upper bound on blocks of any reduction ke
 constexpr int NPART = 4;            // doubles of partial sums per block
 constexpr int NSLOT = 32;           // atomic accumulator slots per scalar sum
 constexpr int SLOT_STRIDE = 16;     // doubles between slots (one 128-byte line)
-constexpr int MAX_CTA_TILES = 16;   // tiles of one of its CTAs
+// Tiles of one of its CTAs.  Never what decides whether a plan is taken: a CTA of more has at least
+// this many full tiles, whose points alone exceed a CTA's shared memory (pcg_smem_bytes).
+constexpr int MAX_CTA_TILES = 32;
 constexpr int MAX_PBLOCKS = 256;    // CTAs of the persistent PCG kernel (one per SM)
 // Exchange area of the persistent PCG kernels: two alternating sets of XCH_NV sums of every CTA,
 // 16 bytes each (two 64-bit words), cleared before every launch.
