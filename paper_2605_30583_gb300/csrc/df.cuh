@@ -1,5 +1,6 @@
 // Double-float ("df") arithmetic: a value is the unevaluated sum hi + lo of two FP32
-// numbers with |lo| <= ulp(hi) / 2, about 48 significant bits, from FP32 operations only
+// numbers with |lo| <= ulp(hi) / 2 (results of the _raw operations excepted), about 48
+// significant bits, from FP32 operations only
 // (Dekker, "A floating-point technique for extending the available precision", 1971;
 // Knuth's TwoSum; the exact product by FMA).  On this GPU FP64 runs at 1/64 of the FP32
 // rate, so the one quantity of the mixed form that needs more than FP32 -- the
@@ -17,8 +18,6 @@ namespace gbba {
 struct DF {
     float hi, lo;
 };
-
-__device__ __forceinline__ DF df_from(float a) { return {a, 0.0f}; }
 
 // hi + lo of a double, rounded twice (conversions on the integer units: narrow, widen).
 __device__ __forceinline__ DF df_from_double(double a) {
@@ -42,46 +41,42 @@ __device__ __forceinline__ DF fast_two_sum_f(float a, float b) {
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
-// a b as the exact product of the high parts (fma gives its error) plus the cross terms; not
-// renormalised: |lo| may reach a few ulp of hi, which the sums and products below take.
-__device__ __forceinline__ DF df_mul(DF a, DF b) {
+// The operations ending in _raw leave out the last renormalisation: |lo| may reach a few ulp of
+// hi, which the operations that take the result allow for; df_norm makes up for it.
+__device__ __forceinline__ DF df_norm(DF a) { return fast_two_sum_f(a.hi, a.lo); }
+
+// a b as the exact product of the high parts (fma gives its error) plus the cross terms.
+__device__ __forceinline__ DF df_mul_raw(DF a, DF b) {
     const float p = __fmul_rn(a.hi, b.hi);
     float e = __fmaf_rn(a.hi, b.hi, -p);
     e = __fmaf_rn(a.hi, b.lo, e);
     return {p, __fmaf_rn(a.lo, b.hi, e)};
 }
 
-// a + b: the high parts' sum and its error exactly, the low parts added (not renormalised).
-__device__ __forceinline__ DF df_add(DF a, DF b) {
+__device__ __forceinline__ DF df_mul(DF a, DF b) { return df_norm(df_mul_raw(a, b)); }
+
+// a + b: the high parts' sum and its error exactly, the low parts added.
+__device__ __forceinline__ DF df_add_raw(DF a, DF b) {
     const DF s = two_sum_f(a.hi, b.hi);
     return {s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
 }
 
+__device__ __forceinline__ DF df_add(DF a, DF b) { return df_norm(df_add_raw(a, b)); }
+
 __device__ __forceinline__ DF df_add_f(DF a, float b) {
     const DF s = two_sum_f(a.hi, b);
-    return {s.hi, __fadd_rn(s.lo, a.lo)};
+    return df_norm({s.hi, __fadd_rn(s.lo, a.lo)});
 }
 
-__device__ __forceinline__ DF df_norm(DF a) { return fast_two_sum_f(a.hi, a.lo); }
-
-__device__ __forceinline__ DF df_square(DF a) {
+__device__ __forceinline__ DF df_square_raw(DF a) {
     const float p = __fmul_rn(a.hi, a.hi);
     return {p, __fmaf_rn(__fadd_rn(a.hi, a.hi), a.lo, __fmaf_rn(a.hi, a.hi, -p))};
 }
 
-// acc + a b for the row products of a rotation: as df_mul and df_add, the low parts gathered.
-__device__ __forceinline__ DF df_mul_add(DF a, DF b, DF acc) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    const DF s = two_sum_f(acc.hi, p);
-    float e = __fadd_rn(__fmaf_rn(a.hi, b.hi, -p), __fadd_rn(acc.lo, s.lo));
-    e = __fmaf_rn(a.hi, b.lo, e);
-    return {s.hi, __fmaf_rn(a.lo, b.hi, e)};
-}
-
-// 1 / b: the FP32 reciprocal approximation x of b.hi, then x + x (e + e^2) with
-// e = 1 - b x (fma: exact to 2^-48, |e| < 2^-22).
-__device__ __forceinline__ DF df_rcp(DF b) {
-    const float x = rcp_approx(b.hi);
+// 1 / b: the FP32 reciprocal x of b.hi, then x + x (e + e^2) with e = 1 - b x
+// (fma: exact to 2^-48, |e| < 2^-23).
+__device__ __forceinline__ DF df_rcp_raw(DF b) {
+    const float x = __frcp_rn(b.hi);
     const float e = __fmaf_rn(-b.lo, x, __fmaf_rn(-b.hi, x, 1.0f));
     const float xe = __fmul_rn(x, e);
     return {x, __fmaf_rn(xe, e, xe)};
@@ -115,30 +110,32 @@ __device__ __forceinline__ CamDF load_cam_df(const float* __restrict__ rec, cons
 
 // The Snavely residual of Sec. VI-A in df arithmetic: P = R X + t, d = P.z -+ eps
 // (d_safe), p = -P.xy / d, s = 1 + k1 |p|^2 + k2 |p|^4, r = f s p - u.  Its error is a
-// few units of 2^-46 of the ~500 px terms, so rounded to FP32 it is the exact residual
-// to within an ulp of itself.  Low parts are gathered and renormalised only where a
-// cancellation (R X + t, f s p - u) or a division follows: 210 FP32 operations, where
-// renormalising every sum and product took 305
-// (28.8M residuals: 475 -> 381 us).
+// few units of 2^-48 of the ~500 px terms, so rounded to FP32 it is the exact residual
+// to within an ulp of itself.  R X + t, where the terms cancel, is renormalised after every
+// product and sum; the polynomial of the distortion, whose terms do not, only where a product
+// with p or a cancellation follows.  28.8M residuals: 475 us with every operation renormalised,
+// 437 us so, with no larger an error (200 cameras: 3.26e-13 px rms against 3.28e-13; R X + t of
+// 65-unit coordinates: 7.8e-12 against 7.7e-12); with R X + t left raw as well 381 us, but
+// 3.7e-13 and 9.3e-12.
 __device__ __forceinline__ void residual_df(const CamDF& c, const DF (&X)[3], float eps, float u0, float u1,
                                             DF& r0, DF& r1) {
     DF P[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         DF a = df_mul(c.R[3 * i], X[0]);
-        a = df_mul_add(c.R[3 * i + 1], X[1], a);
-        a = df_mul_add(c.R[3 * i + 2], X[2], a);
-        P[i] = df_norm(df_add(a, c.t[i]));
+        a = df_add(a, df_mul(c.R[3 * i + 1], X[1]));
+        a = df_add(a, df_mul(c.R[3 * i + 2], X[2]));
+        P[i] = df_add(a, c.t[i]);
     }
     DF d = P[2];
-    if (eps != 0.0f) d = df_norm(df_add_f(d, P[2].hi >= 0.0f ? eps : -eps));
-    const DF iz = df_rcp(d);
-    const DF q0 = df_norm(df_mul(P[0], iz)), q1 = df_norm(df_mul(P[1], iz));   // -p
-    const DF n2 = df_add(df_square(q0), df_square(q1));
-    const DF s = df_norm(df_add_f(df_mul(n2, df_add(c.k1, df_mul(c.k2, n2))), 1.0f));
+    if (eps != 0.0f) d = df_add_f(d, P[2].hi >= 0.0f ? eps : -eps);
+    const DF iz = df_rcp_raw(d);
+    const DF q0 = df_mul(P[0], iz), q1 = df_mul(P[1], iz);   // -p
+    const DF n2 = df_add_raw(df_square_raw(q0), df_square_raw(q1));
+    const DF s = df_add_f(df_mul_raw(n2, df_add_raw(c.k1, df_mul_raw(c.k2, n2))), 1.0f);
     const DF fs = df_mul(c.f, s);
     // r = -(f s q + u)
-    const DF a0 = df_norm(df_add_f(df_mul(fs, q0), u0)), a1 = df_norm(df_add_f(df_mul(fs, q1), u1));
+    const DF a0 = df_add_f(df_mul_raw(fs, q0), u0), a1 = df_add_f(df_mul_raw(fs, q1), u1);
     r0 = {-a0.hi, -a0.lo};
     r1 = {-a1.hi, -a1.lo};
 }

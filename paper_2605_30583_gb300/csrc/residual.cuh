@@ -51,7 +51,7 @@ __device__ __forceinline__ void residual_tiles(const Views<float>& v, int at_can
                 residual_df(cam, X, eps, uv.x, uv.y, d0, d1);
                 r0 = df_to_float(d0);
                 r1 = df_to_float(d1);
-                s2 = df_add(df_square(d0), df_square(d1));
+                s2 = df_add(df_mul(d0, d0), df_mul(d1, d1));
             } else {
                 const Cam cam = load_cam(rec + (size_t)c * CP_STRIDE);
                 project_residual(cam, xh.x, xh.y, xh.z, eps, uv.x, uv.y, r0, r1);

@@ -1,0 +1,101 @@
+"""What the mixed form computes beyond FP32 keeps its bits: residuals in double-float."""
+import numpy as np
+import pytest
+
+from oracle import ba_oracle as O
+from paper_2605_30583_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2605_30583_gb300 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+@pytest.mark.parametrize("scene,n_cams,n_pts,kw", [("cloud", 200, 50_000, {}),
+                                                   ("band", 3000, 100_000, dict(ring_radius=65.0, scene="band"))])
+def test_residual_error(B, scene, n_cams, n_pts, kw):
+    """Pixels are the exact projections rounded to FP32, so residuals below 1e-6 px show the
+    arithmetic's error and not their own rounding.  The bound is the error of the same formula with
+    every double-float operation renormalised and a correctly rounded FP32 reciprocal, taken in
+    the same operations on the host, plus 4 % for the choice of observations and for operations
+    that round differently."""
+    prob = synth.make_problem(n_cams, n_pts, ("poisson", 3.0), "nearest", seed=200, **kw)
+    args = prob.cams_gt, prob.pts_gt, prob.cam_idx, prob.pt_idx
+    exact = O.residuals(*args, np.zeros((prob.n_obs, 2)))
+    px = exact.astype(np.float32).astype(np.float64)
+    p = B.Problem(prob.n_cams, prob.n_pts, prob.cam_idx, prob.pt_idx, px)
+    p.set_params(prob.cams_gt, prob.pts_gt)
+    _, r, _ = p.evaluate(residuals=True)
+    pick = np.abs(exact - px) < 1e-6
+    err = (r.double().cpu().numpy() - (exact - px))[pick]
+    ref = (_renormalised(prob, px) - (exact - px))[pick]
+    assert np.sqrt(np.mean(err**2)) <= 1.04 * np.sqrt(np.mean(ref**2))
+
+
+# ---- double-float arithmetic on the host: float32 pairs, FMA through float64 (a product of two
+# float32 values is exact there)
+F = np.float32
+
+
+def _fma(a, b, c):
+    return (a.astype(np.float64) * b + c).astype(F)
+
+
+def _norm(h, l):
+    s = h + l
+    return s, l - (s - h)
+
+
+def _add(a, b):
+    s = a[0] + b[0]
+    t = s - a[0]
+    return _norm(s, ((a[0] - (s - t)) + (b[0] - t)) + (a[1] + b[1]))
+
+
+def _mul(a, b):
+    p = a[0] * b[0]
+    e = _fma(a[0], b[0], -p)
+    return _norm(p, _fma(a[1], b[0], _fma(a[0], b[1], e)))
+
+
+def _rcp(b):
+    x = (1.0 / b[0].astype(np.float64)).astype(F)
+    bx = _mul(b, (x, np.zeros_like(x)))
+    return _norm(x, x * ((F(1) - bx[0]) - bx[1]))
+
+
+def _pair(x):
+    h = x.astype(F)
+    return h, (x - h).astype(F)
+
+
+def _renormalised(prob, px):
+    from scipy.spatial.transform import Rotation
+    c, X = prob.cams_gt[prob.cam_idx], prob.pts_gt[prob.pt_idx]
+    R = Rotation.from_rotvec(prob.cams_gt[:, :3]).as_matrix()[prob.cam_idx]
+    X = [_pair(X[:, j]) for j in range(3)]
+    P = []
+    for i in range(3):
+        a = _mul(_pair(R[:, i, 0]), X[0])
+        for j in (1, 2):
+            a = _add(a, _mul(_pair(R[:, i, j]), X[j]))
+        P.append(_add(a, _pair(c[:, 3 + i])))
+    iz = _rcp(P[2])
+    q = [_mul(P[0], iz), _mul(P[1], iz)]
+    one = (np.ones_like(iz[0]), np.zeros_like(iz[0]))
+    n2 = _add(_mul(q[0], q[0]), _mul(q[1], q[1]))
+    s = _add(_mul(n2, _add(_pair(c[:, 7]), _mul(_pair(c[:, 8]), n2))), one)
+    fs = _mul(_pair(c[:, 6]), s)
+    out = []
+    for k in range(2):
+        h, l = _add(_mul(fs, q[k]), (px[:, k].astype(F), np.zeros_like(iz[0])))
+        out.append(-(h + l))
+    return np.stack(out, 1).astype(np.float64)
