@@ -284,12 +284,13 @@ __device__ __forceinline__ void rodrigues_coeffs(double th2, double& A, double& 
         C = 1.0 / 6.0 + th2 * (-1.0 / 120.0 + th2 * (1.0 / 5040.0 + th2 * (-1.0 / 362880.0)));
     } else {
         const double th = sqrt(th2);
-        double sh, ch;
-        sincos(0.5 * th, &sh, &ch);
-        const double s = 2.0 * sh * ch, i = rcp64(th);   // sin(th); FP64 divisions are slow here
-        A = s * i;
-        B = 2.0 * (sh * i) * (sh * i);
-        C = (th - s) * i * i * i;
+        const double s = sin(th), sh = sin(0.5 * th);
+        // Quotients and a sine of their own: sin th from the half angle's sine and cosine and powers
+        // of 1 / th take ~1.7 us less of a camera kernel's FP64 latency, but raise the FP64
+        // form's residual error by a fifth (5.0e-14 -> 6.0e-14 px rms, 200 cameras).
+        A = s / th;
+        B = 2.0 * sh * sh / th2;
+        C = (th - s) / (th2 * th);
     }
 }
 

@@ -30,7 +30,7 @@ namespace gbba {
 // Camera records from the current parameters (their FP64 master copy); zeroes the
 // linearisation sums.
 // Three lanes a camera (camera_record_rows), ten cameras a warp: the kernel is one chain of FP64
-// latency (14 -> 9 us on 1,000 cameras).
+// latency (14 -> 10 us on 1,000 cameras).
 constexpr int ROW_CAMS = 10;
 
 __global__ void k_camera_precompute(Views<float> v) {

@@ -1,4 +1,4 @@
-"""What the mixed form computes beyond FP32 keeps its bits: residuals in double-float."""
+"""What is computed beyond FP32 keeps its bits: double-float residuals, FP64 camera records."""
 import numpy as np
 import pytest
 
@@ -38,6 +38,40 @@ def test_residual_error(B, scene, n_cams, n_pts, kw):
     err = (r.double().cpu().numpy() - (exact - px))[pick]
     ref = (_renormalised(prob, px) - (exact - px))[pick]
     assert np.sqrt(np.mean(err**2)) <= 1.04 * np.sqrt(np.mean(ref**2))
+
+
+@pytest.mark.parametrize("n_cams,n_pts,kw", [(200, 5000, {}), (3000, 20_000, dict(ring_radius=65.0, scene="band"))])
+def test_camera_record_error(B, n_cams, n_pts, kw):
+    """The FP64 form's residuals against extended precision: no further off than the formula with
+    sin th / th, 2 sin^2(th / 2) / th^2 in FP64 on the host, plus 6 % for operations that round
+    differently (FMA)."""
+    prob = synth.make_problem(n_cams, n_pts, ("poisson", 3.0), "nearest", seed=1, **kw)
+    p = B.Problem(prob.n_cams, prob.n_pts, prob.cam_idx, prob.pt_idx, prob.pixels, precision="fp64")
+    p.set_params(prob.cams_gt, prob.pts_gt)
+    _, r, _ = p.evaluate(residuals=True)
+    exact = _residuals(prob, np.longdouble)
+
+    def rms(x):
+        return float(np.sqrt(np.mean((x - exact) ** 2)))
+
+    assert rms(r.cpu().numpy()) <= 1.06 * rms(_residuals(prob, np.float64))
+
+
+def _residuals(prob, dtype):
+    c, X = prob.cams_gt.astype(dtype), prob.pts_gt.astype(dtype)[prob.pt_idx]
+    w, th2 = c[:, :3], (c[:, :3] ** 2).sum(1)
+    th = np.sqrt(th2)
+    K = np.zeros((len(c), 3, 3), dtype)
+    K[:, 2, 1], K[:, 0, 2], K[:, 1, 0] = w.T
+    K -= K.transpose(0, 2, 1)
+    eye = np.eye(3, dtype=dtype)
+    K2 = w[:, :, None] * w[:, None, :] - th2[:, None, None] * eye
+    R = eye + (np.sin(th) / th)[:, None, None] * K + (2 * np.sin(th / 2) ** 2 / th2)[:, None, None] * K2
+    R, c = R[prob.cam_idx], c[prob.cam_idx]
+    P = sum(R[:, :, j] * X[:, j, None] for j in range(3)) + c[:, 3:6]
+    q = -P[:, :2] / P[:, 2:]
+    n2 = (q * q).sum(1)
+    return (c[:, 6] * (1 + n2 * (c[:, 7] + c[:, 8] * n2)))[:, None] * q - prob.pixels
 
 
 # ---- double-float arithmetic on the host: float32 pairs, FMA through float64 (a product of two
