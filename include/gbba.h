@@ -186,7 +186,7 @@ ba_status ba_selftest_wait_timeout(void* scratch, int32_t grid, int32_t timeout_
                                    int32_t* error_word);
 
 /* Self-test of the FP64 reciprocal that the block-Jacobi inversions use (a hardware
- * approximation refined by one third-order step).  y[i] = 1/x[i] for i < n, with
+ * approximation refined by two Newton-Raphson steps).  y[i] = 1/x[i] for i < n, with
  * x and y device arrays of n doubles (n >= 1), enqueued on `stream` (cudaStream_t).
  * Zero, non-finite and |x| outside [1e-300, 1e300] take the IEEE quotient 1.0 / x. */
 ba_status ba_selftest_rcp64(const double* x, double* y, int64_t n, void* stream);

@@ -124,23 +124,19 @@ __device__ __forceinline__ double slot_sum_warp(const double* base, int k) {
     return v;
 }
 
-// 1/x in FP64: hardware approximation (over 18 bits) refined by one third-order step
-// y <- y + y (e + e^2), e = 1 - x y, which triples the correct bits in three dependent FP64
-// operations (an FP64 operation has ~130 cycles of latency on this GPU; two Newton-Raphson
-// steps take four).  Zero, non-finite and
+// 1/x in FP64: hardware approximation refined by two Newton-Raphson steps
+// y <- y + y (1 - x y), each roughly doubling the correct bits.  (One third-order step
+// y + y (e + e^2) is an FP64 operation, ~130 cycles, shorter, but leaves up to 0.505 ulp where
+// this leaves 0.500: 0.03 % of the results are then not the rounded quotient.)  Zero, non-finite and
 // |x| outside [1e-300, 1e300] (where x y or the approximation could leave the normal
 // range, flushing or overflowing before the refinement) take the IEEE quotient.
-__device__ __forceinline__ double rcp64_fast(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
 __device__ __forceinline__ double rcp64(double x) {
     const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;   // the range test on the high word
     if (h - 0x01a56e20u > 0x7e37e43bu - 0x01a56e20u) return 1.0 / x;
-    return rcp64_fast(x);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
 }
 
 // float -> double and double -> float (round to nearest even) with integer instructions.  The
@@ -516,7 +512,7 @@ __device__ __forceinline__ bool camera_inverse9(const T* __restrict__ H, double 
         // positive, finite and within rcp64's range, from the high word: an integer test stays off
         // the chain of FP64 operations (~130 cycles each)
         ok = ok && (uint32_t)__double2hiint(piv) - 0x01a56e20u <= 0x7e37e43bu - 0x01a56e20u;
-        const double ip = rcp64_fast(piv);
+        const double ip = rcp64(piv);
         const bool own = L.i == k;
         const double rk = own ? ip : col[k] * ip;   // row k of the updated matrix, this lane's column
 #pragma unroll

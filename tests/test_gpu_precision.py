@@ -57,6 +57,16 @@ def test_camera_record_error(B, n_cams, n_pts, kw):
     assert rms(r.cpu().numpy()) <= 1.06 * rms(_residuals(prob, np.float64))
 
 
+def test_reciprocal_is_the_rounded_quotient(B):
+    """Two Newton-Raphson steps from the hardware's ~20 bits leave 2^-70 before the last rounding, so
+    a result differs from the rounded quotient only where that lies within 2^-17 ulp of the middle
+    between two numbers: 2^-16 of the arguments at most."""
+    import torch
+    x = np.concatenate([1.0 + np.random.default_rng(3).random(1_000_000), np.logspace(-299, 299, 200_001)])
+    y = B.selftest_rcp64(torch.from_numpy(x).cuda()).cpu().numpy()
+    assert np.mean(y != 1.0 / x) <= 2.0**-16
+
+
 def _residuals(prob, dtype):
     c, X = prob.cams_gt.astype(dtype), prob.pts_gt.astype(dtype)[prob.pt_idx]
     w, th2 = c[:, :3], (c[:, :3] ** 2).sum(1)
