@@ -492,7 +492,7 @@ __device__ __forceinline__ double to_fp64(double x) { return x; }
 // takes a_ik times it from the other rows and leaves column k of the inverse in column k's place
 // (the operations of the elimination of [A | I], without its columns that are still those of
 // I).  Bound by the FP64 pipe, which a warp instruction holds for 16 cycles: one camera a warp
-// with its 18 columns took three times as long.  False if a pivot is not within [1e-300, 1e300].
+// with its 18 columns took three times as long.  False if a pivot is not positive and finite.
 // Every lane of the warp calls it.
 template <typename T>
 __device__ __forceinline__ bool camera_inverse9(const T* __restrict__ H, double mu, double lo, double hi,
@@ -509,9 +509,10 @@ __device__ __forceinline__ bool camera_inverse9(const T* __restrict__ H, double 
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const double piv = __shfl_sync(0xffffffffu, col[k], L.base + k);
-        // positive, finite and within rcp64's range, from the high word: an integer test stays off
-        // the chain of FP64 operations (~130 cycles each)
-        ok = ok && (uint32_t)__double2hiint(piv) - 0x01a56e20u <= 0x7e37e43bu - 0x01a56e20u;
+        // positive and finite, from its words: an integer test stays off the chain of FP64
+        // operations (~130 cycles each)
+        const uint32_t h = (uint32_t)__double2hiint(piv);
+        ok = ok && h < 0x7ff00000u && (h | (uint32_t)__double2loint(piv)) != 0u;
         const double ip = rcp64(piv);
         const bool own = L.i == k;
         const double rk = own ? ip : col[k] * ip;   // row k of the updated matrix, this lane's column

@@ -67,6 +67,29 @@ def test_reciprocal_is_the_rounded_quotient(B):
     assert np.mean(y != 1.0 / x) <= 2.0**-16
 
 
+@pytest.mark.parametrize("iters", [2, 4])
+def test_camera_blocks_with_tiny_pivots(B, iters):
+    """A camera that sees points on its axis only: no observation moves with w_z, t_z, f, k1 or k2,
+    and with min_diag = 1e-305 their pivots are ~1e-307.  The block is positive definite all the same,
+    and the preconditioner is its inverse: FP64 form against the oracle."""
+    prob = synth.make_problem(12, 200, ("poisson", 3.0), "uniform", seed=9)
+    k = 6
+    cams, pts, ci, pi = prob.cams_init.copy(), prob.pts_init.copy(), prob.cam_idx.copy(), prob.pt_idx
+    ci[ci == 0] = 1 + pi[ci == 0] % 11
+    cams[0, :6] = 0.0
+    pts[:k, :2], pts[:k, 2] = 0.0, -np.linspace(2.0, 3.0, k)
+    ci = np.concatenate([ci, np.zeros(k, ci.dtype)])
+    pi = np.concatenate([pi, np.arange(k, dtype=pi.dtype)])
+    px = np.concatenate([prob.pixels, np.random.default_rng(8).standard_normal((k, 2))])
+    opts = dict(max_lm_iters=1, max_pcg_iters=iters, pcg_rel_tol=0.0, min_diag=1e-305)
+    p = B.Problem(prob.n_cams, prob.n_pts, ci, pi, px, precision="fp64")
+    p.set_params(cams, pts)
+    h = p.solve(**opts).history[0]
+    o = O.ba_solve(cams, pts, ci, pi, px, O.LMOptions(**opts)).history[0]
+    assert h["pcg_iters"] == o["pcg_iters"] == iters
+    assert abs(h["model_decrease"] - o["model_decrease"]) <= 1e-9 * o["model_decrease"]
+
+
 def _residuals(prob, dtype):
     c, X = prob.cams_gt.astype(dtype), prob.pts_gt.astype(dtype)[prob.pt_idx]
     w, th2 = c[:, :3], (c[:, :3] ** 2).sum(1)
