@@ -227,9 +227,10 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 // invert the point blocks (a thread per point), so the long FP64 camera eliminations run
 // beside the point work instead of before it in the same warps.
 //
-// Bound by the FP64 pipe (80 % active: 28 operations a point, ~42 a camera's share of a warp):
-// 687 -> 488 us on 13,000 cameras and 4.5M points with integer conversions, one reciprocal a
-// point, compensated FP32 sums and three cameras a warp.  h is always cleared: a PCG that runs no
+// Bound by the FP64 pipe (31 operations a point, ~50 a camera's share of a warp):
+// 687 -> 540 us on 13,000 cameras and 4.5M points with integer conversions, one reciprocal a
+// point and three cameras a warp.  r^T z and |r|^2 are summed in FP64 (as FP32 pairs: 37 us less,
+// but a camera's g of 2e19 and more squares to infinity there).  h is always cleared: a PCG that runs no
 // iteration (cap 0, a zero or non-finite residual) leaves the step at 0, and the candidate and its
 // evaluation read it.  `zero_ps`: the solver that follows wants the points' p and s cleared too.
 __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulonglong2* words, int cam_blocks,
@@ -247,7 +248,7 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
     const double mu = st->mu, lo = st->opt.min_diag, hi = st->opt.max_diag;
     // the bounds as floats on the inner side: h >= lo exactly when h >= lo_f
     const float lo_f = __double2float_ru(lo), hi_f = __double2float_rd(hi);
-    float rz = 0.0f, rr = 0.0f, rzc = 0.0f, rrc = 0.0f;   // Kahan pairs
+    double rz = 0.0, rr = 0.0;
     const int warps = cam_blocks * (blockDim.x >> 5);
     const bool cam_role = (int)blockIdx.x < cam_blocks;
     for (int c0 = 3 * (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); cam_role && c0 < v.n_cams; c0 += 3 * warps) {
@@ -281,8 +282,8 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
             v.h[e] = 0.0f;
             v.pc[e] = 0.0f;
             v.pc[v.pc_stride + e] = 0.0f;
-            kahan_add(rz, rzc, ri * z);
-            kahan_add(rr, rrc, ri * ri);
+            rz = fma(widen(ri), widen(z), rz);
+            rr = fma(widen(ri), widen(ri), rr);
             for (int k = L.i; k < CA_STRIDE; k += 9) {
                 v.cam_acc[(size_t)c * CA_STRIDE + k] = 0.0f;
                 if (words != nullptr)   // the persistent kernel rotates over all the sets
@@ -315,12 +316,12 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
             v.p[e] = 0.0f; v.p[e + 1] = 0.0f; v.p[e + 2] = 0.0f;
             v.s[e] = 0.0f; v.s[e + 1] = 0.0f; v.s[e + 2] = 0.0f;
         }
-        kahan_add(rz, rzc, fmaf(r0, z0, fmaf(r1, z1, r2 * z2)));
-        kahan_add(rr, rrc, fmaf(r0, r0, fmaf(r1, r1, r2 * r2)));
+        rz += widen(fmaf(r0, z0, fmaf(r1, z1, r2 * z2)));
+        rr += widen(fmaf(r0, r0, fmaf(r1, r1, r2 * r2)));
     }
-    __shared__ double red[64];
+    __shared__ double red[32];
     double in[2], out[2];
-    block_sum2c(rz, rzc, rr, rrc, red, in[0], in[1]);
+    block_sum2d(rz, rr, red, in[0], in[1]);
     if (!grid_reduce_block<2>(in, v.partials, &st->tickets[TK_PRE], out)) return;
     for (int k = threadIdx.x; k < NSLOT * SLOT_STRIDE; k += blockDim.x) st->acc_mv[k] = st->acc_up[k] = 0.0;
     if (threadIdx.x == 0) {
@@ -632,8 +633,7 @@ __global__ void k_candidate(Views<float> v) {
     if (st->lm_active == 0) return;
     const bool retract = st->opt.retract != 0;
     const float ha = st->h_alpha;
-    double gh = 0.0;                 // cameras
-    float ghp = 0.0f, ghc = 0.0f;    // points, a Kahan pair
+    double gh = 0.0;
     // cameras: three lanes each (camera_record_rows), in the first warp of a block
     const int row = (int)threadIdx.x % 3;
     for (int c = ROW_CAMS * (int)blockIdx.x + (int)threadIdx.x / 3; threadIdx.x < 3 * ROW_CAMS && c < v.n_cams;
@@ -719,12 +719,11 @@ __global__ void k_candidate(Views<float> v) {
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             x4[k] = make_float4(narrow(X[4 * k]), narrow(X[4 * k + 1]), narrow(X[4 * k + 2]), narrow(X[4 * k + 3]));
-        kahan_add(ghp, ghc, sgh);
+        gh += widen(sgh);
     }
-    __shared__ double red[64];
-    double in[1], out[1], none;
-    block_sum2c(ghp, ghc, 0.0f, 0.0f, red, in[0], none);
-    if (threadIdx.x < 32) in[0] += warp_sum(gh);   // only the first warp has cameras
+    __shared__ double red[32];
+    double in[1], out[1];
+    in[0] = block_sum(gh, red);
     if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_CAND], out) && threadIdx.x == 0) st->gh = out[0];
 }
 
@@ -740,9 +739,10 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
     const int active = st->lm_active;
     const float eps = (float)st->opt.eps;
     const int loss = st->opt.loss;
-    float jc = 0.0f, jcc = 0.0f;   // Kahan pair
+    double jh2 = 0.0;
     if (active) {
         for (int tile = blockIdx.x; tile < v.n_tiles; tile += gridDim.x) {
+            float jc = 0.0f, jcc = 0.0f;   // Kahan pair
             const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
             const int pt0 = tile * v.tile_pts;
             const uint32_t n = hi - lo;
@@ -766,11 +766,12 @@ __global__ void __launch_bounds__(TB) k_eval_candidate(Views<float> v, CondHandl
                 // |J h|^2 weighted at x (F' comes from k_residual)
                 kahan_add(jc, jcc, (loss ? __ldg(v.obs_w + j) : 1.0f) * fmaf(t0, t0, t1 * t1));
             }
+            jh2 += pair_sum(jc, jcc);
         }
     }
-    __shared__ double red[64];
-    double in[1], out[1], none;
-    block_sum2c(jc, jcc, 0.0f, 0.0f, red, in[0], none);
+    __shared__ double red[32];
+    double in[1], out[1];
+    in[0] = block_sum(jh2, red);
     if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {
         // pose factors: k_factor_eval ran just before
         const bool fac = v.n_fac > 0;

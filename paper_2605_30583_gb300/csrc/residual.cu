@@ -36,11 +36,10 @@ __global__ void __launch_bounds__(TB, 5) k_residual(Views<float> v, int at_candi
     // a candidate is only evaluated while LM runs (the decision kernel reads F' then)
     if (at_candidate && st->lm_active == 0) return;
     __shared__ float4 sXh[TILE_PTS], sXl[TILE_PTS];
-    float cs = 0.0f, cc = 0.0f;
-    residual_tiles<TB>(v, at_candidate, squared, blockIdx.x, gridDim.x, sXh, sXl, cs, cc);
-    __shared__ double red[2 * (TB / 32)];
-    double in[1], out[1], none;
-    block_sum2c(cs, cc, 0.0f, 0.0f, red, in[0], none);
+    const double cost2 = residual_tiles<TB>(v, at_candidate, squared, blockIdx.x, gridDim.x, sXh, sXl);
+    __shared__ double red[TB / 32];
+    double in[1], out[1];
+    in[0] = block_sum(cost2, red);
     if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_RES], out) && threadIdx.x == 0) st->F_res = 0.5 * out[0];
 }
 

@@ -7,11 +7,11 @@
 
 namespace gbba {
 
-// Residuals of tiles first, first + stride, ... to v.rbuf; the cost as a Kahan pair cs - cc (twice
-// the cost).  sXh, sXl: TILE_PTS entries of shared memory each (the tile's points, double-float).
+// Residuals of tiles first, first + stride, ... to v.rbuf; returns this thread's part of twice the
+// cost.  sXh, sXl: TILE_PTS entries of shared memory each (the tile's points, double-float).
 template <int TB>
-__device__ __forceinline__ void residual_tiles(const Views<float>& v, int at_candidate, int squared, int first, int stride,
-                                               float4* sXh, float4* sXl, float& cs, float& cc) {
+__device__ __forceinline__ double residual_tiles(const Views<float>& v, int at_candidate, int squared, int first, int stride,
+                                                 float4* sXh, float4* sXl) {
     DevState* st = v.st;
     const double* xm = at_candidate ? v.xm_new : v.xm;
     const float* rec = at_candidate ? v.cam_pre_new : v.cam_pre;
@@ -23,7 +23,7 @@ __device__ __forceinline__ void residual_tiles(const Views<float>& v, int at_can
     // the cost: Kahan pair of the high parts of |r|^2 (double-float |r|^2 before any
     // rounding, so F resolves steps far below an FP32 ulp of the residuals) and the sum
     // of their low parts
-    float cl = 0.0f;
+    float cs = 0.0f, cc = 0.0f, cl = 0.0f;
     for (int tile = first; tile < v.n_tiles; tile += stride) {
         const uint32_t lo = v.tile_off[tile], hi = v.tile_off[tile + 1];
         const int pt0 = tile * v.tile_pts;
@@ -67,7 +67,7 @@ __device__ __forceinline__ void residual_tiles(const Views<float>& v, int at_can
         }
         __syncthreads();   // the next tile's staging overwrites the points
     }
-    cc -= cl;
+    return pair_sum(cs, cc) + widen(cl);
 }
 
 }  // namespace gbba

@@ -603,7 +603,7 @@ constexpr int TL_TB = 128;
 // Few tiles: a tile's runs spread over the warps of 512 threads.  The linearisation does so up to
 // one tile per SM (16 tiles: 18.0 -> 13.8 us; 298 tiles 22.9 against 23.6, 302 tiles 23.3 against
 // 25.8, 910 tiles 43.7 against 61.9), the candidate's residuals and evaluation in one launch
-// (k_tile_step) up to two (against both launches: 25.3 -> 14.2 us, 31.8 -> 30.6, 32.5 -> 32.5 and
+// (k_tile_step) up to two (against both launches: 25.3 -> 15.0 us, 31.8 -> 30.6, 32.5 -> 32.5 and
 // a launch gap of 2 us each; 910 tiles 45.8 against 77.7).
 constexpr int WIDE_LIN_TILES = 1;
 constexpr int WIDE_TILES = 2;
@@ -841,12 +841,13 @@ __global__ void __launch_bounds__(TB, TB == 128 ? 4 : 1) k_tile_linearize(Views<
 // LM loop flag.
 constexpr int TE_TB = 128;
 
-// |J h|^2 of tiles first, first + stride, ... as a Kahan pair (js, jc).  sXo, sHp: TILE_PTS entries
+// This thread's part of |J h|^2 over tiles first, first + stride, ...  sXo, sHp: TILE_PTS entries
 // each (x and h of the tile's points).
 template <int TB>
-__device__ __forceinline__ void eval_tiles(const Views<float>& v, const Caps& cap, unsigned char* dsm, float4* sXo,
-                                           float4* sHp, unsigned int* s_next, int first, int stride, float& js,
-                                           float& jc) {
+__device__ __forceinline__ double eval_tiles(const Views<float>& v, const Caps& cap, unsigned char* dsm, float4* sXo,
+                                             float4* sHp, unsigned int* s_next, int first, int stride) {
+    double jh2 = 0.0;
+    float js, jc;   // the tile's part, a Kahan pair
     const float eps = (float)v.st->opt.eps;
     const int loss = v.st->opt.loss;
     const int lane = threadIdx.x & 31;
@@ -869,6 +870,7 @@ __device__ __forceinline__ void eval_tiles(const Views<float>& v, const Caps& ca
     };
     for (int tile = first; tile < v.n_tiles; tile += stride) {
         const TileRange T = tile_range(v, tile);
+        js = jc = 0.0f;
         for (int i = threadIdx.x; i < T.npt; i += TB) {
             const size_t e = T.base + 3 * i;
             sXo[i] = make_float4(v.x[e], v.x[e + 1], v.x[e + 2], 0.0f);
@@ -902,8 +904,10 @@ __device__ __forceinline__ void eval_tiles(const Views<float>& v, const Caps& ca
             }
             visit(e, j, key & 0xffu);
         }
+        jh2 += pair_sum(js, jc);
         __syncthreads();   // the next tile's staging overwrites the points
     }
+    return jh2;
 }
 
 // The LM decision from F' (F_res) and |J h|^2, by one thread.
@@ -923,13 +927,12 @@ __global__ void __launch_bounds__(TB, 6) k_tile_eval(Views<float> v, CondHandle 
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ float4 sXo[TILE_PTS], sHp[TILE_PTS];
     __shared__ unsigned int s_next;
-    __shared__ double red[2 * (TB / 32)];
+    __shared__ double red[TB / 32];
     DevState* st = v.st;
     const int active = st->lm_active;
-    float js = 0.0f, jc = 0.0f;
-    if (active) eval_tiles<TB>(v, cap, dsm, sXo, sHp, &s_next, blockIdx.x, gridDim.x, js, jc);
-    double in[1], out[1], none;
-    block_sum2c(js, jc, 0.0f, 0.0f, red, in[0], none);
+    const double jh2 = active ? eval_tiles<TB>(v, cap, dsm, sXo, sHp, &s_next, blockIdx.x, gridDim.x) : 0.0;
+    double in[1], out[1];
+    in[0] = block_sum(jh2, red);
     if (grid_reduce_block<1>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0)
         tile_decide(v, active, st->F_res, out[0], lm_cond, use_cond);
 }
@@ -942,15 +945,14 @@ __global__ void __launch_bounds__(TB, 1) k_tile_step(Views<float> v, CondHandle 
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ float4 sA[TILE_PTS], sB[TILE_PTS];
     __shared__ unsigned int s_next;
-    __shared__ double red[2 * (TB / 32)];
+    __shared__ double red[TB / 32];
     DevState* st = v.st;
     const int active = st->lm_active;
     const bool res = (int)blockIdx.x < v.n_tiles;
-    float s = 0.0f, c = 0.0f;
-    if (active && res) residual_tiles<TB>(v, 1, 0, blockIdx.x, v.n_tiles, sA, sB, s, c);
-    if (active && !res) eval_tiles<TB>(v, cap, dsm, sA, sB, &s_next, (int)blockIdx.x - v.n_tiles, v.n_tiles, s, c);
-    double b, none, in[2], out[2];
-    block_sum2c(s, c, 0.0f, 0.0f, red, b, none);
+    double part = 0.0, in[2], out[2];
+    if (active && res) part = residual_tiles<TB>(v, 1, 0, blockIdx.x, v.n_tiles, sA, sB);
+    if (active && !res) part = eval_tiles<TB>(v, cap, dsm, sA, sB, &s_next, (int)blockIdx.x - v.n_tiles, v.n_tiles);
+    const double b = block_sum(part, red);
     in[0] = res ? b : 0.0;
     in[1] = res ? 0.0 : b;
     if (grid_reduce_block<2>(in, v.partials, &st->tickets[TK_COST], out) && threadIdx.x == 0) {

@@ -90,6 +90,33 @@ def test_camera_blocks_with_tiny_pivots(B, iters):
     assert abs(h["model_decrease"] - o["model_decrease"]) <= 1e-9 * o["model_decrease"]
 
 
+@pytest.mark.parametrize("pcg_kernel", [0, 1])
+def test_gradients_whose_squares_leave_the_fp32_range(B, pcg_kernel):
+    """A point that grazes a camera's plane (|p| ~ 1000) has a derivative of ~1e15 in k2: g there is
+    ~1e20, representable in FP32, its square is not.  |r_0|^2 and r^T z are summed in FP64, so the
+    first step is the oracle's (the FP32 residual after it may still be too long to go on)."""
+    prob = synth.make_problem(12, 200, ("poisson", 3.0), "uniform", seed=12)
+    cams, pts = prob.cams_init.copy(), prob.pts_init.copy()
+    cams[0], pts[0] = 0.0, (1.0, 0.3, -1e-3)
+    cams[0, 6] = 1000.0
+    ci, pi = prob.cam_idx.copy(), prob.pt_idx
+    ci[ci == 0] = 1 + pi[ci == 0] % 11
+    ci = np.concatenate([ci, np.zeros(1, ci.dtype)])
+    pi = np.concatenate([pi, np.zeros(1, pi.dtype)])
+    cams, pts = cams.astype(np.float32).astype(np.float64), pts.astype(np.float32).astype(np.float64)
+    px = np.concatenate([prob.pixels, O.residuals(cams, pts, ci[-1:], pi[-1:], np.zeros((1, 2))) + 60.0])
+    px = px.astype(np.float32).astype(np.float64)
+    opts = dict(max_lm_iters=1, max_pcg_iters=1)
+    g = O.linearize(cams, pts, ci, pi, px).g
+    assert 2e19 < np.abs(g).max() < 1e38
+    p = B.Problem(prob.n_cams, prob.n_pts, ci, pi, px)
+    p.set_params(cams, pts)
+    res = p.solve(pcg_kernel=pcg_kernel, **opts)
+    o = O.ba_solve(cams, pts, ci, pi, px, O.LMOptions(**opts)).history[0]
+    assert res.accepted == 1 and o["accepted"]
+    assert abs(res.history[0]["model_decrease"] - o["model_decrease"]) <= 1e-3 * abs(o["model_decrease"])
+
+
 def _residuals(prob, dtype):
     c, X = prob.cams_gt.astype(dtype), prob.pts_gt.astype(dtype)[prob.pt_idx]
     w, th2 = c[:, :3], (c[:, :3] ** 2).sum(1)
