@@ -108,8 +108,8 @@ __device__ __forceinline__ void bdecide(float a, float b, float* sh, F&& decide)
     __syncthreads();
 }
 
-// Block sums of two FP32 per-thread values, or of two compensated ones (Kahan pairs s - c),
-// broadcast to every thread.  `sh` holds 64 doubles.
+// Block sums of two FP32 per-thread values, or of two FP64 ones, broadcast to every thread.
+// `sh` holds 64 doubles.
 __device__ __forceinline__ void bsum2(float a, float b, double* sh, double& ra, double& rb) {
     bdecide(a, b, reinterpret_cast<float*>(sh), [&](double x, double y) { sh[62] = x; sh[63] = y; });
     ra = sh[62];
@@ -117,8 +117,8 @@ __device__ __forceinline__ void bsum2(float a, float b, double* sh, double& ra, 
     __syncthreads();
 }
 
-__device__ __forceinline__ void bsum2c(float sa, float ca, float sb, float cb, double* sh, double& ra, double& rb) {
-    block_sum2c(sa, ca, sb, cb, sh, ra, rb);
+__device__ __forceinline__ void bsum2d(double a, double b, double* sh, double& ra, double& rb) {
+    block_sum2d(a, b, sh, ra, rb);
     if (threadIdx.x == 0) { sh[62] = ra; sh[63] = rb; }
     __syncthreads();
     ra = sh[62];
@@ -227,7 +227,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
         const bool head = seg_reduce<BLIN>(cur, acc);
         if (head && cur != NO_CAM) b_flush_lin(b, P.c0 + cur, acc);
     }
-    float cost = 0.0f, costc = 0.0f;   // Kahan pair
+    double cost = 0.0;
     for (int i = threadIdx.x; i < P.np; i += blockDim.x) {
         const int gp = P.p0 + i;
         const float* X = b.x + P.v0 + 9 * P.nc + 3 * i;
@@ -241,7 +241,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
             const float fs = cam.f * g.s;
             const float r0 = fmaf(fs, g.p[0], -b.obs_uv[2 * (size_t)j]);
             const float r1 = fmaf(fs, g.p[1], -b.obs_uv[2 * (size_t)j + 1]);
-            kahan_add(cost, costc, fmaf(r0, r0, r1 * r1));
+            cost += widen(fmaf(r0, r0, r1 * r1));
             float jx0[3], jx1[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
@@ -262,7 +262,7 @@ __device__ double b_linearize(const BatchView& b, const Prob& P, float eps, doub
         for (int q = 0; q < 6; ++q) b.pt_H[(size_t)gp * 6 + q] = hq[q];
     }
     double F, unused;
-    bsum2c(cost, costc, 0.0f, 0.0f, sh, F, unused);   // its barriers also publish the camera sums
+    bsum2d(cost, 0.0, sh, F, unused);   // its barriers also publish the camera sums
     return 0.5 * F;
 }
 
@@ -507,7 +507,7 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
             const double denom = sj + sp;
             const bool fine = denom > 0.0 && isfinite(denom);
             step.stop = fine ? 0 : (isfinite(denom) ? 1 : 4);
-            step.a = fine ? (float)(rz * rcp64(denom)) : 0.0f;
+            step.a = fine ? (float)(rz / denom) : 0.0f;
         });
         if (step.stop) {
             if (step.stop == 4) status = 4;
@@ -585,7 +585,7 @@ __device__ int b_pcg(const BatchView& b, const Prob& P, double mu, double rz, do
             step.stop = !isfinite(rzn) || !isfinite(rrn) ? 4
                         : (rrn <= o.tol * o.tol * rr0 || k >= o.max_pcg || !(rzn > 0.0) ? 1 : 0);
             if (!step.stop) {
-                step.a = (float)(rzn * rcp64(rz));
+                step.a = (float)(rzn / rz);
                 rz = rzn;   // thread 0's; the others' is not read
             }
         });
@@ -612,18 +612,12 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
     float* xn = b.x_new + P.v0;
     const float* h = b.h + P.v0;
     const float* gv = b.g + P.v0;
-    double lgh = 0.0;                 // cameras
-    float sgh = 0.0f, cgh = 0.0f;     // points: exact products, summed as a Kahan pair
+    double lgh = 0.0;
     for (int e = tid; e < n; e += TB) {
         const float he = h[e];
         xn[e] = x[e] + he;
-        if (e < 9 * P.nc) {
-            lgh += b.cam_g[(size_t)(P.c0 + e / 9) * CL_STRIDE + e % 9] * (double)he;
-        } else {
-            const float ge = gv[e], pr = ge * he;
-            kahan_add(sgh, cgh, pr);
-            cgh -= fmaf(ge, he, -pr);
-        }
+        const double ge = e < 9 * P.nc ? b.cam_g[(size_t)(P.c0 + e / 9) * CL_STRIDE + e % 9] : widen(gv[e]);
+        lgh = fma(ge, widen(he), lgh);
     }
     __syncthreads();
     if (b.opt.retract) {   // rotations: R' = Exp(h_w) R(w)
@@ -645,7 +639,7 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         for (int q = 3; q < 9; ++q) sDir[SDIR * c + q] = hc[q];
     }
     __syncthreads();
-    float lf = 0.0f, lfc = 0.0f, ljh = 0.0f, ljhc = 0.0f;   // Kahan pairs
+    double lf = 0.0, ljh = 0.0;
     for (int64_t j = P.o0 + tid; j < P.o0 + P.no; j += TB) {
         const uint32_t key = b.obs_key[j];
         const uint32_t c = key >> 16, lp = key & 0xffffu;
@@ -653,7 +647,7 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         const Cam cn = cam_plain(b.cam_pre_new + (size_t)(P.c0 + c) * CP_STRIDE);
         float r0, r1;
         project_residual(cn, xn[e3], xn[e3 + 1], xn[e3 + 2], eps, b.obs_uv[2 * j], b.obs_uv[2 * j + 1], r0, r1);
-        kahan_add(lf, lfc, fmaf(r0, r0, r1 * r1));
+        lf += widen(fmaf(r0, r0, r1 * r1));
         const float4* r4 = reinterpret_cast<const float4*>(sCam + SCAM * c);
         const float4 c0 = r4[0], c1 = r4[1], c2 = r4[2], c3 = r4[3];
         Cam co;
@@ -677,16 +671,11 @@ __device__ void b_candidate(const BatchView& b, const Prob& P, const float* sCam
         apply_A(g, dP0, dP1, dP2, t0, t1);
         t0 = fmaf(ci, g.p[0], t0);
         t1 = fmaf(ci, g.p[1], t1);
-        kahan_add(ljh, ljhc, fmaf(t0, t0, t1 * t1));
+        ljh += widen(fmaf(t0, t0, t1 * t1));
     }
-    double fs;
-    bsum2c(lf, lfc, ljh, ljhc, sh, fs, jh2);
-    double gc = block_sum(lgh, sh), gp, none;   // in thread 0
-    block_sum2c(sgh, cgh, 0.0f, 0.0f, sh, gp, none);
-    if (tid == 0) sh[62] = gc + gp;
-    __syncthreads();
-    gh = sh[62];
-    __syncthreads();
+    double fs, unused;
+    bsum2d(lf, ljh, sh, fs, jh2);
+    bsum2d(lgh, 0.0, sh, gh, unused);
     Fn = 0.5 * fs;
 }
 

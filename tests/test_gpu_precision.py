@@ -117,6 +117,21 @@ def test_gradients_whose_squares_leave_the_fp32_range(B, pcg_kernel):
     assert abs(res.history[0]["model_decrease"] - o["model_decrease"]) <= 1e-3 * abs(o["model_decrease"])
 
 
+def test_batch_costs_beyond_the_fp32_range(B):
+    """Squared residuals of ~1e37 each are FP32 numbers; their sum is not, and the cost is an FP64
+    sum.  Terms round to FP32: 1e-6 relative."""
+    import dataclasses
+    prob = synth.round_to_f32(synth.make_problem(8, 100, ("poisson", 3.0), "uniform", seed=14))
+    scaled = synth.round_to_f32(dataclasses.replace(prob, pixels=prob.pixels * 1e16))
+    ref = [0.5 * np.sum(O.residuals(p.cams_init, p.pts_init, p.cam_idx, p.pt_idx, p.pixels) ** 2) for p in (prob, scaled)]
+    assert ref[1] > 3.5e38
+    b = B.Batch([prob, scaled])
+    b.set_params(np.concatenate([prob.cams_init] * 2), np.concatenate([prob.pts_init] * 2))
+    res = b.solve(max_lm_iters=0)
+    for r, want in zip(res, ref):
+        assert abs(r.initial_cost - want) <= 1e-6 * want
+
+
 def _residuals(prob, dtype):
     c, X = prob.cams_gt.astype(dtype), prob.pts_gt.astype(dtype)[prob.pt_idx]
     w, th2 = c[:, :3], (c[:, :3] ** 2).sum(1)
