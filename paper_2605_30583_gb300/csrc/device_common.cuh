@@ -214,9 +214,6 @@ __device__ __forceinline__ float2 warp_pair(float hi, float lo) {
 // FP32 pairs inside each warp, FP64 across warps (in the first warp alone: FP64 work that
 // every warp repeats costs 16 cycles of the SM's FP64 pipe per instruction).  Results valid in
 // thread 0.  `sh` holds 2 * (blockDim.x / 32) doubles.  Contains __syncthreads.
-// Against FP64 additions inside the warps too, the sums r^T z, |r|^2 and z^T D z of eight problems
-// (16 to 1,000 cameras, 1,000 to 200,000 points) are no further from their 64-bit values: 3.99856e-10
-// rms relative error both ways, all of it the rounding of the FP32 terms.
 __device__ __forceinline__ void block_sum2c(float sa, float ca, float sb, float cb, double* sh, double& ra,
                                             double& rb) {
     const float2 a = warp_pair(sa, -ca), b = warp_pair(sb, -cb);
@@ -241,20 +238,29 @@ __device__ __forceinline__ void block_sum2c(float sa, float ca, float sb, float 
     }
 }
 
-// A Kahan pair's sum s - c in FP64.
-__device__ __forceinline__ double pair_sum(float s, float c) { return widen(s) - widen(c); }
+// A Kahan pair's sum s - c in FP64 (c is 0 where a thread had one term: no FP64 operation then).
+__device__ __forceinline__ double pair_sum(float s, float c) {
+    return c == 0.0f ? widen(s) : widen(s) - widen(c);
+}
 
-// Block sums of two FP64 values a thread, valid in thread 0.  A warp's lanes 0 to 15 go on with the
+// Warp sums of two FP64 values a lane: a's in lane 0, b's in lane 16.  Lanes 0 to 15 go on with the
 // sums of a and the others with those of b, so that two sums take the five additions of one (each
-// holds the SM's FP64 pipe for 16 cycles).  At most 512 threads; `sh` holds 2 * (blockDim.x / 32)
-// doubles.  Contains __syncthreads.
-__device__ __forceinline__ void block_sum2d(double a, double b, double* sh, double& ra, double& rb) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    const bool second = lane >= 16;
+// holds the SM's FP64 pipe for 16 cycles).
+__device__ __forceinline__ double warp_sum2(double a, double b) {
+    const bool second = (threadIdx.x & 31) >= 16;
     double v = second ? b : a;
     v += __shfl_xor_sync(0xffffffffu, second ? a : b, 16);
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Block sums of two FP64 values a thread, valid in thread 0.  At most 512 threads; `sh` holds
+// 2 * (blockDim.x / 32) doubles.  Contains __syncthreads.
+__device__ __forceinline__ void block_sum2d(double a, double b, double* sh, double& ra, double& rb) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const bool second = lane >= 16;
+    double v = warp_sum2(a, b);
     __syncthreads();
     if ((lane & 15) == 0) sh[(second ? nw : 0) + w] = v;
     __syncthreads();

@@ -348,7 +348,6 @@ __global__ void k_precond(Views<float> v, CondHandle pcg_cond, int use_cond, ulo
 // rows of phi recompute the camera's p_w themselves.
 __global__ void k_cam_direction(Views<float> v, const int32_t* gate, const float* zs, int use_beta) {
     if (gated_off(gate)) return;
-    __shared__ double red[32];
     DevState* st = v.st;
     const int par = st->pcg_iter & 1;
     const float beta = use_beta ? (float)st->beta : 0.0f;
@@ -372,9 +371,10 @@ __global__ void k_cam_direction(Views<float> v, const int32_t* gate, const float
         }
         v.cam_dir[(size_t)c * CD_STRIDE + k] = d;   // CD_PHI = 0, CD_T = 3, CD_I = 6
     }
-    double bp, none;
-    block_sum2c(pdp, pdpc, 0.0f, 0.0f, red, bp, none);
-    if (threadIdx.x == 0) slot_add(st->acc_mv, 1, bp);
+    // a warp's sum straight to the slots: a block's would wait for two barriers and three more FP64
+    // additions (~130 cycles each) in a kernel that is one chain of latency
+    const double wp = warp_sum(pair_sum(pdp, pdpc));
+    if ((threadIdx.x & 31) == 0) slot_add(st->acc_mv, 1, wp);
 }
 
 // One PCG direction step fused with the damped normal operator, after k_cam_direction:
@@ -472,7 +472,6 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
 // block decides whether PCG continues, sets the loop flag and clears the accumulators.
 __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int cam_blocks, int cameras_only) {
     DevState* st = v.st;
-    __shared__ double red[64];
     __shared__ double sh_mv[3];   // |J p|^2, p^T D p, alpha
     __shared__ float sh_f[2];     // alpha, mu
     __shared__ bool is_last, sh_bad;
@@ -576,13 +575,10 @@ __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int 
             }
         }
     }
-    double brz, brr;
-    block_sum2c(rz, rzc, rr, rrc, red, brz, brr);
+    const double sums = warp_sum2(pair_sum(rz, rzc), pair_sum(rr, rrc));   // to the slots, as in k_cam_direction
+    if (active && !bad && (threadIdx.x & 15) == 0) slot_add(st->acc_up, (threadIdx.x & 31) >> 4, sums);
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (active && !bad) {
-            slot_add(st->acc_up, 0, brz);
-            slot_add(st->acc_up, 1, brr);
-        }
         __threadfence();
         const unsigned int t = atomicAdd(&st->tickets[TK_UPD], 1u);
         is_last = (t == gridDim.x - 1);
