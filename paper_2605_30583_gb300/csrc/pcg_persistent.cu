@@ -65,26 +65,25 @@ struct WaitLimit {
     }
 };
 
-// One published sum: a float pair, each half in a 64-bit word with the exchange's number in its
-// upper 32 bits (64-bit accesses are not torn, so a reader needs no order between the words).
-__device__ __forceinline__ void publish(ulonglong2* to, float hi, float lo, uint32_t epoch) {
+// One published FP64 sum: each half of it in a 64-bit word with the exchange's number in the upper
+// 32 bits (64-bit accesses are not torn, so a reader needs no order between the words).
+__device__ __forceinline__ void publish(ulonglong2* to, double x, uint32_t epoch) {
     const unsigned long long e = (unsigned long long)epoch << 32;
-    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(to), "l"(e | __float_as_uint(hi)),
-                 "l"(e | __float_as_uint(lo))
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(to), "l"(e | (uint32_t)__double2hiint(x)),
+                 "l"(e | (uint32_t)__double2loint(x))
                  : "memory");
 }
 
 // Waits until the sums of `n` <= MAX_PBLOCKS CTAs at `from` carry `epoch` and adds them up, in the
 // same order in every CTA; one warp, the total in every lane.  False when the wait's limit ran out.
-__device__ __forceinline__ bool gather(const ulonglong2* from, int n, uint32_t epoch, WaitLimit limit, float& hi,
-                                       float& lo) {
+__device__ __forceinline__ bool gather(const ulonglong2* from, int n, uint32_t epoch, WaitLimit limit, double& sum) {
     constexpr int PER = MAX_PBLOCKS / 32;
     const int lane = threadIdx.x & 31;
-    float h[PER], l[PER];
+    double x[PER];
     unsigned missing = 0;
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
-        h[i] = l[i] = 0.0f;
+        x[i] = 0.0;
         if (lane + 32 * i < n) missing |= 1u << i;
     }
     for (;;) {
@@ -94,8 +93,7 @@ __device__ __forceinline__ bool gather(const ulonglong2* from, int n, uint32_t e
                 unsigned long long a, b;
                 asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(from + lane + 32 * i) : "memory");
                 if ((uint32_t)(a >> 32) == epoch && (uint32_t)(b >> 32) == epoch) {
-                    h[i] = __uint_as_float((uint32_t)a);
-                    l[i] = __uint_as_float((uint32_t)b);
+                    x[i] = __hiloint2double((int)(uint32_t)a, (int)(uint32_t)b);
                     missing &= ~(1u << i);
                 }
             }
@@ -104,22 +102,15 @@ __device__ __forceinline__ bool gather(const ulonglong2* from, int n, uint32_t e
         if (lane == 0) over = limit.over() ? 1 : 0;
         if (__shfl_sync(FULL, over, 0)) return false;
     }
-    hi = lo = 0.0f;
+    // a tree over the lane's values, then over the lanes; an FP64 addition is ~130 cycles, so none
+    // for values that the grid does not have
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        float s, e;
-        two_sum(hi, h[i], s, e);
-        hi = s;
-        lo += l[i] + e;
-    }
+    for (int o = 1; o < PER; o <<= 1)
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float h2 = __shfl_xor_sync(FULL, hi, o), l2 = __shfl_xor_sync(FULL, lo, o);
-        float s, e;
-        two_sum(hi, h2, s, e);
-        hi = s;
-        lo = (lo + l2) + e;
-    }
+        for (int i = 0; i + o < PER; i += 2 * o)
+            if (32 * (i + o) < n) x[i] += x[i + o];
+    sum = x[0];
+    for (int o = 1; o < 32 && o < n; o <<= 1) sum += __shfl_xor_sync(FULL, sum, o);
     return true;
 }
 
@@ -140,7 +131,10 @@ struct PcgStep {
 // atomics, a release on a counter, the wait and the read of the slots: ~5.5 us.)  Two sets of
 // words alternate: a CTA that publishes exchange e + 2 has seen every CTA's e + 1, which each
 // published after reading all of e.  What the CTAs wrote before (camera sums) is visible after:
-// the last value's publisher and readers carry the fences.  Thread 0 calls decide(totals), which
+// the last value's publisher and readers carry the fences.  The sums are FP64 from the warps on:
+// float pairs took 0.64 us less an exchange (the solve of 16 cameras and 1,000 points 1,062 us, so
+// 1,130), but the squares of a residual can add up beyond FP32 although no warp's part does.
+// Thread 0 calls decide(totals), which
 // writes the shared step.  Call with the partials published (a barrier before); returns after
 // a barrier.
 template <int NW, typename F>
@@ -153,29 +147,22 @@ __device__ __forceinline__ void exchange(DevState* st, ulonglong2* words, uint32
     if (w < XCH_NV) {
         const bool last = w == XCH_NV - 1;
         ulonglong2* cur = words + (size_t)((epoch & 1u) * XCH_NV + w) * MAX_PBLOCKS;
-        float hi = 0.0f, lo = 0.0f;
+        double x = 0.0;
         if (lane < NW && (last || !last_only)) {
             const float2 p = red[NW * w + lane];
-            hi = p.x;
-            lo = p.y;
+            x = widen(p.x) + widen(p.y);
         }
 #pragma unroll
-        for (int o = NW / 2; o > 0; o >>= 1) {
-            const float h2 = __shfl_down_sync(FULL, hi, o), l2 = __shfl_down_sync(FULL, lo, o);
-            float s, e;
-            two_sum(hi, h2, s, e);
-            hi = s;
-            lo = (lo + l2) + e;
-        }
+        for (int o = NW / 2; o > 0; o >>= 1) x += __shfl_down_sync(FULL, x, o);
         if (lane == 0) {
             if (last) asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            publish(cur + blockIdx.x, hi, lo, epoch);
+            publish(cur + blockIdx.x, x, epoch);
         }
         __syncwarp();
-        const bool ok = gather(cur, gridDim.x, epoch, WaitLimit{&st->bar_err, st->opt.wait_ns}, hi, lo);
+        const bool ok = gather(cur, gridDim.x, epoch, WaitLimit{&st->bar_err, st->opt.wait_ns}, x);
         if (last) asm volatile("fence.acq_rel.gpu;" ::: "memory");
         if (lane == 0) {
-            s_tot[w] = widen(hi) + widen(lo);
+            s_tot[w] = x;
             s_ok[w] = ok;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * XCH_NV) : "memory");
@@ -948,6 +935,8 @@ __global__ void __launch_bounds__(TB, 1) k_pcg_persistent_1x(Views<float> v, con
                 return;
             }
             gam = g_k;
+            // alpha and beta are used in FP32: of 10^8 random quotients none differs there from
+            // the IEEE one, which takes 0.25 us longer each
             alpha = g_k * rcp64(denom);
             step.act = ACT_UPDATE;
             step.alpha = narrow(alpha);
@@ -1069,8 +1058,8 @@ __device__ ulonglong2 selftest_words[1];
 __global__ void k_selftest_wait(unsigned long long* scratch, long long timeout_ns) {
     int* err = reinterpret_cast<int*>(scratch + 1);
     if (threadIdx.x >= 32) return;
-    float hi, lo;
-    const bool ok = gather(selftest_words, 1, 1u, WaitLimit{err, timeout_ns}, hi, lo);
+    double sum;
+    const bool ok = gather(selftest_words, 1, 1u, WaitLimit{err, timeout_ns}, sum);
     if (!ok && threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned int*>(err) + 1, 1u);
 }
 

@@ -117,6 +117,36 @@ def test_gradients_whose_squares_leave_the_fp32_range(B, pcg_kernel):
     assert abs(res.history[0]["model_decrease"] - o["model_decrease"]) <= 1e-3 * abs(o["model_decrease"])
 
 
+@pytest.mark.parametrize("pcg_kernel", [0, 2])
+def test_residuals_whose_squares_add_up_beyond_fp32(B, pcg_kernel):
+    """Sixty cameras with g ~ 3e18 in k2 (a grazing point each, as above): every square is an FP32 number,
+    their sum over the grid's CTAs is not.  The exchanged totals carry it."""
+    k = 60
+    base = synth.make_problem(12, 200, ("poisson", 3.0), "uniform", seed=13)
+    centre = np.zeros((k, 3))
+    centre[:, 0] = 10.0 * np.arange(k)
+    far = np.array([300.0, 0.0, 700.0])
+    cams = np.zeros((k + 1, 9))
+    cams[:k, 3:6], cams[k, 3:6], cams[:, 6] = -centre, -far, 1000.0
+    cams = np.concatenate([base.cams_init, cams]).astype(np.float32).astype(np.float64)
+    pts = np.concatenate([base.pts_init, centre + (1.0, 0.3, -1e-3)]).astype(np.float32).astype(np.float64)
+    i = np.arange(k)
+    ci = np.concatenate([base.cam_idx, 12 + i, np.full(k, 12 + k)]).astype(np.uint32)
+    pi = np.concatenate([base.pt_idx, 200 + i, 200 + i]).astype(np.uint32)
+    px = np.concatenate([base.pixels, O.residuals(cams, pts, ci, pi, np.zeros((len(ci), 2)))[len(base.pixels):]])
+    px[len(base.pixels):len(base.pixels) + k, 0] += 2.5
+    px = px.astype(np.float32).astype(np.float64)
+    g = O.linearize(cams, pts, ci, pi, px).g
+    assert np.abs(g).max() < 1e19 and np.sum(g**2) > 3.5e38
+    opts = dict(max_lm_iters=1, max_pcg_iters=1)
+    p = B.Problem(len(cams), len(pts), ci, pi, px)
+    p.set_params(cams, pts)
+    res = p.solve(pcg_kernel=pcg_kernel, **opts)
+    o = O.ba_solve(cams, pts, ci, pi, px, O.LMOptions(**opts)).history[0]
+    assert res.accepted == 1 and o["accepted"] and res.history[0]["pcg_iters"] == 1
+    assert abs(res.history[0]["model_decrease"] - o["model_decrease"]) <= 1e-3 * abs(o["model_decrease"])
+
+
 def test_batch_costs_beyond_the_fp32_range(B):
     """Squared residuals of ~1e37 each are FP32 numbers; their sum is not, and the cost is an FP64
     sum.  Terms round to FP32: 1e-6 relative."""
