@@ -807,8 +807,10 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
     p->fits_one = fits(PCG_ONE_EXCHANGE, worst_one);
     p->fits_two = fits(PCG_TWO_EXCHANGE, worst_two);
     if (!p->fits_one && !p->fits_two) return BA_OK;
-    GBBA_CUDA(cudaMemcpy(p->blk_cam_off, coff.data(), 4 * coff.size(), cudaMemcpyHostToDevice));
-    GBBA_CUDA(cudaMemcpy(p->blk_cams, cams.data(), 4 * cams.size(), cudaMemcpyHostToDevice));
+    // on the bound stream: a cudaMemcpy of pageable memory may return before its transfer has ended,
+    // and a non-blocking stream does not wait for it
+    GBBA_CUDA(cudaMemcpyAsync(p->blk_cam_off, coff.data(), 4 * coff.size(), cudaMemcpyHostToDevice, p->stream));
+    GBBA_CUDA(cudaMemcpyAsync(p->blk_cams, cams.data(), 4 * cams.size(), cudaMemcpyHostToDevice, p->stream));
     // the factors in the order of their CTAs
     std::vector<uint32_t> foff((size_t)G + 1, 0), fcam;
     std::vector<double> fmeas, fsqrt;
@@ -820,11 +822,11 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
         }
         foff[b + 1] = foff[b] + (uint32_t)fac_of[b].size();
     }
-    GBBA_CUDA(cudaMemcpy(p->blk_fac, foff.data(), 4 * foff.size(), cudaMemcpyHostToDevice));
+    GBBA_CUDA(cudaMemcpyAsync(p->blk_fac, foff.data(), 4 * foff.size(), cudaMemcpyHostToDevice, p->stream));
     if (p->n_fac > 0) {
-        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_cam, fcam.data(), 4 * fcam.size(), cudaMemcpyHostToDevice));
-        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_meas, fmeas.data(), 8 * fmeas.size(), cudaMemcpyHostToDevice));
-        GBBA_CUDA(cudaMemcpy(p->ws + p->lay.fac_sqrt, fsqrt.data(), 8 * fsqrt.size(), cudaMemcpyHostToDevice));
+        GBBA_CUDA(cudaMemcpyAsync(p->ws + p->lay.fac_cam, fcam.data(), 4 * fcam.size(), cudaMemcpyHostToDevice, p->stream));
+        GBBA_CUDA(cudaMemcpyAsync(p->ws + p->lay.fac_meas, fmeas.data(), 8 * fmeas.size(), cudaMemcpyHostToDevice, p->stream));
+        GBBA_CUDA(cudaMemcpyAsync(p->ws + p->lay.fac_sqrt, fsqrt.data(), 8 * fsqrt.size(), cudaMemcpyHostToDevice, p->stream));
     }
     p->persistent = true;
     p->p_grid = G;
