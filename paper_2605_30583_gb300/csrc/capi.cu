@@ -9,6 +9,7 @@
 #include <cstring>
 #include <iterator>
 #include <new>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -528,7 +529,13 @@ ObsCheck check_and_copy_observations(int32_t n_cams, int32_t n_pts, int64_t n_ob
     };
     auto run = [&](auto&& f) {
         std::vector<std::thread> th;
-        for (int t = 1; t < nt; ++t) th.emplace_back(f, t);
+        th.reserve((size_t)nt);
+        int t = 1;
+        try {
+            for (; t < nt; ++t) th.emplace_back(f, t);
+        } catch (const std::system_error&) {   // no more threads to be had: the rest runs here
+        }
+        for (; t < nt; ++t) f(t);
         f(0);
         for (auto& x : th) x.join();
     };
@@ -590,8 +597,15 @@ ba_status ba_problem_create(int32_t n_cams, int32_t n_pts, int64_t n_obs, const 
         set_error("ba_problem_create: out of host memory");
         return BA_ERR_INVALID_ARG;
     }
-    const ObsCheck chk = check_and_copy_observations(n_cams, n_pts, n_obs, cam_idx, pt_idx, pixels, p->cam_idx.data(),
-                                                     p->pt_idx.data(), p->pixels.data());
+    ObsCheck chk;
+    try {
+        chk = check_and_copy_observations(n_cams, n_pts, n_obs, cam_idx, pt_idx, pixels, p->cam_idx.data(),
+                                          p->pt_idx.data(), p->pixels.data());
+    } catch (...) {
+        delete p;
+        set_error("ba_problem_create: out of host memory");
+        return BA_ERR_INVALID_ARG;
+    }
     if (chk.bad_obs >= 0 || chk.bad_pt >= 0) {
         if (chk.bad_obs >= 0 && chk.range)
             set_error("ba_problem_create: observation %lld has camera %u / point %u out of range",
@@ -836,6 +850,27 @@ static ba_status plan_persistent(ba_problem* p, int sms) {
     return BA_OK;
 }
 
+// The mixed form's plans: the persistent PCG's, and the tile kernels' tables for the largest tile.
+static ba_status plan_kernels(ba_problem* p, int sms, bool plain_q) {
+    ba_status pst = plan_persistent(p, sms);
+    if (pst) return pst;
+    const size_t nt = (size_t)p->n_tiles;
+    std::vector<uint32_t> toff(nt + 1), loff(nt + 1), sst(nt);
+    GBBA_CUDA(cudaMemcpy(toff.data(), p->vf.tile_off, 4 * toff.size(), cudaMemcpyDeviceToHost));
+    GBBA_CUDA(cudaMemcpy(loff.data(), p->vf.long_off, 4 * loff.size(), cudaMemcpyDeviceToHost));
+    GBBA_CUDA(cudaMemcpy(sst.data(), p->vf.short_start, 4 * sst.size(), cudaMemcpyDeviceToHost));
+    uint32_t most_long = 1, most_short = 1, most_runs = 1;
+    for (size_t t = 0; t < nt; ++t) {
+        most_long = std::max(most_long, sst[t] - toff[t]);
+        most_short = std::max(most_short, toff[t + 1] - sst[t]);
+        most_runs = std::max(most_runs, loff[t + 1] - loff[t]);
+    }
+    plan_tile_kernels(p->L, p->n_tiles, sms, (int)most_long, (int)most_short, (int)most_runs);
+    p->L.tn_plain_q = plain_q;
+    GBBA_CUDA(cudaGetLastError());
+    return BA_OK;
+}
+
 ba_status ba_bind_workspace(ba_problem* p, void* ws, size_t bytes, void* stream) {
     if (!p || !ws) {
         set_error("ba_bind_workspace: null pointer");
@@ -922,22 +957,14 @@ ba_status ba_bind_workspace(ba_problem* p, void* ws, size_t bytes, void* stream)
     p->xch = (ulonglong2*)(w + l.xch);
     p->persistent = p->fits_one = p->fits_two = false;
     if (p->precision == BA_PREC_MIXED) {
-        ba_status pst = plan_persistent(p, sms);
-        if (pst) return pst;
-        const size_t nt = (size_t)p->n_tiles;
-        std::vector<uint32_t> toff(nt + 1), loff(nt + 1), sst(nt);
-        GBBA_CUDA(cudaMemcpy(toff.data(), p->vf.tile_off, 4 * toff.size(), cudaMemcpyDeviceToHost));
-        GBBA_CUDA(cudaMemcpy(loff.data(), p->vf.long_off, 4 * loff.size(), cudaMemcpyDeviceToHost));
-        GBBA_CUDA(cudaMemcpy(sst.data(), p->vf.short_start, 4 * sst.size(), cudaMemcpyDeviceToHost));
-        uint32_t most_long = 1, most_short = 1, most_runs = 1;
-        for (size_t t = 0; t < nt; ++t) {
-            most_long = std::max(most_long, sst[t] - toff[t]);
-            most_short = std::max(most_short, toff[t + 1] - sst[t]);
-            most_runs = std::max(most_runs, loff[t + 1] - loff[t]);
+        ba_status pst;
+        try {
+            pst = plan_kernels(p, sms, repeated == 0u);
+        } catch (const std::bad_alloc&) {
+            set_error("ba_bind_workspace: out of host memory");
+            pst = BA_ERR_INVALID_ARG;
         }
-        plan_tile_kernels(p->L, p->n_tiles, sms, (int)most_long, (int)most_short, (int)most_runs);
-        p->L.tn_plain_q = repeated == 0u;
-        GBBA_CUDA(cudaGetLastError());
+        if (pst) return pst;
     }
     p->bound = true;
     return BA_OK;
