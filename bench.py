@@ -194,16 +194,19 @@ def operator_model(prob):
     return nb, 120 * prob.n_obs
 
 
-def pcg_iter_tile_model(prob):
+def pcg_iter_tile_model(prob, deferred_h=False):
     """Algorithmic bytes of one PCG iteration of the separate-kernel form (operator with
     the point direction step p = z + beta p fused in, then k_update).
 
     Per point: z, p_prev, D, X read and p, q written by the operator (6 x 12 B); p, h, r,
     q read and h, r, z written by the update (7 x 12 B); its M^-1 block (24 B): 180 B.
+    deferred_h: as the kernels do it, with the points' h += alpha p taken by the next
+    operator, which reads p anyway (h read and written there, 8 x 12 B; the update reads r, q
+    and writes r, z, 4 x 12 B): 168 B.
     Per observation its key (4 B).  Per camera the operator's 364 B plus the update's
     (p, h, r, D and the accumulator read, h, r, z, p written: 9 x 36 B; M^-1 324 B; J_l
     36 B): 1,048 B."""
-    return 4 * prob.n_obs + 180 * prob.n_pts + 1048 * prob.n_cams
+    return 4 * prob.n_obs + (168 if deferred_h else 180) * prob.n_pts + 1048 * prob.n_cams
 
 
 def lm_iter_model(prob):
@@ -559,7 +562,7 @@ def run_ours(args, rank, world, local_rank):
     roofline = roof_pp if roof_pp is not None else roof_op
     # the separate-kernel PCG iteration as a whole (operator + update) against its bytes
     pcg_us = kernel_us["matvec"] + kernel_us["update"]
-    pcg_bytes = pcg_iter_tile_model(prob)
+    pcg_bytes = pcg_iter_tile_model(prob, deferred_h=True)
     roof_iter = {"us_per_pcg_iter": pcg_us, "algorithmic_bytes": pcg_bytes,
                  "achieved": pcg_bytes / (pcg_us / 1e6) / 1e9, "frac": pcg_bytes / (pcg_us / 1e6) / 1e9 / hbm_peak,
                  "unit": "GB/s", "kernels": "k_cam_direction + k_tile_normal + k_update (isolated launches)",

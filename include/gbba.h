@@ -289,8 +289,10 @@ ba_status ba_repeat_normal(ba_problem* problem, int32_t launches);
  * `reps` launches each (after one warm-up launch), every launch timed alone with its
  * gates opened just before it, after a prior ba_evaluate or ba_solve.  Writes
  * the average microseconds per launch into us_out[0..n) in this order: camera
- * records, linearisation, preconditioner, normal operator (matvec), PCG update,
- * candidate step, candidate evaluation, commit; then [8] one launch of the persistent
+ * records, linearisation, preconditioner, normal operator (matvec, with the direction
+ * step and the points' step of the last update, as in an iteration past the first), PCG
+ * update, candidate step, candidate evaluation (with the residual pass where both run in one
+ * launch: at most two tiles per SM), commit; then [8] one launch of the persistent
  * PCG kernel (a whole PCG solve capped at 50 iterations with zero tolerance, each
  * launch after a preconditioner launch that resets its state, events around the PCG
  * launch alone) and [9] the PCG iterations that launch ran; -1 and 0 there when the

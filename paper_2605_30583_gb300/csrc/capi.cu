@@ -1365,7 +1365,15 @@ ba_status ba_profile_kernels(ba_problem* p, int32_t reps, double* us, int32_t n)
     out[0] = timeit([&] { launch_camera_precompute(v, p->L, s); });
     out[1] = timeit([&] { launch_linearize(v, p->L, s, 1, nullptr, nullptr, 0, 0); });
     out[2] = timeit([&] { launch_precond(v, p->L, s, 0, 0, nullptr, 0); });
-    out[3] = timeit([&] { launch_matvec(v, p->L, s, nullptr, v.z, 1); });
+    {
+        // an iteration past the first: the direction and the points' step of the last update are
+        // taken on the way (beta and h_alpha not 0)
+        const double beta = 0.5;
+        const float h_alpha = 1e-6f;
+        GBBA_CUDA(cudaMemcpyAsync(&v.st->beta, &beta, sizeof(beta), cudaMemcpyHostToDevice, s));
+        GBBA_CUDA(cudaMemcpyAsync(&v.st->h_alpha, &h_alpha, sizeof(h_alpha), cudaMemcpyHostToDevice, s));
+        out[3] = timeit([&] { launch_matvec(v, p->L, s, nullptr, v.z, 1); });
+    }
     {
         // the update skips its work once the operator sums it consumes are cleared, so
         // each timed launch follows a re-armed |J p|^2 slot and is timed alone
