@@ -191,6 +191,12 @@ ba_status ba_selftest_wait_timeout(void* scratch, int32_t grid, int32_t timeout_
  * Zero, non-finite and |x| outside [1e-300, 1e300] take the IEEE quotient 1.0 / x. */
 ba_status ba_selftest_rcp64(const double* x, double* y, int64_t n, void* stream);
 
+/* Self-test of the FP32 / FP64 conversions that the kernels do with integer instructions:
+ * wide[i] = (double)x32[i] and narrowed[i] = (float)x64[i] (round to nearest even) for i < n, device
+ * arrays of n >= 1 entries, enqueued on `stream` (cudaStream_t). */
+ba_status ba_selftest_conversions(const float* x32, double* wide, const double* x64, float* narrowed, int64_t n,
+                                  void* stream);
+
 /* Fills *opts with the defaults listed at ba_options. */
 ba_status ba_options_default(ba_options* opts);
 

@@ -72,6 +72,7 @@ SIGNATURES = {
     "ba_set_pose_factors": (I32, [P, I32, P, P, P, P]),
     "ba_selftest_wait_timeout": (I32, [P, I32, I32, P, ctypes.POINTER(I32), ctypes.POINTER(I32)]),
     "ba_selftest_rcp64": (I32, [P, P, I64, P]),
+    "ba_selftest_conversions": (I32, [P, P, P, P, I64, P]),
     "ba_bind_workspace": (I32, [P, P, SZ, P]),
     "ba_set_params": (I32, [P, P, P]),
     "ba_get_params": (I32, [P, P, P]),
@@ -150,6 +151,19 @@ def selftest_rcp64(x):
     y = torch.empty_like(x)
     check(lib().ba_selftest_rcp64(x.data_ptr(), y.data_ptr(), x.numel(), torch.cuda.current_stream().cuda_stream))
     return y
+
+
+def selftest_conversions(x32, x64):
+    """(x32 as float64, x64 as float32) through the kernels' integer conversions
+    (ba_selftest_conversions) for CUDA tensors of one length; returns new tensors."""
+    torch = _torch()
+    x32, x64 = x32.contiguous(), x64.contiguous()
+    assert x32.is_cuda and x32.dtype == torch.float32 and x64.is_cuda and x64.dtype == torch.float64
+    assert x32.numel() == x64.numel()
+    wide, narrowed = torch.empty_like(x32, dtype=torch.float64), torch.empty_like(x64, dtype=torch.float32)
+    check(lib().ba_selftest_conversions(x32.data_ptr(), wide.data_ptr(), x64.data_ptr(), narrowed.data_ptr(), x32.numel(),
+                                        torch.cuda.current_stream().cuda_stream))
+    return wide, narrowed
 
 
 def default_options(**kw) -> Options:

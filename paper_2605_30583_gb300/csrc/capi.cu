@@ -438,6 +438,17 @@ ba_status ba_selftest_rcp64(const double* x, double* y, int64_t n, void* stream)
     return BA_OK;
 }
 
+ba_status ba_selftest_conversions(const float* x32, double* wide, const double* x64, float* narrowed, int64_t n,
+                                  void* stream) {
+    if (!x32 || !wide || !x64 || !narrowed || n < 1) {
+        set_error("ba_selftest_conversions: null pointer or n < 1");
+        return BA_ERR_INVALID_ARG;
+    }
+    launch_selftest_conversions(x32, wide, x64, narrowed, n, (cudaStream_t)stream);
+    GBBA_CUDA(cudaGetLastError());
+    return BA_OK;
+}
+
 ba_status ba_options_default(ba_options* o) {
     if (!o) {
         set_error("ba_options_default: null pointer");

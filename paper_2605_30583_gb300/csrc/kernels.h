@@ -109,6 +109,8 @@ constexpr uint32_t BLK_CAM_OWNER = 0x80000000u;
 int persistent_max_smem();
 // Self-test of the FP64 reciprocal of the block inversions: y[i] = rcp64(x[i]).
 void launch_selftest_rcp64(const double* x, double* y, int64_t n, cudaStream_t s);
+void launch_selftest_conversions(const float* x32, double* wide, const double* x64, float* narrowed, int64_t n,
+                                 cudaStream_t s);
 // Self-test of the bounded grid wait (16 bytes of device scratch).
 cudaError_t launch_selftest_wait(void* scratch, int grid, long long timeout_ns, cudaStream_t s);
 cudaError_t persistent_prepare(int form, int smem_bytes, int* blocks_per_sm);

@@ -1073,6 +1073,20 @@ void launch_selftest_rcp64(const double* x, double* y, int64_t n, cudaStream_t s
     k_selftest_rcp64<<<(unsigned int)(b < 1024 ? b : 1024), 256, 0, s>>>(x, y, n);
 }
 
+__global__ void k_selftest_conversions(const float* __restrict__ x32, double* __restrict__ wide,
+                                       const double* __restrict__ x64, float* __restrict__ narrowed, int64_t n) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        wide[i] = widen(x32[i]);
+        narrowed[i] = narrow(x64[i]);
+    }
+}
+
+void launch_selftest_conversions(const float* x32, double* wide, const double* x64, float* narrowed, int64_t n,
+                                 cudaStream_t s) {
+    const int64_t b = (n + 255) / 256;
+    k_selftest_conversions<<<(unsigned int)(b < 1024 ? b : 1024), 256, 0, s>>>(x32, wide, x64, narrowed, n);
+}
+
 cudaError_t launch_selftest_wait(void* scratch, int grid, long long timeout_ns, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
