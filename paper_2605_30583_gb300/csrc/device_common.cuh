@@ -21,12 +21,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__device__ __forceinline__ float warp_sumf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // Sum of v over the block, in a fixed order; valid in thread 0.  `sh` holds at
 // least blockDim.x / 32 doubles.  Contains __syncthreads.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -181,22 +175,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // Warp sum of per-lane compensated values hi + lo in FP32 pairs: every level adds the
 // partner's high parts with TwoSum and carries the rounding error into the low parts,
 // so the result has about twice FP32's precision (FP64 shuffles cost ~67x more on this
-// GPU).  Result valid in lane 0 as a double.
-__device__ __forceinline__ double warp_sum_pair(float hi, float lo) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h2 = __shfl_down_sync(0xffffffffu, hi, o);
-        const float l2 = __shfl_down_sync(0xffffffffu, lo, o);
-        float s, e;
-        two_sum(hi, h2, s, e);
-        hi = s;
-        lo = lo + l2 + e;
-    }
-    return (double)hi + (double)lo;
-}
-
-// Compensated warp sum of per-lane values hi + lo as a pair (warp_sum_pair without its FP64
-// finish), valid in lane 0.
+// GPU).  A pair, valid in lane 0.
 __device__ __forceinline__ float2 warp_pair(float hi, float lo) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

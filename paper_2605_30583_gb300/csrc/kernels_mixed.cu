@@ -8,7 +8,7 @@
 // point: on this hardware the ~100 FP32 operations per observation cost less than
 // streaming 96 bytes of stored Jacobian per observation from HBM.
 //
-// Work decomposition: a tile is TILE_PTS consecutive points (locality order) and all
+// Work decomposition: a tile is up to TILE_PTS consecutive points (locality order) and all
 // their observations, sorted by camera inside the tile.  One CTA handles a tile;
 // each thread takes a contiguous chunk of the tile's observations, keeps the camera
 // sums of the current camera run in registers, and at the end of its chunk a
@@ -212,7 +212,8 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 
 // ------------------------------------------------------------------ K3 --------
 // Block-Jacobi preconditioner (Sec. V: one block per node) of J^T J + mu D, inverted
-// by FP64 Cholesky, and the start of PCGNR: h = 0, r = -g, z = M^-1 r, p = 0.
+// in FP64 (camera blocks by Gauss-Jordan elimination, point blocks by the adjugate), and the
+// start of PCGNR: h = 0, r = -g, z = M^-1 r, p = 0.
 // Camera c of an item kernel runs in lane c % 32 of warp 0 of block (c / 32) % gridDim:
 // 32 cameras share every warp instruction (the FP64 pipe takes whole warps, so a warp
 // with one busy lane costs as much as a full one) and the cameras spread over the SMs.

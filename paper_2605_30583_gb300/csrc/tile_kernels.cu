@@ -1,8 +1,8 @@
 // Tile kernels of the mixed-precision form: the damped normal operator of the
 // separate-kernel PCG, the linearisation and the candidate evaluation.
 //
-// Work decomposition.  A tile is TILE_PTS consecutive points (locality order) and all
-// their observations.  Inside a tile each camera's observations form one run, and the
+// Work decomposition.  A tile is tile_points(n_pts) <= TILE_PTS consecutive points (locality
+// order) and all their observations.  Inside a tile each camera's observations form one run, and the
 // runs of at least LONG_RUN observations come first (order.cu); on the large workloads
 // they hold most of the observations.  A CTA stages in shared memory, in one round
 // trip, the tile's points, its compact observation table (a one-byte point slot per long-run
@@ -132,14 +132,6 @@ __device__ __forceinline__ void stage_compact(const Views<float>& v, const TileR
 // Brings [p, p + bytes) into the L2 (16-byte aligned, a multiple of 16 bytes).
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// Block sums of compensated per-thread partials (Kahan pairs s - c): FP32 pairs inside
-// each warp, FP64 across the warps; valid in thread 0.  `sh` holds 2 * (TB / 32) doubles.
-template <int TB>
-__device__ __forceinline__ void block_pair_sums(float sa, float ca, float sb, float cb, double* sh, double& ra,
-                                                double& rb) {
-    block_sum2c(sa, ca, sb, cb, sh, ra, rb);
 }
 
 // The normal operator over a tile's observations (points and directions staged in sX4, sP4):
@@ -301,7 +293,7 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
                 const int slot = 4 * g / 3, k = 4 * g - 3 * slot;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {   // entry (slot, k + q) in rows of four floats
-                    const int o = 4 * slot + k + q + (k + q >= 3 ? 1 : 0) + (k + q >= 6 ? 1 : 0);
+                    const int o = 4 * slot + k + q + (k + q >= 3 ? 1 : 0);   // k + q <= 5
                     sPf[o] = pk[q];
                     sXf[o] = xk[q];
                 }
@@ -338,7 +330,7 @@ __global__ void __launch_bounds__(TB, 8) k_tile_normal(Views<float> v, const int
         *reinterpret_cast<float4*>(v.q + T.base + 4 * (size_t)i) = qi;
     }
     double bj, bp;
-    block_pair_sums<TB>(jp_s, jp_c, pd_s, pd_c, red, bj, bp);
+    block_sum2c(jp_s, jp_c, pd_s, pd_c, red, bj, bp);
     if (threadIdx.x == 0) {
         slot_add(st->acc_mv, 0, bj);
         slot_add(st->acc_mv, 1, bp);
@@ -939,7 +931,7 @@ __global__ void __launch_bounds__(TB, 6) k_tile_eval(Views<float> v, CondHandle 
 
 // Few tiles: the residual pass at x' and the evaluation of |J h|^2 in one launch (both are bound by
 // latency there, and neither needs the other): blocks below n_tiles take a tile's residuals, the
-// others a tile's |J h|^2.  1,000 points: 18 + 14 -> 14 us and a launch less.
+// others a tile's |J h|^2.  1,000 points: 18 + 14 -> 15 us and a launch less.
 template <int TB>
 __global__ void __launch_bounds__(TB, 1) k_tile_step(Views<float> v, CondHandle lm_cond, int use_cond, Caps cap) {
     extern __shared__ __align__(16) unsigned char dsm[];
