@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(TB, 8) k_matvec(Views<float> v, const int32_t*
 // Blocks [0, cam_blocks) take the cameras, nine lanes each and three to a warp: a camera's sums, r
 // and z travel by shuffles, so its update is one round of loads (a thread per camera, with its 81
 // preconditioner entries one after the other, took ~8 us of this kernel whatever the size).  102 ->
-// 68 us on 4.5M points with the points' h left to the operator; the bytes take 48.  The
+// 69 us on 4.5M points with the points' h left to the operator; the bytes take 48.  The
 // other blocks take the points, four at a time with float4 accesses.  Never gated: its last
 // block decides whether PCG continues, sets the loop flag and clears the accumulators.
 __global__ void k_update(Views<float> v, CondHandle pcg_cond, int use_cond, int cam_blocks, int cameras_only) {

@@ -595,8 +595,9 @@ constexpr int TL_TB = 128;
 // Few tiles: a tile's runs spread over the warps of 512 threads.  The linearisation does so up to
 // one tile per SM (16 tiles: 18.0 -> 13.8 us; 298 tiles 22.9 against 23.6, 302 tiles 23.3 against
 // 25.8, 910 tiles 43.7 against 61.9), the candidate's residuals and evaluation in one launch
-// (k_tile_step) up to two (against both launches: 25.3 -> 15.0 us, 31.8 -> 30.6, 32.5 -> 32.5 and
-// a launch gap of 2 us each; 910 tiles 45.8 against 77.7).
+// (k_tile_step) up to two (both launches against the one: 16 tiles 25.4 and 14.4 us, 152 tiles 32.5
+// and 23.2, 298 tiles 32.4 and 34.7, 302 tiles 35.3 and 37.2, where it saves a launch gap of 2 us
+// each; 910 tiles 45.8 and 77.7 in an earlier form).
 constexpr int WIDE_LIN_TILES = 1;
 constexpr int WIDE_TILES = 2;
 constexpr int WIDE_TB = 512;
