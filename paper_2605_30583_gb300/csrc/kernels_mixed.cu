@@ -51,11 +51,11 @@ __global__ void k_camera_precompute(Views<float> v) {
 
 // ------------------------------------------------------------------ K1 --------
 // Linearisation (fused score + Jacobian products, Sec. V-A): cost F = 1/2 |r|^2,
-// g = J^T r and the diagonal blocks J_c^T J_c, J_p^T J_p.  Two passes per tile:
-//   camera pass: the tile's camera-sorted observations, camera sums in registers,
-//     one set of atomics per camera run (g in FP64, J_c^T J_c in FP32 float4 atomics);
-//   point pass: one thread per point over its observations (point-major index), point
-//     sums in registers, no atomics; it also sums the cost.
+// g = J^T r and the diagonal blocks J_c^T J_c, J_p^T J_p, for problems whose tiles' tables do not
+// fit in shared memory (else k_tile_linearize).  One pass over the tile's camera-sorted
+// observations: camera sums in registers, one set of atomics per camera run (g in FP64,
+// J_c^T J_c in FP32 float4 atomics), point sums in shared memory; r and the cost come from
+// k_residual.
 // `mode`: 0 = first linearisation of a solve (initialises the LM state), 1 =
 // relinearisation after an accepted step (gated by st->relin), 2 = evaluation only
 // (optional r and J output in the caller's observation order).
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(TB, 6) k_linearize(Views<float> v, int mode, f
 // invert the point blocks (a thread per point), so the long FP64 camera eliminations run
 // beside the point work instead of before it in the same warps.
 //
-// Bound by the FP64 pipe (31 operations a point, ~50 a camera's share of a warp):
+// Bound by the FP64 pipe (30 operations a point, ~46 a camera's share of a warp):
 // 687 -> 540 us on 13,000 cameras and 4.5M points with integer conversions, one reciprocal a
 // point and three cameras a warp.  r^T z and |r|^2 are summed in FP64 (as FP32 pairs: 37 us less,
 // but a camera's g of 2e19 and more squares to infinity there).  h is always cleared: a PCG that runs no

@@ -138,7 +138,7 @@ __device__ __forceinline__ void store_residual(float* out, float r0, float r1) {
 // the diagonal where A is not positive definite.  lo_f, hi_f: the bounds as floats on the inner
 // side, so that h >= lo exactly when h >= lo_f.  Writes M (packed) and D in FP32.  FP64 runs
 // at 1/64 of the FP32 rate here (a warp instruction holds the SM's FP64 pipe for 16 cycles):
-// only the 29 instructions of the inverse itself are FP64; clamping, comparisons and
+// only the 28 instructions of the inverse itself are FP64; clamping, comparisons and
 // conversions run on the integer and FP32 units (the 28.8M-observation workload's
 // preconditioner took 688 us with them in FP64).
 __device__ __forceinline__ void point_inverse(const float (&H)[6], double mu, double lo, double hi, float lo_f,

@@ -12,15 +12,14 @@
 //
 // Two forms of the same Krylov iteration:
 //
-// k_pcg_persistent (the default form): the textbook recurrences, two
-// exchanges per iteration:
+// k_pcg_persistent (pcg_kernel 0): the textbook recurrences, two exchanges per iteration:
 //   A  p = z + beta p (points in smem; cameras double-buffered in global), then
 //      q = J^T J p + mu D p with |J p|^2 and p^T D p;            -> exchange
 //   B  alpha = r^T z / (|J p|^2 + mu p^T D p); h += alpha p; r -= alpha q; z = M^-1 r;
 //      r^T z, |r|^2                                              -> exchange
 //   C  stop test (|r| <= tol |r_0| or the iteration cap), beta.
 //
-// k_pcg_persistent_1x: one exchange per iteration.  The recurrences are arranged as in
+// k_pcg_persistent_1x (the default): one exchange per iteration.  The recurrences are arranged as in
 // the CG of Chronopoulos and Gear (J. Comput. Appl. Math. 25, 1989): with u = M^-1 r,
 // w = A u and s = A p carried by s = w + beta s,
 //   gamma = r^T u,  delta = u^T A u = |J u|^2 + mu u^T D u,
