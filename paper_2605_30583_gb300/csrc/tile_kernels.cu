@@ -1127,7 +1127,6 @@ __global__ void __launch_bounds__(TB) k_tile_schur(Views<float> v, const int32_t
     __shared__ float4 sX4[TILE_PTS], sZ4[TILE_PTS];
     __shared__ float sY[NW * 3 * TILE_PTS];
     __shared__ unsigned int s_next[2];
-    __shared__ double red[2 * NW];
     DevState* st = v.st;
     const float eps = (float)st->opt.eps;
     const bool weighted = st->opt.loss != 0;
@@ -1135,10 +1134,9 @@ __global__ void __launch_bounds__(TB) k_tile_schur(Views<float> v, const int32_t
     float ts = 0.0f, tc = 0.0f;   // Kahan pair
     if (weighted || eps != 0.0f) tile_schur<TB, MODE, true>(v, T, cap, dsm, sX4, sY, sZ4, s_next, eps, weighted, ts, tc);
     else tile_schur<TB, MODE, false>(v, T, cap, dsm, sX4, sY, sZ4, s_next, eps, weighted, ts, tc);
-    if (MODE == SCHUR_MV) {
-        double b, none;
-        block_sum2c(ts, tc, 0.0f, 0.0f, red, b, none);
-        if (threadIdx.x == 0) slot_add(st->acc_mv, 0, b);
+    if (MODE == SCHUR_MV) {   // FP64, a warp's sum straight to the slots (as k_cam_direction)
+        const double w = warp_sum(pair_sum(ts, tc));
+        if ((threadIdx.x & 31) == 0) slot_add(st->acc_mv, 0, w);
     }
 }
 
